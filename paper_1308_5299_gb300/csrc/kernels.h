@@ -8,6 +8,13 @@
 
 namespace cr {
 
+// Tables of the digit-slice kernels (legendre_ds.cu), position ds_off(Lc, m) + k
+struct DsTab {
+  double *A = nullptr, *B = nullptr, *AB = nullptr;    // coefficients of the step that produces q_k
+  double *sg = nullptr, *e0 = nullptr, *e1 = nullptr;  // sigma_k, and times e_o and e_{o+1}
+  int Lc = -1;
+};
+
 template <typename T>
 struct LegArgs {
   const typename Tr<T>::C* alm = nullptr;  // synthesis input, layout off_m(L)
@@ -36,6 +43,26 @@ struct LegArgs {
   int mt_synth = 1, mt_adj = 1;            // m tile: 1 (one m per CTA) or 2 (m and L - m per CTA)
   int tc_variant = 0;                      // tensor-core kernels: stage shape (legendre_tc.cu)
   int tc_split = 0;                        // tensor-core kernels: hi + lo BF16 operands
+  const DsTab* ds = nullptr;               // FP64: tables of the digit-slice kernels (null: not used)
+  int nis = 0;                             // pairs [0, nis) with z above their equatorial zone
+};
+
+// Arguments of the digit-slice kernels.
+struct DsArgs {
+  DsTab t;
+  const double2* alm = nullptr;   // [nr][ld_alm]
+  int64_t ld_alm = 0;
+  double2* phase = nullptr;       // [nr][nring][ldp]
+  int64_t ld_phase = 0, ldp = 0;
+  double* partial = nullptr;      // adjoint: [nr][nblk][nkk][4]
+  int64_t nkk = 0;
+  int nblk = 0;                   // tiles of ring pairs
+  int L = 0, Lc = 0, nr = 1;
+  const double *c = nullptr, *s = nullptr, *dl = nullptr, *z = nullptr;
+  const int* ls = nullptr;
+  const double2* st = nullptr;
+  int ld_seed = 0, npairs = 0, nring = 0;
+  int nis = 0, nt_is = 0;         // pairs and tiles of the two-step sequence
 };
 
 template <typename T>
@@ -116,6 +143,16 @@ int launch_leg_adjoint_mr(const LegArgs<double>& a, const double2* phase, int64_
 int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, double2* y, const double* dl_in,
                    const double* pix, const double* dl_out, const double* dadd, const double2* bsub);
 int ensure_mr_workspace(cr_plan* P, const Grid& g, int L);
+// FP64 stages by digit slices on the tensor cores (legendre_ds.cu)
+int ds_tab_build(DsTab& t, int Lc, cudaStream_t st);
+void ds_tab_free(DsTab& t);
+int ds_first_equatorial(const double* z, int npairs);
+int64_t ds_partial_bytes(int nis, int npairs, int L, int nr);
+bool ds_use(const LegArgs<double>& a);
+int launch_ds_synth(const LegArgs<double>& la, const double2* alm, int64_t ld_alm, int nr, double2* phase,
+                    cudaStream_t st);
+int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, double* partial,
+                      const FinalizeArgs<double>* f, cudaStream_t st);
 int launch_leg_diag(cr_plan* P, const double* ringval, double2* out);
 template <typename T> int launch_ring_fft(const RingArgs<T>& a, int mode, cudaStream_t st);
 

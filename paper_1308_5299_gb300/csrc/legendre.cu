@@ -929,7 +929,10 @@ template <typename T>
 int launch_leg_synth(const LegArgs<T>& a, cudaStream_t st) {
   if (a.L < 0) return CR_OK;
   if constexpr (sizeof(T) == 8)
+  {
     if (a.df) return launch_leg_synth_df(a, st);
+    if (ds_use(a)) return launch_ds_synth(a, a.alm, n_lm(a.L), 1, a.phase, st);
+  }
   int nbp, nbe;
   const int rp = legal_rp(a.rp_synth);
   pair_blocks(a.npolar, a.npairs, rp, &nbp, &nbe, sizeof(T) == 4 ? L32_NT : LEG_NT);
@@ -950,6 +953,8 @@ int launch_leg_adjoint(const LegArgs<T>& a, const FinalizeArgs<T>& f, cudaStream
       int rc = launch_leg_adjoint_df(a, &nbe, st);
       if (rc) return rc;
       done = true;
+    } else if (ds_use(a)) {
+      return launch_ds_adjoint(a, a.phase, 1, reinterpret_cast<double*>(a.partial), &f, st);
     }
   }
   if (!done) {

@@ -1,0 +1,1025 @@
+// FP64 Legendre stages on the tensor cores, by digit slices.
+//
+// On this GPU the FP64 pipe runs at 1/64 of the FP32 rate, so a Legendre
+// stage whose sums are FP64 fused multiply-adds is bound by that pipe.  Here
+// the FP64 pipe only advances the recurrence; the sums over l (synthesis) or
+// over ring pairs (adjoint) are exact integer products on the tensor cores.
+//
+// Digit slices.  Every operand is written as a fixed-point number of seven
+// signed base-256 digits (54 bits below a bound that holds for the whole row
+// or block).  Digits are small integers, exact in FP16; products of two
+// digits summed over at most 128 terms and at most seven digit pairs of the
+// same weight stay below 2^24, so the FP32 accumulators of the tensor cores
+// are exact, and the sums of equal weight (order s = i + j of the digits'
+// positions) can share one accumulator.  Orders 0..7 are kept: the dropped
+// ones are below the last digit of either operand.  Per term the error is
+// thus an absolute 2^-54 of the operands' bounds, where a chain of FP64
+// multiply-adds rounds to 2^-53 of the running sum at each step.  (The
+// splitting of an accurate product into exact low-precision products is the
+// scheme of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012.)
+//
+// The recurrence.  For one m let e_l = sqrt((l^2 - m^2) / (4 l^2 - 1)), so
+// that z P~_l = e_{l+1} P~_{l+1} + e_l P~_{l-1}.  With p_k = P~_o / z,
+// o = m + 1 + 2k (an even polynomial times sin^m),
+//   P~_o = z p_k,   P~_{o+1} = e_{o+2} p_{k+1} + e_{o+1} p_k,
+// so one sequence serves both parities of l - m:
+//   sum_l a_l P~_l(+-z) = sum_k p_k c_k +- z sum_k p_k d_k,
+//   c_k = e_o a_{o-1} + e_{o+1} a_{o+1},  d_k = a_o,
+// and p_k obeys a three-term recurrence in z^2 (Ishioka, J. Meteor. Soc.
+// Japan 96, 2018).  Rescaled by sigma_k so that the last coefficient is one,
+//   q_{k+1} = (A_k z^2 + B_k) q_k - q_{k-1},
+// two FP64 operations per two l instead of four.  z^2 is rounded once for the
+// whole sequence, which would add up coherently; four copies of it that
+// differ in the last place and average to the exact square are used in turn,
+// and near the poles (z^2 > 1/2) the same is done with 1 - z^2 and
+// A_k + B_k.  Near the equator p_k grows like 1/z while P~ does not and the
+// even sums would cancel, so pairs with z <= DS_ZEQ run the one-step
+// recurrence of legendre.cu instead (every l its own column of the sums).
+// Against extended precision at Nside 2048 / lmax 3000 both forms are at or
+// below the error of the one-step form for z > 0.2 and far below it near the
+// poles (1e-12 instead of 3e-11 in the first rings).
+//
+// What bounds it: the FP64 pipe (2 instructions per two l and ring pair, 4
+// near the equator, plus 1/8 for collecting the accumulators), with about 45
+// integer and shared-memory instructions per two l hidden behind it.
+#include <cuda_fp16.h>
+
+#include <cmath>
+
+#include "common.cuh"
+#include "kernels.h"
+#include "tc.cuh"
+
+namespace cr {
+
+constexpr int DS_PAIRS = 128;             // ring pairs per CTA, one per producer thread
+constexpr int DS_NT = 160;                // four producer warps and the MMA warp
+constexpr int DS_DIG = 7;                 // digits per operand
+constexpr int DS_ORD = 8;                 // orders of the digit products kept
+constexpr double DS_ZEQ = 0.25;           // pairs with z at or below run the one-step recurrence
+constexpr uint32_t DS_WAIT = 1u << 26;    // polls of a bounded mbarrier wait
+constexpr int DS_NONE = 0x3fffffff;       // start index of a pair that never starts
+constexpr uint64_t DS_BIAS = 0x8080808080808080ull;  // 128 in every digit (and half a unit of the dropped byte)
+
+// position of m's first k in tables of band limit L: room for
+// (L - m) / 2 + 1 entries each
+__host__ __device__ inline int64_t ds_off(int L, int m) { return (lm_off(L, m) >> 1) + m; }
+int64_t ds_len(int L) { return ds_off(L, L + 1) + 2; }
+
+// ---- plan tables -------------------------------------------------------------
+// Double-double helpers (Knuth's TwoSum, Dekker's product by FMA).
+struct dd2 {
+  double h, l;
+};
+__device__ __forceinline__ dd2 dd_prod(double a, double b) {
+  const double p = a * b;
+  return {p, fma(a, b, -p)};
+}
+__device__ __forceinline__ dd2 dd_norm(double h, double l) {
+  const double s = h + l;
+  return {s, l - (s - h)};
+}
+__device__ __forceinline__ dd2 dd_mul(dd2 a, dd2 b) {
+  dd2 p = dd_prod(a.h, b.h);
+  p.l += a.h * b.l + a.l * b.h;
+  return dd_norm(p.h, p.l);
+}
+__device__ __forceinline__ dd2 dd_div(dd2 a, dd2 b) {
+  const double q = a.h / b.h;
+  const dd2 p = dd_prod(q, b.h);
+  const double r = (a.h - p.h) - p.l + a.l - q * b.l;
+  return dd_norm(q, r / b.h);
+}
+__device__ __forceinline__ dd2 dd_sqrt(dd2 a) {
+  const double q = sqrt(a.h);
+  const dd2 p = dd_prod(q, q);
+  const double r = (a.h - p.h) - p.l + a.l;
+  return dd_norm(q, 0.5 * r / q);
+}
+
+// sigma_{k-1}^2 / sigma_{k+1}^2 = e_{o+1}^2 e_{o+2}^2 / (e_o^2 e_{o-1}^2), o = m + 1 + 2k, k >= 1
+__device__ __forceinline__ dd2 ds_ratio(int m, int k) {
+  const double o = m + 1.0 + 2.0 * k, dm = m;
+  auto n = [&](double l) { return (l - dm) * (l + dm); };
+  const dd2 num = dd_mul(dd_prod(n(o + 1), n(o + 2)), {(2 * o - 1) * (2 * o - 1) * (2 * o - 3), 0.0});
+  const dd2 den = dd_mul(dd_prod(n(o), n(o - 1)), {(2 * o + 3) * (2 * o + 3) * (2 * o + 5), 0.0});
+  return dd_div(num, den);
+}
+
+// One CTA per m.  sigma_k^2 runs down from 1 at the last two k by ds_ratio,
+// each parity of k its own chain: every thread multiplies the ratios of its
+// stretch of k, one warp combines the stretches, and a second pass forms the
+// coefficients.  In double-double, so that the tables are rounded once.
+constexpr int DST_NT = 128;
+__global__ void __launch_bounds__(DST_NT) ds_tab_kernel(DsTab t) {
+  const int m = blockIdx.x, tid = threadIdx.x;
+  const int nk = (t.Lc - m) / 2 + 1;
+  const int64_t off = ds_off(t.Lc, m);
+  __shared__ dd2 seg[2][DST_NT];
+  // stretch of this thread in the order from the last k down, of even length
+  const int len = (((nk + DST_NT - 1) / DST_NT) + 1) & ~1;
+  const int j0 = tid * len, j1 = min(nk, j0 + len);
+  dd2 c[2] = {{1.0, 0.0}, {1.0, 0.0}};
+  for (int j = j0; j < j1; ++j)  // k = nk - 1 - j; sigma_k^2 from sigma_{k+2}^2 by the ratio at k + 1
+    if (j >= 2) c[j & 1] = dd_mul(c[j & 1], ds_ratio(m, nk - j));
+  seg[0][tid] = c[0];
+  seg[1][tid] = c[1];
+  __syncthreads();
+  if (tid < 2) {
+    dd2 s = {1.0, 0.0};
+    for (int i = 0; i < DST_NT; ++i) {
+      const dd2 v = seg[tid][i];
+      seg[tid][i] = s;
+      s = dd_mul(s, v);
+    }
+  }
+  __syncthreads();
+  dd2 s2[2] = {seg[0][tid], seg[1][tid]};  // the chains' values at the last j before this stretch
+  const double dm = m;
+  for (int j = j0; j < j1; ++j) {
+    const int k = nk - 1 - j;
+    const double o = m + 1.0 + 2.0 * k;
+    const dd2 up = s2[(j & 1) ^ 1];  // sigma_{k+1}^2 (for j = 0 unused)
+    if (j >= 2) s2[j & 1] = dd_mul(s2[j & 1], ds_ratio(m, nk - j));
+    const dd2 cur = s2[j & 1];
+    auto n = [&](double l) { return (l - dm) * (l + dm); };
+    auto d = [&](double l) { return (2 * l - 1) * (2 * l + 1); };
+    if (j > 0) {
+      // A_k = sigma_k / (sigma_{k+1} e_{o+1} e_{o+2}), stored with the q it produces, k + 1
+      const dd2 x = dd_div(dd_mul(cur, dd_prod(d(o + 1), d(o + 2))), dd_mul(up, dd_prod(n(o + 1), n(o + 2))));
+      const dd2 A = dd_sqrt(x);
+      const dd2 g = dd_prod(2 * o - 1, 2 * o + 3);
+      const dd2 S = dd_div({2.0 * (o * o + o - dm * dm) - 1.0, 0.0}, g);           // e_{o+1}^2 + e_o^2
+      const dd2 S1 = dd_div({2.0 * (o * o + o + dm * dm) - 2.0, 0.0}, g);          // 1 - that
+      t.A[off + k + 1] = A.h;
+      t.B[off + k + 1] = -dd_mul(A, S).h;
+      t.AB[off + k + 1] = dd_mul(A, S1).h;
+    }
+    t.sg[off + k] = dd_sqrt(cur).h;
+    t.e0[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o), 0.0}), {d(o), 0.0})).h;
+    t.e1[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o + 1), 0.0}), {d(o + 1), 0.0})).h;
+    if (k == 0) t.A[off] = t.B[off] = t.AB[off] = 0.0;
+  }
+}
+
+void ds_tab_free(DsTab& t) {
+  if (t.A) cudaFree(t.A);
+  t = DsTab();
+}
+
+// the tables for band limits up to Lc (one allocation, six arrays)
+int ds_tab_build(DsTab& t, int Lc, cudaStream_t st) {
+  ds_tab_free(t);
+  const int64_t n = ds_len(Lc);
+  CR_CUDA(cudaMalloc(&t.A, 6 * n * sizeof(double)));
+  t.B = t.A + n;
+  t.AB = t.B + n;
+  t.sg = t.AB + n;
+  t.e0 = t.sg + n;
+  t.e1 = t.e0 + n;
+  t.Lc = Lc;
+  { ds_tab_kernel<<<Lc + 1, DST_NT, 0, st>>>(t); count_launch(); }
+  CR_CHECK_LAUNCH("ds_tab_kernel");
+  return CR_OK;
+}
+
+// ---- device helpers ----------------------------------------------------------
+
+__device__ __forceinline__ void ds_arrive(uint64_t* mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(mbar)) : "memory");
+}
+// the four producer warps
+__device__ __forceinline__ void ds_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// kind::f16 instruction descriptor, FP16 inputs, FP32 accumulation
+__host__ __device__ constexpr uint32_t ds_idesc(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// MN-major offset (see legendre_tc.cu)
+__device__ __forceinline__ uint32_t ds_mn_off(int mn, int k, int MN) {
+  return (uint32_t)(((mn >> 3) << 7) + (k >> 3) * (MN / 8) * 128 + ((k & 7) << 4) + ((mn & 7) << 1));
+}
+
+__device__ __forceinline__ int ds_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// round(v 2^62 / 2^(eb - 1023)) + DS_BIAS as 64 bits, |v| < 2^(eb - 1023):
+// the mantissa at bit 62, shifted right by the exponent's distance from the
+// bound.  Bytes 7..1 are the digits + 128; the bias of byte 0 rounds.
+__device__ __forceinline__ uint64_t ds_fix(double v, int eb) {
+  const int hi = __double2hiint(v);
+  const uint32_t lo = (uint32_t)__double2loint(v);
+  const int ex = (hi >> 20) & 0x7ff;
+  const int r = max(0, min(63, eb - ex));
+  const uint32_t mh = ((uint32_t)hi & 0xfffffu) | (ex ? 0x100000u : 0u);
+  const uint64_t x = ((((uint64_t)mh << 32) | lo) << 10) >> r;
+  const uint64_t s = (uint64_t)(int64_t)(hi >> 31);
+  return (x ^ s) - s + DS_BIAS;
+}
+
+// digits of weight byte b of 8 values as 8 FP16: 0x6400 | byte is 1024 + byte
+__device__ __forceinline__ uint32_t ds_pair(uint32_t w0, uint32_t w1, int bb) {
+  const uint32_t v = (__byte_perm(w0, w1, bb | ((4 + bb) << 8)) & 0x00ff00ffu) | 0x64006400u;
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&v), __half2half2(__ushort_as_half(0x6480)));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ uint4 ds_digits8(const uint32_t w[8], int bb) {
+  return make_uint4(ds_pair(w[0], w[1], bb), ds_pair(w[2], w[3], bb), ds_pair(w[4], w[5], bb), ds_pair(w[6], w[7], bb));
+}
+// digit i (0 the most significant) of one value
+__device__ __forceinline__ __half ds_digit(uint64_t y, int i) {
+  return __int2half_rn((int)((uint32_t)(y >> (8 * (7 - i))) & 255u) - 128);
+}
+
+// sum_s D_s 256^-s of the eight exact orders, times 256^3
+__device__ __forceinline__ double ds_collect(const float f[DS_ORD]) {
+  const long long hi = ((long long)((int)f[0] * 256 + (int)f[1]) << 16) + ((int)f[2] * 256 + (int)f[3]);
+  const long long lo = ((long long)(int)f[4] << 24) + ((long long)(int)f[5] << 16) + ((long long)(int)f[6] << 8) + (int)f[7];
+  // |hi|, |lo| < 2^51: to FP64 through the mantissa of 1.5 2^52
+  const double dh = __longlong_as_double(0x4338000000000000ll + hi) - 6755399441055744.0;
+  const double dl = __longlong_as_double(0x4338000000000000ll + lo) - 6755399441055744.0;
+  return fma(dl, 0x1p-32, dh);
+}
+// 2^(eb - 1023 - 36): ds_collect's 2^-24 and the 2^-6 of either operand's
+// leading digit; NaN where the block held an infinity or a NaN
+__device__ __forceinline__ double ds_scale(int eb) {
+  if (eb > 2047) return __longlong_as_double(0x7ff8000000000000ll);
+  const int e = eb - 36;
+  return e > 0 ? __hiloint2double(e << 20, 0) : 0.0;
+}
+
+// columns 16 o + c .. 16 o + c + 3 of the eight orders o, of this warp's lanes;
+// the wait names the registers, so that nothing reads them before it
+__device__ __forceinline__ void ds_ld_orders(uint32_t taddr, float f[DS_ORD][4]) {
+#pragma unroll
+  for (int o = 0; o < DS_ORD; ++o)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(f[o][0]), "=f"(f[o][1]), "=f"(f[o][2]), "=f"(f[o][3])
+                 : "r"(taddr + 16 * o));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(f[0][0]), "+f"(f[0][1]), "+f"(f[0][2]), "+f"(f[0][3]), "+f"(f[1][0]), "+f"(f[1][1]),
+                 "+f"(f[1][2]), "+f"(f[1][3]), "+f"(f[2][0]), "+f"(f[2][1]), "+f"(f[2][2]), "+f"(f[2][3]),
+                 "+f"(f[3][0]), "+f"(f[3][1]), "+f"(f[3][2]), "+f"(f[3][3]), "+f"(f[4][0]), "+f"(f[4][1]),
+                 "+f"(f[4][2]), "+f"(f[4][3]), "+f"(f[5][0]), "+f"(f[5][1]), "+f"(f[5][2]), "+f"(f[5][3]),
+                 "+f"(f[6][0]), "+f"(f[6][1]), "+f"(f[6][2]), "+f"(f[6][3]), "+f"(f[7][0]), "+f"(f[7][1]),
+                 "+f"(f[7][2]), "+f"(f[7][3])
+               :
+               : "memory");
+}
+
+// One ring pair's sequence: state, argument and bound.
+template <bool EQ>
+struct DsPair {
+  double q1 = 0.0, q2 = 0.0;
+  double Z[4] = {0.0, 0.0, 0.0, 0.0};  // EQ: Z[0] = z
+  int k0 = DS_NONE;                    // first index of the sequence
+  int eb = 1023;                       // |q| < 2^(eb - 1023)
+
+  // four copies of v + lo that average to it within an eighth of the last place
+  __device__ __forceinline__ void dither(double v, double lo) {
+    const double up = __longlong_as_double(__double_as_longlong(v) + 1) - v;
+    const int t = (int)rint(4.0 * lo / up);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Z[j] = v + (j < abs(t) ? copysign(up, lo) : 0.0);
+  }
+
+  // p: pair; polar: the warp runs on 1 - z^2
+  __device__ __forceinline__ void load(const DsArgs& a, int m, int p, bool polar) {
+    const int64_t o = (int64_t)m * a.ld_seed + p;
+    const double z = a.z[p];
+    const double zz = z * z;
+    if (EQ) {
+      Z[0] = z;
+    } else if (polar) {
+      const double w = 1.0 - z;  // exact for z >= 1/2
+      const double w2 = w * w, e = fma(w, w, -w2), t = 2.0 * w;
+      const double s = t - w2;
+      dither(s, ((t - s) - w2) - e);
+    } else {
+      dither(zz, fma(z, z, -zz));
+    }
+    const int L = a.L;
+    const int ls = a.ls[o];
+    // bounds |P~_lm| <= sqrt((2 l + 1) / 4 pi) and 0.3 (l + 1)^(1/4) / sqrt(sin)
+    // (the supremum over l, m and z is 0.29965 at every l tried to 3000),
+    // over the rescaling at its smallest
+    const float fl = (float)(L + 1);
+    float b = fminf(0.2821f * sqrtf(2.f * fl), 0.305f * sqrtf(sqrtf(fl)) * rsqrtf(sqrtf(fmaxf((float)(1.0 - zz), 1e-20f))));
+    if (EQ) {
+      const int64_t c = lm_off(a.Lc, m) + (L - m);
+      const double s = fmin(a.s[c], L > m ? a.s[c - 1] : 1.0);
+      b /= (float)fmin(s, 1.0);
+    } else {
+      b /= (float)z;
+    }
+    eb = 1023 + (int)ceilf(log2f(b) + 0.1f);
+    if (ls > L) return;
+    const double2 st = a.st[o];
+    if (EQ) {
+      k0 = ls - m;
+      q1 = st.x;
+      q2 = st.y;
+      return;
+    }
+    // (q_{k0-1}, q_{k0-2}) from the one-step state (Q_{ls-1}, Q_{ls-2})
+    k0 = (ls - m) >> 1;
+    const int64_t oc = lm_off(a.Lc, m) + (ls - m), ok = ds_off(a.t.Lc, m) + k0;
+    const double Q = fma((ls > m ? a.c[oc] : 0.0) * z, st.x, -st.y);
+    const double P = a.s[oc] * Q;
+    double qk;
+    if ((ls - m) & 1) {
+      if (k0 > 0) q1 = a.s[oc - 2] * st.y / (z * a.t.sg[ok - 1]);
+      qk = P / (z * a.t.sg[ok]);
+    } else {
+      if (k0 > 0) q1 = a.s[oc - 1] * st.x / (z * a.t.sg[ok - 1]);
+      qk = (k0 > 0 ? P - a.t.e1[ok - 1] * q1 : P) / a.t.e0[ok];
+    }
+    // the second value, such that the recurrence's next step returns q_{k0}
+    const double A = a.t.A[ok], B = polar ? a.t.AB[ok] : a.t.B[ok];
+    const double Zk = (k0 & 2) ? ((k0 & 1) ? Z[3] : Z[2]) : ((k0 & 1) ? Z[1] : Z[0]);
+    q2 = fma(fma(polar ? -A : A, Zk, B), q1, -qk);
+  }
+
+  __device__ __forceinline__ double step(double2 c, int u) {
+    const double e = EQ ? c.x * Z[0] : fma(c.x, Z[u & 3], c.y);
+    return fma(e, q1, -q2);
+  }
+};
+
+// Coefficients of the step that produces index k of the sequence.
+template <bool EQ>
+__device__ __forceinline__ double2 ds_coef(const DsArgs& a, int m, int k, int nk, bool polar) {
+  if (k >= nk) return make_double2(0.0, 0.0);
+  if (EQ) return make_double2(a.c[lm_off(a.Lc, m) + k], 0.0);
+  const int64_t o = ds_off(a.t.Lc, m) + k;
+  return polar ? make_double2(-a.t.A[o], a.t.AB[o]) : make_double2(a.t.A[o], a.t.B[o]);
+}
+
+struct DsShared {
+  double2 sc[4][32];      // recurrence coefficients, one copy per producer warp
+  uint64_t full[2], empty[2], done;
+  int eb[2][16];          // largest exponents of a block's columns
+  uint32_t taddr;
+  int kmin;
+  volatile int abort_;
+};
+
+// The 8 values k..k+7 of a warp's sequences as digits: calls store(i, digits)
+// for each digit i.  Idle before the warp's first start; per-lane start tests
+// while some lanes have not started.
+template <bool EQ, typename F>
+__device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const double2* sc, int k, int wmin, int wmax, F store) {
+  if (k + 8 <= wmin) {
+#pragma unroll
+    for (int i = 0; i < DS_DIG; ++i) store(i, make_uint4(0u, 0u, 0u, 0u));
+    return;
+  }
+  uint32_t yh[8], yl[8];
+  if (k >= wmax) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double q = s.step(sc[u], u);
+      s.q2 = s.q1;
+      s.q1 = q;
+      const uint64_t y = ds_fix(q, s.eb);
+      yh[u] = (uint32_t)(y >> 32);
+      yl[u] = (uint32_t)y;
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool on = k + u >= s.k0;
+      const double q = s.step(sc[u], u);
+      s.q2 = on ? s.q1 : s.q2;
+      s.q1 = on ? q : s.q1;
+      const uint64_t y = on ? ds_fix(q, s.eb) : DS_BIAS;
+      yh[u] = (uint32_t)(y >> 32);
+      yl[u] = (uint32_t)y;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) store(i, ds_digits8(yh, 3 - i));
+#pragma unroll
+  for (int i = 4; i < DS_DIG; ++i) store(i, ds_digits8(yl, 7 - i));
+}
+
+// this thread's pair, and the warp's and the CTA's first (and the warp's
+// last) start index
+template <bool EQ>
+__device__ __forceinline__ void ds_setup(const DsArgs& a, DsShared& sh, DsPair<EQ>& s, int m, int p, int pend,
+                                         bool producer, bool* polar, int* wmin, int* wmax) {
+  *polar = false;
+  if (producer) {
+    // one form per warp, from its last pair's cosine
+    const int wl = min((p | 31), pend - 1);
+    if (!EQ && p < pend) {
+      const double zl = a.z[wl];
+      *polar = zl * zl > 0.5;
+    }
+    *polar = __any_sync(0xffffffffu, *polar);
+    if (p < pend) s.load(a, m, p, *polar);
+  }
+  *wmin = __reduce_min_sync(0xffffffffu, s.k0);
+  *wmax = __reduce_max_sync(0xffffffffu, s.k0 == DS_NONE ? 0 : s.k0);
+  if (threadIdx.x == 0) {
+    sh.kmin = DS_NONE;
+    sh.abort_ = 0;
+  }
+  __syncthreads();
+  if (producer && (threadIdx.x & 31) == 0) atomicMin(&sh.kmin, *wmin);
+  __syncthreads();
+}
+
+// ---- synthesis ---------------------------------------------------------------
+// CTA: one m, 128 ring pairs (tensor-core rows), up to NR right-hand sides.
+// A operand: the pairs' digits, 16 sequence values per stage (two stages).
+// B operand: the digits of (c_k, d_k) x (Re, Im) of the right-hand sides, 16
+// columns per digit, for a block of 128 k with one exponent per column.  The
+// accumulator of digit pair (i, j) starts at column 16 i, so equal orders add
+// up in place.  After each block the four producer warps collect the eight
+// orders of their own pairs into FP64 sums.
+constexpr int DSS_STAGE = DS_DIG * DS_PAIRS * 16 * 2;     // 28 KB
+constexpr int DSS_BSTEP = 16 * DS_ORD * 16 * 2;           // 16 columns x 8 digits (the last zero) x K 16
+constexpr int DSS_KB = 128;                               // k per block
+constexpr int DSS_SMEM = 2 * DSS_STAGE + (DSS_KB / 16) * DSS_BSTEP;
+constexpr int DSS_TMEM = 128;
+
+template <int NR, bool EQ>
+__device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uint8_t* sm, int base, int pend) {
+  const int m = blockIdx.y, L = a.L;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool producer = warp < 4;
+  const int p = base + tid;
+  DsPair<EQ> s;
+  bool polar;
+  int wmin, wmax;
+  ds_setup<EQ>(a, sh, s, m, p, pend, producer, &polar, &wmin, &wmax);
+  const int nk = EQ ? L - m + 1 : (L - m) / 2 + 1;
+  const int kbeg = sh.kmin & ~3;
+  const bool any = sh.kmin < nk;
+  uint8_t* Bs = sm + 2 * DSS_STAGE;
+  double acc[4 * NR];
+#pragma unroll
+  for (int j = 0; j < 4 * NR; ++j) acc[j] = 0.0;
+  bool ok = true;
+  uint32_t taddr = 0;
+  if (any) {
+    for (int e = tid; e < (DSS_KB / 16) * DSS_BSTEP / 16; e += DS_NT)
+      reinterpret_cast<uint4*>(Bs)[e] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < 32) sh.eb[tid >> 4][tid & 15] = 0;
+    if (warp == 4) tc::tmem_alloc(&sh.taddr, DSS_TMEM);
+    if (tid == 0) {
+      for (int i = 0; i < 2; ++i) {
+        tc::mbar_init(&sh.full[i], 128);
+        tc::mbar_init(&sh.empty[i], 1);
+      }
+      tc::mbar_init(&sh.done, 1);
+      tc::mbar_fence_init();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    taddr = sh.taddr;
+    int gst = 0, nblk = 0;  // stages and blocks so far
+    if (producer) {
+      const int64_t offa = lm_off(L, m);
+      const int64_t ok_ = ds_off(a.t.Lc, m), oc = lm_off(a.Lc, m);
+      double2 cf = make_double2(0.0, 0.0);
+      if (lane < 16) cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar);
+      for (int kc = kbeg; kc < nk; kc += DSS_KB, ++nblk) {
+        // coefficients of this block: thread = k
+        const int k = kc + tid;
+        double v[4 * NR];
+#pragma unroll
+        for (int j = 0; j < 4 * NR; ++j) v[j] = 0.0;
+        if (k < nk) {
+          if (EQ) {
+            const double f = a.s[oc + k] * (a.dl ? a.dl[m + k] : 1.0);
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+              if (r < a.nr) {
+                const double2 x = a.alm[r * a.ld_alm + offa + k];
+                const int odd = 2 * (k & 1);
+                v[4 * r + 0] = odd ? 0.0 : f * x.x;
+                v[4 * r + 1] = odd ? 0.0 : f * x.y;
+                v[4 * r + 2] = odd ? f * x.x : 0.0;
+                v[4 * r + 3] = odd ? f * x.y : 0.0;
+              }
+          } else {
+            const int l = m + 2 * k;  // a_l, a_{l+1} = a_o, a_{l+2}
+            const double f0 = a.t.e0[ok_ + k] * (a.dl ? a.dl[l] : 1.0);
+            const double f1 = l + 1 <= L ? a.t.sg[ok_ + k] * (a.dl ? a.dl[l + 1] : 1.0) : 0.0;
+            const double f2 = l + 2 <= L ? a.t.e1[ok_ + k] * (a.dl ? a.dl[l + 2] : 1.0) : 0.0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+              if (r < a.nr) {
+                const double2* x = a.alm + r * a.ld_alm + offa + 2 * k;
+                const double2 x0 = x[0];
+                const double2 x1 = l + 1 <= L ? x[1] : make_double2(0.0, 0.0);
+                const double2 x2 = l + 2 <= L ? x[2] : make_double2(0.0, 0.0);
+                v[4 * r + 0] = fma(f0, x0.x, f2 * x2.x);
+                v[4 * r + 1] = fma(f0, x0.y, f2 * x2.y);
+                v[4 * r + 2] = f1 * x1.x;
+                v[4 * r + 3] = f1 * x1.y;
+              }
+          }
+          if (m == 0) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) v[4 * r + 1] = v[4 * r + 3] = 0.0;
+          }
+        }
+        int* eb = sh.eb[nblk & 1];
+#pragma unroll
+        for (int j = 0; j < 4 * NR; ++j) {
+          const int e = __reduce_max_sync(0xffffffffu, ds_exp(v[j]));
+          if (lane == 0) atomicMax(&eb[j], e + 1);  // |v| < 2^(eb - 1023); 2048: not finite
+        }
+        ds_bar();
+        if (tid < 16) sh.eb[(nblk + 1) & 1][tid] = 0;  // last read before this barrier
+        uint8_t* Bk = Bs + (tid >> 4) * DSS_BSTEP;
+#pragma unroll
+        for (int j = 0; j < 4 * NR; ++j) {
+          const uint64_t y = ds_fix(v[j], eb[j]);
+#pragma unroll
+          for (int i = 0; i < DS_DIG; ++i)
+            *reinterpret_cast<__half*>(Bk + tc::kmajor_offset(16 * i + j, tid & 15, 16)) = ds_digit(y, i);
+        }
+        const int nst = min(DSS_KB / 16, (nk - kc + 15) / 16);
+        for (int st = 0; st < nst; ++st, ++gst) {
+          const int stg = gst & 1, ks = kc + 16 * st;
+          if (gst >= 2 && ok) {
+            const bool w = tc::mbar_wait(&sh.empty[stg], ((gst >> 1) - 1) & 1, DS_WAIT);
+            if (!__all_sync(0xffffffffu, w)) {
+              if (lane == 0) sh.abort_ = 1;
+              ok = false;
+            }
+          }
+          __syncwarp();
+          if (lane < 16) {
+            sh.sc[warp][lane] = cf;
+            cf = ds_coef<EQ>(a, m, ks + 16 + lane, nk, polar);
+          }
+          __syncwarp();
+          uint8_t* S = sm + stg * DSS_STAGE;
+#pragma unroll
+          for (int g = 0; g < 2; ++g) {
+            const uint32_t off = tc::kmajor_offset(tid, 8 * g, 16);
+            ds_produce8<EQ>(s, sh.sc[warp] + 8 * g, ks + 8 * g, wmin, wmax, [&](int i, uint4 d) {
+              *reinterpret_cast<uint4*>(S + i * (DSS_STAGE / DS_DIG) + off) = d;
+            });
+          }
+          tc::fence_proxy_async();
+          tc::fence_before_sync();
+          ds_arrive(&sh.full[stg]);
+        }
+        if (ok) {
+          const bool w = tc::mbar_wait(&sh.done, nblk & 1, DS_WAIT);
+          if (!__all_sync(0xffffffffu, w)) {
+            if (lane == 0) sh.abort_ = 1;
+            ok = false;
+          }
+        }
+        if (ok) {
+          tc::fence_after_sync();
+          const uint32_t tw = taddr + ((uint32_t)(warp * 32) << 16);
+          const bool on = kc + DSS_KB > s.k0;
+#pragma unroll
+          for (int r = 0; r < NR; ++r) {
+            if (r < a.nr) {
+              float f[DS_ORD][4];
+              ds_ld_orders(tw + 4 * r, f);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                float c[DS_ORD];
+#pragma unroll
+                for (int o = 0; o < DS_ORD; ++o) c[o] = f[o][j];
+                const double x = fma(ds_collect(c), ds_scale(eb[4 * r + j]), acc[4 * r + j]);
+                if (on) acc[4 * r + j] = x;
+              }
+            }
+          }
+          tc::fence_before_sync();
+        }
+      }
+    } else {
+      for (int kc = kbeg; kc < nk && ok; kc += DSS_KB, ++nblk) {
+        const int nst = min(DSS_KB / 16, (nk - kc + 15) / 16);
+        for (int st = 0; st < nst; ++st, ++gst) {
+          const int stg = gst & 1;
+          const bool w = tc::mbar_wait(&sh.full[stg], (gst >> 1) & 1, DS_WAIT);
+          if (!__all_sync(0xffffffffu, w) || __any_sync(0xffffffffu, sh.abort_ != 0)) {
+            if (lane == 0) sh.abort_ = 1;
+            ok = false;
+            break;
+          }
+          tc::fence_after_sync();
+          if (lane == 0) {
+            const uint32_t sa = tc::smem_addr(sm + stg * DSS_STAGE), sb = tc::smem_addr(Bs + st * DSS_BSTEP);
+            const uint64_t bd = tc::smem_desc(sb, 128, 256);
+#pragma unroll
+            for (int i = 0; i < DS_DIG; ++i) {
+              // digit i meets digits 0 .. min(6, 7 - i); i = 0 also the zero
+              // digit, which clears the last order on the block's first step
+              const int nj = i == 0 ? DS_ORD : min(DS_DIG, DS_ORD - i);
+              tc::mma_bf16(taddr + 16 * i, tc::smem_desc(sa + i * (DSS_STAGE / DS_DIG), 128, 256), bd,
+                           ds_idesc(128, 16 * nj), (st > 0 || i > 0) ? 1u : 0u);
+            }
+            tc::mma_commit(&sh.empty[stg]);
+            if (st == nst - 1) tc::mma_commit(&sh.done);
+          }
+          __syncwarp();
+        }
+      }
+      // commits are cumulative: the last one issued covers every MMA
+      if (gst > 0) {
+        const bool w = tc::mbar_wait(&sh.empty[(gst - 1) & 1], ((gst - 1) >> 1) & 1, DS_WAIT);
+        if (!__all_sync(0xffffffffu, w)) ok = false;
+      }
+    }
+    tc::fence_before_sync();
+    ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    tc::fence_after_sync();
+    if (warp == 4) tc::tmem_dealloc(taddr, DSS_TMEM);
+  }
+  if (producer && p < pend) {
+    const int rn = p, rs = a.nring - 1 - p;
+    const bool live = s.k0 < nk;
+    // a wait that gave up must not pass for a result
+    const double sc = ok ? __hiloint2double(s.eb << 20, 0) : __longlong_as_double(0x7ff8000000000000ll);
+    const double zd = EQ ? sc : sc * a.z[p];
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (r < a.nr) {
+        double2 n = make_double2(0.0, 0.0), t = n;
+        if (live || !ok) {
+          const double cx = acc[4 * r] * sc, cy = acc[4 * r + 1] * sc;
+          const double dx = acc[4 * r + 2] * zd, dy = acc[4 * r + 3] * zd;
+          n = make_double2(cx + dx, cy + dy);
+          t = make_double2(cx - dx, cy - dy);
+        }
+        a.phase[r * a.ld_phase + (int64_t)rn * a.ldp + m] = n;
+        if (rs != rn) a.phase[r * a.ld_phase + (int64_t)rs * a.ldp + m] = t;
+      }
+  }
+}
+
+template <int NR>
+__global__ void __launch_bounds__(DS_NT, 2) ds_synth_kernel(DsArgs a) {
+  extern __shared__ __align__(1024) uint8_t ds_sm[];
+  __shared__ DsShared sh;
+  const int tile = blockIdx.x;
+  if (tile < a.nt_is) ds_synth_body<NR, false>(a, sh, ds_sm, tile * DS_PAIRS, a.nis);
+  else ds_synth_body<NR, true>(a, sh, ds_sm, a.nis + (tile - a.nt_is) * DS_PAIRS, a.npairs);
+}
+
+// ---- adjoint -----------------------------------------------------------------
+// CTA: one m, 128 ring pairs (the contraction index).  The pairs' phases
+// G = (even combination, z times the odd one) x (Re, Im) of up to NR
+// right-hand sides are split into digits once: row (digit, column) of a
+// K-major operand that starts with 6 CB zero rows, so that the operand read
+// from CB i rows earlier is the digits shifted down by i and row (s, column)
+// of the accumulator collects order s whatever the digit i of the other
+// operand.  That one holds 32 sequence values (N) of the 128 pairs per stage,
+// MN-major, so a thread writes 8 consecutive values of its own pair.  CB = 8
+// columns make 64 rows for one or two right-hand sides, CB = 16 make 128 for
+// up to four.  One partial row per (tile, right-hand side): (u_k, v_k) with
+// a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k, a_{o+1} += sigma_k e_{o+1} u_k,
+// or the two parities' values themselves near the equator.
+constexpr int DSA_N = 32;                                  // sequence values per stage
+constexpr int DSA_BD = DSA_N * DS_PAIRS * 2;               // one digit of a stage
+constexpr int DSA_FS = 40;                                 // row stride of the collected accumulators
+template <int NR>
+struct DsaLayout {
+  static constexpr int CB = NR <= 2 ? 8 : 16;
+  static constexpr int A_ROWS = 14 * CB;                   // zeros, digits, zeros
+  static constexpr int A_BYTES = A_ROWS * DS_PAIRS * 2;
+  static constexpr int B0 = A_BYTES;
+  static constexpr int F0 = B0 + DS_DIG * DSA_BD;
+  static constexpr int BYTES = F0 + DS_ORD * 4 * NR * DSA_FS * 4;
+};
+
+template <int NR, bool EQ>
+__device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, uint8_t* sm, int base, int pend) {
+  using Lay = DsaLayout<NR>;
+  constexpr int CB = Lay::CB, NC = 4 * NR;
+  const int m = blockIdx.y, L = a.L, blk = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool producer = warp < 4;
+  const int p = base + tid;
+  DsPair<EQ> s;
+  bool polar;
+  int wmin, wmax;
+  ds_setup<EQ>(a, sh, s, m, p, pend, producer, &polar, &wmin, &wmax);
+  const int nk = EQ ? L - m + 1 : (L - m) / 2 + 1;
+  const int nk2 = (L - m) / 2 + 1;
+  const int kbeg = min(sh.kmin, nk) & ~3;
+  // partial row of right-hand side r: doubles 4 k + column
+  const int64_t rstride = (int64_t)a.nblk * a.nkk * 4;
+  double* part = a.partial + ((int64_t)blk * a.nkk + ds_off(L, m)) * 4;
+  // zero before the tile's first start
+  for (int r = 0; r < a.nr; ++r)
+    for (int i = tid; i < (sh.kmin < nk ? (EQ ? 2 * kbeg : 4 * kbeg) : 4 * nk2); i += DS_NT) part[r * rstride + i] = 0.0;
+  if (sh.kmin >= nk) return;
+
+  for (int e = tid; e < Lay::A_BYTES / 16; e += DS_NT) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < 16) sh.eb[0][tid] = 0;
+  if (warp == 4) tc::tmem_alloc(&sh.taddr, 32);
+  if (tid == 0) {
+    tc::mbar_init(&sh.full[0], 128);
+    tc::mbar_init(&sh.done, 1);
+    tc::mbar_fence_init();
+  }
+  __syncthreads();
+  double g[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) g[j] = 0.0;
+  if (producer) {
+    if (s.k0 < nk) {
+      const int rn = p, rs = a.nring - 1 - p;
+      const double zo = EQ ? 1.0 : a.z[p];
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        if (r < a.nr) {
+          const double2 gn = a.phase[r * a.ld_phase + (int64_t)rn * a.ldp + m];
+          const double2 gs = (rs != rn) ? a.phase[r * a.ld_phase + (int64_t)rs * a.ldp + m] : make_double2(0.0, 0.0);
+          g[4 * r] = gn.x + gs.x;
+          g[4 * r + 1] = gn.y + gs.y;
+          g[4 * r + 2] = zo * (gn.x - gs.x);
+          g[4 * r + 3] = zo * (gn.y - gs.y);
+        }
+    }
+    // the pair's bound goes to this operand: |g| 2^(eb_pair) < 2^(eb - 1023)
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+      const int x = ds_exp(g[j]);
+      const int e = __reduce_max_sync(0xffffffffu, x == 0 ? 0 : (x == 2047 ? 1 << 20 : x + s.eb - 1023));
+      if (lane == 0) atomicMax(&sh.eb[0][j], e + 1);
+    }
+  }
+  __syncthreads();
+  if (producer) {
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+      const uint64_t y = ds_fix(g[j], sh.eb[0][j] - (s.eb - 1023));
+#pragma unroll
+      for (int i = 0; i < DS_DIG; ++i)
+        *reinterpret_cast<__half*>(sm + tc::kmajor_offset((6 + i) * CB + j, tid, DS_PAIRS)) = ds_digit(y, i);
+    }
+  }
+  tc::fence_proxy_async();
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t taddr = sh.taddr;
+  bool ok = true;
+  const int nit = (nk - kbeg + DSA_N - 1) / DSA_N;
+  if (producer) {
+    float* fb = reinterpret_cast<float*>(sm + Lay::F0);
+    // accumulators of iteration `it` to the partial rows
+    auto flush = [&](int it) {
+      if (ok) {
+        const bool w = tc::mbar_wait(&sh.done, it & 1, DS_WAIT);
+        if (!__all_sync(0xffffffffu, w)) {
+          if (lane == 0) sh.abort_ = 1;
+          ok = false;
+        }
+      }
+      tc::fence_after_sync();
+      float f[DSA_N];
+      tc::tmem_ld32(taddr + ((uint32_t)(warp * 32) << 16), f);
+      // 64 rows live in lanes 0..15 of each warp's quarter, 128 rows in all
+      const int so = 2 * warp + lane / CB, col = lane % CB;
+      if (lane < 2 * CB && col < NC) {
+        float4* d = reinterpret_cast<float4*>(fb + (so * NC + col) * DSA_FS);
+#pragma unroll
+        for (int i = 0; i < DSA_N / 4; ++i) d[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
+      }
+      tc::fence_before_sync();
+      ds_bar();
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        if (r < a.nr) {
+          const int j = 4 * r + (tid & 3), kk = tid >> 2, k = kbeg + it * DSA_N + kk;
+          float c[DS_ORD];
+#pragma unroll
+          for (int o = 0; o < DS_ORD; ++o) c[o] = fb[(o * NC + j) * DSA_FS + kk];
+          double x = ds_collect(c) * ds_scale(sh.eb[0][j]);
+          if (!ok) x = __longlong_as_double(0x7ff8000000000000ll);
+          if (k < nk) {
+            double* d = part + r * rstride;
+            if (!EQ) d[4 * (int64_t)k + (tid & 3)] = x;
+            else if ((k & 1) == ((tid >> 1) & 1)) d[2 * (int64_t)k + (tid & 1)] = x;
+          }
+        }
+      }
+    };
+    double2 cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar);
+    for (int it = 0; it < nit; ++it) {
+      const int ks = kbeg + it * DSA_N;
+      if (it > 0) flush(it - 1);
+      __syncwarp();
+      sh.sc[warp][lane] = cf;
+      cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar);
+      __syncwarp();
+#pragma unroll 1
+      for (int gq = 0; gq < DSA_N / 8; ++gq) {
+        uint8_t* B = sm + Lay::B0 + ds_mn_off(8 * gq, tid, DSA_N);
+        ds_produce8<EQ>(s, sh.sc[warp] + 8 * gq, ks + 8 * gq, wmin, wmax,
+                        [&](int i, uint4 d) { *reinterpret_cast<uint4*>(B + i * DSA_BD) = d; });
+      }
+      tc::fence_proxy_async();
+      ds_arrive(&sh.full[0]);
+    }
+    flush(nit - 1);
+  } else {
+    int issued = 0;
+    for (int it = 0; it < nit && ok; ++it) {
+      const bool w = tc::mbar_wait(&sh.full[0], it & 1, DS_WAIT);
+      if (!__all_sync(0xffffffffu, w) || __any_sync(0xffffffffu, sh.abort_ != 0)) {
+        if (lane == 0) sh.abort_ = 1;
+        ok = false;
+        break;
+      }
+      tc::fence_after_sync();
+      if (lane == 0) {
+        constexpr uint32_t id = ds_idesc(8 * CB, DSA_N) | (1u << 16);  // B MN-major
+        constexpr uint32_t rg = (DS_PAIRS / 8) * 128;                  // 8 rows of the K-major operand
+        constexpr uint32_t bk = (DSA_N / 8) * 128;                     // 8 pairs of the MN-major one
+        const uint32_t sa = tc::smem_addr(sm), sb = tc::smem_addr(sm + Lay::B0);
+#pragma unroll
+        for (int i = 0; i < DS_DIG; ++i)
+#pragma unroll
+          for (int kk = 0; kk < DS_PAIRS / 16; ++kk)
+            tc::mma_bf16(taddr, tc::smem_desc(sa + (6 - i) * (CB / 8) * rg + kk * 256, 128, rg),
+                         tc::smem_desc(sb + i * DSA_BD + kk * 2 * bk, bk, 128), id, (i > 0 || kk > 0) ? 1u : 0u);
+        tc::mma_commit(&sh.done);
+      }
+      __syncwarp();
+      issued = it + 1;
+    }
+    if (issued > 0) {
+      const bool w = tc::mbar_wait(&sh.done, (issued - 1) & 1, DS_WAIT);
+      if (!__all_sync(0xffffffffu, w)) ok = false;
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  if (warp == 4) tc::tmem_dealloc(taddr, 32);
+}
+
+template <int NR>
+__global__ void __launch_bounds__(DS_NT, NR <= 2 ? 2 : 1) ds_adjoint_kernel(DsArgs a) {
+  extern __shared__ __align__(1024) uint8_t ds_sm[];
+  __shared__ DsShared sh;
+  const int tile = blockIdx.x;
+  if (tile < a.nt_is) ds_adjoint_body<NR, false>(a, sh, ds_sm, tile * DS_PAIRS, a.nis);
+  else ds_adjoint_body<NR, true>(a, sh, ds_sm, a.nis + (tile - a.nt_is) * DS_PAIRS, a.npairs);
+}
+
+// The tiles' partial rows to coefficients (fixed order), with the epilogue of
+// leg_finalize_kernel.  Thread: one k, i.e. l = m + 2 k and l + 1.
+__global__ void __launch_bounds__(128) ds_finalize_kernel(DsArgs a, const double* partial, FinalizeArgs<double> f) {
+  const int m = blockIdx.y, L = a.L;
+  const int nk = (L - m) / 2 + 1;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.x * blockDim.x >= nk) return;  // whole CTA
+  const double2* row = reinterpret_cast<const double2*>(partial) + ds_off(L, m) * 2;
+  const int64_t bs = a.nkk * 2;
+  auto sum = [&](int kk, int w, int b0, int b1) {
+    double2 x = make_double2(0.0, 0.0);
+    for (int b = b0; b < b1; ++b) x = cadd(x, row[b * bs + 2 * (int64_t)kk + w]);
+    return x;
+  };
+  const bool in = k < nk;
+  double2 u = make_double2(0.0, 0.0), v = u;
+  if (in) {
+    u = sum(k, 0, 0, a.nt_is);
+    v = sum(k, 1, 0, a.nt_is);
+  }
+  double2 um;  // u_{k-1}
+  um.x = __shfl_up_sync(0xffffffffu, u.x, 1);
+  um.y = __shfl_up_sync(0xffffffffu, u.y, 1);
+  if (!in) return;
+  if ((threadIdx.x & 31) == 0) um = k > 0 ? sum(k - 1, 0, 0, a.nt_is) : make_double2(0.0, 0.0);
+  const int64_t ok = ds_off(a.t.Lc, m) + k, oc = lm_off(a.Lc, m) + 2 * k;
+  const double g0 = a.t.e0[ok], g1 = k > 0 ? a.t.e1[ok - 1] : 0.0;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int l = m + 2 * k + w;
+    if (l > L) break;
+    const double2 q = sum(k, w, a.nt_is, a.nblk);
+    const double sl = a.s[oc + w];
+    double2 y = make_double2(sl * q.x, sl * q.y);
+    if (w == 0) {
+      y.x += g0 * u.x + (k > 0 ? g1 * um.x : 0.0);
+      y.y += g0 * u.y + (k > 0 ? g1 * um.y : 0.0);
+    } else {
+      y.x = fma(a.t.sg[ok], v.x, y.x);
+      y.y = fma(a.t.sg[ok], v.y, y.y);
+    }
+    const int64_t i = lm_off(L, m) + (l - m);
+    if (f.dl_out) y = cscale(y, f.dl_out[l]);
+    if (f.dadd) {
+      const double2 x = f.xadd[i];
+      y.x = fma(f.dadd[l], x.x, y.x);
+      y.y = fma(f.dadd[l], x.y, y.y);
+    }
+    if (f.bsub) {
+      const double2 b = f.bsub[i];
+      y = make_double2(b.x - y.x, b.y - y.y);
+    }
+    if (m == 0) y.y = 0.0;
+    if (f.accumulate) y = cadd(y, f.out[i]);
+    f.out[i] = y;
+  }
+}
+
+// ---- launchers ---------------------------------------------------------------
+
+int ds_tiles(int nis, int npairs) { return (nis + DS_PAIRS - 1) / DS_PAIRS + (npairs - nis + DS_PAIRS - 1) / DS_PAIRS; }
+int ds_first_equatorial(const double* z, int npairs) {
+  int n = 0;
+  while (n < npairs && z[n] > DS_ZEQ) ++n;
+  return n;
+}
+int64_t ds_partial_bytes(int nis, int npairs, int L, int nr) {
+  return (int64_t)nr * ds_tiles(nis, npairs) * ds_len(L) * 4 * (int64_t)sizeof(double);
+}
+
+bool ds_use(const LegArgs<double>& a) { return a.ds && !a.df && a.npairs >= 64 && a.L >= 64; }
+
+static DsArgs ds_args(const LegArgs<double>& la, int nr) {
+  DsArgs a;
+  a.t = *la.ds;
+  a.phase = la.phase;
+  a.ldp = la.ldp;
+  a.ld_phase = (int64_t)la.nring * la.ldp;
+  a.L = la.L;
+  a.Lc = la.Lc;
+  a.nr = nr;
+  a.c = la.c;
+  a.s = la.s;
+  a.dl = la.dl;
+  a.z = la.z;
+  a.ls = la.ls;
+  a.st = la.st;
+  a.ld_seed = la.ld_seed;
+  a.npairs = la.npairs;
+  a.nring = la.nring;
+  a.nis = la.nis;
+  a.nt_is = (la.nis + DS_PAIRS - 1) / DS_PAIRS;
+  a.nblk = ds_tiles(la.nis, la.npairs);
+  a.nkk = ds_len(la.L);
+  return a;
+}
+
+// nr right-hand sides (vectors at stride ld_alm, phases at nring * ldp), four at a time
+int launch_ds_synth(const LegArgs<double>& la, const double2* alm, int64_t ld_alm, int nr, double2* phase,
+                    cudaStream_t st) {
+  for (int r0 = 0; r0 < nr; r0 += 4) {
+    DsArgs a = ds_args(la, std::min(4, nr - r0));
+    a.alm = alm + r0 * ld_alm;
+    a.ld_alm = ld_alm;
+    a.phase = phase + r0 * a.ld_phase;
+    const dim3 grid(a.nblk, la.L + 1);
+    if (a.nr == 1) {
+      CR_CUDA(cudaFuncSetAttribute(ds_synth_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSS_SMEM));
+      { ds_synth_kernel<1><<<grid, DS_NT, DSS_SMEM, st>>>(a); count_launch(); }
+    } else {
+      CR_CUDA(cudaFuncSetAttribute(ds_synth_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSS_SMEM));
+      { ds_synth_kernel<4><<<grid, DS_NT, DSS_SMEM, st>>>(a); count_launch(); }
+    }
+    CR_CHECK_LAUNCH("ds_synth_kernel");
+  }
+  return CR_OK;
+}
+
+template <int NR>
+static int ds_adjoint_launch(const DsArgs& a, cudaStream_t st) {
+  CR_CUDA(cudaFuncSetAttribute(ds_adjoint_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, DsaLayout<NR>::BYTES));
+  { ds_adjoint_kernel<NR><<<dim3(a.nblk, a.L + 1), DS_NT, DsaLayout<NR>::BYTES, st>>>(a); count_launch(); }
+  CR_CHECK_LAUNCH("ds_adjoint_kernel");
+  return CR_OK;
+}
+
+// phases of nr right-hand sides -> f[0..nr-1].out, through partial rows in `partial`
+// (ds_partial_bytes of up to four right-hand sides)
+int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, double* partial,
+                      const FinalizeArgs<double>* f, cudaStream_t st) {
+  for (int r0 = 0; r0 < nr; r0 += 4) {
+    DsArgs a = ds_args(la, std::min(4, nr - r0));
+    a.phase = const_cast<double2*>(phase) + r0 * a.ld_phase;
+    a.partial = partial;
+    int rc = a.nr == 1 ? ds_adjoint_launch<1>(a, st) : a.nr == 2 ? ds_adjoint_launch<2>(a, st) : ds_adjoint_launch<4>(a, st);
+    if (rc) return rc;
+    const dim3 grid((la.L / 2 + 1 + 127) / 128, la.L + 1);
+    for (int r = 0; r < a.nr; ++r) {
+      { ds_finalize_kernel<<<grid, 128, 0, st>>>(a, partial + (int64_t)r * a.nblk * a.nkk * 4, f[r0 + r]); count_launch(); }
+      CR_CHECK_LAUNCH("ds_finalize_kernel");
+    }
+  }
+  return CR_OK;
+}
+
+}  // namespace cr

@@ -212,6 +212,7 @@ int grid_upload(Grid& g, int Lseed, cudaStream_t st) {
   CR_CUDA(cudaMemcpyAsync(g.d_z, g.z.data(), g.nring * sizeof(double), cudaMemcpyHostToDevice, st));
   CR_CUDA(cudaMemcpyAsync(g.d_z32, z32.data(), g.nring * sizeof(float), cudaMemcpyHostToDevice, st));
   CR_CUDA(cudaMemcpyAsync(g.d_sth, g.sth.data(), g.nring * sizeof(double), cudaMemcpyHostToDevice, st));
+  g.nis = ds_first_equatorial(g.z.data(), g.npairs);
   int rc = build_fft_tables(g, st);
   if (rc) return rc;
   return build_seeds(g, Lseed, st);
@@ -265,7 +266,8 @@ static int build_coef(cr_plan* P, int Lc) {
   CR_CUDA(cudaMemcpy(P->d_c32, c32.data(), nlm * sizeof(float), cudaMemcpyHostToDevice));
   CR_CUDA(cudaMemcpy(P->d_s32, s32.data(), nlm * sizeof(float), cudaMemcpyHostToDevice));
   P->Lcoef = Lc;
-  return CR_OK;
+  if (!P->ds) P->ds = new DsTab();
+  return ds_tab_build(*P->ds, Lc, P->stream);
 }
 
 // Recurrence tables for a larger band limit (the plan's transforms at any
@@ -302,7 +304,8 @@ int grid_reseed(Grid& g, int Lseed, cudaStream_t st) {
 
 int ensure_workspace(cr_plan* P, const Grid& g, int L) {
   const int64_t phase = (int64_t)g.nring * (L + 1) * (int64_t)sizeof(double2);
-  const int64_t partial = (int64_t)leg_partial_blocks(g.npairs) * n_lm(L) * (int64_t)sizeof(double2);
+  const int64_t partial = std::max((int64_t)leg_partial_blocks(g.npairs) * n_lm(L) * (int64_t)sizeof(double2),
+                                   ds_partial_bytes(g.nis, g.npairs, L, 1));
   if (phase > P->ws.phase_bytes) {
     if (P->ws.phase) cudaFree(P->ws.phase);
     P->ws.phase = nullptr;
@@ -320,6 +323,8 @@ int ensure_workspace(cr_plan* P, const Grid& g, int L) {
 
 static void plan_free(cr_plan* P) {
   free_hierarchy(P);
+  if (P->ds) ds_tab_free(*P->ds);
+  delete P->ds;
   grid_free(P->obs);
   for (Grid* g : P->level_grids) {
     grid_free(*g);
@@ -408,6 +413,8 @@ static LegArgs<T> leg_args(cr_plan* P, const Grid& g, int L) {
     a.st = g.d_st64b;
     a.npolar = 0;
     a.df = P->fp64_df;
+    a.ds = P->ds;
+    a.nis = g.nis;
     a.ls_df = g.d_ls32;
     a.st_df = g.d_st64b;
     a.npolar_df = g.npolar32;
@@ -581,7 +588,8 @@ int ensure_mr_workspace(cr_plan* P, const Grid& g, int L) {
   const int64_t nlm = n_lm(L), ld_phase = (int64_t)g.nring * (L + 1);
   const int nblk = mr_blocks(g.npairs);
   const int64_t phase = 8 * ld_phase * (int64_t)sizeof(double2);
-  const int64_t partial = 8 * (int64_t)nblk * nlm * (int64_t)sizeof(double2);
+  const int64_t partial = std::max(8 * (int64_t)nblk * nlm * (int64_t)sizeof(double2),
+                                   ds_partial_bytes(g.nis, g.npairs, L, 4));
   if (phase > P->ws_mr.phase_bytes || partial > P->ws_mr.partial_bytes) {
     if (P->capturing) return fail(CR_ESTATE, "FP64 batch: buffers missing (run once outside a capture)");
     if (phase > P->ws_mr.phase_bytes) {
@@ -612,7 +620,8 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
   a.dl = dl_in;
   {
     TimerScope ts(P->timing, P->stream, "legendre_synth_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
-    rc = launch_leg_synth_mr(a, x, nlm, nr, ph, ld_phase, P->stream);
+    rc = ds_use(a) ? launch_ds_synth(a, x, nlm, nr, ph, P->stream)
+                   : launch_leg_synth_mr(a, x, nlm, nr, ph, ld_phase, P->stream);
   }
   for (int r = 0; r < nr && !rc; ++r) {
     RingArgs<double> ra = ring_args<double>(P, g, L);
@@ -623,22 +632,23 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
     rc = launch_ring_fft<double>(ra, 2, P->stream);
   }
   if (rc) return rc;
-  int nb = 0;
-  {
-    TimerScope ts(P->timing, P->stream, "legendre_adjoint_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
-    rc = launch_leg_adjoint_mr(a, ph, ld_phase, nr, part, &nb, P->stream);
+  FinalizeArgs<double> f[8];
+  for (int r = 0; r < nr; ++r) {
+    f[r].L = L;
+    f[r].dl_out = dl_out;
+    f[r].dadd = dadd;
+    f[r].xadd = x + r * nlm;
+    f[r].bsub = bsub ? bsub + r * nlm : nullptr;
+    f[r].out = y + r * nlm;
   }
+  TimerScope ts(P->timing, P->stream, "legendre_adjoint_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
+  if (ds_use(a)) return launch_ds_adjoint(a, ph, nr, reinterpret_cast<double*>(part), f, P->stream);
+  int nb = 0;
+  rc = launch_leg_adjoint_mr(a, ph, ld_phase, nr, part, &nb, P->stream);
   for (int r = 0; r < nr && !rc; ++r) {
-    FinalizeArgs<double> f;
-    f.partial = part + (int64_t)r * nb * nlm;
-    f.nblk = nb;
-    f.L = L;
-    f.dl_out = dl_out;
-    f.dadd = dadd;
-    f.xadd = x + r * nlm;
-    f.bsub = bsub ? bsub + r * nlm : nullptr;
-    f.out = y + r * nlm;
-    rc = launch_leg_finalize<double>(f, P->stream);
+    f[r].partial = part + (int64_t)r * nb * nlm;
+    f[r].nblk = nb;
+    rc = launch_leg_finalize<double>(f[r], P->stream);
   }
   return rc;
 }
@@ -692,6 +702,7 @@ static int tune_stage(cr_plan* P, const Grid& g, int L, int stage, int reps) {
     if (i >= nchoice) continue;
     LegArgs<T> a = leg_args<T>(P, g, L);
     a.df = 0;
+    a.ds = nullptr;  // the shapes are those of the CUDA-core kernels
     a.alm = alm;
     a.rp_synth = a.rp_adj = rps[i];
     a.mt_synth = a.mt_adj = mt;

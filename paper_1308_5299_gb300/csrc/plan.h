@@ -30,6 +30,7 @@ struct Grid {
   int nside = 0;
   int nring = 0;
   int npairs = 0;  // north/south ring pairs (the middle ring pairs with itself)
+  int nis = 0;     // pairs above the equatorial zone of the digit-slice kernels
   int64_t npix = 0;
   int Lseed = -1;  // seeds exist for m <= Lseed
   int Mmax = 1;    // largest FFT size
@@ -123,6 +124,7 @@ struct Level {
 
 namespace cr {
 struct Hierarchy;
+struct DsTab;
 }
 
 struct cr_plan {
@@ -139,6 +141,7 @@ struct cr_plan {
   float* d_c32 = nullptr;
   float* d_c2_32 = nullptr;  // c - 2, FP32 (polar difference form)
   float* d_s32 = nullptr;
+  cr::DsTab* ds = nullptr;   // tables of the digit-slice FP64 kernels
   // operator diagonals (l-indexed, [lmax+1])
   bool has_op = false;
   double* d_bl = nullptr;    // b_l p_l, 0 where C_l = 0
