@@ -59,7 +59,7 @@ constexpr int DS_ORD = 8;                 // orders of the digit products kept
 constexpr double DS_ZEQ = 0.25;           // pairs with z at or below run the one-step recurrence
 constexpr uint32_t DS_WAIT = 1u << 26;    // polls of a bounded mbarrier wait
 constexpr int DS_NONE = 0x3fffffff;       // start index of a pair that never starts
-constexpr uint64_t DS_BIAS = 0x8080808080808080ull;  // 128 in every digit (and half a unit of the dropped byte)
+constexpr uint64_t DS_BIAS = 0x8000000000000080ull;  // zero (sign bit flipped) and half a unit of the dropped byte
 
 // position of m's first k in tables of band limit L: room for
 // (L - m) / 2 + 1 entries each
@@ -151,14 +151,25 @@ __global__ void __launch_bounds__(DST_NT) ds_tab_kernel(DsTab t) {
       const dd2 g = dd_prod(2 * o - 1, 2 * o + 3);
       const dd2 S = dd_div({2.0 * (o * o + o - dm * dm) - 1.0, 0.0}, g);           // e_{o+1}^2 + e_o^2
       const dd2 S1 = dd_div({2.0 * (o * o + o + dm * dm) - 2.0, 0.0}, g);          // 1 - that
+      const dd2 B = dd_mul(A, {-S.h, -S.l});
       t.A[off + k + 1] = A.h;
-      t.B[off + k + 1] = -dd_mul(A, S).h;
+      t.B[off + k + 1] = B.h;
       t.AB[off + k + 1] = dd_mul(A, S1).h;
+      // fixed point: A 2^58 and (B + 4) 2^61 (modulo 2^64); the integer steps
+      // start where A < 31
+      const double n = rint(B.h);
+      t.Ai[off + k + 1] = A.h < 31.5 ? (uint64_t)(__double2ll_rn(A.h * 0x1p58) + __double2ll_rn(A.l * 0x1p58)) : 0;
+      t.Bi[off + k + 1] = A.h < 31.5 ? ((uint64_t)((int64_t)n + 4) << 61) + (uint64_t)__double2ll_rn((B.h - n) * 0x1p61) +
+                                           (uint64_t)__double2ll_rn(B.l * 0x1p61)
+                                     : 0;
     }
     t.sg[off + k] = dd_sqrt(cur).h;
     t.e0[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o), 0.0}), {d(o), 0.0})).h;
     t.e1[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o + 1), 0.0}), {d(o + 1), 0.0})).h;
-    if (k == 0) t.A[off] = t.B[off] = t.AB[off] = 0.0;
+    if (k == 0) {
+      t.A[off] = t.B[off] = t.AB[off] = 0.0;
+      t.Ai[off] = t.Bi[off] = 0;
+    }
   }
 }
 
@@ -167,16 +178,18 @@ void ds_tab_free(DsTab& t) {
   t = DsTab();
 }
 
-// the tables for band limits up to Lc (one allocation, six arrays)
+// the tables for band limits up to Lc (one allocation, eight arrays)
 int ds_tab_build(DsTab& t, int Lc, cudaStream_t st) {
   ds_tab_free(t);
   const int64_t n = ds_len(Lc);
-  CR_CUDA(cudaMalloc(&t.A, 6 * n * sizeof(double)));
+  CR_CUDA(cudaMalloc(&t.A, 8 * n * sizeof(double)));
   t.B = t.A + n;
   t.AB = t.B + n;
   t.sg = t.AB + n;
   t.e0 = t.sg + n;
   t.e1 = t.e0 + n;
+  t.Ai = reinterpret_cast<uint64_t*>(t.e1 + n);
+  t.Bi = t.Ai + n;
   t.Lc = Lc;
   { ds_tab_kernel<<<Lc + 1, DST_NT, 0, st>>>(t); count_launch(); }
   CR_CHECK_LAUNCH("ds_tab_kernel");
@@ -203,9 +216,9 @@ __device__ __forceinline__ uint32_t ds_mn_off(int mn, int k, int MN) {
 
 __device__ __forceinline__ int ds_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
-// round(v 2^62 / 2^(eb - 1023)) + DS_BIAS as 64 bits, |v| < 2^(eb - 1023):
-// the mantissa at bit 62, shifted right by the exponent's distance from the
-// bound.  Bytes 7..1 are the digits + 128; the bias of byte 0 rounds.
+// round(v 2^62 / 2^(eb - 1023)) + DS_BIAS, |v| < 2^(eb - 1023): the mantissa
+// at bit 62, shifted right by the exponent's distance from the bound.  Bytes
+// 7..1 are the digits: the leading one plus 128, the others as they are.
 __device__ __forceinline__ uint64_t ds_fix(double v, int eb) {
   const int hi = __double2hiint(v);
   const uint32_t lo = (uint32_t)__double2loint(v);
@@ -217,24 +230,56 @@ __device__ __forceinline__ uint64_t ds_fix(double v, int eb) {
   return (x ^ s) - s + DS_BIAS;
 }
 
-// digits of weight byte b of 8 values as 8 FP16: 0x6400 | byte is 1024 + byte
-__device__ __forceinline__ uint32_t ds_pair(uint32_t w0, uint32_t w1, int bb) {
-  const uint32_t v = (__byte_perm(w0, w1, bb | ((4 + bb) << 8)) & 0x00ff00ffu) | 0x64006400u;
-  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&v), __half2half2(__ushort_as_half(0x6480)));
-  return *reinterpret_cast<const uint32_t*>(&h);
+// The digits of the sequence (the operand with many values) are FP16
+// subnormals d 2^-24: the bits of an unsigned digit are its value, so it
+// takes a byte permutation and no conversion.  yh, yl: the two words of 8
+// values; calls store(i, digits) for the digits i = 0..6.
+template <typename F>
+__device__ __forceinline__ void ds_digits8(const uint32_t yh[8], const uint32_t yl[8], F store) {
+  uint4 d[DS_DIG];
+  uint32_t* w = reinterpret_cast<uint32_t*>(d);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t h0 = yh[2 * j], h1 = yh[2 * j + 1], l0 = yl[2 * j], l1 = yl[2 * j + 1];
+    const uint32_t a = __byte_perm(h0, h1, 0x7632), b = __byte_perm(h0, h1, 0x5410), c = __byte_perm(l0, l1, 0x7632);
+    // the leading digit: 1024 + byte, less 1152, times 2^-24
+    const uint32_t t = __byte_perm(a, 0x64646464u, 0x4341);
+    const __half2 v = __hfma2(*reinterpret_cast<const __half2*>(&t), __half2half2(__ushort_as_half(0x0001)),
+                              __half2half2(__ushort_as_half(0x8480)));
+    w[0 * 4 + j] = *reinterpret_cast<const uint32_t*>(&v);
+    w[1 * 4 + j] = __byte_perm(a, 0u, 0x4240);
+    w[2 * 4 + j] = __byte_perm(b, 0u, 0x4341);
+    w[3 * 4 + j] = __byte_perm(b, 0u, 0x4240);
+    w[4 * 4 + j] = __byte_perm(c, 0u, 0x4341);
+    w[5 * 4 + j] = __byte_perm(c, 0u, 0x4240);
+    w[6 * 4 + j] = __byte_perm(l0, l1, 0x5410) >> 8 & 0x00ff00ffu;
+  }
+#pragma unroll
+  for (int i = 0; i < DS_DIG; ++i) store(i, d[i]);
 }
-__device__ __forceinline__ uint4 ds_digits8(const uint32_t w[8], int bb) {
-  return make_uint4(ds_pair(w[0], w[1], bb), ds_pair(w[2], w[3], bb), ds_pair(w[4], w[5], bb), ds_pair(w[6], w[7], bb));
-}
-// digit i (0 the most significant) of one value
+// digit i (0 the most significant) of one value of the other operand, signed
+// digits -128..127 of y = ds_fix + DS_SIGNED
+constexpr uint64_t DS_SIGNED = 0x0080808080808000ull;
 __device__ __forceinline__ __half ds_digit(uint64_t y, int i) {
   return __int2half_rn((int)((uint32_t)(y >> (8 * (7 - i))) & 255u) - 128);
 }
 
-// sum_s D_s 256^-s of the eight exact orders, times 256^3
+// high 64 bits of a product, without its lowest partial product and rounded
+// so that the mean error is zero (truncation would bias every step the same way)
+__device__ __forceinline__ uint64_t ds_mulhi(uint64_t a, uint64_t b) {
+  const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+  const uint64_t t1 = (uint64_t)al * bh + 0xC0000000u;
+  const uint64_t t2 = (uint64_t)ah * bl + (uint32_t)t1;
+  return (uint64_t)ah * bh + (t1 >> 32) + (t2 >> 32);
+}
+
+// sum_s D_s 256^-s of the eight orders f = D 2^-24, times 256^3
 __device__ __forceinline__ double ds_collect(const float f[DS_ORD]) {
-  const long long hi = ((long long)((int)f[0] * 256 + (int)f[1]) << 16) + ((int)f[2] * 256 + (int)f[3]);
-  const long long lo = ((long long)(int)f[4] << 24) + ((long long)(int)f[5] << 16) + ((long long)(int)f[6] << 8) + (int)f[7];
+  long long d[DS_ORD];
+#pragma unroll
+  for (int s = 0; s < DS_ORD; ++s) d[s] = (int)(f[s] * 0x1p24f);
+  const long long hi = (d[0] << 24) + (d[1] << 16) + (d[2] << 8) + d[3];
+  const long long lo = (d[4] << 24) + (d[5] << 16) + (d[6] << 8) + d[7];
   // |hi|, |lo| < 2^51: to FP64 through the mantissa of 1.5 2^52
   const double dh = __longlong_as_double(0x4338000000000000ll + hi) - 6755399441055744.0;
   const double dl = __longlong_as_double(0x4338000000000000ll + lo) - 6755399441055744.0;
@@ -274,6 +319,8 @@ struct DsPair {
   double Z[4] = {0.0, 0.0, 0.0, 0.0};  // EQ: Z[0] = z
   int k0 = DS_NONE;                    // first index of the sequence
   int eb = 1023;                       // |q| < 2^(eb - 1023)
+  // integer steps: q 2^62 / 2^(eb - 1023) + 2^63, and z^2 2^64 (EQ: z 2^64)
+  uint64_t Q1 = 1ull << 63, Q2 = 1ull << 63, zi = 0;
 
   // four copies of v + lo that average to it within an eighth of the last place
   __device__ __forceinline__ void dither(double v, double lo) {
@@ -288,6 +335,7 @@ struct DsPair {
     const int64_t o = (int64_t)m * a.ld_seed + p;
     const double z = a.z[p];
     const double zz = z * z;
+    zi = EQ ? __double2ull_rn(z * 0x1p64) : __double2ull_rn(zz * 0x1p64) + (uint64_t)__double2ll_rn(fma(z, z, -zz) * 0x1p64);
     if (EQ) {
       Z[0] = z;
     } else if (polar) {
@@ -344,19 +392,69 @@ struct DsPair {
     const double e = EQ ? c.x * Z[0] : fma(c.x, Z[u & 3], c.y);
     return fma(e, q1, -q2);
   }
+
+  // The same step in 64-bit integers: e + 4 = A z^2 + (B + 4) times 2^61, and
+  // with Q = q + 2^63 (up to the common scale) e q - q' is
+  // 8 mulhi(e + 4, Q) - 4 (e + 4 + Q) - Q' modulo 2^64.
+  __device__ __forceinline__ uint64_t istep(ulonglong2 c) {
+    const uint64_t e = (ds_mulhi(c.x, zi) << 3) + c.y;
+    const uint64_t q = (ds_mulhi(e, Q1) << 3) - ((e + Q1) << 2) - Q2;
+    Q2 = Q1;
+    Q1 = q;
+    return q;
+  }
+
+  // Whether this pair can go on in integers, c0 and c1 being the next two
+  // steps' coefficients: |e| < 4 (it falls with k), and an amplitude at which
+  // the fixed point's 2^-62 of the bound is below FP64's rounding.
+  __device__ __forceinline__ bool can_int(double2 c0, double2 c1) const {
+    if (k0 == DS_NONE) return true;
+    const double e0 = EQ ? c0.x * Z[0] : fma(c0.x, Z[0], c0.y), e1 = EQ ? c1.x * Z[0] : fma(c1.x, Z[0], c1.y);
+    return fabs(e0) < 3.5 && fabs(e1) < 3.5 && max(ds_exp(q1), ds_exp(q2)) >= eb - 10;
+  }
+  __device__ __forceinline__ void to_int() {
+    Q1 = ds_fix(q1, eb) - 0x80;
+    Q2 = ds_fix(q2, eb) - 0x80;
+  }
 };
 
-// Coefficients of the step that produces index k of the sequence.
+// Coefficients of the step that produces index k of the sequence, for the
+// FP64 steps (two doubles) or the integer ones.
 template <bool EQ>
-__device__ __forceinline__ double2 ds_coef(const DsArgs& a, int m, int k, int nk, bool polar) {
-  if (k >= nk) return make_double2(0.0, 0.0);
-  if (EQ) return make_double2(a.c[lm_off(a.Lc, m) + k], 0.0);
-  const int64_t o = ds_off(a.t.Lc, m) + k;
-  return polar ? make_double2(-a.t.A[o], a.t.AB[o]) : make_double2(a.t.A[o], a.t.B[o]);
+__device__ __forceinline__ ulonglong2 ds_coef(const DsArgs& a, int m, int k, int nk, bool polar, bool ints) {
+  if (k >= nk) return make_ulonglong2(0, 0);
+  double2 d = make_double2(0.0, 0.0);
+  if (EQ) {
+    d.x = a.c[lm_off(a.Lc, m) + k];
+    if (ints) return make_ulonglong2(__double2ull_rn(d.x * 0x1p58), 1ull << 63);
+  } else {
+    const int64_t o = ds_off(a.t.Lc, m) + k;
+    if (ints) return make_ulonglong2(a.t.Ai[o], a.t.Bi[o]);
+    d = polar ? make_double2(-a.t.A[o], a.t.AB[o]) : make_double2(a.t.A[o], a.t.B[o]);
+  }
+  return make_ulonglong2((uint64_t)__double_as_longlong(d.x), (uint64_t)__double_as_longlong(d.y));
+}
+__device__ __forceinline__ double2 ds_coef_d(ulonglong2 c) {
+  return make_double2(__longlong_as_double((long long)c.x), __longlong_as_double((long long)c.y));
+}
+
+// At the start of a stage (first index ks, cf its coefficients, one per
+// lane): changes the warp to integer steps once all its pairs can.
+template <bool EQ>
+__device__ __forceinline__ void ds_try_int(const DsArgs& a, DsPair<EQ>& s, int m, int ks, int nk, bool polar, int wmin,
+                                           int wmax, ulonglong2& cf, bool& ints) {
+  if (ints || ks < wmax || wmin == DS_NONE) return;
+  const double2 d = ds_coef_d(cf);
+  const double2 c0 = make_double2(__shfl_sync(0xffffffffu, d.x, 0), __shfl_sync(0xffffffffu, d.y, 0));
+  const double2 c1 = make_double2(__shfl_sync(0xffffffffu, d.x, 1), __shfl_sync(0xffffffffu, d.y, 1));
+  if (!__all_sync(0xffffffffu, fabs(d.x) < 31.0 && s.can_int(c0, c1))) return;
+  s.to_int();
+  ints = true;
+  cf = ds_coef<EQ>(a, m, ks + (threadIdx.x & 31), nk, polar, true);
 }
 
 struct DsShared {
-  double2 sc[4][32];      // recurrence coefficients, one copy per producer warp
+  ulonglong2 sc[4][32];   // recurrence coefficients, one copy per producer warp
   uint64_t full[2], empty[2], done;
   int eb[2][16];          // largest exponents of a block's columns
   uint32_t taddr;
@@ -366,30 +464,28 @@ struct DsShared {
 
 // The 8 values k..k+7 of a warp's sequences as digits: calls store(i, digits)
 // for each digit i.  Idle before the warp's first start; per-lane start tests
-// while some lanes have not started.
+// while some lanes have not started; integer steps once ds_try_int has set
+// `ints`.
 template <bool EQ, typename F>
-__device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const double2* sc, int k, int wmin, int wmax, F store) {
-  if (k + 8 <= wmin) {
-#pragma unroll
-    for (int i = 0; i < DS_DIG; ++i) store(i, make_uint4(0u, 0u, 0u, 0u));
-    return;
-  }
+__device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const ulonglong2* sc, int k, int wmin, int wmax, bool ints,
+                                            F store) {
   uint32_t yh[8], yl[8];
-  if (k >= wmax) {
+  if (ints) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const double q = s.step(sc[u], u);
-      s.q2 = s.q1;
-      s.q1 = q;
-      const uint64_t y = ds_fix(q, s.eb);
+      const uint64_t y = s.istep(sc[u]);
       yh[u] = (uint32_t)(y >> 32);
       yl[u] = (uint32_t)y;
     }
+  } else if (k + 8 <= wmin) {
+#pragma unroll
+    for (int i = 0; i < DS_DIG; ++i) store(i, make_uint4(0u, 0u, 0u, 0u));
+    return;
   } else {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const bool on = k + u >= s.k0;
-      const double q = s.step(sc[u], u);
+      const double q = s.step(ds_coef_d(sc[u]), u);
       s.q2 = on ? s.q1 : s.q2;
       s.q1 = on ? q : s.q1;
       const uint64_t y = on ? ds_fix(q, s.eb) : DS_BIAS;
@@ -397,10 +493,7 @@ __device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const double2* sc, in
       yl[u] = (uint32_t)y;
     }
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) store(i, ds_digits8(yh, 3 - i));
-#pragma unroll
-  for (int i = 4; i < DS_DIG; ++i) store(i, ds_digits8(yl, 7 - i));
+  ds_digits8(yh, yl, store);
 }
 
 // this thread's pair, and the warp's and the CTA's first (and the warp's
@@ -484,8 +577,9 @@ __device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uin
     if (producer) {
       const int64_t offa = lm_off(L, m);
       const int64_t ok_ = ds_off(a.t.Lc, m), oc = lm_off(a.Lc, m);
-      double2 cf = make_double2(0.0, 0.0);
-      if (lane < 16) cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar);
+      bool ints = false;
+      ulonglong2 cf = make_ulonglong2(0, 0);
+      if (lane < 16) cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
       for (int kc = kbeg; kc < nk; kc += DSS_KB, ++nblk) {
         // coefficients of this block: thread = k
         const int k = kc + tid;
@@ -539,7 +633,7 @@ __device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uin
         uint8_t* Bk = Bs + (tid >> 4) * DSS_BSTEP;
 #pragma unroll
         for (int j = 0; j < 4 * NR; ++j) {
-          const uint64_t y = ds_fix(v[j], eb[j]);
+          const uint64_t y = ds_fix(v[j], eb[j]) + DS_SIGNED;
 #pragma unroll
           for (int i = 0; i < DS_DIG; ++i)
             *reinterpret_cast<__half*>(Bk + tc::kmajor_offset(16 * i + j, tid & 15, 16)) = ds_digit(y, i);
@@ -554,17 +648,18 @@ __device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uin
               ok = false;
             }
           }
+          ds_try_int<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, ints);
           __syncwarp();
           if (lane < 16) {
             sh.sc[warp][lane] = cf;
-            cf = ds_coef<EQ>(a, m, ks + 16 + lane, nk, polar);
+            cf = ds_coef<EQ>(a, m, ks + 16 + lane, nk, polar, ints);
           }
           __syncwarp();
           uint8_t* S = sm + stg * DSS_STAGE;
 #pragma unroll
           for (int g = 0; g < 2; ++g) {
             const uint32_t off = tc::kmajor_offset(tid, 8 * g, 16);
-            ds_produce8<EQ>(s, sh.sc[warp] + 8 * g, ks + 8 * g, wmin, wmax, [&](int i, uint4 d) {
+            ds_produce8<EQ>(s, sh.sc[warp] + 8 * g, ks + 8 * g, wmin, wmax, ints, [&](int i, uint4 d) {
               *reinterpret_cast<uint4*>(S + i * (DSS_STAGE / DS_DIG) + off) = d;
             });
           }
@@ -760,7 +855,7 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
   if (producer) {
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
-      const uint64_t y = ds_fix(g[j], sh.eb[0][j] - (s.eb - 1023));
+      const uint64_t y = ds_fix(g[j], sh.eb[0][j] - (s.eb - 1023)) + DS_SIGNED;
 #pragma unroll
       for (int i = 0; i < DS_DIG; ++i)
         *reinterpret_cast<__half*>(sm + tc::kmajor_offset((6 + i) * CB + j, tid, DS_PAIRS)) = ds_digit(y, i);
@@ -813,18 +908,20 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
         }
       }
     };
-    double2 cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar);
+    bool ints = false;
+    ulonglong2 cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
     for (int it = 0; it < nit; ++it) {
       const int ks = kbeg + it * DSA_N;
       if (it > 0) flush(it - 1);
+      ds_try_int<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, ints);
       __syncwarp();
       sh.sc[warp][lane] = cf;
-      cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar);
+      cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar, ints);
       __syncwarp();
 #pragma unroll 1
       for (int gq = 0; gq < DSA_N / 8; ++gq) {
         uint8_t* B = sm + Lay::B0 + ds_mn_off(8 * gq, tid, DSA_N);
-        ds_produce8<EQ>(s, sh.sc[warp] + 8 * gq, ks + 8 * gq, wmin, wmax,
+        ds_produce8<EQ>(s, sh.sc[warp] + 8 * gq, ks + 8 * gq, wmin, wmax, ints,
                         [&](int i, uint4 d) { *reinterpret_cast<uint4*>(B + i * DSA_BD) = d; });
       }
       tc::fence_proxy_async();
