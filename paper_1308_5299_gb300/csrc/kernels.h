@@ -12,7 +12,7 @@ namespace cr {
 struct DsTab {
   double *A = nullptr, *B = nullptr, *AB = nullptr;    // coefficients of the step that produces q_k
   double *sg = nullptr, *e0 = nullptr, *e1 = nullptr;  // sigma_k, and times e_o and e_{o+1}
-  uint64_t *Ai = nullptr, *Bi = nullptr;               // A 2^58, (B + 4) 2^61: the integer steps' coefficients
+  uint64_t *Ai = nullptr, *Bi = nullptr;               // A 2^57, (B + 8) 2^60: the integer steps' coefficients
   int Lc = -1;
 };
 

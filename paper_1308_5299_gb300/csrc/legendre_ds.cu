@@ -52,11 +52,10 @@
 
 namespace cr {
 
-constexpr int DS_PAIRS = 128;             // ring pairs per CTA, one per producer thread
-constexpr int DS_NT = 160;                // four producer warps and the MMA warp
+constexpr int DS_PAIRS = 128;             // ring pairs and threads per CTA
 constexpr int DS_DIG = 7;                 // digits per operand
 constexpr int DS_ORD = 8;                 // orders of the digit products kept
-constexpr double DS_ZEQ = 0.25;           // pairs with z at or below run the one-step recurrence
+constexpr double DS_ZEQ = 0.06;           // pairs with z at or below run the one-step recurrence
 constexpr uint32_t DS_WAIT = 1u << 26;    // polls of a bounded mbarrier wait
 constexpr int DS_NONE = 0x3fffffff;       // start index of a pair that never starts
 constexpr uint64_t DS_BIAS = 0x8000000000000080ull;  // zero (sign bit flipped) and half a unit of the dropped byte
@@ -155,13 +154,14 @@ __global__ void __launch_bounds__(DST_NT) ds_tab_kernel(DsTab t) {
       t.A[off + k + 1] = A.h;
       t.B[off + k + 1] = B.h;
       t.AB[off + k + 1] = dd_mul(A, S1).h;
-      // fixed point: A 2^58 and (B + 4) 2^61 (modulo 2^64); the integer steps
-      // start where A < 31
+      // fixed point: A 2^57 and (B + 8) 2^60 (modulo 2^64); the integer steps
+      // start where A < 100
       const double n = rint(B.h);
-      t.Ai[off + k + 1] = A.h < 31.5 ? (uint64_t)(__double2ll_rn(A.h * 0x1p58) + __double2ll_rn(A.l * 0x1p58)) : 0;
-      t.Bi[off + k + 1] = A.h < 31.5 ? ((uint64_t)((int64_t)n + 4) << 61) + (uint64_t)__double2ll_rn((B.h - n) * 0x1p61) +
-                                           (uint64_t)__double2ll_rn(B.l * 0x1p61)
-                                     : 0;
+      const bool in = A.h < 127.0;
+      t.Ai[off + k + 1] = in ? __double2ull_rn(A.h * 0x1p57) + (uint64_t)__double2ll_rn(A.l * 0x1p57) : 0;
+      t.Bi[off + k + 1] = in ? ((uint64_t)((int64_t)n + 8) << 60) + (uint64_t)__double2ll_rn((B.h - n) * 0x1p60) +
+                                   (uint64_t)__double2ll_rn(B.l * 0x1p60)
+                             : 0;
     }
     t.sg[off + k] = dd_sqrt(cur).h;
     t.e0[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o), 0.0}), {d(o), 0.0})).h;
@@ -197,12 +197,6 @@ int ds_tab_build(DsTab& t, int Lc, cudaStream_t st) {
 }
 
 // ---- device helpers ----------------------------------------------------------
-
-__device__ __forceinline__ void ds_arrive(uint64_t* mbar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(mbar)) : "memory");
-}
-// the four producer warps
-__device__ __forceinline__ void ds_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 // kind::f16 instruction descriptor, FP16 inputs, FP32 accumulation
 __host__ __device__ constexpr uint32_t ds_idesc(int M, int N) {
@@ -264,13 +258,14 @@ __device__ __forceinline__ __half ds_digit(uint64_t y, int i) {
   return __int2half_rn((int)((uint32_t)(y >> (8 * (7 - i))) & 255u) - 128);
 }
 
-// high 64 bits of a product, without its lowest partial product and rounded
-// so that the mean error is zero (truncation would bias every step the same way)
-__device__ __forceinline__ uint64_t ds_mulhi(uint64_t a, uint64_t b) {
+// High 64 bits of a product from its three upper partial products, plus
+// `up`: each of the two middle ones loses half a unit to truncation and the
+// lowest product a quarter, so `up` = 1, 1, 1, 2 in turn keeps the mean error
+// of four steps at zero (a bias would push every step the same way).
+__device__ __forceinline__ uint64_t ds_mulhi(uint64_t a, uint64_t b, uint32_t up) {
   const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
-  const uint64_t t1 = (uint64_t)al * bh + 0xC0000000u;
-  const uint64_t t2 = (uint64_t)ah * bl + (uint32_t)t1;
-  return (uint64_t)ah * bh + (t1 >> 32) + (t2 >> 32);
+  const uint64_t mid = (uint64_t)__umulhi(al, bh) + __umulhi(ah, bl) + up;
+  return (uint64_t)ah * bh + mid;
 }
 
 // sum_s D_s 256^-s of the eight orders f = D 2^-24, times 256^3
@@ -312,42 +307,31 @@ __device__ __forceinline__ void ds_ld_orders(uint32_t taddr, float f[DS_ORD][4])
                : "memory");
 }
 
-// One ring pair's sequence: state, argument and bound.
+// One ring pair's sequence.  The first few steps, where the functions can grow
+// by large factors, run in FP64 (mode 0); then in integers with an exponent
+// per pair (mode 1: (Q - 2^63) 2^-62 2^(eb - 1023 - x), x falling to zero as
+// the functions grow out of 2^-60); then, when every pair of the warp has
+// x = 0, in plain fixed point (mode 2).
 template <bool EQ>
 struct DsPair {
-  double q1 = 0.0, q2 = 0.0;
-  double Z[4] = {0.0, 0.0, 0.0, 0.0};  // EQ: Z[0] = z
+  double q1 = 0.0, q2 = 0.0, Z = 0.0;  // mode 0; Z = z^2 or 1 - z^2 (EQ: z)
+  uint64_t Q1 = 1ull << 63, Q2 = 1ull << 63, zi = 0;  // zi = z^2 2^64 (EQ: z 2^64)
+  int x = 0;
   int k0 = DS_NONE;                    // first index of the sequence
   int eb = 1023;                       // |q| < 2^(eb - 1023)
-  // integer steps: q 2^62 / 2^(eb - 1023) + 2^63, and z^2 2^64 (EQ: z 2^64)
-  uint64_t Q1 = 1ull << 63, Q2 = 1ull << 63, zi = 0;
+  bool calm = true;                    // |e| at k0 is small enough for integer steps
 
-  // four copies of v + lo that average to it within an eighth of the last place
-  __device__ __forceinline__ void dither(double v, double lo) {
-    const double up = __longlong_as_double(__double_as_longlong(v) + 1) - v;
-    const int t = (int)rint(4.0 * lo / up);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) Z[j] = v + (j < abs(t) ? copysign(up, lo) : 0.0);
-  }
-
-  // p: pair; polar: the warp runs on 1 - z^2
+  // p: pair; polar: FP64 steps on 1 - z^2, A + B
   __device__ __forceinline__ void load(const DsArgs& a, int m, int p, bool polar) {
     const int64_t o = (int64_t)m * a.ld_seed + p;
+    const int ls = a.ls[o];
+    const double2 st = a.st[o];
     const double z = a.z[p];
     const double zz = z * z;
     zi = EQ ? __double2ull_rn(z * 0x1p64) : __double2ull_rn(zz * 0x1p64) + (uint64_t)__double2ll_rn(fma(z, z, -zz) * 0x1p64);
-    if (EQ) {
-      Z[0] = z;
-    } else if (polar) {
-      const double w = 1.0 - z;  // exact for z >= 1/2
-      const double w2 = w * w, e = fma(w, w, -w2), t = 2.0 * w;
-      const double s = t - w2;
-      dither(s, ((t - s) - w2) - e);
-    } else {
-      dither(zz, fma(z, z, -zz));
-    }
+    const double w = 1.0 - z;
+    Z = EQ ? z : polar ? fma(-w, w, 2.0 * w) : zz;
     const int L = a.L;
-    const int ls = a.ls[o];
     // bounds |P~_lm| <= sqrt((2 l + 1) / 4 pi) and 0.3 (l + 1)^(1/4) / sqrt(sin)
     // (the supremum over l, m and z is 0.29965 at every l tried to 3000),
     // over the rescaling at its smallest
@@ -355,67 +339,78 @@ struct DsPair {
     float b = fminf(0.2821f * sqrtf(2.f * fl), 0.305f * sqrtf(sqrtf(fl)) * rsqrtf(sqrtf(fmaxf((float)(1.0 - zz), 1e-20f))));
     if (EQ) {
       const int64_t c = lm_off(a.Lc, m) + (L - m);
-      const double s = fmin(a.s[c], L > m ? a.s[c - 1] : 1.0);
-      b /= (float)fmin(s, 1.0);
+      b /= fminf((float)fmin(a.s[c], L > m ? a.s[c - 1] : 1.0), 1.f);
     } else {
       b /= (float)z;
     }
     eb = 1023 + (int)ceilf(log2f(b) + 0.1f);
     if (ls > L) return;
-    const double2 st = a.st[o];
+    const int64_t oc = lm_off(a.Lc, m) + (ls - m);
+    const double c = ls > m ? a.c[oc] : 0.0;
     if (EQ) {
       k0 = ls - m;
       q1 = st.x;
       q2 = st.y;
+      calm = k0 > 0 && c * z < 7.0;
       return;
     }
     // (q_{k0-1}, q_{k0-2}) from the one-step state (Q_{ls-1}, Q_{ls-2})
     k0 = (ls - m) >> 1;
-    const int64_t oc = lm_off(a.Lc, m) + (ls - m), ok = ds_off(a.t.Lc, m) + k0;
-    const double Q = fma((ls > m ? a.c[oc] : 0.0) * z, st.x, -st.y);
-    const double P = a.s[oc] * Q;
-    double qk;
-    if ((ls - m) & 1) {
-      if (k0 > 0) q1 = a.s[oc - 2] * st.y / (z * a.t.sg[ok - 1]);
-      qk = P / (z * a.t.sg[ok]);
-    } else {
-      if (k0 > 0) q1 = a.s[oc - 1] * st.x / (z * a.t.sg[ok - 1]);
-      qk = (k0 > 0 ? P - a.t.e1[ok - 1] * q1 : P) / a.t.e0[ok];
-    }
-    // the second value, such that the recurrence's next step returns q_{k0}
+    const int64_t ok = ds_off(a.t.Lc, m) + k0;
+    const double P = a.s[oc] * fma(c * z, st.x, -st.y);
     const double A = a.t.A[ok], B = polar ? a.t.AB[ok] : a.t.B[ok];
-    const double Zk = (k0 & 2) ? ((k0 & 1) ? Z[3] : Z[2]) : ((k0 & 1) ? Z[1] : Z[0]);
-    q2 = fma(fma(polar ? -A : A, Zk, B), q1, -qk);
+    const bool odd = (ls - m) & 1;
+    double n1 = 0.0, d1 = 1.0;  // q_{k0-1} = n1 / d1
+    if (k0 > 0) {
+      n1 = odd ? a.s[oc - 2] * st.y : a.s[oc - 1] * st.x;
+      d1 = z * a.t.sg[ok - 1];
+    }
+    q1 = n1 / d1;
+    const double qk = (odd ? P : fma(k0 > 0 ? -a.t.e1[ok - 1] : 0.0, q1, P)) / (odd ? z * a.t.sg[ok] : a.t.e0[ok]);
+    // the second value, such that the recurrence's next step returns q_{k0}
+    const double e = fma(polar ? -A : A, Z, B);
+    q2 = fma(e, q1, -qk);
+    calm = k0 > 0 && A < 100.0 && fabs(e) < 7.0;
   }
 
-  __device__ __forceinline__ double step(double2 c, int u) {
-    const double e = EQ ? c.x * Z[0] : fma(c.x, Z[u & 3], c.y);
-    return fma(e, q1, -q2);
+  __device__ __forceinline__ double step(double2 c) { return fma(EQ ? c.x * Z : fma(c.x, Z, c.y), q1, -q2); }
+
+  // The same step in 64-bit integers: e + 8 = A z^2 + (B + 8) times 2^60, and
+  // with Q = q + 2^63 (up to the common scale) e q - q' + 2^63 is
+  // 16 mulhi(e + 8, Q) - 8 (e + 8 + Q) - Q' modulo 2^64.
+  __device__ __forceinline__ uint64_t istep(ulonglong2 c, int u) const {
+    const uint32_t up = (u & 3) == 3 ? 2u : 1u;
+    const uint64_t e = (ds_mulhi(c.x, zi, up) << 3) + c.y;
+    const uint64_t r = 0 - ((e + Q1) << 3) - Q2;  // beside the product
+    return (ds_mulhi(e, Q1, up) << 4) + r;
   }
 
-  // The same step in 64-bit integers: e + 4 = A z^2 + (B + 4) times 2^61, and
-  // with Q = q + 2^63 (up to the common scale) e q - q' is
-  // 8 mulhi(e + 4, Q) - 4 (e + 4 + Q) - Q' modulo 2^64.
-  __device__ __forceinline__ uint64_t istep(ulonglong2 c) {
-    const uint64_t e = (ds_mulhi(c.x, zi) << 3) + c.y;
-    const uint64_t q = (ds_mulhi(e, Q1) << 3) - ((e + Q1) << 2) - Q2;
-    Q2 = Q1;
-    Q1 = q;
-    return q;
-  }
-
-  // Whether this pair can go on in integers, c0 and c1 being the next two
-  // steps' coefficients: |e| < 4 (it falls with k), and an amplitude at which
-  // the fixed point's 2^-62 of the bound is below FP64's rounding.
-  __device__ __forceinline__ bool can_int(double2 c0, double2 c1) const {
+  // mode 0 -> 1: whether this pair can (c0, c1: the coefficients of the next
+  // two steps; |e| falls with k), and the change, to at most 2^55
+  __device__ __forceinline__ bool can_int(double2 c0, double2 c1, int ks) const {
     if (k0 == DS_NONE) return true;
-    const double e0 = EQ ? c0.x * Z[0] : fma(c0.x, Z[0], c0.y), e1 = EQ ? c1.x * Z[0] : fma(c1.x, Z[0], c1.y);
-    return fabs(e0) < 3.5 && fabs(e1) < 3.5 && max(ds_exp(q1), ds_exp(q2)) >= eb - 10;
+    if (k0 > ks) return calm;
+    const double e0 = EQ ? c0.x * Z : fma(c0.x, Z, c0.y), e1 = EQ ? c1.x * Z : fma(c1.x, Z, c1.y);
+    return fabs(e0) < 7.0 && fabs(e1) < 7.0;
   }
   __device__ __forceinline__ void to_int() {
-    Q1 = ds_fix(q1, eb) - 0x80;
-    Q2 = ds_fix(q2, eb) - 0x80;
+    x = k0 == DS_NONE ? 0 : max(0, eb - max(ds_exp(q1), ds_exp(q2)) - 8);
+    Q1 = ds_fix(q1, eb - x) - 0x80;
+    Q2 = ds_fix(q2, eb - x) - 0x80;
   }
+  __device__ __forceinline__ void shift(int s) {
+    constexpr uint64_t off = 1ull << 63;
+    Q1 = (uint64_t)((int64_t)(Q1 ^ off) >> s) ^ off;
+    Q2 = (uint64_t)((int64_t)(Q2 ^ off) >> s) ^ off;
+    x -= s;
+  }
+  // bits of the larger of the two values, 32 to 63
+  __device__ __forceinline__ int bits() const {
+    const int h1 = (int)((uint32_t)(Q1 >> 32) ^ 0x80000000u), h2 = (int)((uint32_t)(Q2 >> 32) ^ 0x80000000u);
+    return 64 - __clz((h1 ^ (h1 >> 31)) | (h2 ^ (h2 >> 31)));
+  }
+  // back to at most 2^55: two steps with |e| < 8 stay below 2^62
+  __device__ __forceinline__ void renorm() { shift(min(x, max(0, bits() - 55))); }
 };
 
 // Coefficients of the step that produces index k of the sequence, for the
@@ -426,7 +421,7 @@ __device__ __forceinline__ ulonglong2 ds_coef(const DsArgs& a, int m, int k, int
   double2 d = make_double2(0.0, 0.0);
   if (EQ) {
     d.x = a.c[lm_off(a.Lc, m) + k];
-    if (ints) return make_ulonglong2(__double2ull_rn(d.x * 0x1p58), 1ull << 63);
+    if (ints) return make_ulonglong2(__double2ull_rn(d.x * 0x1p57), 1ull << 63);
   } else {
     const int64_t o = ds_off(a.t.Lc, m) + k;
     if (ints) return make_ulonglong2(a.t.Ai[o], a.t.Bi[o]);
@@ -439,41 +434,47 @@ __device__ __forceinline__ double2 ds_coef_d(ulonglong2 c) {
 }
 
 // At the start of a stage (first index ks, cf its coefficients, one per
-// lane): changes the warp to integer steps once all its pairs can.
+// lane): the warp's next mode, once all its pairs are fit for it.
 template <bool EQ>
-__device__ __forceinline__ void ds_try_int(const DsArgs& a, DsPair<EQ>& s, int m, int ks, int nk, bool polar, int wmin,
-                                           int wmax, ulonglong2& cf, bool& ints) {
-  if (ints || ks < wmax || wmin == DS_NONE) return;
-  const double2 d = ds_coef_d(cf);
-  const double2 c0 = make_double2(__shfl_sync(0xffffffffu, d.x, 0), __shfl_sync(0xffffffffu, d.y, 0));
-  const double2 c1 = make_double2(__shfl_sync(0xffffffffu, d.x, 1), __shfl_sync(0xffffffffu, d.y, 1));
-  if (!__all_sync(0xffffffffu, fabs(d.x) < 31.0 && s.can_int(c0, c1))) return;
-  s.to_int();
-  ints = true;
-  cf = ds_coef<EQ>(a, m, ks + (threadIdx.x & 31), nk, polar, true);
+__device__ __forceinline__ void ds_mode(const DsArgs& a, DsPair<EQ>& s, int m, int ks, int nk, bool polar, int wmin,
+                                        int wmax, ulonglong2& cf, int& mode) {
+  if (mode == 2 || wmin == DS_NONE) return;
+  if (mode == 0) {
+    const double2 d = ds_coef_d(cf);
+    const double2 c0 = make_double2(__shfl_sync(0xffffffffu, d.x, 0), __shfl_sync(0xffffffffu, d.y, 0));
+    const double2 c1 = make_double2(__shfl_sync(0xffffffffu, d.x, 1), __shfl_sync(0xffffffffu, d.y, 1));
+    const bool fit = fabs(d.x) < 100.0 || wmin > ks + 31;  // pairs yet to start know their own coefficient
+    if (!__all_sync(0xffffffffu, fit && s.can_int(c0, c1, ks))) return;
+    s.to_int();
+    mode = 1;
+    cf = ds_coef<EQ>(a, m, ks + (threadIdx.x & 31), nk, polar, true);
+  }
+  // plain fixed point: all started, and what the shift leaves is above FP64's precision
+  if (ks >= wmax && __all_sync(0xffffffffu, s.k0 == DS_NONE || s.x == 0 || s.bits() - s.x >= 51)) {
+    s.shift(s.x);
+    mode = 2;
+  }
 }
 
 struct DsShared {
-  ulonglong2 sc[4][32];   // recurrence coefficients, one copy per producer warp
-  uint64_t full[2], empty[2], done;
+  ulonglong2 sc[4][32];   // recurrence coefficients, one copy per warp
+  uint64_t done;
   int eb[2][16];          // largest exponents of a block's columns
   uint32_t taddr;
   int kmin;
-  volatile int abort_;
 };
 
 // The 8 values k..k+7 of a warp's sequences as digits: calls store(i, digits)
-// for each digit i.  Idle before the warp's first start; per-lane start tests
-// while some lanes have not started; integer steps once ds_try_int has set
-// `ints`.
+// for each digit i.  Nothing before the warp's first start.
 template <bool EQ, typename F>
-__device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const ulonglong2* sc, int k, int wmin, int wmax, bool ints,
-                                            F store) {
+__device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const ulonglong2* sc, int k, int wmin, int mode, F store) {
   uint32_t yh[8], yl[8];
-  if (ints) {
+  if (mode == 2) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const uint64_t y = s.istep(sc[u]);
+      const uint64_t y = s.istep(sc[u], u);
+      s.Q2 = s.Q1;
+      s.Q1 = y;
       yh[u] = (uint32_t)(y >> 32);
       yl[u] = (uint32_t)y;
     }
@@ -481,11 +482,23 @@ __device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const ulonglong2* sc,
 #pragma unroll
     for (int i = 0; i < DS_DIG; ++i) store(i, make_uint4(0u, 0u, 0u, 0u));
     return;
+  } else if (mode == 1) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool on = k + u >= s.k0;
+      const uint64_t q = s.istep(sc[u], u);
+      s.Q2 = on ? s.Q1 : s.Q2;
+      s.Q1 = on ? q : s.Q1;
+      const uint64_t y = on ? (uint64_t)((int64_t)(q ^ (1ull << 63)) >> min(s.x, 63)) ^ (1ull << 63) : 1ull << 63;
+      yh[u] = (uint32_t)(y >> 32);
+      yl[u] = (uint32_t)y;
+      if (u & 1) s.renorm();
+    }
   } else {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const bool on = k + u >= s.k0;
-      const double q = s.step(ds_coef_d(sc[u]), u);
+      const double q = s.step(ds_coef_d(sc[u]));
       s.q2 = on ? s.q1 : s.q2;
       s.q1 = on ? q : s.q1;
       const uint64_t y = on ? ds_fix(q, s.eb) : DS_BIAS;
@@ -500,136 +513,129 @@ __device__ __forceinline__ void ds_produce8(DsPair<EQ>& s, const ulonglong2* sc,
 // last) start index
 template <bool EQ>
 __device__ __forceinline__ void ds_setup(const DsArgs& a, DsShared& sh, DsPair<EQ>& s, int m, int p, int pend,
-                                         bool producer, bool* polar, int* wmin, int* wmax) {
+                                         bool* polar, int* wmin, int* wmax) {
+  // one form per warp, from its last pair's cosine
   *polar = false;
-  if (producer) {
-    // one form per warp, from its last pair's cosine
-    const int wl = min((p | 31), pend - 1);
-    if (!EQ && p < pend) {
-      const double zl = a.z[wl];
-      *polar = zl * zl > 0.5;
-    }
-    *polar = __any_sync(0xffffffffu, *polar);
-    if (p < pend) s.load(a, m, p, *polar);
+  if (!EQ) {
+    const double zl = a.z[min(p | 31, pend - 1)];
+    *polar = __any_sync(0xffffffffu, zl * zl > 0.5);
   }
+  if (p < pend) s.load(a, m, p, *polar);
   *wmin = __reduce_min_sync(0xffffffffu, s.k0);
   *wmax = __reduce_max_sync(0xffffffffu, s.k0 == DS_NONE ? 0 : s.k0);
-  if (threadIdx.x == 0) {
-    sh.kmin = DS_NONE;
-    sh.abort_ = 0;
-  }
+  if (threadIdx.x == 0) sh.kmin = DS_NONE;
   __syncthreads();
-  if (producer && (threadIdx.x & 31) == 0) atomicMin(&sh.kmin, *wmin);
+  if ((threadIdx.x & 31) == 0) atomicMin(&sh.kmin, *wmin);
   __syncthreads();
 }
 
+// wait for the MMAs committed with phase `n`; once a wait has given up none
+// is tried again (the results are marked, the barriers still pair up)
+__device__ __forceinline__ void ds_wait(DsShared& sh, int n, bool& ok) {
+  if (ok) ok = tc::mbar_wait(&sh.done, n & 1, DS_WAIT);
+}
+
 // ---- synthesis ---------------------------------------------------------------
-// CTA: one m, 128 ring pairs (tensor-core rows), up to NR right-hand sides.
-// A operand: the pairs' digits, 16 sequence values per stage (two stages).
-// B operand: the digits of (c_k, d_k) x (Re, Im) of the right-hand sides, 16
-// columns per digit, for a block of 128 k with one exponent per column.  The
-// accumulator of digit pair (i, j) starts at column 16 i, so equal orders add
-// up in place.  After each block the four producer warps collect the eight
-// orders of their own pairs into FP64 sums.
+// CTA: one m, 128 ring pairs (tensor-core rows, one per thread), up to NR
+// right-hand sides.  A operand: the pairs' digits, 16 sequence values at a
+// time.  B operand: the digits of (c_k, d_k) x (Re, Im) of the right-hand
+// sides, 16 columns per digit, for a block of DSS_KB k with one exponent per
+// column.  The accumulator of digit pair (i, j) starts at column 16 i, so
+// equal orders add up in place.  After each block the warps collect the eight
+// orders of their own pairs into FP64 sums.  Four CTAs per SM (53 KB of
+// shared memory, 128 tensor-memory columns and 128 registers each): while one
+// waits for its products the others step their recurrences.
 constexpr int DSS_STAGE = DS_DIG * DS_PAIRS * 16 * 2;     // 28 KB
 constexpr int DSS_BSTEP = 16 * DS_ORD * 16 * 2;           // 16 columns x 8 digits (the last zero) x K 16
-constexpr int DSS_KB = 128;                               // k per block
-constexpr int DSS_SMEM = 2 * DSS_STAGE + (DSS_KB / 16) * DSS_BSTEP;
+constexpr int DSS_KB = 96;                                // k per block
+constexpr int DSS_SMEM = DSS_STAGE + (DSS_KB / 16) * DSS_BSTEP;
 constexpr int DSS_TMEM = 128;
 
 template <int NR, bool EQ>
 __device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uint8_t* sm, int base, int pend) {
   const int m = blockIdx.y, L = a.L;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool producer = warp < 4;
   const int p = base + tid;
   DsPair<EQ> s;
   bool polar;
   int wmin, wmax;
-  ds_setup<EQ>(a, sh, s, m, p, pend, producer, &polar, &wmin, &wmax);
+  ds_setup<EQ>(a, sh, s, m, p, pend, &polar, &wmin, &wmax);
   const int nk = EQ ? L - m + 1 : (L - m) / 2 + 1;
-  const int kbeg = sh.kmin & ~3;
-  const bool any = sh.kmin < nk;
-  uint8_t* Bs = sm + 2 * DSS_STAGE;
+  const int kbeg = sh.kmin;
+  uint8_t* Bs = sm + DSS_STAGE;
   double acc[4 * NR];
 #pragma unroll
   for (int j = 0; j < 4 * NR; ++j) acc[j] = 0.0;
   bool ok = true;
-  uint32_t taddr = 0;
-  if (any) {
-    for (int e = tid; e < (DSS_KB / 16) * DSS_BSTEP / 16; e += DS_NT)
+  if (kbeg < nk) {
+    for (int e = tid; e < (DSS_KB / 16) * DSS_BSTEP / 16; e += DS_PAIRS)
       reinterpret_cast<uint4*>(Bs)[e] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < 32) sh.eb[tid >> 4][tid & 15] = 0;
-    if (warp == 4) tc::tmem_alloc(&sh.taddr, DSS_TMEM);
+    if (warp == 0) tc::tmem_alloc(&sh.taddr, DSS_TMEM);
     if (tid == 0) {
-      for (int i = 0; i < 2; ++i) {
-        tc::mbar_init(&sh.full[i], 128);
-        tc::mbar_init(&sh.empty[i], 1);
-      }
       tc::mbar_init(&sh.done, 1);
       tc::mbar_fence_init();
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    taddr = sh.taddr;
-    int gst = 0, nblk = 0;  // stages and blocks so far
-    if (producer) {
-      const int64_t offa = lm_off(L, m);
-      const int64_t ok_ = ds_off(a.t.Lc, m), oc = lm_off(a.Lc, m);
-      bool ints = false;
-      ulonglong2 cf = make_ulonglong2(0, 0);
-      if (lane < 16) cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
-      for (int kc = kbeg; kc < nk; kc += DSS_KB, ++nblk) {
-        // coefficients of this block: thread = k
-        const int k = kc + tid;
-        double v[4 * NR];
+    const uint32_t taddr = sh.taddr;
+    const int64_t offa = lm_off(L, m);
+    const int64_t ok_ = ds_off(a.t.Lc, m), oc = lm_off(a.Lc, m);
+    int mode = 0, gst = 0, nblk = 0;  // stages and blocks so far
+    ulonglong2 cf = make_ulonglong2(0, 0);
+    if (lane < 16) cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
+    for (int kc = kbeg; kc < nk; kc += DSS_KB, ++nblk) {
+      // coefficients of this block: thread = k
+      const int k = kc + tid;
+      double v[4 * NR];
 #pragma unroll
-        for (int j = 0; j < 4 * NR; ++j) v[j] = 0.0;
-        if (k < nk) {
-          if (EQ) {
-            const double f = a.s[oc + k] * (a.dl ? a.dl[m + k] : 1.0);
+      for (int j = 0; j < 4 * NR; ++j) v[j] = 0.0;
+      if (k < nk && tid < DSS_KB) {
+        if (EQ) {
+          const double f = a.s[oc + k] * (a.dl ? a.dl[m + k] : 1.0);
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
-              if (r < a.nr) {
-                const double2 x = a.alm[r * a.ld_alm + offa + k];
-                const int odd = 2 * (k & 1);
-                v[4 * r + 0] = odd ? 0.0 : f * x.x;
-                v[4 * r + 1] = odd ? 0.0 : f * x.y;
-                v[4 * r + 2] = odd ? f * x.x : 0.0;
-                v[4 * r + 3] = odd ? f * x.y : 0.0;
-              }
-          } else {
-            const int l = m + 2 * k;  // a_l, a_{l+1} = a_o, a_{l+2}
-            const double f0 = a.t.e0[ok_ + k] * (a.dl ? a.dl[l] : 1.0);
-            const double f1 = l + 1 <= L ? a.t.sg[ok_ + k] * (a.dl ? a.dl[l + 1] : 1.0) : 0.0;
-            const double f2 = l + 2 <= L ? a.t.e1[ok_ + k] * (a.dl ? a.dl[l + 2] : 1.0) : 0.0;
+          for (int r = 0; r < NR; ++r)
+            if (r < a.nr) {
+              const double2 x = a.alm[r * a.ld_alm + offa + k];
+              const bool odd = k & 1;
+              v[4 * r + 0] = odd ? 0.0 : f * x.x;
+              v[4 * r + 1] = odd ? 0.0 : f * x.y;
+              v[4 * r + 2] = odd ? f * x.x : 0.0;
+              v[4 * r + 3] = odd ? f * x.y : 0.0;
+            }
+        } else {
+          const int l = m + 2 * k;  // a_l, a_{l+1} = a_o, a_{l+2}
+          const double f0 = a.t.e0[ok_ + k] * (a.dl ? a.dl[l] : 1.0);
+          const double f1 = l + 1 <= L ? a.t.sg[ok_ + k] * (a.dl ? a.dl[l + 1] : 1.0) : 0.0;
+          const double f2 = l + 2 <= L ? a.t.e1[ok_ + k] * (a.dl ? a.dl[l + 2] : 1.0) : 0.0;
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
-              if (r < a.nr) {
-                const double2* x = a.alm + r * a.ld_alm + offa + 2 * k;
-                const double2 x0 = x[0];
-                const double2 x1 = l + 1 <= L ? x[1] : make_double2(0.0, 0.0);
-                const double2 x2 = l + 2 <= L ? x[2] : make_double2(0.0, 0.0);
-                v[4 * r + 0] = fma(f0, x0.x, f2 * x2.x);
-                v[4 * r + 1] = fma(f0, x0.y, f2 * x2.y);
-                v[4 * r + 2] = f1 * x1.x;
-                v[4 * r + 3] = f1 * x1.y;
-              }
-          }
-          if (m == 0) {
-#pragma unroll
-            for (int r = 0; r < NR; ++r) v[4 * r + 1] = v[4 * r + 3] = 0.0;
-          }
+          for (int r = 0; r < NR; ++r)
+            if (r < a.nr) {
+              const double2* x = a.alm + r * a.ld_alm + offa + 2 * k;
+              const double2 x0 = x[0];
+              const double2 x1 = l + 1 <= L ? x[1] : make_double2(0.0, 0.0);
+              const double2 x2 = l + 2 <= L ? x[2] : make_double2(0.0, 0.0);
+              v[4 * r + 0] = fma(f0, x0.x, f2 * x2.x);
+              v[4 * r + 1] = fma(f0, x0.y, f2 * x2.y);
+              v[4 * r + 2] = f1 * x1.x;
+              v[4 * r + 3] = f1 * x1.y;
+            }
         }
-        int* eb = sh.eb[nblk & 1];
+        if (m == 0) {
 #pragma unroll
-        for (int j = 0; j < 4 * NR; ++j) {
-          const int e = __reduce_max_sync(0xffffffffu, ds_exp(v[j]));
-          if (lane == 0) atomicMax(&eb[j], e + 1);  // |v| < 2^(eb - 1023); 2048: not finite
+          for (int r = 0; r < NR; ++r) v[4 * r + 1] = v[4 * r + 3] = 0.0;
         }
-        ds_bar();
-        if (tid < 16) sh.eb[(nblk + 1) & 1][tid] = 0;  // last read before this barrier
+      }
+      int* eb = sh.eb[nblk & 1];
+#pragma unroll
+      for (int j = 0; j < 4 * NR; ++j) {
+        const int e = __reduce_max_sync(0xffffffffu, ds_exp(v[j]));
+        if (lane == 0) atomicMax(&eb[j], e + 1);  // |v| < 2^(eb - 1023); 2048: not finite
+      }
+      __syncthreads();
+      if (tid < 16) sh.eb[(nblk + 1) & 1][tid] = 0;  // last read before this barrier
+      if (tid < DSS_KB) {
         uint8_t* Bk = Bs + (tid >> 4) * DSS_BSTEP;
 #pragma unroll
         for (int j = 0; j < 4 * NR; ++j) {
@@ -638,105 +644,72 @@ __device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uin
           for (int i = 0; i < DS_DIG; ++i)
             *reinterpret_cast<__half*>(Bk + tc::kmajor_offset(16 * i + j, tid & 15, 16)) = ds_digit(y, i);
         }
-        const int nst = min(DSS_KB / 16, (nk - kc + 15) / 16);
-        for (int st = 0; st < nst; ++st, ++gst) {
-          const int stg = gst & 1, ks = kc + 16 * st;
-          if (gst >= 2 && ok) {
-            const bool w = tc::mbar_wait(&sh.empty[stg], ((gst >> 1) - 1) & 1, DS_WAIT);
-            if (!__all_sync(0xffffffffu, w)) {
-              if (lane == 0) sh.abort_ = 1;
-              ok = false;
-            }
-          }
-          ds_try_int<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, ints);
-          __syncwarp();
-          if (lane < 16) {
-            sh.sc[warp][lane] = cf;
-            cf = ds_coef<EQ>(a, m, ks + 16 + lane, nk, polar, ints);
-          }
-          __syncwarp();
-          uint8_t* S = sm + stg * DSS_STAGE;
-#pragma unroll
-          for (int g = 0; g < 2; ++g) {
-            const uint32_t off = tc::kmajor_offset(tid, 8 * g, 16);
-            ds_produce8<EQ>(s, sh.sc[warp] + 8 * g, ks + 8 * g, wmin, wmax, ints, [&](int i, uint4 d) {
-              *reinterpret_cast<uint4*>(S + i * (DSS_STAGE / DS_DIG) + off) = d;
-            });
-          }
-          tc::fence_proxy_async();
-          tc::fence_before_sync();
-          ds_arrive(&sh.full[stg]);
+      }
+      const int nst = min(DSS_KB / 16, (nk - kc + 15) / 16);
+      for (int st = 0; st < nst; ++st, ++gst) {
+        const int ks = kc + 16 * st;
+        ds_mode<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, mode);
+        __syncwarp();
+        if (lane < 16) {
+          sh.sc[warp][lane] = cf;
+          cf = ds_coef<EQ>(a, m, ks + 16 + lane, nk, polar, mode > 0);
         }
-        if (ok) {
-          const bool w = tc::mbar_wait(&sh.done, nblk & 1, DS_WAIT);
-          if (!__all_sync(0xffffffffu, w)) {
-            if (lane == 0) sh.abort_ = 1;
-            ok = false;
-          }
+        __syncwarp();
+        if (st > 0) ds_wait(sh, gst - 1, ok);
+#pragma unroll 1
+        for (int g = 0; g < 2; ++g) {
+          uint8_t* S = sm + tc::kmajor_offset(tid, 8 * g, 16);
+          ds_produce8<EQ>(s, sh.sc[warp] + 8 * g, ks + 8 * g, wmin, mode,
+                          [&](int i, uint4 d) { *reinterpret_cast<uint4*>(S + i * (DSS_STAGE / DS_DIG)) = d; });
         }
-        if (ok) {
+        tc::fence_proxy_async();
+        tc::fence_before_sync();
+        __syncthreads();
+        if (tid == 0) {
           tc::fence_after_sync();
-          const uint32_t tw = taddr + ((uint32_t)(warp * 32) << 16);
-          const bool on = kc + DSS_KB > s.k0;
+          const uint32_t sa = tc::smem_addr(sm);
+          const uint64_t bd = tc::smem_desc(tc::smem_addr(Bs + st * DSS_BSTEP), 128, 256);
 #pragma unroll
-          for (int r = 0; r < NR; ++r) {
-            if (r < a.nr) {
-              float f[DS_ORD][4];
-              ds_ld_orders(tw + 4 * r, f);
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                float c[DS_ORD];
-#pragma unroll
-                for (int o = 0; o < DS_ORD; ++o) c[o] = f[o][j];
-                const double x = fma(ds_collect(c), ds_scale(eb[4 * r + j]), acc[4 * r + j]);
-                if (on) acc[4 * r + j] = x;
-              }
-            }
+          for (int i = 0; i < DS_DIG; ++i) {
+            // digit i meets digits 0 .. min(6, 7 - i); i = 0 also the zero
+            // digit, which clears the last order on the block's first step
+            const int nj = i == 0 ? DS_ORD : min(DS_DIG, DS_ORD - i);
+            tc::mma_bf16(taddr + 16 * i, tc::smem_desc(sa + i * (DSS_STAGE / DS_DIG), 128, 256), bd,
+                         ds_idesc(128, 16 * nj), (st > 0 || i > 0) ? 1u : 0u);
           }
-          tc::fence_before_sync();
+          tc::mma_commit(&sh.done);
+        }
+        __syncwarp();
+      }
+      ds_wait(sh, gst - 1, ok);
+      tc::fence_after_sync();
+      __syncwarp();
+      const uint32_t tw = taddr + ((uint32_t)(warp * 32) << 16);
+      const bool on = kc + DSS_KB > s.k0;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        if (r < a.nr) {
+          float f[DS_ORD][4];
+          ds_ld_orders(tw + 4 * r, f);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float c[DS_ORD];
+#pragma unroll
+            for (int o = 0; o < DS_ORD; ++o) c[o] = f[o][j];
+            const double x = fma(ds_collect(c), ds_scale(eb[4 * r + j]), acc[4 * r + j]);
+            if (on) acc[4 * r + j] = x;
+          }
         }
       }
-    } else {
-      for (int kc = kbeg; kc < nk && ok; kc += DSS_KB, ++nblk) {
-        const int nst = min(DSS_KB / 16, (nk - kc + 15) / 16);
-        for (int st = 0; st < nst; ++st, ++gst) {
-          const int stg = gst & 1;
-          const bool w = tc::mbar_wait(&sh.full[stg], (gst >> 1) & 1, DS_WAIT);
-          if (!__all_sync(0xffffffffu, w) || __any_sync(0xffffffffu, sh.abort_ != 0)) {
-            if (lane == 0) sh.abort_ = 1;
-            ok = false;
-            break;
-          }
-          tc::fence_after_sync();
-          if (lane == 0) {
-            const uint32_t sa = tc::smem_addr(sm + stg * DSS_STAGE), sb = tc::smem_addr(Bs + st * DSS_BSTEP);
-            const uint64_t bd = tc::smem_desc(sb, 128, 256);
-#pragma unroll
-            for (int i = 0; i < DS_DIG; ++i) {
-              // digit i meets digits 0 .. min(6, 7 - i); i = 0 also the zero
-              // digit, which clears the last order on the block's first step
-              const int nj = i == 0 ? DS_ORD : min(DS_DIG, DS_ORD - i);
-              tc::mma_bf16(taddr + 16 * i, tc::smem_desc(sa + i * (DSS_STAGE / DS_DIG), 128, 256), bd,
-                           ds_idesc(128, 16 * nj), (st > 0 || i > 0) ? 1u : 0u);
-            }
-            tc::mma_commit(&sh.empty[stg]);
-            if (st == nst - 1) tc::mma_commit(&sh.done);
-          }
-          __syncwarp();
-        }
-      }
-      // commits are cumulative: the last one issued covers every MMA
-      if (gst > 0) {
-        const bool w = tc::mbar_wait(&sh.empty[(gst - 1) & 1], ((gst - 1) >> 1) & 1, DS_WAIT);
-        if (!__all_sync(0xffffffffu, w)) ok = false;
-      }
+      tc::fence_before_sync();
     }
-    tc::fence_before_sync();
     ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    // a wait that gave up: once more, before the tensor memory goes back
+    if (!ok) tc::mbar_wait_block(&sh.done, (gst - 1) & 1, DS_WAIT);
     tc::fence_after_sync();
-    if (warp == 4) tc::tmem_dealloc(taddr, DSS_TMEM);
+    if (warp == 0) tc::tmem_dealloc(taddr, DSS_TMEM);
   }
-  if (producer && p < pend) {
+  if (p < pend) {
     const int rn = p, rs = a.nring - 1 - p;
     const bool live = s.k0 < nk;
     // a wait that gave up must not pass for a result
@@ -759,7 +732,7 @@ __device__ __forceinline__ void ds_synth_body(const DsArgs& a, DsShared& sh, uin
 }
 
 template <int NR>
-__global__ void __launch_bounds__(DS_NT, 2) ds_synth_kernel(DsArgs a) {
+__global__ void __launch_bounds__(DS_PAIRS, NR == 1 ? 4 : 3) ds_synth_kernel(DsArgs a) {
   extern __shared__ __align__(1024) uint8_t ds_sm[];
   __shared__ DsShared sh;
   const int tile = blockIdx.x;
@@ -768,98 +741,89 @@ __global__ void __launch_bounds__(DS_NT, 2) ds_synth_kernel(DsArgs a) {
 }
 
 // ---- adjoint -----------------------------------------------------------------
-// CTA: one m, 128 ring pairs (the contraction index).  The pairs' phases
-// G = (even combination, z times the odd one) x (Re, Im) of up to NR
-// right-hand sides are split into digits once: row (digit, column) of a
-// K-major operand that starts with 6 CB zero rows, so that the operand read
-// from CB i rows earlier is the digits shifted down by i and row (s, column)
-// of the accumulator collects order s whatever the digit i of the other
-// operand.  That one holds 32 sequence values (N) of the 128 pairs per stage,
-// MN-major, so a thread writes 8 consecutive values of its own pair.  CB = 8
-// columns make 64 rows for one or two right-hand sides, CB = 16 make 128 for
-// up to four.  One partial row per (tile, right-hand side): (u_k, v_k) with
-// a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k, a_{o+1} += sigma_k e_{o+1} u_k,
-// or the two parities' values themselves near the equator.
+// CTA: one m, 128 ring pairs (the contraction index, one per thread).  The
+// pairs' phases G = (even combination, z times the odd one) x (Re, Im) of up
+// to NR right-hand sides are split into digits once: row (digit, column) of a
+// K-major operand, 8 columns per digit (64 rows), with zero rows around.  The
+// other operand holds 32 sequence values of the 128 pairs per stage, MN-major,
+// so a thread writes 8 consecutive values of its own pair.  A tensor-core
+// instruction takes at least 48 cycles here up to N = 64 and N / 2 beyond,
+// whatever M, so four digits of the sequence share one instruction (N = 128,
+// then 96 for the other three, read against G's digits shifted down by four):
+// 16 per stage instead of 56, which the instruction rate would bind (30 ms
+// against 18 at Nside 2048 / lmax 3000).  Row s of the accumulator of digits
+// d and d + 4 is order s + d.  One partial row per (tile, right-hand side):
+// (u_k, v_k) with a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k,
+// a_{o+1} += sigma_k e_{o+1} u_k, or the two parities' values themselves near
+// the equator.
 constexpr int DSA_N = 32;                                  // sequence values per stage
-constexpr int DSA_BD = DSA_N * DS_PAIRS * 2;               // one digit of a stage
+constexpr int DSA_CB = 8;                                  // columns per digit of G
+constexpr int DSA_A = 12 * DSA_CB * DS_PAIRS * 2;          // G: 4 CB zero rows, the digits, CB zero rows
+constexpr int DSA_B = DS_DIG * DSA_N * DS_PAIRS * 2;       // a stage: digits 0..3, digits 4..6
 constexpr int DSA_FS = 40;                                 // row stride of the collected accumulators
-template <int NR>
-struct DsaLayout {
-  static constexpr int CB = NR <= 2 ? 8 : 16;
-  static constexpr int A_ROWS = 14 * CB;                   // zeros, digits, zeros
-  static constexpr int A_BYTES = A_ROWS * DS_PAIRS * 2;
-  static constexpr int B0 = A_BYTES;
-  static constexpr int F0 = B0 + DS_DIG * DSA_BD;
-  static constexpr int BYTES = F0 + DS_ORD * 4 * NR * DSA_FS * 4;
-};
+constexpr int DSA_SMEM = DSA_A + DSA_B + 4 * DS_ORD * 4 * DSA_FS * 4;
+constexpr int DSA_TMEM = 128;
 
 template <int NR, bool EQ>
 __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, uint8_t* sm, int base, int pend) {
-  using Lay = DsaLayout<NR>;
-  constexpr int CB = Lay::CB, NC = 4 * NR;
+  constexpr int NC = 4 * NR;
   const int m = blockIdx.y, L = a.L, blk = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool producer = warp < 4;
   const int p = base + tid;
   DsPair<EQ> s;
   bool polar;
   int wmin, wmax;
-  ds_setup<EQ>(a, sh, s, m, p, pend, producer, &polar, &wmin, &wmax);
+  ds_setup<EQ>(a, sh, s, m, p, pend, &polar, &wmin, &wmax);
   const int nk = EQ ? L - m + 1 : (L - m) / 2 + 1;
   const int nk2 = (L - m) / 2 + 1;
-  const int kbeg = min(sh.kmin, nk) & ~3;
+  const int kbeg = sh.kmin;
   // partial row of right-hand side r: doubles 4 k + column
   const int64_t rstride = (int64_t)a.nblk * a.nkk * 4;
   double* part = a.partial + ((int64_t)blk * a.nkk + ds_off(L, m)) * 4;
   // zero before the tile's first start
   for (int r = 0; r < a.nr; ++r)
-    for (int i = tid; i < (sh.kmin < nk ? (EQ ? 2 * kbeg : 4 * kbeg) : 4 * nk2); i += DS_NT) part[r * rstride + i] = 0.0;
-  if (sh.kmin >= nk) return;
+    for (int i = tid; i < (kbeg < nk ? (EQ ? 2 * kbeg : 4 * kbeg) : 4 * nk2); i += DS_PAIRS) part[r * rstride + i] = 0.0;
+  if (kbeg >= nk) return;
 
-  for (int e = tid; e < Lay::A_BYTES / 16; e += DS_NT) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0u, 0u, 0u, 0u);
+  for (int e = tid; e < DSA_A / 16; e += DS_PAIRS) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0u, 0u, 0u, 0u);
   if (tid < 16) sh.eb[0][tid] = 0;
-  if (warp == 4) tc::tmem_alloc(&sh.taddr, 32);
+  if (warp == 0) tc::tmem_alloc(&sh.taddr, DSA_TMEM);
   if (tid == 0) {
-    tc::mbar_init(&sh.full[0], 128);
     tc::mbar_init(&sh.done, 1);
     tc::mbar_fence_init();
   }
-  __syncthreads();
   double g[NC];
 #pragma unroll
   for (int j = 0; j < NC; ++j) g[j] = 0.0;
-  if (producer) {
-    if (s.k0 < nk) {
-      const int rn = p, rs = a.nring - 1 - p;
-      const double zo = EQ ? 1.0 : a.z[p];
+  if (s.k0 < nk) {
+    const int rn = p, rs = a.nring - 1 - p;
+    const double zo = EQ ? 1.0 : a.z[p];
 #pragma unroll
-      for (int r = 0; r < NR; ++r)
-        if (r < a.nr) {
-          const double2 gn = a.phase[r * a.ld_phase + (int64_t)rn * a.ldp + m];
-          const double2 gs = (rs != rn) ? a.phase[r * a.ld_phase + (int64_t)rs * a.ldp + m] : make_double2(0.0, 0.0);
-          g[4 * r] = gn.x + gs.x;
-          g[4 * r + 1] = gn.y + gs.y;
-          g[4 * r + 2] = zo * (gn.x - gs.x);
-          g[4 * r + 3] = zo * (gn.y - gs.y);
-        }
-    }
-    // the pair's bound goes to this operand: |g| 2^(eb_pair) < 2^(eb - 1023)
-#pragma unroll
-    for (int j = 0; j < NC; ++j) {
-      const int x = ds_exp(g[j]);
-      const int e = __reduce_max_sync(0xffffffffu, x == 0 ? 0 : (x == 2047 ? 1 << 20 : x + s.eb - 1023));
-      if (lane == 0) atomicMax(&sh.eb[0][j], e + 1);
-    }
+    for (int r = 0; r < NR; ++r)
+      if (r < a.nr) {
+        const double2 gn = a.phase[r * a.ld_phase + (int64_t)rn * a.ldp + m];
+        const double2 gs = (rs != rn) ? a.phase[r * a.ld_phase + (int64_t)rs * a.ldp + m] : make_double2(0.0, 0.0);
+        g[4 * r] = gn.x + gs.x;
+        g[4 * r + 1] = gn.y + gs.y;
+        g[4 * r + 2] = zo * (gn.x - gs.x);
+        g[4 * r + 3] = zo * (gn.y - gs.y);
+      }
   }
   __syncthreads();
-  if (producer) {
+  // the pair's bound goes to this operand: |g| 2^(eb_pair) < 2^(eb - 1023)
 #pragma unroll
-    for (int j = 0; j < NC; ++j) {
-      const uint64_t y = ds_fix(g[j], sh.eb[0][j] - (s.eb - 1023)) + DS_SIGNED;
+  for (int j = 0; j < NC; ++j) {
+    const int x = ds_exp(g[j]);
+    const int e = __reduce_max_sync(0xffffffffu, x == 0 ? 0 : (x == 2047 ? 1 << 20 : x + s.eb - 1023));
+    if (lane == 0) atomicMax(&sh.eb[0][j], e + 1);
+  }
+  __syncthreads();
 #pragma unroll
-      for (int i = 0; i < DS_DIG; ++i)
-        *reinterpret_cast<__half*>(sm + tc::kmajor_offset((6 + i) * CB + j, tid, DS_PAIRS)) = ds_digit(y, i);
-    }
+  for (int j = 0; j < NC; ++j) {
+    const uint64_t y = ds_fix(g[j], sh.eb[0][j] - (s.eb - 1023)) + DS_SIGNED;
+#pragma unroll
+    for (int i = 0; i < DS_DIG; ++i)
+      *reinterpret_cast<__half*>(sm + tc::kmajor_offset((4 + i) * DSA_CB + j, tid, DS_PAIRS)) = ds_digit(y, i);
   }
   tc::fence_proxy_async();
   tc::fence_before_sync();
@@ -868,105 +832,97 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
   const uint32_t taddr = sh.taddr;
   bool ok = true;
   const int nit = (nk - kbeg + DSA_N - 1) / DSA_N;
-  if (producer) {
-    float* fb = reinterpret_cast<float*>(sm + Lay::F0);
-    // accumulators of iteration `it` to the partial rows
-    auto flush = [&](int it) {
-      if (ok) {
-        const bool w = tc::mbar_wait(&sh.done, it & 1, DS_WAIT);
-        if (!__all_sync(0xffffffffu, w)) {
-          if (lane == 0) sh.abort_ = 1;
-          ok = false;
-        }
-      }
-      tc::fence_after_sync();
-      float f[DSA_N];
-      tc::tmem_ld32(taddr + ((uint32_t)(warp * 32) << 16), f);
-      // 64 rows live in lanes 0..15 of each warp's quarter, 128 rows in all
-      const int so = 2 * warp + lane / CB, col = lane % CB;
-      if (lane < 2 * CB && col < NC) {
-        float4* d = reinterpret_cast<float4*>(fb + (so * NC + col) * DSA_FS);
+  float* fb = reinterpret_cast<float*>(sm + DSA_A + DSA_B);
+  // accumulators of iteration `it` to the partial rows
+  auto flush = [&](int it) {
+    ds_wait(sh, it, ok);
+    tc::fence_after_sync();
+    __syncwarp();
+    // the 64 rows live in lanes 0..15 of each warp's quarter
+    const int so = 2 * warp + (lane >> 3), col = lane & 7;
 #pragma unroll
-        for (int i = 0; i < DSA_N / 4; ++i) d[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
-      }
-      tc::fence_before_sync();
-      ds_bar();
+    for (int r = 0; r < NR; ++r) {
+      if (r < a.nr) {
+        if (r > 0) __syncthreads();  // the previous right-hand side is collected
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        if (r < a.nr) {
-          const int j = 4 * r + (tid & 3), kk = tid >> 2, k = kbeg + it * DSA_N + kk;
-          float c[DS_ORD];
+        for (int d = 0; d < 4; ++d) {
+          float f[DSA_N];
+          tc::tmem_ld32(taddr + ((uint32_t)(warp * 32) << 16) + DSA_N * d, f);
+          if (lane < 16 && (col >> 2) == r) {
+            float4* q = reinterpret_cast<float4*>(fb + ((d * DS_ORD + so) * 4 + (col & 3)) * DSA_FS);
 #pragma unroll
-          for (int o = 0; o < DS_ORD; ++o) c[o] = fb[(o * NC + j) * DSA_FS + kk];
-          double x = ds_collect(c) * ds_scale(sh.eb[0][j]);
-          if (!ok) x = __longlong_as_double(0x7ff8000000000000ll);
-          if (k < nk) {
-            double* d = part + r * rstride;
-            if (!EQ) d[4 * (int64_t)k + (tid & 3)] = x;
-            else if ((k & 1) == ((tid >> 1) & 1)) d[2 * (int64_t)k + (tid & 1)] = x;
+            for (int i = 0; i < DSA_N / 4; ++i) q[i] = make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
           }
         }
+        tc::fence_before_sync();
+        __syncthreads();
+        const int w = tid & 3, kk = tid >> 2, k = kbeg + it * DSA_N + kk;
+        float c[DS_ORD];
+#pragma unroll
+        for (int o = 0; o < DS_ORD; ++o) {
+          c[o] = fb[(o * 4 + w) * DSA_FS + kk];
+#pragma unroll
+          for (int d = 1; d < 4; ++d)
+            if (d <= o) c[o] += fb[((d * DS_ORD + o - d) * 4 + w) * DSA_FS + kk];
+        }
+        double x = ds_collect(c) * ds_scale(sh.eb[0][4 * r + w]);
+        if (!ok) x = __longlong_as_double(0x7ff8000000000000ll);
+        if (k < nk) {
+          double* q = part + r * rstride;
+          if (!EQ) q[4 * (int64_t)k + w] = x;
+          else if ((k & 1) == (w >> 1)) q[2 * (int64_t)k + (w & 1)] = x;
+        }
       }
-    };
-    bool ints = false;
-    ulonglong2 cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
-    for (int it = 0; it < nit; ++it) {
-      const int ks = kbeg + it * DSA_N;
-      if (it > 0) flush(it - 1);
-      ds_try_int<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, ints);
-      __syncwarp();
-      sh.sc[warp][lane] = cf;
-      cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar, ints);
-      __syncwarp();
+    }
+  };
+  int mode = 0;
+  ulonglong2 cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
+  for (int it = 0; it < nit; ++it) {
+    const int ks = kbeg + it * DSA_N;
+    ds_mode<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, mode);
+    __syncwarp();
+    sh.sc[warp][lane] = cf;
+    cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar, mode > 0);
+    __syncwarp();
+    if (it > 0) flush(it - 1);
 #pragma unroll 1
-      for (int gq = 0; gq < DSA_N / 8; ++gq) {
-        uint8_t* B = sm + Lay::B0 + ds_mn_off(8 * gq, tid, DSA_N);
-        ds_produce8<EQ>(s, sh.sc[warp] + 8 * gq, ks + 8 * gq, wmin, wmax, ints,
-                        [&](int i, uint4 d) { *reinterpret_cast<uint4*>(B + i * DSA_BD) = d; });
-      }
-      tc::fence_proxy_async();
-      ds_arrive(&sh.full[0]);
+    for (int gq = 0; gq < DSA_N / 8; ++gq) {
+      uint8_t* B = sm + DSA_A;
+      const uint32_t o4 = ds_mn_off(8 * gq, tid, 4 * DSA_N), o3 = 4 * DSA_N * DS_PAIRS * 2 + ds_mn_off(8 * gq, tid, 3 * DSA_N);
+      ds_produce8<EQ>(s, sh.sc[warp] + 8 * gq, ks + 8 * gq, wmin, mode, [&](int i, uint4 d) {
+        *reinterpret_cast<uint4*>(B + (i < 4 ? o4 : o3) + (i & 3) * (DSA_N / 8) * 128) = d;
+      });
     }
-    flush(nit - 1);
-  } else {
-    int issued = 0;
-    for (int it = 0; it < nit && ok; ++it) {
-      const bool w = tc::mbar_wait(&sh.full[0], it & 1, DS_WAIT);
-      if (!__all_sync(0xffffffffu, w) || __any_sync(0xffffffffu, sh.abort_ != 0)) {
-        if (lane == 0) sh.abort_ = 1;
-        ok = false;
-        break;
-      }
+    tc::fence_proxy_async();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (tid == 0) {
       tc::fence_after_sync();
-      if (lane == 0) {
-        constexpr uint32_t id = ds_idesc(8 * CB, DSA_N) | (1u << 16);  // B MN-major
-        constexpr uint32_t rg = (DS_PAIRS / 8) * 128;                  // 8 rows of the K-major operand
-        constexpr uint32_t bk = (DSA_N / 8) * 128;                     // 8 pairs of the MN-major one
-        const uint32_t sa = tc::smem_addr(sm), sb = tc::smem_addr(sm + Lay::B0);
+      constexpr uint32_t rg = (DS_PAIRS / 8) * 128;  // 8 rows of the K-major operand
+      const uint32_t sa = tc::smem_addr(sm), sb = tc::smem_addr(sm + DSA_A);
 #pragma unroll
-        for (int i = 0; i < DS_DIG; ++i)
+      for (int h = 0; h < 2; ++h) {
+        const int n = h == 0 ? 4 * DSA_N : 3 * DSA_N;
+        const uint32_t bk = (n / 8) * 128;           // 8 pairs of the MN-major operand
+        const uint32_t id = ds_idesc(8 * DSA_CB, n) | (1u << 16);
 #pragma unroll
-          for (int kk = 0; kk < DS_PAIRS / 16; ++kk)
-            tc::mma_bf16(taddr, tc::smem_desc(sa + (6 - i) * (CB / 8) * rg + kk * 256, 128, rg),
-                         tc::smem_desc(sb + i * DSA_BD + kk * 2 * bk, bk, 128), id, (i > 0 || kk > 0) ? 1u : 0u);
-        tc::mma_commit(&sh.done);
+        for (int kk = 0; kk < DS_PAIRS / 16; ++kk)
+          tc::mma_bf16(taddr, tc::smem_desc(sa + (h == 0 ? 4 : 0) * (DSA_CB / 8) * rg + kk * 256, 128, rg),
+                       tc::smem_desc(sb + h * 4 * DSA_N * DS_PAIRS * 2 + kk * 2 * bk, bk, 128), id,
+                       (h > 0 || kk > 0) ? 1u : 0u);
       }
-      __syncwarp();
-      issued = it + 1;
+      tc::mma_commit(&sh.done);
     }
-    if (issued > 0) {
-      const bool w = tc::mbar_wait(&sh.done, (issued - 1) & 1, DS_WAIT);
-      if (!__all_sync(0xffffffffu, w)) ok = false;
-    }
+    __syncwarp();
   }
-  tc::fence_before_sync();
-  __syncthreads();
+  flush(nit - 1);
+  if (!__syncthreads_and(ok ? 1 : 0)) tc::mbar_wait_block(&sh.done, (nit - 1) & 1, DS_WAIT);
   tc::fence_after_sync();
-  if (warp == 4) tc::tmem_dealloc(taddr, 32);
+  if (warp == 0) tc::tmem_dealloc(taddr, DSA_TMEM);
 }
 
 template <int NR>
-__global__ void __launch_bounds__(DS_NT, NR <= 2 ? 2 : 1) ds_adjoint_kernel(DsArgs a) {
+__global__ void __launch_bounds__(DS_PAIRS, 2) ds_adjoint_kernel(DsArgs a) {
   extern __shared__ __align__(1024) uint8_t ds_sm[];
   __shared__ DsShared sh;
   const int tile = blockIdx.x;
@@ -1082,10 +1038,10 @@ int launch_ds_synth(const LegArgs<double>& la, const double2* alm, int64_t ld_al
     const dim3 grid(a.nblk, la.L + 1);
     if (a.nr == 1) {
       CR_CUDA(cudaFuncSetAttribute(ds_synth_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSS_SMEM));
-      { ds_synth_kernel<1><<<grid, DS_NT, DSS_SMEM, st>>>(a); count_launch(); }
+      { ds_synth_kernel<1><<<grid, DS_PAIRS, DSS_SMEM, st>>>(a); count_launch(); }
     } else {
       CR_CUDA(cudaFuncSetAttribute(ds_synth_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSS_SMEM));
-      { ds_synth_kernel<4><<<grid, DS_NT, DSS_SMEM, st>>>(a); count_launch(); }
+      { ds_synth_kernel<4><<<grid, DS_PAIRS, DSS_SMEM, st>>>(a); count_launch(); }
     }
     CR_CHECK_LAUNCH("ds_synth_kernel");
   }
@@ -1094,21 +1050,22 @@ int launch_ds_synth(const LegArgs<double>& la, const double2* alm, int64_t ld_al
 
 template <int NR>
 static int ds_adjoint_launch(const DsArgs& a, cudaStream_t st) {
-  CR_CUDA(cudaFuncSetAttribute(ds_adjoint_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, DsaLayout<NR>::BYTES));
-  { ds_adjoint_kernel<NR><<<dim3(a.nblk, a.L + 1), DS_NT, DsaLayout<NR>::BYTES, st>>>(a); count_launch(); }
+  CR_CUDA(cudaFuncSetAttribute(ds_adjoint_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSA_SMEM));
+  { ds_adjoint_kernel<NR><<<dim3(a.nblk, a.L + 1), DS_PAIRS, DSA_SMEM, st>>>(a); count_launch(); }
   CR_CHECK_LAUNCH("ds_adjoint_kernel");
   return CR_OK;
 }
 
-// phases of nr right-hand sides -> f[0..nr-1].out, through partial rows in `partial`
-// (ds_partial_bytes of up to four right-hand sides)
+// phases of nr right-hand sides -> f[0..nr-1].out, two at a time, through
+// partial rows in `partial` (ds_partial_bytes of two right-hand sides, of one
+// when nr = 1)
 int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, double* partial,
                       const FinalizeArgs<double>* f, cudaStream_t st) {
-  for (int r0 = 0; r0 < nr; r0 += 4) {
-    DsArgs a = ds_args(la, std::min(4, nr - r0));
+  for (int r0 = 0; r0 < nr; r0 += 2) {
+    DsArgs a = ds_args(la, std::min(2, nr - r0));
     a.phase = const_cast<double2*>(phase) + r0 * a.ld_phase;
     a.partial = partial;
-    int rc = a.nr == 1 ? ds_adjoint_launch<1>(a, st) : a.nr == 2 ? ds_adjoint_launch<2>(a, st) : ds_adjoint_launch<4>(a, st);
+    int rc = a.nr == 1 ? ds_adjoint_launch<1>(a, st) : ds_adjoint_launch<2>(a, st);
     if (rc) return rc;
     const dim3 grid((la.L / 2 + 1 + 127) / 128, la.L + 1);
     for (int r = 0; r < a.nr; ++r) {

@@ -589,7 +589,7 @@ int ensure_mr_workspace(cr_plan* P, const Grid& g, int L) {
   const int nblk = mr_blocks(g.npairs);
   const int64_t phase = 8 * ld_phase * (int64_t)sizeof(double2);
   const int64_t partial = std::max(8 * (int64_t)nblk * nlm * (int64_t)sizeof(double2),
-                                   ds_partial_bytes(g.nis, g.npairs, L, 4));
+                                   ds_partial_bytes(g.nis, g.npairs, L, 2));
   if (phase > P->ws_mr.phase_bytes || partial > P->ws_mr.partial_bytes) {
     if (P->capturing) return fail(CR_ESTATE, "FP64 batch: buffers missing (run once outside a capture)");
     if (phase > P->ws_mr.phase_bytes) {
