@@ -307,6 +307,20 @@ __device__ __forceinline__ void ds_ld_orders(uint32_t taddr, float f[DS_ORD][4])
                : "memory");
 }
 
+// 16 columns of this warp's lanes
+__device__ __forceinline__ void ds_ld16(uint32_t taddr, float f[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]), "=f"(f[4]), "=f"(f[5]), "=f"(f[6]), "=f"(f[7]), "=f"(f[8]),
+        "=f"(f[9]), "=f"(f[10]), "=f"(f[11]), "=f"(f[12]), "=f"(f[13]), "=f"(f[14]), "=f"(f[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(f[0]), "+f"(f[1]), "+f"(f[2]), "+f"(f[3]), "+f"(f[4]), "+f"(f[5]), "+f"(f[6]), "+f"(f[7]),
+                 "+f"(f[8]), "+f"(f[9]), "+f"(f[10]), "+f"(f[11]), "+f"(f[12]), "+f"(f[13]), "+f"(f[14]), "+f"(f[15])
+               :
+               : "memory");
+}
+
 // One ring pair's sequence.  The first few steps, where the functions can grow
 // by large factors, run in FP64 (mode 0); then in integers with an exponent
 // per pair (mode 1: (Q - 2^63) 2^-62 2^(eb - 1023 - x), x falling to zero as
@@ -756,13 +770,14 @@ __global__ void __launch_bounds__(DS_PAIRS, NR == 1 ? 4 : 3) ds_synth_kernel(DsA
 // (u_k, v_k) with a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k,
 // a_{o+1} += sigma_k e_{o+1} u_k, or the two parities' values themselves near
 // the equator.
-constexpr int DSA_N = 32;                                  // sequence values per stage
+constexpr int DSA_N = 16;                                  // sequence values per stage
 constexpr int DSA_CB = 8;                                  // columns per digit of G
 constexpr int DSA_A = 12 * DSA_CB * DS_PAIRS * 2;          // G: 4 CB zero rows, the digits, CB zero rows
 constexpr int DSA_B = DS_DIG * DSA_N * DS_PAIRS * 2;       // a stage: digits 0..3, digits 4..6
-constexpr int DSA_FS = 40;                                 // row stride of the collected accumulators
-constexpr int DSA_SMEM = DSA_A + DSA_B + 4 * DS_ORD * 4 * DSA_FS * 4;
-constexpr int DSA_TMEM = 128;
+constexpr int DSA_FS = 24;                                 // row stride of the collected accumulators
+constexpr int DSA_SMEM = DSA_A + DSA_B;
+constexpr int DSA_TMEM = 64;
+static_assert(4 * DS_ORD * 4 * DSA_FS * 4 <= DSA_B, "the collected accumulators reuse the stage");
 
 template <int NR, bool EQ>
 __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, uint8_t* sm, int base, int pend) {
@@ -832,7 +847,7 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
   const uint32_t taddr = sh.taddr;
   bool ok = true;
   const int nit = (nk - kbeg + DSA_N - 1) / DSA_N;
-  float* fb = reinterpret_cast<float*>(sm + DSA_A + DSA_B);
+  float* fb = reinterpret_cast<float*>(sm + DSA_A);  // the stage's operand is read by then
   // accumulators of iteration `it` to the partial rows
   auto flush = [&](int it) {
     ds_wait(sh, it, ok);
@@ -847,7 +862,7 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
           float f[DSA_N];
-          tc::tmem_ld32(taddr + ((uint32_t)(warp * 32) << 16) + DSA_N * d, f);
+          ds_ld16(taddr + ((uint32_t)(warp * 32) << 16) + DSA_N * d, f);
           if (lane < 16 && (col >> 2) == r) {
             float4* q = reinterpret_cast<float4*>(fb + ((d * DS_ORD + so) * 4 + (col & 3)) * DSA_FS);
 #pragma unroll
@@ -857,6 +872,7 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
         tc::fence_before_sync();
         __syncthreads();
         const int w = tid & 3, kk = tid >> 2, k = kbeg + it * DSA_N + kk;
+        if (kk >= DSA_N) continue;
         float c[DS_ORD];
 #pragma unroll
         for (int o = 0; o < DS_ORD; ++o) {
@@ -876,15 +892,21 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
     }
   };
   int mode = 0;
-  ulonglong2 cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
+  ulonglong2 cf = make_ulonglong2(0, 0);
+  if (lane < DSA_N) cf = ds_coef<EQ>(a, m, kbeg + lane, nk, polar, false);
   for (int it = 0; it < nit; ++it) {
     const int ks = kbeg + it * DSA_N;
     ds_mode<EQ>(a, s, m, ks, nk, polar, wmin, wmax, cf, mode);
     __syncwarp();
-    sh.sc[warp][lane] = cf;
-    cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar, mode > 0);
+    if (lane < DSA_N) {
+      sh.sc[warp][lane] = cf;
+      cf = ds_coef<EQ>(a, m, ks + DSA_N + lane, nk, polar, mode > 0);
+    }
     __syncwarp();
-    if (it > 0) flush(it - 1);
+    if (it > 0) {
+      flush(it - 1);
+      __syncthreads();
+    }
 #pragma unroll 1
     for (int gq = 0; gq < DSA_N / 8; ++gq) {
       uint8_t* B = sm + DSA_A;
@@ -922,7 +944,7 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
 }
 
 template <int NR>
-__global__ void __launch_bounds__(DS_PAIRS, 2) ds_adjoint_kernel(DsArgs a) {
+__global__ void __launch_bounds__(DS_PAIRS, 4) ds_adjoint_kernel(DsArgs a) {
   extern __shared__ __align__(1024) uint8_t ds_sm[];
   __shared__ DsShared sh;
   const int tile = blockIdx.x;
