@@ -13,6 +13,7 @@ struct DsTab {
   double *A = nullptr, *B = nullptr, *AB = nullptr;    // coefficients of the step that produces q_k
   double *sg = nullptr, *e0 = nullptr, *e1 = nullptr;  // sigma_k, and times e_o and e_{o+1}
   uint64_t *Ai = nullptr, *Bi = nullptr;               // A 2^57, (B + 8) 2^60: the integer steps' coefficients
+  float4 *rf = nullptr, *cf = nullptr;                 // FP32: (A, A + B - 2, B, B + 2); sigma_k times (1, e_o, e_{o+1})
   int Lc = -1;
 };
 
@@ -40,12 +41,17 @@ struct LegArgs {
   int npairs = 0, nring = 0;
   typename Tr<T>::C* partial = nullptr;    // adjoint: [nblk][n_lm(L)]
   const T* ringval = nullptr;              // SQ variant: per-ring value
-  int rp_synth = 4, rp_adj = 4;            // ring pairs per thread (2, 4, 8) of the two stages
+  int rp_synth = 0, rp_adj = 0;            // ring pairs per thread (2, 4, 8) of the two stages; 0: not tuned
   int mt_synth = 1, mt_adj = 1;            // m tile: 1 (one m per CTA) or 2 (m and L - m per CTA)
   int tc_variant = 0;                      // tensor-core kernels: stage shape (legendre_tc.cu)
   int tc_split = 0;                        // tensor-core kernels: hi + lo BF16 operands
   const DsTab* ds = nullptr;               // FP64: tables of the digit-slice kernels (null: not used)
   int nis = 0;                             // pairs [0, nis) with z above their equatorial zone
+  // FP32 kernels (legendre_f32.cu): tables of DsTab, per-ring arguments, start
+  // states, and the first pair of the middle and of the equatorial zone
+  const float4 *rf = nullptr, *cf = nullptr, *zi = nullptr;
+  const float2* sti = nullptr;
+  int n1 = 0, n2 = 0;
 };
 
 // Arguments of the digit-slice kernels.
@@ -154,6 +160,13 @@ int launch_ds_synth(const LegArgs<double>& la, const double2* alm, int64_t ld_al
                     cudaStream_t st);
 int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, double* partial,
                       const FinalizeArgs<double>* f, cudaStream_t st);
+// FP32 stages (legendre_f32.cu)
+int64_t ds_len(int L);
+void lf_zones(const double* z, int npairs, int* n1, int* n2);
+void lf_args(const double* z, int npairs, int n1, int n2, float4* out);
+int64_t lf_partial_bytes(int npairs, int L);
+int launch_lf_synth(const LegArgs<float>& a, cudaStream_t st);
+int launch_lf_adjoint(const LegArgs<float>& a, const FinalizeArgs<float>& f, cudaStream_t st);
 int launch_leg_diag(cr_plan* P, const double* ringval, double2* out);
 template <typename T> int launch_ring_fft(const RingArgs<T>& a, int mode, cudaStream_t st);
 

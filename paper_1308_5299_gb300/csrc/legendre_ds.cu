@@ -63,7 +63,7 @@ constexpr uint64_t DS_BIAS = 0x8000000000000080ull;  // zero (sign bit flipped) 
 // position of m's first k in tables of band limit L: room for
 // (L - m) / 2 + 1 entries each
 __host__ __device__ inline int64_t ds_off(int L, int m) { return (lm_off(L, m) >> 1) + m; }
-int64_t ds_len(int L) { return ds_off(L, L + 1) + 2; }
+int64_t ds_len(int L) { return (ds_off(L, L + 1) + 3) & ~(int64_t)1; }  // even: 16-byte alignment of what follows
 
 // ---- plan tables -------------------------------------------------------------
 // Double-double helpers (Knuth's TwoSum, Dekker's product by FMA).
@@ -153,7 +153,9 @@ __global__ void __launch_bounds__(DST_NT) ds_tab_kernel(DsTab t) {
       const dd2 B = dd_mul(A, {-S.h, -S.l});
       t.A[off + k + 1] = A.h;
       t.B[off + k + 1] = B.h;
-      t.AB[off + k + 1] = dd_mul(A, S1).h;
+      const dd2 AB = dd_mul(A, S1);
+      t.AB[off + k + 1] = AB.h;
+      t.rf[off + k + 1] = make_float4((float)A.h, (float)((AB.h - 2.0) + AB.l), (float)B.h, (float)((B.h + 2.0) + B.l));
       // fixed point: A 2^57 and (B + 8) 2^60 (modulo 2^64); the integer steps
       // start where A < 100
       const double n = rint(B.h);
@@ -163,12 +165,17 @@ __global__ void __launch_bounds__(DST_NT) ds_tab_kernel(DsTab t) {
                                    (uint64_t)__double2ll_rn(B.l * 0x1p60)
                              : 0;
     }
-    t.sg[off + k] = dd_sqrt(cur).h;
-    t.e0[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o), 0.0}), {d(o), 0.0})).h;
-    t.e1[off + k] = dd_sqrt(dd_div(dd_mul(cur, {n(o + 1), 0.0}), {d(o + 1), 0.0})).h;
+    const double sg = dd_sqrt(cur).h;
+    const double e0 = dd_sqrt(dd_div(dd_mul(cur, {n(o), 0.0}), {d(o), 0.0})).h;
+    const double e1 = dd_sqrt(dd_div(dd_mul(cur, {n(o + 1), 0.0}), {d(o + 1), 0.0})).h;
+    t.sg[off + k] = sg;
+    t.e0[off + k] = e0;
+    t.e1[off + k] = e1;
+    t.cf[off + k] = make_float4((float)sg, (float)e0, (float)e1, 0.f);
     if (k == 0) {
       t.A[off] = t.B[off] = t.AB[off] = 0.0;
       t.Ai[off] = t.Bi[off] = 0;
+      t.rf[off] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
 }
@@ -178,11 +185,11 @@ void ds_tab_free(DsTab& t) {
   t = DsTab();
 }
 
-// the tables for band limits up to Lc (one allocation, eight arrays)
+// the tables for band limits up to Lc (one allocation)
 int ds_tab_build(DsTab& t, int Lc, cudaStream_t st) {
   ds_tab_free(t);
   const int64_t n = ds_len(Lc);
-  CR_CUDA(cudaMalloc(&t.A, 8 * n * sizeof(double)));
+  CR_CUDA(cudaMalloc(&t.A, 8 * n * sizeof(double) + 2 * n * sizeof(float4)));
   t.B = t.A + n;
   t.AB = t.B + n;
   t.sg = t.AB + n;
@@ -190,6 +197,8 @@ int ds_tab_build(DsTab& t, int Lc, cudaStream_t st) {
   t.e1 = t.e0 + n;
   t.Ai = reinterpret_cast<uint64_t*>(t.e1 + n);
   t.Bi = t.Ai + n;
+  t.rf = reinterpret_cast<float4*>(t.Bi + n);
+  t.cf = t.rf + n;
   t.Lc = Lc;
   { ds_tab_kernel<<<Lc + 1, DST_NT, 0, st>>>(t); count_launch(); }
   CR_CHECK_LAUNCH("ds_tab_kernel");

@@ -1,0 +1,548 @@
+// FP32 Legendre stages on the CUDA cores.
+//
+// The two-step sequence of legendre_ds.cu: with p_k = P~_o / z, o = m + 1 + 2k,
+//   sum_l a_l P~_l(+-z) = sum_k p_k c_k +- z sum_k p_k d_k,
+//   c_k = e_o a_{o-1} + e_{o+1} a_{o+1},  d_k = a_o,
+// and q_k = p_k / sigma_k obeys q_{k+1} = e_k q_k - q_{k-1}, e_k = A_k z^2 + B_k.
+// Per two l and ring pair that is 2 (or 3) operations of recurrence and 4 of
+// sums, where the one-step recurrence took 4 (or 6) and 4.  Three forms of the
+// step keep FP32's rounding down, each on a range of pairs (a warp has one):
+//  - polar, z > LF_ZPOLAR: the difference form on s = 1 - z^2,
+//      d = ((A + B - 2) - A s) q + d, q = q + d
+//    (q varies slowly in k there; e - 2 is carried at full relative precision);
+//  - middle: q_{k+1} = (A z^2 + B) q_k - q_{k-1} with four copies of z^2 that
+//    differ in the last place and average to the exact square, used in turn
+//    (one rounded square would act the same way at every k);
+//  - equatorial, z < LF_ZEQ: q alternates in sign; v_k = (-1)^k q_k takes the
+//    difference form with -(B + 2) - A z^2, and the sign goes to the
+//    coefficients (synthesis) or the sums (adjoint).
+// In FP32 emulated against extended precision (white spectrum, Nside 2048 /
+// lmax 3000) the error is 5e-6 where the one-step form's was 1.5e-5.
+//
+// One warp per block of 32 RP pairs of one m (RP per thread), without block
+// barriers; m in blockIdx.y, so the longest warps start first.  Each warp
+// stages the chunk's coefficients itself; a group of 8 k runs unchecked once
+// all of the warp's pairs have started (start tables, |P~| >= 2^-60).  Bound by
+// FP32 issue: 6.5 operations per pair and k beside two shared loads per k and
+// warp.
+#include "common.cuh"
+#include "kernels.h"
+
+namespace cr {
+
+constexpr double LF_ZPOLAR = 0.8, LF_ZEQ = 0.15;
+constexpr int LF_CH = 128;       // k per staged chunk
+constexpr int LF_FUSED = 8;      // most warps of one m whose sums one CTA collects
+
+void lf_zones(const double* z, int npairs, int* n1, int* n2) {
+  int i = 0;
+  while (i < npairs && z[i] > LF_ZPOLAR) ++i;
+  *n1 = i;
+  while (i < npairs && z[i] >= LF_ZEQ) ++i;
+  *n2 = i;
+}
+
+// arguments of a pair's steps: four copies of z^2 (middle), or 1 - z^2, or z^2
+void lf_args(const double* z, int npairs, int n1, int n2, float4* out) {
+  for (int p = 0; p < npairs; ++p) {
+    const long double x = (long double)z[p] * z[p];
+    if (p < n1) {
+      const double w = 1.0 - z[p];
+      const float s = (float)(w * (2.0 - w));
+      out[p] = make_float4(s, s, s, s);
+    } else if (p >= n2) {
+      const float s = (float)x;
+      out[p] = make_float4(s, s, s, s);
+    } else {
+      const float h = (float)x;
+      const float up = nextafterf(h, 2.f) - h;
+      const int t = (int)lrint(4.0 * (double)(x - (long double)h) / up);
+      float c[4];
+      for (int j = 0; j < 4; ++j) c[j] = h + (j < abs(t) ? (t > 0 ? up : -up) : 0.f);
+      out[p] = make_float4(c[0], c[1], c[2], c[3]);
+    }
+  }
+}
+
+// One warp's pairs: arguments, states, start indices.
+template <int ZONE, int RP>
+struct LfPairs {
+  static constexpr int NZ = ZONE == 1 ? 4 : 1;
+  float q1[RP], q2[RP], Z[RP][NZ];
+  int k0[RP], p[RP];
+  int kmin, kmax;  // first and last start of the warp's live pairs
+
+  __device__ __forceinline__ void load(const LegArgs<float>& a, int m, int base, int pend) {
+    const int lane = threadIdx.x & 31;
+    const int none = 0x3fffffff;
+    int lo = none, hi = 0;
+#pragma unroll
+    for (int j = 0; j < RP; ++j) {
+      p[j] = base + 32 * j + lane;
+      k0[j] = none;
+      q1[j] = q2[j] = 0.f;
+      float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (p[j] < pend) {
+        z = a.zi[p[j]];
+        const int64_t o = (int64_t)m * a.ld_seed + p[j];
+        const int l = a.ls[o];
+        if (l <= a.L) {
+          const float2 st = a.sti[o];
+          k0[j] = (l - m) >> 1;
+          q1[j] = st.x;
+          q2[j] = st.y;
+          lo = min(lo, k0[j]);
+          hi = max(hi, k0[j]);
+        }
+      }
+      Z[j][0] = z.x;
+      if (NZ == 4) {
+        Z[j][NZ > 1 ? 1 : 0] = z.y;
+        Z[j][NZ > 2 ? 2 : 0] = z.z;
+        Z[j][NZ > 3 ? 3 : 0] = z.w;
+      }
+    }
+    kmin = __reduce_min_sync(0xffffffffu, lo);
+    kmax = __reduce_max_sync(0xffffffffu, hi);
+  }
+  // the next value of pair j; u: its k modulo 4
+  __device__ __forceinline__ float next(float2 r, int j, int u, float& second) const {
+    const float e = fmaf(r.x, Z[j][NZ == 4 ? u & 3 : 0], r.y);
+    if (ZONE == 1) {
+      second = q1[j];
+      return fmaf(e, q1[j], -q2[j]);
+    }
+    const float d = fmaf(e, q1[j], q2[j]);
+    second = d;
+    return q1[j] + d;
+  }
+};
+
+// (factor of the argument, constant) of a zone's step, from (A, A + B - 2, B, B + 2)
+template <int ZONE>
+__device__ __forceinline__ float2 lf_coef(float4 t) {
+  if (ZONE == 0) return make_float2(-t.x, t.y);
+  if (ZONE == 1) return make_float2(t.x, t.z);
+  return make_float2(-t.x, -t.w);
+}
+
+struct LfStage {
+  float2 r[LF_CH];
+  float4 c[LF_CH];
+};
+
+// ---- synthesis ---------------------------------------------------------------
+
+template <int ZONE, int RP>
+__device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, int m, int base, int pend) {
+  const int L = a.L, lane = threadIdx.x;
+  const int nk = (L - m) / 2 + 1;
+  LfPairs<ZONE, RP> s;
+  s.load(a, m, base, pend);
+  float cx[RP], cy[RP], dx[RP], dy[RP];
+#pragma unroll
+  for (int j = 0; j < RP; ++j) cx[j] = cy[j] = dx[j] = dy[j] = 0.f;
+  const int64_t offa = lm_off(L, m), offk = (lm_off(a.Lc, m) >> 1) + m;
+  // chunks start at a multiple of 8
+  for (int kc = s.kmin & ~7; kc < nk; kc += LF_CH) {
+    const int n = min(LF_CH, nk - kc);
+    __syncwarp();
+#pragma unroll
+    for (int i = lane; i < LF_CH; i += 32) {
+      const int k = kc + i;
+      if (i < n) {
+        const int l = m + 2 * k;
+        const float4 t = a.rf[offk + k], g = a.cf[offk + k];
+        const float2* x = a.alm + offa + 2 * k;
+        const float2 x0 = x[0];
+        const float2 x1 = l + 1 <= L ? x[1] : make_float2(0.f, 0.f);
+        const float2 x2 = l + 2 <= L ? x[2] : make_float2(0.f, 0.f);
+        float f0 = g.y, f1 = g.x, f2 = g.z;
+        if (a.dl) {
+          f0 *= a.dl[l];
+          f1 *= l + 1 <= L ? a.dl[l + 1] : 0.f;
+          f2 *= l + 2 <= L ? a.dl[l + 2] : 0.f;
+        }
+        float4 c = make_float4(fmaf(f0, x0.x, f2 * x2.x), fmaf(f0, x0.y, f2 * x2.y), f1 * x1.x, f1 * x1.y);
+        if (m == 0) c.y = c.w = 0.f;
+        if (ZONE == 2 && (k & 1)) c = make_float4(-c.x, -c.y, -c.z, -c.w);
+        sh.c[i] = c;
+        sh.r[i] = lf_coef<ZONE>(t);
+      }
+    }
+    __syncwarp();
+    for (int i8 = 0; i8 < n; i8 += 8) {
+      const int k = kc + i8;
+      if (s.kmin >= k + 8) continue;
+      if (s.kmax <= k && i8 + 8 <= n) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float2 r = sh.r[i8 + u];
+          const float4 c = sh.c[i8 + u];
+#pragma unroll
+          for (int j = 0; j < RP; ++j) {
+            float d;
+            const float q = s.next(r, j, u, d);
+            s.q2[j] = d;
+            s.q1[j] = q;
+            cx[j] = fmaf(q, c.x, cx[j]);
+            cy[j] = fmaf(q, c.y, cy[j]);
+            dx[j] = fmaf(q, c.z, dx[j]);
+            dy[j] = fmaf(q, c.w, dy[j]);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (i8 + u >= n) break;
+          const float2 r = sh.r[i8 + u];
+          const float4 c = sh.c[i8 + u];
+#pragma unroll
+          for (int j = 0; j < RP; ++j) {
+            float d;
+            const float q = s.next(r, j, u, d);
+            if (k + u >= s.k0[j]) {
+              s.q2[j] = d;
+              s.q1[j] = q;
+              cx[j] = fmaf(q, c.x, cx[j]);
+              cy[j] = fmaf(q, c.y, cy[j]);
+              dx[j] = fmaf(q, c.z, dx[j]);
+              dy[j] = fmaf(q, c.w, dy[j]);
+            }
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < RP; ++j)
+    if (s.p[j] < pend) {
+      const int rn = s.p[j], rs = a.nring - 1 - rn;
+      const float z = a.z[rn];
+      a.phase[(int64_t)rn * a.ldp + m] = make_float2(fmaf(z, dx[j], cx[j]), fmaf(z, dy[j], cy[j]));
+      if (rs != rn) a.phase[(int64_t)rs * a.ldp + m] = make_float2(fmaf(-z, dx[j], cx[j]), fmaf(-z, dy[j], cy[j]));
+    }
+}
+
+// warp blocks of the three zones
+template <int RP>
+__host__ __device__ inline int lf_blocks(int n) { return (n + 32 * RP - 1) / (32 * RP); }
+
+template <int RP, int MT>
+__global__ void __launch_bounds__(32) lf_synth_kernel(LegArgs<float> a) {
+  __shared__ LfStage sh;
+  const int b0 = lf_blocks<RP>(a.n1), b1 = lf_blocks<RP>(a.n2 - a.n1);
+  const int b = blockIdx.x;
+#pragma unroll 1
+  for (int mi = 0; mi < MT; ++mi) {
+    const int m = mi == 0 ? (int)blockIdx.y : a.L - (int)blockIdx.y;
+    if (mi > 0 && m <= (int)blockIdx.y) break;
+    if (b < b0) lf_synth<0, RP>(a, sh, m, b * 32 * RP, a.n1);
+    else if (b < b0 + b1) lf_synth<1, RP>(a, sh, m, a.n1 + (b - b0) * 32 * RP, a.n2);
+    else lf_synth<2, RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, a.npairs);
+    __syncwarp();
+  }
+}
+
+// ---- adjoint -----------------------------------------------------------------
+// u_k = sum_pairs q_k (G_m(z) + G_m(-z)), v_k = sum_pairs q_k z (G_m(z) - G_m(-z));
+// a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k, a_{o+1} += sigma_k e_{o+1} u_k.
+// The four real sums of a k over a thread's RP pairs go to a shared-memory
+// row; per 8 k, lane (k, part) adds every fourth lane's entry and two exchange
+// steps leave one of the four sums per lane, 128 contiguous bytes of the
+// warp's row.  Rows are 36 entries apart: 16-byte reads of two rows fall on
+// different banks.
+constexpr int LF_RS = 36;
+typedef unsigned long long lf_u64;
+__device__ __forceinline__ lf_u64 lf_add2(lf_u64 a, lf_u64 b) {
+  lf_u64 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+struct LfAdjStage {
+  float2 r[LF_CH];
+  float4 b[8][LF_RS];
+};
+
+// row: this warp's sums, 4 floats per k
+template <int ZONE, int RP>
+__device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& sh, int m, int base, int pend,
+                                           float* row) {
+  const int L = a.L, lane = threadIdx.x & 31;
+  const int nk = (L - m) / 2 + 1;
+  LfPairs<ZONE, RP> s;
+  s.load(a, m, base, pend);
+  float2 ge[RP], go[RP];
+#pragma unroll
+  for (int j = 0; j < RP; ++j) {
+    ge[j] = go[j] = make_float2(0.f, 0.f);
+    if (s.k0[j] < nk) {
+      const int rn = s.p[j], rs = a.nring - 1 - rn;
+      const float z = a.z[rn];
+      const float2 gn = a.phase[(int64_t)rn * a.ldp + m];
+      const float2 gs = rs != rn ? a.phase[(int64_t)rs * a.ldp + m] : make_float2(0.f, 0.f);
+      ge[j] = cadd(gn, gs);
+      go[j] = make_float2(z * (gn.x - gs.x), z * (gn.y - gs.y));
+    }
+  }
+  const int64_t offk = (lm_off(a.Lc, m) >> 1) + m;
+  const int kbeg = min(s.kmin, nk) & ~7;
+  for (int i = lane; i < 4 * kbeg; i += 32) row[i] = 0.f;  // before the first start
+  if (s.kmin >= nk) {
+    for (int i = 4 * kbeg + lane; i < 4 * nk; i += 32) row[i] = 0.f;
+    return;
+  }
+  for (int kc = kbeg; kc < nk; kc += LF_CH) {
+    const int n = min(LF_CH, nk - kc);
+    __syncwarp();
+#pragma unroll
+    for (int i = lane; i < LF_CH; i += 32)
+      if (i < n) sh.r[i] = lf_coef<ZONE>(a.rf[offk + kc + i]);
+    __syncwarp();
+    for (int i8 = 0; i8 < n; i8 += 8) {
+      const int k = kc + i8;
+      const bool full = s.kmax <= k && i8 + 8 <= n;
+      if (full) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float2 r = sh.r[i8 + u];
+          float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int j = 0; j < RP; ++j) {
+            float d;
+            const float q = s.next(r, j, u, d);
+            s.q2[j] = d;
+            s.q1[j] = q;
+            t.x = fmaf(q, ge[j].x, t.x);
+            t.y = fmaf(q, ge[j].y, t.y);
+            t.z = fmaf(q, go[j].x, t.z);
+            t.w = fmaf(q, go[j].y, t.w);
+          }
+          sh.b[u][lane] = t;
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (i8 + u < n) {
+            const float2 r = sh.r[i8 + u];
+#pragma unroll
+            for (int j = 0; j < RP; ++j) {
+              float d;
+              const float q = s.next(r, j, u, d);
+              if (k + u >= s.k0[j]) {
+                s.q2[j] = d;
+                s.q1[j] = q;
+                t.x = fmaf(q, ge[j].x, t.x);
+                t.y = fmaf(q, ge[j].y, t.y);
+                t.z = fmaf(q, go[j].x, t.z);
+                t.w = fmaf(q, go[j].y, t.w);
+              }
+            }
+          }
+          sh.b[u][lane] = t;
+        }
+      }
+      __syncwarp();
+      const int u = lane >> 2, part = lane & 3;
+      const ulonglong2* e = reinterpret_cast<const ulonglong2*>(&sh.b[u][part]);
+      ulonglong2 t = e[0];
+#pragma unroll
+      for (int i = 1; i < 8; ++i) {
+        const ulonglong2 w = e[4 * i];
+        t.x = lf_add2(t.x, w.x);
+        t.y = lf_add2(t.y, w.y);
+      }
+      __syncwarp();  // the rows are rewritten by the next group
+      const float2 tu = *reinterpret_cast<const float2*>(&t.x), tv = *reinterpret_cast<const float2*>(&t.y);
+      // parts 0, 1 keep u and 2, 3 keep v; then even parts the real part
+      const bool hi = part & 2, im = part & 1;
+      const float s0 = __shfl_xor_sync(0xffffffffu, hi ? tu.x : tv.x, 2);
+      const float s1 = __shfl_xor_sync(0xffffffffu, hi ? tu.y : tv.y, 2);
+      const float w0 = (hi ? tv.x : tu.x) + s0, w1 = (hi ? tv.y : tu.y) + s1;
+      float w = (im ? w1 : w0) + __shfl_xor_sync(0xffffffffu, im ? w0 : w1, 1);
+      if (ZONE == 2 && (u & 1)) w = -w;  // k is a multiple of 8
+      if (i8 + u < n) row[4 * (k + u) + part] = w;
+    }
+  }
+}
+
+template <int RP, int MT>
+__global__ void __launch_bounds__(32) lf_adjoint_kernel(LegArgs<float> a, float* partial, int64_t nkk) {
+  __shared__ LfAdjStage sh;
+  const int b0 = lf_blocks<RP>(a.n1), b1 = lf_blocks<RP>(a.n2 - a.n1);
+  const int b = blockIdx.x;
+#pragma unroll 1
+  for (int mi = 0; mi < MT; ++mi) {
+    const int m = mi == 0 ? (int)blockIdx.y : a.L - (int)blockIdx.y;
+    if (mi > 0 && m <= (int)blockIdx.y) break;
+    float* row = partial + ((int64_t)b * nkk + ((lm_off(a.L, m) >> 1) + m)) * 4;
+    if (b < b0) lf_adjoint<0, RP>(a, sh, m, b * 32 * RP, a.n1, row);
+    else if (b < b0 + b1) lf_adjoint<1, RP>(a, sh, m, a.n1 + (b - b0) * 32 * RP, a.n2, row);
+    else lf_adjoint<2, RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, a.npairs, row);
+    __syncwarp();
+  }
+}
+
+// a_l (l = m + 2k + w) from the summed (u_k, v_k), u_{k-1}, and the epilogue of
+// leg_finalize_kernel
+__device__ __forceinline__ void lf_emit(const LegArgs<float>& a, const FinalizeArgs<float>& f, int m, int k, float4 t,
+                                        float2 um) {
+  const int L = a.L;
+  const int64_t ok = (lm_off(a.Lc, m) >> 1) + m + k;
+  const float4 g = a.cf[ok];
+  const float g1 = k > 0 ? a.cf[ok - 1].z : 0.f;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int l = m + 2 * k + w;
+    if (l > L) break;
+    float2 y = w == 0 ? make_float2(fmaf(g.y, t.x, g1 * um.x), fmaf(g.y, t.y, g1 * um.y))
+                      : make_float2(g.x * t.z, g.x * t.w);
+    const int64_t i = lm_off(L, m) + (l - m);
+    if (f.dl_out) y = cscale(y, f.dl_out[l]);
+    if (f.dadd) {
+      const float2 x = f.xadd[i];
+      y.x = fmaf(f.dadd[l], x.x, y.x);
+      y.y = fmaf(f.dadd[l], x.y, y.y);
+    }
+    if (f.bsub) {
+      const float2 b = f.bsub[i];
+      y = make_float2(b.x - y.x, b.y - y.y);
+    }
+    if (m == 0) y.y = 0.f;
+    if (f.accumulate) y = cadd(y, f.out[i]);
+    f.out[i] = y;
+  }
+}
+
+// The warps' rows in a fixed order; thread = one k.
+__global__ void __launch_bounds__(128) lf_finalize_kernel(LegArgs<float> a, FinalizeArgs<float> f, const float4* partial,
+                                                          int64_t nkk, int nblk) {
+  const int m = blockIdx.y;
+  const int nk = (a.L - m) / 2 + 1;
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if ((int)(blockIdx.x * blockDim.x) >= nk) return;  // whole CTA
+  const float4* row = partial + ((lm_off(a.L, m) >> 1) + m);
+  auto sum = [&](int kk) {
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int b = 0; b < nblk; ++b) {
+      const float4 w = row[b * nkk + kk];
+      t = make_float4(t.x + w.x, t.y + w.y, t.z + w.z, t.w + w.w);
+    }
+    return t;
+  };
+  float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (k < nk) t = sum(k);
+  float2 um = make_float2(__shfl_up_sync(0xffffffffu, t.x, 1), __shfl_up_sync(0xffffffffu, t.y, 1));
+  if (k >= nk) return;
+  if ((threadIdx.x & 31) == 0) {
+    um = make_float2(0.f, 0.f);
+    if (k > 0) {
+      const float4 w = sum(k - 1);
+      um = make_float2(w.x, w.y);
+    }
+  }
+  lf_emit(a, f, m, k, t, um);
+}
+
+// All warps of one m in one CTA (grids of few pairs): the rows stay in shared
+// memory and the same kernel finishes the coefficients -- one launch instead
+// of two, no partial rows.
+template <int RP>
+__global__ void __launch_bounds__(32 * LF_FUSED) lf_adjoint_fused_kernel(LegArgs<float> a, FinalizeArgs<float> f) {
+  extern __shared__ __align__(16) unsigned char lf_dyn[];
+  const int b0 = lf_blocks<RP>(a.n1), b1 = lf_blocks<RP>(a.n2 - a.n1);
+  const int b = threadIdx.x >> 5, nw = blockDim.x >> 5, m = blockIdx.x;
+  const int nk = (a.L - m) / 2 + 1;
+  LfAdjStage& sh = reinterpret_cast<LfAdjStage*>(lf_dyn)[b];
+  float4* rows = reinterpret_cast<float4*>(lf_dyn + nw * sizeof(LfAdjStage));
+  const int ld = a.L / 2 + 1;
+  float* row = reinterpret_cast<float*>(rows + b * ld);
+  if (b < b0) lf_adjoint<0, RP>(a, sh, m, b * 32 * RP, a.n1, row);
+  else if (b < b0 + b1) lf_adjoint<1, RP>(a, sh, m, a.n1 + (b - b0) * 32 * RP, a.n2, row);
+  else lf_adjoint<2, RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, a.npairs, row);
+  __syncthreads();
+  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 um = make_float2(0.f, 0.f);
+    for (int w = 0; w < nw; ++w) {
+      const float4 x = rows[w * ld + k];
+      t = make_float4(t.x + x.x, t.y + x.y, t.z + x.z, t.w + x.w);
+      if (k > 0) {
+        const float4 y = rows[w * ld + k - 1];
+        um = make_float2(um.x + y.x, um.y + y.y);
+      }
+    }
+    lf_emit(a, f, m, k, t, um);
+  }
+}
+
+// ---- launchers ---------------------------------------------------------------
+
+static int lf_nblocks(const LegArgs<float>& a, int rp) {
+  auto nb = [&](int n) { return (n + 32 * rp - 1) / (32 * rp); };
+  return nb(a.n1) + nb(a.n2 - a.n1) + nb(a.npairs - a.n2);
+}
+int64_t lf_partial_bytes(int npairs, int L) {
+  return (int64_t)((npairs + 63) / 64 + 3) * ds_len(L) * (int64_t)sizeof(float4);
+}
+
+// ring pairs per thread where nothing was tuned: 4, or 2 where 4 would leave
+// fewer than 16 warps per SM
+static int lf_default_rp(const LegArgs<float>& a) {
+  return (int64_t)lf_nblocks(a, 4) * (a.L + 1) < 152 * 16 ? 2 : 4;
+}
+
+template <int RP>
+static void lf_synth_launch(const LegArgs<float>& a, cudaStream_t st) {
+  const int nb = lf_nblocks(a, RP);
+  if (a.mt_synth == 2) lf_synth_kernel<RP, 2><<<dim3(nb, (a.L + 2) / 2), 32, 0, st>>>(a);
+  else lf_synth_kernel<RP, 1><<<dim3(nb, a.L + 1), 32, 0, st>>>(a);
+  count_launch();
+}
+
+int launch_lf_synth(const LegArgs<float>& a, cudaStream_t st) {
+  const int rp = a.rp_synth ? a.rp_synth : lf_default_rp(a);
+  if (rp == 2) lf_synth_launch<2>(a, st);
+  else if (rp == 8) lf_synth_launch<8>(a, st);
+  else lf_synth_launch<4>(a, st);
+  CR_CHECK_LAUNCH("lf_synth_kernel");
+  return CR_OK;
+}
+
+template <int RP>
+static int lf_adjoint_launch(const LegArgs<float>& a, const FinalizeArgs<float>& f, cudaStream_t st) {
+  const int nb = lf_nblocks(a, RP);
+  const size_t smem = nb * (sizeof(LfAdjStage) + (size_t)(a.L / 2 + 1) * sizeof(float4));
+  if constexpr (RP <= 4) {
+    // few pairs: one CTA per m (up to LF_FUSED warps, 64 KB: three CTAs per SM)
+    if (a.mt_adj == 1 && nb <= LF_FUSED && smem <= 64 * 1024) {
+      CR_CUDA(cudaFuncSetAttribute(lf_adjoint_fused_kernel<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      { lf_adjoint_fused_kernel<RP><<<a.L + 1, 32 * nb, smem, st>>>(a, f); count_launch(); }
+      CR_CHECK_LAUNCH("lf_adjoint_fused_kernel");
+      return CR_OK;
+    }
+  }
+  float* part = reinterpret_cast<float*>(a.partial);
+  const int64_t nkk = ds_len(a.L);
+  if (a.mt_adj == 2) lf_adjoint_kernel<RP, 2><<<dim3(nb, (a.L + 2) / 2), 32, 0, st>>>(a, part, nkk);
+  else lf_adjoint_kernel<RP, 1><<<dim3(nb, a.L + 1), 32, 0, st>>>(a, part, nkk);
+  count_launch();
+  CR_CHECK_LAUNCH("lf_adjoint_kernel");
+  const dim3 grid((a.L / 2 + 1 + 127) / 128, a.L + 1);
+  { lf_finalize_kernel<<<grid, 128, 0, st>>>(a, f, reinterpret_cast<const float4*>(part), nkk, nb); count_launch(); }
+  CR_CHECK_LAUNCH("lf_finalize_kernel");
+  return CR_OK;
+}
+
+int launch_lf_adjoint(const LegArgs<float>& a, const FinalizeArgs<float>& f, cudaStream_t st) {
+  const int rp = a.rp_adj ? a.rp_adj : lf_default_rp(a);
+  if (rp == 2) return lf_adjoint_launch<2>(a, f, st);
+  if (rp == 8) return lf_adjoint_launch<8>(a, f, st);
+  if (rp == 16) return lf_adjoint_launch<16>(a, f, st);
+  return lf_adjoint_launch<4>(a, f, st);
+}
+
+}  // namespace cr

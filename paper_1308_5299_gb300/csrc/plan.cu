@@ -213,6 +213,11 @@ int grid_upload(Grid& g, int Lseed, cudaStream_t st) {
   CR_CUDA(cudaMemcpyAsync(g.d_z32, z32.data(), g.nring * sizeof(float), cudaMemcpyHostToDevice, st));
   CR_CUDA(cudaMemcpyAsync(g.d_sth, g.sth.data(), g.nring * sizeof(double), cudaMemcpyHostToDevice, st));
   g.nis = ds_first_equatorial(g.z.data(), g.npairs);
+  lf_zones(g.z.data(), g.npairs, &g.n1, &g.n2);
+  std::vector<float4> zi(g.npairs);
+  lf_args(g.z.data(), g.npairs, g.n1, g.n2, zi.data());
+  CR_CUDA(cudaMalloc(&g.d_zi, g.npairs * sizeof(float4)));
+  CR_CUDA(cudaMemcpyAsync(g.d_zi, zi.data(), g.npairs * sizeof(float4), cudaMemcpyHostToDevice, st));
   int rc = build_fft_tables(g, st);
   if (rc) return rc;
   return build_seeds(g, Lseed, st);
@@ -221,7 +226,7 @@ int grid_upload(Grid& g, int Lseed, cudaStream_t st) {
 void grid_free(Grid& g) {
   void* ptrs[] = {g.d_z, g.d_z32, g.d_w32, g.d_sth, g.d_fft, g.d_tab, g.d_tab32, g.d_vhat, g.d_vhat32,
                   g.d_tw, g.d_tw32, g.d_seed, g.d_lev, g.d_seed32, g.d_lev32, g.d_ls64, g.d_st64, g.d_ls32,
-                  g.d_st32, g.d_st64b, g.d_rings};
+                  g.d_st32, g.d_st64b, g.d_sti, g.d_zi, g.d_rings};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -287,7 +292,7 @@ int rebuild_coef(cr_plan* P, int Lc) {
 // Legendre seeds of a grid for a larger band limit.
 int grid_reseed(Grid& g, int Lseed, cudaStream_t st) {
   CR_CUDA(cudaStreamSynchronize(st));
-  void* ptrs[] = {g.d_seed, g.d_lev, g.d_seed32, g.d_lev32, g.d_ls64, g.d_st64, g.d_ls32, g.d_st32, g.d_st64b};
+  void* ptrs[] = {g.d_seed, g.d_lev, g.d_seed32, g.d_lev32, g.d_ls64, g.d_st64, g.d_ls32, g.d_st32, g.d_st64b, g.d_sti};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   g.d_seed = nullptr;
@@ -299,13 +304,14 @@ int grid_reseed(Grid& g, int Lseed, cudaStream_t st) {
   g.d_ls32 = nullptr;
   g.d_st32 = nullptr;
   g.d_st64b = nullptr;
+  g.d_sti = nullptr;
   return build_seeds(g, Lseed, st);
 }
 
 int ensure_workspace(cr_plan* P, const Grid& g, int L) {
   const int64_t phase = (int64_t)g.nring * (L + 1) * (int64_t)sizeof(double2);
   const int64_t partial = std::max((int64_t)leg_partial_blocks(g.npairs) * n_lm(L) * (int64_t)sizeof(double2),
-                                   ds_partial_bytes(g.nis, g.npairs, L, 1));
+                                   std::max(ds_partial_bytes(g.nis, g.npairs, L, 1), lf_partial_bytes(g.npairs, L)));
   if (phase > P->ws.phase_bytes) {
     if (P->ws.phase) cudaFree(P->ws.phase);
     P->ws.phase = nullptr;
@@ -348,7 +354,8 @@ __global__ void ninv32_kernel(const double* in, float* out, int64_t n) {
 // Choices of the Legendre autotuner: ring pairs per thread (2, 4 or 8, the
 // ring-block size of one CTA) per (grid shape, band limit, precision,
 // stage 0 synthesis / 1 adjoint), kept for the process and shared by every
-// plan with the same shapes; 4 where nothing was tuned.
+// plan with the same shapes; the launchers have their own rule where nothing
+// was tuned.
 struct TuneKey {
   int nring;
   int64_t npix;
@@ -374,11 +381,11 @@ static bool rp_allowed(int rp, int bytes, int stage) {
 static std::mutex g_tune_mu;
 static std::map<TuneKey, TuneVal> g_tune;
 
-// the cached (pairs per thread, m tile) of a stage; (4, 1) when not tuned
+// the cached (pairs per thread, m tile) of a stage; (0, 1) when not tuned: the launcher's own rule
 static void tuned_shape(const Grid& g, int L, int bytes, int stage, int* rp, int* mt) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find(TuneKey{g.nring, g.npix, L, bytes, stage});
-  *rp = it == g_tune.end() ? 4 : it->second.rp;
+  *rp = it == g_tune.end() ? 0 : it->second.rp;
   *mt = it == g_tune.end() ? 1 : it->second.mt;
 }
 
@@ -427,6 +434,12 @@ static LegArgs<T> leg_args(cr_plan* P, const Grid& g, int L) {
     a.npolar = g.npolar32;
     a.ls = g.d_ls32;
     a.st = g.d_st32;
+    a.rf = P->ds->rf;
+    a.cf = P->ds->cf;
+    a.zi = g.d_zi;
+    a.sti = g.d_sti;
+    a.n1 = g.n1;
+    a.n2 = g.n2;
   }
   a.ld_seed = g.npairs;
   a.npairs = g.npairs;
