@@ -291,6 +291,7 @@ static int load_impl(cr_plan* plan, const char* path) {
     lev.amax = lv[i].amax;
     lev.lambda_max = lv[i].lambda_max;
     lev.lt_valid = false;
+    if ((rc = build_dense_inverse(plan, lev))) return rc;
   }
   H.top_lambda = top_lambda;
   H.top_scale = top_scale;

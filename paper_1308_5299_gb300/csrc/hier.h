@@ -64,6 +64,8 @@ struct PixLevel {
   float* d_L = nullptr;    // factor blocks (diagonal blocks hold inv(L_pp))
   float* d_LT = nullptr;   // backward-sweep copy: per position p, column p's blocks transposed, then inv(L_pp)^T
   bool lt_valid = false;
+  float* d_inv = nullptr;  // explicit inverse [n][n], RING order (levels with few tiles)
+  bool inv_valid = false;
   int* d_perm = nullptr;   // tile-ordered level pixel -> RING index
   int* d_colour_start = nullptr;  // device copy of pat.colour_start
   int coop_grid = 0;       // CTAs of the one-launch cooperative sweeps (0: one launch per colour)

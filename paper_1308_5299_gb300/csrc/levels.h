@@ -40,6 +40,7 @@ template <typename T> int apply_smoother(cr_plan* P, PixLevel& lev, T* map_in, T
 template <typename T>
 int apply_smoother_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map_out, int64_t ld);
 int ensure_smoother_batch(cr_plan* P);
+int build_dense_inverse(cr_plan* P, PixLevel& lev);
 int sweep_status(cr_plan* P);
 void free_smoother(PixLevel& lev);
 

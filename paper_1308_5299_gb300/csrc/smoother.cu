@@ -1091,7 +1091,7 @@ int factorise(cr_plan* P, PixLevel& lev, float alpha, bool* ok) {
   const size_t smem = 4 * TK * (TK + 1) * sizeof(float);
   CR_CUDA(cudaFuncSetAttribute(icc_colour_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   CR_CUDA(cudaMemsetAsync(lev.d_fail, 0, sizeof(int), P->stream));
-  lev.lt_valid = false;
+  lev.lt_valid = lev.inv_valid = false;
   for (size_t c = 0; c + 1 < pat.colour_start.size(); ++c) {
     const int p0 = pat.colour_start[c], p1 = pat.colour_start[c + 1];
     if (p1 > p0) { icc_colour_kernel<<<p1 - p0, MR_NT, smem, P->stream>>>(a, p0); count_launch(); }
@@ -1424,6 +1424,50 @@ int smoother_numeric(cr_plan* P, PixLevel& lev, double ridge_factor, int bisecti
   return CR_OK;
 }
 
+// ---- explicit inverse on the coarsest levels ---------------------------------
+// With at most DI_TILES tiles the 14 or so dependent tile solves of the sweeps
+// take 45 to 65 us on one to a dozen SMs, whatever their size; the inverse M
+// itself is small (n = 768: 2.4 MB, n = 3072: 38 MB, read from L2 between
+// visits), and applying it is one matrix-vector product over the whole chip:
+// 4 and 9 us.  At n = 12288 (604 MB) the product would take longer than the
+// 68 us of the sweeps.  M's columns are the sweeps' results for unit vectors,
+// 16 at a time, averaged with their transpose.
+constexpr int DI_TILES = 48;
+
+__global__ void unit_panel_kernel(float* v, int n, int j0) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < SM_NR * n; i += gridDim.x * blockDim.x)
+    v[i] = (i % n == j0 + i / n) ? 1.f : 0.f;
+}
+__global__ void average_transpose_kernel(float* M, int n) {
+  const int i = blockIdx.y * blockDim.y + threadIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n || j >= i) return;
+  const float a = 0.5f * (M[(int64_t)i * n + j] + M[(int64_t)j * n + i]);
+  M[(int64_t)i * n + j] = a;
+  M[(int64_t)j * n + i] = a;
+}
+
+// out = M in, one warp per row; n a multiple of 128
+template <typename T>
+__global__ void __launch_bounds__(256) dense_apply_kernel(const float* __restrict__ M, const T* __restrict__ in, T* out,
+                                                          int n) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const float4* m4 = reinterpret_cast<const float4*>(M + (int64_t)row * n);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 6
+  for (int i = lane; i < n / 4; i += 32) {
+    const float4 a = m4[i];
+    const T* v = in + 4 * i;
+    acc.x = fmaf(a.x, (float)v[0], acc.x);
+    acc.y = fmaf(a.y, (float)v[1], acc.y);
+    acc.z = fmaf(a.z, (float)v[2], acc.z);
+    acc.w = fmaf(a.w, (float)v[3], acc.w);
+  }
+  float s = (acc.x + acc.y) + (acc.z + acc.w);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[row] = (T)s;
+}
+
 // the backward sweep's transposed copy of the factor, made on first use
 static int ensure_lt(cr_plan* P, PixLevel& lev) {
   if (lev.lt_valid) return CR_OK;
@@ -1442,6 +1486,12 @@ int apply_smoother(cr_plan* P, PixLevel& lev, T* map_in, T* map_out) {
   if (P->hier && P->hier->smoother_kind == 1) {
     { schwarz_apply_kernel<T><<<pat.ntile, TK, 0, P->stream>>>(lev.d_L, lev.d_perm, map_in, map_out); count_launch(); }
     CR_CHECK_LAUNCH("schwarz_apply_kernel");
+    return CR_OK;
+  }
+  if (lev.inv_valid) {
+    const int n = pat.ntile * TK;
+    { dense_apply_kernel<T><<<n / 8, 256, 0, P->stream>>>(lev.d_inv, map_in, map_out, n); count_launch(); }
+    CR_CHECK_LAUNCH("dense_apply_kernel");
     return CR_OK;
   }
   int rc = ensure_lt(P, lev);
@@ -1523,6 +1573,8 @@ template int apply_smoother<float>(cr_plan*, PixLevel&, float*, float*);
 // the one-map path per map.  The tile work vectors of the batch live in
 // the hierarchy's batch buffer (ensure_smoother_batch).
 template <typename T>
+static int sweep_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map_out, int64_t ld, float* y);
+template <typename T>
 int apply_smoother_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map_out, int64_t ld) {
   if (nr < 1 || nr > SM_NR) return fail(CR_EINVAL, "pixel smoother: 1 to 16 maps per call");
   Hierarchy& H = *P->hier;
@@ -1533,14 +1585,20 @@ int apply_smoother_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map
     }
     return CR_OK;
   }
+  if (!H.d_mr_y || H.mr_y_len < (int64_t)lev.pat.ntile * TK)
+    return fail(CR_ESTATE, "pixel smoother: batch buffer missing");
+  return sweep_mr<T>(P, lev, nr, map_in, map_out, ld, H.d_mr_y);
+}
+
+// the sweeps of nr maps; y: tile work vectors [nr][ntile * TK]
+template <typename T>
+static int sweep_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map_out, int64_t ld, float* y) {
   const BlockPattern& pat = lev.pat;
   const int64_t ly = (int64_t)pat.ntile * TK;
-  if (!H.d_mr_y || H.mr_y_len < ly) return fail(CR_ESTATE, "pixel smoother: batch buffer missing");
   int rc = ensure_lt(P, lev);
   if (rc) return rc;
   CR_CUDA(cudaFuncSetAttribute(fwd_colour_mr_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_SMEM));
   CR_CUDA(cudaFuncSetAttribute(bwd_colour_mr_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_SMEM));
-  float* y = H.d_mr_y;
   const int nc = (int)pat.colour_start.size() - 1;
   for (int c = 0; c < nc; ++c) {
     const int p0 = pat.colour_start[c], p1 = pat.colour_start[c + 1];
@@ -1558,6 +1616,35 @@ int apply_smoother_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map
   CR_CHECK_LAUNCH("bwd_colour_mr_kernel");
   return CR_OK;
 }
+// The explicit inverse of a level with few tiles from its present factor
+// (once per factor, at the end of the precompute); only where the form of the
+// sweeps was left to the library.
+int build_dense_inverse(cr_plan* P, PixLevel& lev) {
+  const Hierarchy& H = *P->hier;
+  lev.inv_valid = false;
+  if (H.smoother_kind != 0 || H.sweep_mode != 0 || lev.pat.ntile > DI_TILES) return CR_OK;
+  const int n = lev.pat.ntile * TK;
+  if (!lev.d_inv) CR_CUDA(cudaMalloc(&lev.d_inv, (size_t)n * n * sizeof(float)));
+  float* tmp = nullptr;
+  CR_CUDA(cudaMalloc(&tmp, (size_t)2 * SM_NR * n * sizeof(float)));
+  int rc = CR_OK;
+  for (int j0 = 0; j0 < n && !rc; j0 += SM_NR) {
+    unit_panel_kernel<<<152, 256, 0, P->stream>>>(tmp, n, j0);
+    count_launch();
+    rc = sweep_mr<float>(P, lev, SM_NR, tmp, lev.d_inv + (int64_t)j0 * n, n, tmp + (int64_t)SM_NR * n);
+  }
+  if (!rc) {
+    average_transpose_kernel<<<dim3((n + 31) / 32, (n + 7) / 8), dim3(32, 8), 0, P->stream>>>(lev.d_inv, n);
+    count_launch();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
+    if (e != cudaSuccess) rc = cuda_fail(e, "dense inverse");
+  }
+  cudaFree(tmp);
+  lev.inv_valid = rc == CR_OK;
+  return rc;
+}
+
 template int apply_smoother_mr<double>(cr_plan*, PixLevel&, int, const double*, double*, int64_t);
 template int apply_smoother_mr<float>(cr_plan*, PixLevel&, int, const float*, float*, int64_t);
 
@@ -1585,7 +1672,7 @@ void free_smoother(PixLevel& lev) {
   void* ptrs[] = {lev.d_A, lev.d_L, lev.d_LT, lev.d_perm, lev.d_colour_start, lev.d_row_ptr, lev.d_row_col,
                   lev.d_col_ptr, lev.d_col_row,
                   lev.d_col_blk, lev.d_upd_ptr, lev.d_tgt_blk, lev.d_tgt_u, lev.d_tgt_ptr, lev.d_pair_a, lev.d_pair_b,
-                  lev.d_fail, lev.d_flow_task, lev.d_flow_off};
+                  lev.d_fail, lev.d_flow_task, lev.d_flow_off, lev.d_inv};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }

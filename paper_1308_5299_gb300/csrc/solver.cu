@@ -564,6 +564,8 @@ int build_numeric(cr_plan* P) {
     }
   }
   if ((rc = build_bottom(P, H))) return rc;
+  for (auto& lev : H.pix)
+    if ((rc = build_dense_inverse(P, lev))) return rc;
   CR_CUDA(cudaStreamSynchronize(P->stream));
   H.numeric_ready = true;
   return CR_OK;
