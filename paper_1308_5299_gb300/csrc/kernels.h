@@ -100,6 +100,8 @@ struct RingArgs {
   T* map_out = nullptr;        // mode 0 output; mode 2 optional copy of Y x
   const T* map_in = nullptr;   // mode 1 input
   const T* pixdiag = nullptr;  // mode 2 diagonal
+  const int* live = nullptr;   // mode 2: rings with a non-zero diagonal (null: all)
+  int np_live = 0;             // and the pairs of the Legendre stages around it
   int nring = 0;
   const int* rings = nullptr;  // ring indices ordered by FFT size (device)
   int rbase = 0;               // first entry of this launch's class
@@ -131,8 +133,8 @@ struct TcTail {
 int tc_begin(cr_plan* P, const Grid& g, int L, bool adjoint, bool reset_status);
 int tc_end(cr_plan* P, const char* what);
 float2* tc_slot(cr_plan* P, const Grid& g, int L, int r);
-int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, const float* dl);
-int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t);
+int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, const float* dl, bool masked = false);
+int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t, bool masked = false);
 int tc_ring(cr_plan* P, const Grid& g, int L, int r, int mode, const float* map_in, float* map_out);
 int tc_sandwich(cr_plan* P, const Grid& g, int L, int nr, const float2* x, const float* dl_in, const float* pix,
                 const TcTail& t);

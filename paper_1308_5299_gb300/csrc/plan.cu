@@ -339,7 +339,7 @@ static void plan_free(cr_plan* P) {
   void* ptrs[] = {P->d_c, P->d_s, P->d_c32, P->d_c2_32, P->d_s32, P->d_bl, P->d_sinv, P->d_bl32, P->d_sinv32,
                   P->d_ninv, P->d_ninv32, P->ws.phase, P->ws.partial, P->ws_mr.phase, P->ws_mr.partial, P->d_tc_r64, P->d_pcinv,
                   P->cgv[0], P->cgv[1],
-                  P->cgv[2], P->cgv[3], P->d_cgdot, P->tc_phase, P->d_tc_status, P->tc_partial, P->d_dotpart};
+                  P->cgv[2], P->cgv[3], P->d_ring_live, P->d_cgdot, P->tc_phase, P->d_tc_status, P->tc_partial, P->d_dotpart};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -474,6 +474,32 @@ static RingArgs<T> ring_args(cr_plan* P, const Grid& g, int L) {
   return r;
 }
 
+// In Y^T diag(pix) Y with the plan's own N^-1 a ring whose weights are all zero
+// contributes nothing: its azimuthal stage writes zeros, and the ring pairs
+// after the last one with a weight (the galactic cut of a map in galactic
+// coordinates, 13 % of the pairs at |b| < 10 degrees and the ones with the most
+// terms) take no part in either Legendre stage.
+template <typename T>
+static bool masked_rings(const cr_plan* P, const Grid& g, const T* pix) {
+  return &g == &P->obs && P->d_ring_live &&
+         (const void*)pix == (sizeof(T) == 8 ? (const void*)P->d_ninv : (const void*)P->d_ninv32);
+}
+template <typename T>
+static void limit_pairs(const cr_plan* P, LegArgs<T>& a) {
+  const int n = P->np_live;
+  a.npairs = n;
+  a.nis = std::min(a.nis, n);
+  a.n1 = std::min(a.n1, n);
+  a.n2 = std::min(a.n2, n);
+  a.npolar = std::min(a.npolar, n);
+  a.npolar_df = std::min(a.npolar_df, n);
+}
+template <typename T>
+static void limit_rings(const cr_plan* P, RingArgs<T>& r) {
+  r.live = P->d_ring_live;
+  r.np_live = P->np_live;
+}
+
 template <typename T>
 static const char* ptag() {
   return sizeof(T) == 8 ? "_f64" : "_f32";
@@ -564,6 +590,8 @@ int do_sandwich(cr_plan* P, const Grid& g, int L, const void* x, void* y, const 
   LegArgs<T> a = leg_args<T>(P, g, L);
   a.alm = reinterpret_cast<const typename Tr<T>::C*>(x);
   a.dl = dl_in;
+  const bool masked = !map_copy && masked_rings(P, g, pix);
+  if (masked) limit_pairs(P, a);
   int rc;
   {
     TimerScope ts(P->timing, P->stream, std::string("legendre_synth") + ptag<T>(), leg_work(g, L),
@@ -574,6 +602,7 @@ int do_sandwich(cr_plan* P, const Grid& g, int L, const void* x, void* y, const 
   RingArgs<T> r = ring_args<T>(P, g, L);
   r.pixdiag = pix;
   r.map_out = map_copy;
+  if (masked) limit_rings(P, r);
   {
     // phase read and written back, pixel diagonal read (+ the map copy)
     TimerScope ts(P->timing, P->stream, std::string("ring_fft_apply") + ptag<T>(),
@@ -631,6 +660,8 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
   double2* part = reinterpret_cast<double2*>(P->ws_mr.partial);
   LegArgs<double> a = leg_args<double>(P, g, L);
   a.dl = dl_in;
+  const bool masked = masked_rings(P, g, pix);
+  if (masked) limit_pairs(P, a);
   {
     TimerScope ts(P->timing, P->stream, "legendre_synth_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
     rc = ds_use(a) ? launch_ds_synth(a, x, nlm, nr, ph, P->stream)
@@ -640,6 +671,7 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
     RingArgs<double> ra = ring_args<double>(P, g, L);
     ra.phase = ph + r * ld_phase;
     ra.pixdiag = pix;
+    if (masked) limit_rings(P, ra);
     TimerScope ts(P->timing, P->stream, "ring_fft_apply_f64",
                   fft_bytes<double>(g, L, 1) + (double)g.nring * (L + 1) * sizeof(double2));
     rc = launch_ring_fft<double>(ra, 2, P->stream);
@@ -931,6 +963,8 @@ static int plan_init(cr_plan* P, const cr_params* p) {
         // non-finite residual
         const int64_t chunk = (int64_t)1 << 22;
         std::vector<double> h((size_t)std::min<int64_t>(chunk, npix));
+        std::vector<int> live(P->obs.nring, 0);  // rings with a non-zero weight
+        int ring = 0;
         for (int64_t o = 0; o < npix && !rc; o += chunk) {
           const int64_t n = std::min(chunk, npix - o);
           cudaError_t e = cudaMemcpyAsync(h.data(), P->d_ninv + o, n * sizeof(double), cudaMemcpyDeviceToHost,
@@ -945,6 +979,20 @@ static int plan_init(cr_plan* P, const cr_params* p) {
               rc = fail(CR_EINVAL, "cr_plan_create: N^-1 must be finite and >= 0 (pixel " + std::to_string(o + i) + ")");
               break;
             }
+          for (int64_t i = 0; i < n && !rc;) {
+            while (o + i >= P->obs.fft[ring].off + P->obs.fft[ring].n) ++ring;
+            const int64_t end = std::min(n, P->obs.fft[ring].off + P->obs.fft[ring].n - o);
+            for (; i < end && !live[ring]; ++i) live[ring] = h[i] != 0.0;
+            i = end;
+          }
+        }
+        if (!rc) {
+          P->np_live = 1;
+          for (int k = 0; k < P->obs.npairs; ++k)
+            if (live[k] || live[P->obs.nring - 1 - k]) P->np_live = k + 1;
+          cudaError_t e = cudaMalloc(&P->d_ring_live, live.size() * sizeof(int));
+          if (e == cudaSuccess) e = cudaMemcpy(P->d_ring_live, live.data(), live.size() * sizeof(int), cudaMemcpyHostToDevice);
+          if (e != cudaSuccess) rc = cuda_fail(e, "ring flags");
         }
       }
       if (!rc) {
@@ -1115,9 +1163,10 @@ float2* tc_slot(cr_plan* P, const Grid& g, int L, int r) {
 
 // the synthesis Legendre stage of nr <= 16 right-hand sides x [nr][n_lm(L)]
 // (times dl, may be null) into the phase slots
-int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, const float* dl) {
+int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, const float* dl, bool masked) {
   LegArgs<float> la = leg_args<float>(P, g, L);
   la.dl = dl;
+  if (masked) limit_pairs(P, la);
   TimerScope ts(P->timing, P->stream, "legendre_synth_tc", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
   return launch_tc_synth(la, x, n_lm(L), nr, tc_slot(P, g, L, 0), P->d_tc_status, P->stream);
 }
@@ -1125,8 +1174,9 @@ int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, co
 // the adjoint Legendre stage of nr right-hand sides from the phase slots,
 // then per right-hand side r (vectors at stride n_lm(L)):
 //   out_r (+)= dl_out sum_blk partial + dadd xadd_r   (or bsub_r - that)
-int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t) {
+int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t, bool masked) {
   LegArgs<float> la = leg_args<float>(P, g, L);
+  if (masked) limit_pairs(P, la);
   const int64_t nlm = n_lm(L);
   int nblk = 0, rc;
   {
@@ -1169,17 +1219,19 @@ int tc_ring(cr_plan* P, const Grid& g, int L, int r, int mode, const float* map_
 // tensor cores
 int tc_sandwich(cr_plan* P, const Grid& g, int L, int nr, const float2* x, const float* dl_in, const float* pix,
                 const TcTail& t) {
-  int rc = tc_synth_stage(P, g, L, x, nr, dl_in);
+  const bool masked = masked_rings(P, g, pix);
+  int rc = tc_synth_stage(P, g, L, x, nr, dl_in, masked);
   if (rc) return rc;
   for (int r = 0; r < nr; ++r) {
     RingArgs<float> ra = ring_args<float>(P, g, L);
     ra.phase = tc_slot(P, g, L, r);
     ra.pixdiag = pix;
+    if (masked) limit_rings(P, ra);
     TimerScope ts(P->timing, P->stream, "ring_fft_apply_f32",
                   fft_bytes<float>(g, L, 1) + (double)g.nring * (L + 1) * sizeof(float2));
     if ((rc = launch_ring_fft<float>(ra, 2, P->stream))) return rc;
   }
-  return tc_adjoint_tail(P, g, L, nr, t);
+  return tc_adjoint_tail(P, g, L, nr, t, masked);
 }
 
 }  // namespace cr

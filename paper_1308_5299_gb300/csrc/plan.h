@@ -153,6 +153,8 @@ struct cr_plan {
   float* d_sinv32 = nullptr;
   double* d_ninv = nullptr;  // [npix] obs grid
   float* d_ninv32 = nullptr;
+  int* d_ring_live = nullptr;  // [nring] 1 where the ring has a non-zero weight
+  int np_live = 0;             // ring pairs up to the last one with a weight
   cr::Workspace ws;
   cr::Workspace ws_mr;
   double2* d_tc_r64 = nullptr;  // FP64 residuals of a batch of 16 right-hand sides

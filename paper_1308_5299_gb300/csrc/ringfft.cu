@@ -213,6 +213,11 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
   const int L = a.L;
   const int tid = threadIdx.x;
   const int NT = blockDim.x;
+  if (MODE == 2 && a.live && !a.live[r]) {
+    if (min(r, a.nring - 1 - r) < a.np_live)
+      for (int m = tid; m <= L; m += NT) row[m] = mk((T)0, (T)0);
+    return;
+  }
   // e^{i pi (2 k^2 mod 2n) / n}; 2 k^2 < 2^31 for k < 2^15
   auto chirp = [&](int k) -> C { return tab[(int)((2u * (unsigned)k * (unsigned)k) % (unsigned)twon)]; };
 
