@@ -51,90 +51,106 @@ __device__ __forceinline__ int bitrev(int k, int logM) {
   return logM ? (int)(__brev((unsigned)k) >> (32 - logM)) : 0;
 }
 
-template <typename C>
-__device__ __forceinline__ C twid(const C* __restrict__ tw, int idx, int sign) {
-  const C w = tw[idx];
-  return sign > 0 ? cconj(w) : w;
-}
-// radix-2 butterflies: decimation in time a' = a + w b, b' = a - w b;
-// decimation in frequency a' = a + b, b' = (a - b) w
-template <typename C>
-__device__ __forceinline__ void bf_dit(C& a, C& b, C w) {
-  const C v = cmul(b, w);
-  b = csub(a, v);
-  a = cadd(a, v);
-}
-template <typename C>
-__device__ __forceinline__ void bf_dif(C& a, C& b, C w) {
-  const C u = a;
-  a = cadd(u, b);
-  b = cmul(csub(u, b), w);
-}
+// e^{-2 pi i v / 16}, v < 4, and the half steps of 32: the constant factors of
+// the twiddles inside one pass (cos and sin of 2 pi v / 16)
+__device__ constexpr double RC16[4] = {1.0, 0.923879532511286756128, 0.707106781186547524401, 0.382683432365089771728};
+__device__ constexpr double RS16[4] = {0.0, 0.382683432365089771728, 0.707106781186547524401, 0.923879532511286756128};
 
-// e^{-2 pi i v / 32}, v < 16: the constant factors of the twiddles inside
-// one pass (cos and sin of 2 pi v / 32)
-__device__ constexpr double RC32[16] = {1.0, 0.980785280403230449126, 0.923879532511286756128, 0.831469612302545237079,
-                                        0.707106781186547524401, 0.555570233019602224743, 0.382683432365089771728,
-                                        0.195090322016128267848, 0.0, -0.195090322016128267848, -0.382683432365089771728,
-                                        -0.555570233019602224743, -0.707106781186547524401, -0.831469612302545237079,
-                                        -0.923879532511286756128, -0.980785280403230449126};
-__device__ constexpr double RS32[16] = {0.0, 0.195090322016128267848, 0.382683432365089771728, 0.555570233019602224743,
-                                        0.707106781186547524401, 0.831469612302545237079, 0.923879532511286756128,
-                                        0.980785280403230449126, 1.0, 0.980785280403230449126, 0.923879532511286756128,
-                                        0.831469612302545237079, 0.707106781186547524401, 0.555570233019602224743,
-                                        0.382683432365089771728, 0.195090322016128267848};
+// Radix-2 butterfly a' = a + w b, b' = a - w b in six fused operations: a' by
+// two per component, b' = 2 a - a'.  (Both transforms below are arranged so
+// that the twiddle multiplies an input; the form with the twiddle on the
+// difference takes eight.)
+template <typename C>
+__device__ __forceinline__ void bf_fma(C& a, C& b, C w) {
+  using T = decltype(C().x);
+  const T x = fma(w.x, b.x, fma(-w.y, b.y, a.x));
+  const T y = fma(w.x, b.y, fma(w.y, b.x, a.y));
+  b = mk(fma((T)2, a.x, -x), fma((T)2, a.y, -y));
+  a = mk(x, y);
+}
+// the same with w = 1, and with w = sign i
+template <typename C>
+__device__ __forceinline__ void bf_one(C& a, C& b) {
+  const C t = b;
+  b = csub(a, t);
+  a = cadd(a, t);
+}
+template <typename C>
+__device__ __forceinline__ void bf_rot(C& a, C& b, int sign) {
+  const C t = sign > 0 ? mk(-b.y, b.x) : mk(b.y, -b.x);
+  b = csub(a, t);
+  a = cadd(a, t);
+}
 
 // One pass of NS consecutive radix-2 stages on groups of 2^NS elements
-// j0 + t h (t < 2^NS) held in registers.  Stage s of the pass has span
-// 2^s h; its butterfly on (t, t + 2^s), u = t mod 2^s, uses the twiddle
-// e^{-+2 pi i (k + u h) / (2^(s+1) h)}.  With CTW (computed twiddles) that
-// is base_s e^{-+2 pi i u / 2^(s+1)}: one table value per stage and group
-// (base_s, index k Mmax / (2^(s+1) h)) times a compile-time root of unity --
-// fewer loads for a few FP32 multiplies; without, every distinct twiddle
-// is a table value (FP64, where a multiply costs more than a cached load).
-// DIT runs the stages with spans h, 2h, ... (bit-reversed input, natural
-// output); DIF the reverse (natural input, bit-reversed output).  post (may
-// be null): every element is multiplied by post[its position] before it is
-// stored (the pointwise product of a convolution, fused into the last pass).
-template <typename C, int NS, bool DIT, bool CTW>
-__device__ __forceinline__ void fft_pass(C* buf, int M, int lh, int sign, const C* __restrict__ tw, int Mmax,
+// j0 + i h (i < 2^NS) held in registers.
+//  - FWD (natural input, bit-reversed output, e^{-}): a block of the pass is a
+//    polynomial modulo x^len - c^2, split into x^(len/2) -+ c; at depth d
+//    block B has c = e^{-2 pi i brv_d(B) / 2^(d+1)}, so a group has one c per
+//    stage, c_s = e^{-2 pi i brv_t(B) / 2^(t+s+1)}, times e^{-2 pi i brv_s(j) /
+//    2^(s+1)} for the j-th part of stage s.  post (may be null): the output is
+//    multiplied by post at its positions (the pointwise product of a
+//    convolution, fused into the last pass).
+//  - inverse (bit-reversed input, natural output, e^{+}): stage s joins spans
+//    2^s h with w = e^{2 pi i (k + u h) / (2^(s+1) h)} = c_s e^{2 pi i u / 2^(s+1)}.
+// Either way a stage's upper half of constants is i (or -i) times the lower
+// half, one table value per stage and group serves it, and the pass whose
+// table values are all 1 (TRIV: the first of either transform) has constant
+// twiddles only.
+template <typename C, int NS, bool FWD, bool TRIV>
+__device__ __forceinline__ void fft_pass(C* buf, int M, int lg, const C* __restrict__ tw, int Mmax,
                                          const C* __restrict__ post) {
   using T = decltype(C().x);
   constexpr int R = 1 << NS;
+  constexpr int sign = FWD ? -1 : 1;
+  // FWD: lg = depth t of the pass (2^t blocks), h = len / R; inverse: h = 2^lg
+  const int lh = FWD ? (31 - __clz(M)) - lg - NS : lg;
   const int h = 1 << lh;
   const int ng = M >> NS;
   for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-    const int k = g & (h - 1);
-    const int j0 = ((g - k) << NS) + k;
-    C base[NS];
-    if (CTW) {
+    const int k = g & (h - 1), B = g >> lh;
+    const int j0 = (B << (lh + NS)) + k;
+    C c[NS];
+    if (!TRIV) {
+      const int idx = FWD ? (lg ? (int)(__brev((unsigned)B) >> (32 - lg)) : 0) : k;
 #pragma unroll
-      for (int s = 0; s < NS; ++s) base[s] = twid(tw, k * (Mmax >> (lh + s + 1)), sign);
+      for (int s = 0; s < NS; ++s) {
+        c[s] = tw[idx * (Mmax >> (FWD ? lg + s + 1 : lh + s + 1))];
+        if (!FWD) c[s] = cconj(c[s]);
+      }
     }
     C e[R];
 #pragma unroll
     for (int t = 0; t < R; ++t) e[t] = buf[swz(j0 + t * h)];
 #pragma unroll
-    for (int si = 0; si < NS; ++si) {
-      const int s = DIT ? si : NS - 1 - si;
-      const int S = 1 << s;
+    for (int s = 0; s < NS; ++s) {
+      // span of the stage in i; q-th twiddle of the stage's 2^s
+      const int S = FWD ? R >> (s + 1) : 1 << s;
 #pragma unroll
-      for (int t = 0; t < R; ++t) {
-        if (t & S) continue;
-        const int u = t & (S - 1);
-        C w;
-        if (CTW) {
-          w = base[s];
-          if (u) {
-            const int v = u << (4 - s);
-            const T cr = (T)RC32[v], ci = (T)(sign > 0 ? RS32[v] : -RS32[v]);
-            w = mk(w.x * cr - w.y * ci, w.x * ci + w.y * cr);
-          }
-        } else {
-          w = twid(tw, (k + u * h) * (Mmax >> (lh + s + 1)), sign);
+      for (int q = 0; q < (1 << s); ++q) {
+        // constant e^{sign 2 pi i v / 2^(s+1)}: v = q, or its bit reversal; 16ths
+        int v = q;
+        if (FWD) {
+          v = 0;
+#pragma unroll
+          for (int z = 0; z < s; ++z) v |= ((q >> z) & 1) << (s - 1 - z);
         }
-        if (DIT) bf_dit(e[t], e[t + S], w);
-        else bf_dif(e[t], e[t + S], w);
+        const int v16 = v << (3 - s);
+        const bool rot = v16 >= 4;  // an extra factor sign i
+        const int vv = v16 & 3;
+        C w = mk((T)RC16[vv], (T)(sign > 0 ? RS16[vv] : -RS16[vv]));
+        if (!TRIV) w = vv ? cmul(c[s], w) : c[s];
+        if (rot) w = sign > 0 ? mk(-w.y, w.x) : mk(w.y, -w.x);
+#pragma unroll
+        for (int r = 0; r < R / 2 / (1 << s); ++r) {
+          const int i = FWD ? q * 2 * S + r : r * 2 * S + q;
+          if (TRIV && vv == 0) {
+            if (rot) bf_rot(e[i], e[i + S], sign);
+            else bf_one(e[i], e[i + S]);
+          } else {
+            bf_fma(e[i], e[i + S], w);
+          }
+        }
       }
     }
     if (post) {
@@ -146,56 +162,43 @@ __device__ __forceinline__ void fft_pass(C* buf, int M, int lh, int sign, const 
   }
 }
 
-// BIG: up to 4 stages per pass with computed twiddles (FP32 rings with
-// M >= 4096: fewer barriers and shared-memory round trips, at 75 registers);
-// otherwise up to 3 with table twiddles (fewer registers, so more CTAs per
-// SM, which the small rings need).  Never more stages than leave one group
-// per thread.
+// BIG: up to 4 stages per pass (FP32 rings with M >= 4096: fewer barriers and
+// shared-memory round trips, at 75 registers); otherwise up to 3 (fewer
+// registers, so more CTAs per SM, which the small rings need).  Never more
+// stages than leave one group per thread.
 template <bool BIG>
 __device__ __forceinline__ int fft_pass_cap(int logM) {
   const int lt = 31 - __clz((int)blockDim.x);
   return max(1, min(BIG ? 4 : 3, logM - lt));
 }
 
-template <typename C, bool DIT, bool BIG>
-__device__ __forceinline__ void fft_pass_ns(int ns, C* buf, int M, int lh, int sign, const C* __restrict__ tw,
-                                            int Mmax, const C* __restrict__ post) {
-  if (BIG && ns == 4) fft_pass<C, 4, DIT, true>(buf, M, lh, sign, tw, Mmax, post);
-  else if (ns >= 3) fft_pass<C, 3, DIT, BIG>(buf, M, lh, sign, tw, Mmax, post);
-  else if (ns == 2) fft_pass<C, 2, DIT, BIG>(buf, M, lh, sign, tw, Mmax, post);
-  else fft_pass<C, 1, DIT, BIG>(buf, M, lh, sign, tw, Mmax, post);
+template <typename C, bool FWD, bool TRIV, bool BIG>
+__device__ __forceinline__ void fft_pass_ns(int ns, C* buf, int M, int lg, const C* __restrict__ tw, int Mmax,
+                                            const C* __restrict__ post) {
+  if (BIG && ns == 4) fft_pass<C, 4, FWD, TRIV>(buf, M, lg, tw, Mmax, post);
+  else if (ns >= 3) fft_pass<C, 3, FWD, TRIV>(buf, M, lg, tw, Mmax, post);
+  else if (ns == 2) fft_pass<C, 2, FWD, TRIV>(buf, M, lg, tw, Mmax, post);
+  else fft_pass<C, 1, FWD, TRIV>(buf, M, lg, tw, Mmax, post);
 }
 
-// In-place radix-2 decimation-in-time FFT: bit-reversed input, natural output.
-// sign = -1 forward (e^{-2 pi i jk/M}), +1 inverse (unnormalised).  Passes
-// of several consecutive stages, one barrier per pass.
-template <bool BIG = false, typename C>
-__device__ void fft_dit(C* buf, int M, int logM, int sign, const C* __restrict__ tw, int Mmax) {
-  const int cap = fft_pass_cap<BIG>(logM);
-  int lh = 0;
-  while (lh < logM) {
-    const int ns = min(cap, logM - lh);
-    fft_pass_ns<C, true, BIG>(ns, buf, M, lh, sign, tw, Mmax, nullptr);
-    __syncthreads();
-    lh += ns;
-  }
-}
-
-// In-place radix-2 decimation-in-frequency FFT: natural input, bit-reversed
-// output; passes of several stages (largest span first).  post (may be
-// null): multiply the output, in its bit-reversed positions, by post.
-template <bool BIG = false, typename C>
-__device__ void fft_dif(C* buf, int M, int logM, int sign, const C* __restrict__ tw, int Mmax,
+// In-place transforms, one barrier per pass: inverse (e^{+2 pi i jk/M},
+// unnormalised) from bit-reversed to natural order, forward from natural to
+// bit-reversed order.
+template <bool FWD, bool BIG, typename C>
+__device__ void fft_run(C* buf, int M, int logM, const C* __restrict__ tw, int Mmax,
                         const C* __restrict__ post = nullptr) {
   const int cap = fft_pass_cap<BIG>(logM);
-  int lt = logM;  // stages with span >= 2^lt are done
-  while (lt > 0) {
-    const int ns = min(cap, lt);
-    const int lh = lt - ns;  // smallest span of this pass
-    fft_pass_ns<C, false, BIG>(ns, buf, M, lh, sign, tw, Mmax, lh == 0 ? post : nullptr);
+  int lg = 0;
+  while (lg < logM) {
+    const int ns = min(cap, logM - lg);
+    const C* pp = lg + ns == logM ? post : nullptr;
+    if (lg == 0) fft_pass_ns<C, FWD, true, BIG>(ns, buf, M, lg, tw, Mmax, pp);
+    else fft_pass_ns<C, FWD, false, BIG>(ns, buf, M, lg, tw, Mmax, pp);
     __syncthreads();
-    lt = lh;
+    lg += ns;
   }
+  if (logM == 0 && post && threadIdx.x == 0) buf[swz(0)] = cmul(buf[swz(0)], post[0]);
+  if (logM == 0 && post) __syncthreads();
 }
 
 template <typename T, int MODE, bool BIG>
@@ -222,25 +225,25 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
   auto chirp = [&](int k) -> C { return tab[(int)((2u * (unsigned)k * (unsigned)k) % (unsigned)twon)]; };
 
   if (MODE != 1) {
+    // sum over m = b + q n of F_m e^{i pi s m / n} (tab[s (b + (q mod 2) n)]);
+    // half of m = 0, which the two sums of bin 0 share
     auto fold = [&](int b) -> C {
-      // m = b + q n: e^{i pi s m / n} = tab[s (b + (q mod 2) n)]
       C h = mk((T)0, (T)0);
       int u = f.shift ? b : 0;
       const int du = f.shift ? n : 0;
       for (int m = b; m <= L; m += n) {
-        const C F = row[m];
-        const C v = cmul(F, tab[u]);
-        const T w = (m == 0) ? (T)1 : (T)2;
-        h.x = fma(w, v.x, h.x);
-        h.y = fma(w, v.y, h.y);
+        C v = row[m];
+        if (f.shift) v = cmul(v, tab[u]);
+        if (m == 0) v = cscale(v, (T)0.5);
+        h = cadd(h, v);
         u = (u + du < twon) ? u + du : u + du - twon;
       }
       return h;
     };
-    auto Hp = [&](int b) -> C {
-      const C h1 = fold(b);
-      const C h2 = fold(b == 0 ? 0 : n - b);
-      return cscale(cadd(h1, cconj(h2)), (T)0.5);
+    auto Hp = [&](int b) -> C { return cadd(fold(b), cconj(fold(b == 0 ? 0 : n - b))); };
+    auto put = [&](int k, C Z) {
+      if (!f.bluestein) buf[swz(bitrev(k, lg))] = Z;
+      else buf[swz(k)] = cmul(Z, chirp(k));
     };
     // Rings with fewer bins than threads split each bin's fold over g lanes
     // (a power of two <= 32; lane j of a group takes m = b + q n with
@@ -250,13 +253,14 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
     int g = 1;
     while (g < 32 && nh * g * 2 <= NT) g <<= 1;
     if (g == 1) {
-      for (int k = tid; k < nh; k += NT) {
+      // bins k and nh - k together: with S = H'_k + conj H'_{nh-k} and T = i w^k
+      // (H'_k - conj H'_{nh-k}), Z_k = S + T and Z_{nh-k} = conj(S - T)
+      for (int k = tid; 2 * k <= nh; k += NT) {
         const C A = Hp(k);
         const C B = cconj(Hp(nh - k));
-        const C w = tab[2 * k];
-        const C Z = cadd(cadd(A, B), cmuli(cmul(w, csub(A, B))));
-        if (!f.bluestein) buf[swz(bitrev(k, lg))] = Z;
-        else buf[swz(k)] = cmul(Z, chirp(k));
+        const C S = cadd(A, B), D = cmuli(cmul(tab[2 * k], csub(A, B)));
+        put(k, cadd(S, D));
+        if (k > 0 && 2 * k < nh) put(nh - k, cconj(csub(S, D)));
       }
     } else {
       const int k = tid / g, j = tid & (g - 1);
@@ -265,16 +269,12 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
 #pragma unroll 4
         for (int m = b + j * n; m <= L; m += g * n) {
           const C F = row[m];
-          const T w = (m == 0) ? (T)1 : (T)2;
-          h.x = fma(w, F.x, h.x);
-          h.y = fma(w, F.y, h.y);
+          h = cadd(h, m == 0 ? cscale(F, (T)0.5) : F);
         }
         return f.shift ? cmul(h, tab[b + ((j & 1) ? n : 0)]) : h;
       };
       auto Hpp = [&](int b) -> C {
-        const C h1 = fold_part(b);
-        const C h2 = fold_part(b == 0 ? 0 : n - b);
-        return cscale(cadd(h1, cconj(h2)), (T)0.5);
+        return cadd(fold_part(b), cconj(fold_part(b == 0 ? 0 : n - b)));
       };
       C Z = mk((T)0, (T)0);
       if (k < nh) {
@@ -286,19 +286,16 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
         Z.x += __shfl_xor_sync(0xffffffffu, Z.x, o);
         Z.y += __shfl_xor_sync(0xffffffffu, Z.y, o);
       }
-      if (k < nh && j == 0) {
-        if (!f.bluestein) buf[swz(bitrev(k, lg))] = Z;
-        else buf[swz(k)] = cmul(Z, chirp(k));
-      }
+      if (k < nh && j == 0) put(k, Z);
     }
     if (f.bluestein)
       for (int k = nh + tid; k < M; k += NT) buf[swz(k)] = mk((T)0, (T)0);
     __syncthreads();
     if (!f.bluestein) {
-      fft_dit<BIG>(buf, M, lg, +1, a.tw, a.Mmax);
+      fft_run<false, BIG>(buf, M, lg, a.tw, a.Mmax);
     } else {
-      fft_dif<BIG>(buf, M, lg, -1, a.tw, a.Mmax, vh);  // times the kernel spectrum
-      fft_dit<BIG>(buf, M, lg, +1, a.tw, a.Mmax);
+      fft_run<true, BIG>(buf, M, lg, a.tw, a.Mmax, vh);  // times the kernel spectrum
+      fft_run<false, BIG>(buf, M, lg, a.tw, a.Mmax);
     }
     // z_t = (map_{2t}, map_{2t+1}) = buf[t] (times the chirp for Bluestein rings)
     auto z_of = [&](int t) -> C { return f.bluestein ? cmul(buf[swz(t)], chirp(t)) : buf[swz(t)]; };
@@ -334,14 +331,36 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
 
   // forward length-nh DFT of z_t = y_{2t} + i y_{2t+1}
   if (!f.bluestein) {
-    fft_dif<BIG>(buf, M, lg, -1, a.tw, a.Mmax);  // Z'_k at buf[bitrev(k)]
+    fft_run<true, BIG>(buf, M, lg, a.tw, a.Mmax);  // Z'_k at buf[bitrev(k)]
   } else {
-    fft_dif<BIG>(buf, M, lg, -1, a.tw, a.Mmax, vh);  // times the kernel spectrum
-    fft_dit<BIG>(buf, M, lg, +1, a.tw, a.Mmax);      // Z'_k = conj(buf[k] chirp(k))
+    fft_run<true, BIG>(buf, M, lg, a.tw, a.Mmax, vh);  // times the kernel spectrum
+    fft_run<false, BIG>(buf, M, lg, a.tw, a.Mmax);     // Z'_k = conj(buf[k] chirp(k))
   }
   auto getZ = [&](int k) -> C {
     return f.bluestein ? cconj(cmul(buf[swz(k)], chirp(k))) : buf[swz(bitrev(k, lg))];
   };
+  if (n > L) {
+    // bins b and nh - b together: with E = (Z_b + conj Z_{nh-b}) / 2 and
+    // T = i w^-b (Z_b - conj Z_{nh-b}) / 2, Yhat_b = E - T and Yhat_{nh-b} =
+    // conj(E + T); row m is bin m, or the conjugate of bin n - m
+    auto out = [&](int m, C Y) {
+      if (m <= L) row[m] = f.shift ? cmul(Y, cconj(tab[m])) : Y;
+    };
+    for (int b = tid; 2 * b <= nh; b += NT) {
+      const C Zb = getZ(b);
+      const C Zc = cconj(getZ(b == 0 ? 0 : nh - b));
+      const C E = cscale(cadd(Zb, Zc), (T)0.5);
+      const C D = cmuli(cmul(cconj(tab[2 * b]), cscale(csub(Zb, Zc), (T)0.5)));
+      const C Y0 = csub(E, D), Y1 = cconj(cadd(E, D));
+      out(b, Y0);
+      if (b > 0) out(n - b, cconj(Y0));
+      if (2 * b < nh) {
+        out(nh - b, Y1);
+        if (b > 0) out(nh + b, cconj(Y1));
+      }
+    }
+    return;
+  }
   auto Yhat = [&](int b) -> C {  // b in [0, nh]
     const C Zb = getZ(b == nh ? 0 : b);
     const C Zc = cconj(getZ(b == 0 ? 0 : nh - b));
@@ -448,7 +467,7 @@ __global__ void vhat_kernel(const LenDesc* lens, const double2* tab, const doubl
     buf[swz(k)] = (dd >= 0) ? cconj(tab[d.tab + (int)((2 * (int64_t)dd * dd) % twon)]) : make_double2(0.0, 0.0);
   }
   __syncthreads();
-  fft_dif(buf, d.M, d.logM, -1, tw, Mmax);
+  fft_run<true, false>(buf, d.M, d.logM, tw, Mmax);
   for (int k = threadIdx.x; k < d.M; k += blockDim.x) vhat[d.vhat + k] = cscale(buf[swz(k)], 1.0 / d.M);
 }
 
