@@ -83,6 +83,8 @@ struct FinalizeArgs {
   int accumulate = 0;                      // out += result instead of out = result
   const typename Tr<T>::C* bsub = nullptr; // if set: out = bsub - result (residual)
   typename Tr<T>::C* out = nullptr;
+  int nrhs = 1;                            // right-hand sides of one launch: partial rows follow on each
+  int64_t ld = 0;                          // other, the vectors are ld apart
 };
 
 // Ring FFT stage: mode 0 = synthesis (phase -> map), 1 = adjoint
@@ -100,6 +102,8 @@ struct RingArgs {
   T* map_out = nullptr;        // mode 0 output; mode 2 optional copy of Y x
   const T* map_in = nullptr;   // mode 1 input
   const T* pixdiag = nullptr;  // mode 2 diagonal
+  int nrhs = 1;                // right-hand sides of one launch, phases and maps at these strides
+  int64_t ld_phase = 0, ld_map = 0;
   const int* live = nullptr;   // mode 2: rings with a non-zero diagonal (null: all)
   int np_live = 0;             // and the pairs of the Legendre stages around it
   int nring = 0;
@@ -135,7 +139,7 @@ int tc_end(cr_plan* P, const char* what);
 float2* tc_slot(cr_plan* P, const Grid& g, int L, int r);
 int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, const float* dl, bool masked = false);
 int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t, bool masked = false);
-int tc_ring(cr_plan* P, const Grid& g, int L, int r, int mode, const float* map_in, float* map_out);
+int tc_ring(cr_plan* P, const Grid& g, int L, int r, int nr, int mode, const float* map_in, float* map_out);
 int tc_sandwich(cr_plan* P, const Grid& g, int L, int nr, const float2* x, const float* dl_in, const float* pix,
                 const TcTail& t);
 template <typename T> int launch_leg_finalize(const FinalizeArgs<T>& f, cudaStream_t st);
@@ -161,7 +165,7 @@ bool ds_use(const LegArgs<double>& a);
 int launch_ds_synth(const LegArgs<double>& la, const double2* alm, int64_t ld_alm, int nr, double2* phase,
                     cudaStream_t st);
 int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, double* partial,
-                      const FinalizeArgs<double>* f, cudaStream_t st);
+                      const FinalizeArgs<double>& f, cudaStream_t st);
 // FP32 stages (legendre_f32.cu)
 int64_t ds_len(int L);
 void lf_zones(const double* z, int npairs, int* n1, int* n2);

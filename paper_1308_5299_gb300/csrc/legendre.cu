@@ -385,12 +385,15 @@ __global__ void __launch_bounds__(LEG_NT) leg_adjoint_kernel(LegArgs<double> a) 
 // y_lm = dl_out[l] * sum_blk partial[blk][lm] + dadd[l] * xadd_lm; zero at
 // inactive l (dl_out = dadd = 0 there) and Im(a_l0) = 0.
 template <typename T>
-__global__ void leg_finalize_kernel(FinalizeArgs<T> a) {
+__global__ void __launch_bounds__(256) leg_finalize_kernel(FinalizeArgs<T> a) {
   using C = typename Tr<T>::C;
   const int64_t nlm = n_lm(a.L);
+  const C* part = a.partial + (int64_t)blockIdx.y * a.nblk * nlm;  // blockIdx.y: right-hand side
+  const int64_t v0 = blockIdx.y * a.ld;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlm; i += (int64_t)gridDim.x * blockDim.x) {
-    C s = a.partial[i];
-    for (int b = 1; b < a.nblk; ++b) s = cadd(s, a.partial[(int64_t)b * nlm + i]);
+    C s = part[i];
+#pragma unroll 4
+    for (int b = 1; b < a.nblk; ++b) s = cadd(s, part[(int64_t)b * nlm + i]);
     // recover l, m from the flat index (m-major layout)
     int m = (int)((2.0 * (a.L + 1) + 1.0 - sqrt((2.0 * (a.L + 1) + 1.0) * (2.0 * (a.L + 1) + 1.0) - 8.0 * (double)i)) * 0.5);
     while (m > 0 && lm_off(a.L, m) > i) --m;
@@ -399,17 +402,17 @@ __global__ void leg_finalize_kernel(FinalizeArgs<T> a) {
     T f = a.dl_out ? a.dl_out[l] : (T)1;
     C y = cscale(s, f);
     if (a.dadd) {
-      C x = a.xadd[i];
+      C x = a.xadd[v0 + i];
       y.x = fma(a.dadd[l], x.x, y.x);
       y.y = fma(a.dadd[l], x.y, y.y);
     }
     if (a.bsub) {
-      const C bb = a.bsub[i];
+      const C bb = a.bsub[v0 + i];
       y = mk(bb.x - y.x, (m == 0) ? (T)0 : bb.y - y.y);
     }
     if (m == 0) y.y = 0;
-    if (a.accumulate) y = cadd(y, a.out[i]);
-    a.out[i] = y;
+    if (a.accumulate) y = cadd(y, a.out[v0 + i]);
+    a.out[v0 + i] = y;
   }
 }
 
@@ -468,7 +471,7 @@ int launch_leg_adjoint<double>(const LegArgs<double>& a, const FinalizeArgs<doub
     int rc = launch_leg_adjoint_df(a, &nb, st);
     if (rc) return rc;
   } else if (ds_use(a)) {
-    return launch_ds_adjoint(a, a.phase, 1, reinterpret_cast<double*>(a.partial), &f, st);
+    return launch_ds_adjoint(a, a.phase, 1, reinterpret_cast<double*>(a.partial), f, st);
   } else {
     const int rp = legal_rp(a.rp_adj);
     pair_blocks(a.npairs, rp, &nb);
@@ -488,7 +491,7 @@ template <typename T>
 int launch_leg_finalize(const FinalizeArgs<T>& f, cudaStream_t st) {
   const int64_t nlm = n_lm(f.L);
   int blocks = (int)std::min<int64_t>((nlm + 255) / 256, 152 * 16);
-  { leg_finalize_kernel<T><<<blocks, 256, 0, st>>>(f); count_launch(); }
+  { leg_finalize_kernel<T><<<dim3(blocks, f.nrhs), 256, 0, st>>>(f); count_launch(); }
   CR_CHECK_LAUNCH("leg_finalize_kernel");
   return CR_OK;
 }

@@ -968,33 +968,41 @@ __global__ void __launch_bounds__(128) ds_finalize_kernel(DsArgs a, const double
   const int nk = (L - m) / 2 + 1;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (blockIdx.x * blockDim.x >= nk) return;  // whole CTA
-  const double2* row = reinterpret_cast<const double2*>(partial) + ds_off(L, m) * 2;
+  // blockIdx.z: right-hand side
+  const double2* row = reinterpret_cast<const double2*>(partial) + ((int64_t)blockIdx.z * a.nblk * a.nkk + ds_off(L, m)) * 2;
+  const int64_t v0 = blockIdx.z * f.ld;
   const int64_t bs = a.nkk * 2;
-  auto sum = [&](int kk, int w, int b0, int b1) {
-    double2 x = make_double2(0.0, 0.0);
-    for (int b = b0; b < b1; ++b) x = cadd(x, row[b * bs + 2 * (int64_t)kk + w]);
-    return x;
+  auto sum = [&](int kk, int b0, int b1, double2& x, double2& y) {
+    x = y = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) {
+      const double2* r = row + b * bs + 2 * (int64_t)kk;
+      x = cadd(x, r[0]);
+      y = cadd(y, r[1]);
+    }
   };
   const bool in = k < nk;
   double2 u = make_double2(0.0, 0.0), v = u;
-  if (in) {
-    u = sum(k, 0, 0, a.nt_is);
-    v = sum(k, 1, 0, a.nt_is);
-  }
+  if (in) sum(k, 0, a.nt_is, u, v);
   double2 um;  // u_{k-1}
   um.x = __shfl_up_sync(0xffffffffu, u.x, 1);
   um.y = __shfl_up_sync(0xffffffffu, u.y, 1);
   if (!in) return;
-  if ((threadIdx.x & 31) == 0) um = k > 0 ? sum(k - 1, 0, 0, a.nt_is) : make_double2(0.0, 0.0);
+  if ((threadIdx.x & 31) == 0) {
+    um = make_double2(0.0, 0.0);
+    double2 vm;
+    if (k > 0) sum(k - 1, 0, a.nt_is, um, vm);
+  }
+  double2 q[2];  // the equatorial pairs' values of l and l + 1
+  sum(k, a.nt_is, a.nblk, q[0], q[1]);
   const int64_t ok = ds_off(a.t.Lc, m) + k, oc = lm_off(a.Lc, m) + 2 * k;
   const double g0 = a.t.e0[ok], g1 = k > 0 ? a.t.e1[ok - 1] : 0.0;
 #pragma unroll
   for (int w = 0; w < 2; ++w) {
     const int l = m + 2 * k + w;
     if (l > L) break;
-    const double2 q = sum(k, w, a.nt_is, a.nblk);
     const double sl = a.s[oc + w];
-    double2 y = make_double2(sl * q.x, sl * q.y);
+    double2 y = make_double2(sl * q[w].x, sl * q[w].y);
     if (w == 0) {
       y.x += g0 * u.x + (k > 0 ? g1 * um.x : 0.0);
       y.y += g0 * u.y + (k > 0 ? g1 * um.y : 0.0);
@@ -1002,7 +1010,7 @@ __global__ void __launch_bounds__(128) ds_finalize_kernel(DsArgs a, const double
       y.x = fma(a.t.sg[ok], v.x, y.x);
       y.y = fma(a.t.sg[ok], v.y, y.y);
     }
-    const int64_t i = lm_off(L, m) + (l - m);
+    const int64_t i = v0 + lm_off(L, m) + (l - m);
     if (f.dl_out) y = cscale(y, f.dl_out[l]);
     if (f.dadd) {
       const double2 x = f.xadd[i];
@@ -1087,22 +1095,24 @@ static int ds_adjoint_launch(const DsArgs& a, cudaStream_t st) {
   return CR_OK;
 }
 
-// phases of nr right-hand sides -> f[0..nr-1].out, two at a time, through
+// phases of nr right-hand sides -> f.out (vectors f.ld apart), two at a time, through
 // partial rows in `partial` (ds_partial_bytes of two right-hand sides, of one
 // when nr = 1)
 int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, double* partial,
-                      const FinalizeArgs<double>* f, cudaStream_t st) {
+                      const FinalizeArgs<double>& f0, cudaStream_t st) {
   for (int r0 = 0; r0 < nr; r0 += 2) {
     DsArgs a = ds_args(la, std::min(2, nr - r0));
     a.phase = const_cast<double2*>(phase) + r0 * a.ld_phase;
     a.partial = partial;
     int rc = a.nr == 1 ? ds_adjoint_launch<1>(a, st) : ds_adjoint_launch<2>(a, st);
     if (rc) return rc;
-    const dim3 grid((la.L / 2 + 1 + 127) / 128, la.L + 1);
-    for (int r = 0; r < a.nr; ++r) {
-      { ds_finalize_kernel<<<grid, 128, 0, st>>>(a, partial + (int64_t)r * a.nblk * a.nkk * 4, f[r0 + r]); count_launch(); }
-      CR_CHECK_LAUNCH("ds_finalize_kernel");
-    }
+    FinalizeArgs<double> f = f0;
+    f.out += r0 * f.ld;
+    if (f.xadd) f.xadd += r0 * f.ld;
+    if (f.bsub) f.bsub += r0 * f.ld;
+    const dim3 grid((la.L / 2 + 1 + 127) / 128, la.L + 1, a.nr);
+    { ds_finalize_kernel<<<grid, 128, 0, st>>>(a, partial, f); count_launch(); }
+    CR_CHECK_LAUNCH("ds_finalize_kernel");
   }
   return CR_OK;
 }

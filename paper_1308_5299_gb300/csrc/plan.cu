@@ -667,35 +667,33 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
     rc = ds_use(a) ? launch_ds_synth(a, x, nlm, nr, ph, P->stream)
                    : launch_leg_synth_mr(a, x, nlm, nr, ph, ld_phase, P->stream);
   }
-  for (int r = 0; r < nr && !rc; ++r) {
+  if (rc) return rc;
+  {
     RingArgs<double> ra = ring_args<double>(P, g, L);
-    ra.phase = ph + r * ld_phase;
+    ra.phase = ph;
     ra.pixdiag = pix;
+    ra.nrhs = nr;
+    ra.ld_phase = ld_phase;
     if (masked) limit_rings(P, ra);
     TimerScope ts(P->timing, P->stream, "ring_fft_apply_f64",
-                  fft_bytes<double>(g, L, 1) + (double)g.nring * (L + 1) * sizeof(double2));
+                  nr * (fft_bytes<double>(g, L, 1) + (double)g.nring * (L + 1) * sizeof(double2)));
     rc = launch_ring_fft<double>(ra, 2, P->stream);
   }
   if (rc) return rc;
-  FinalizeArgs<double> f[8];
-  for (int r = 0; r < nr; ++r) {
-    f[r].L = L;
-    f[r].dl_out = dl_out;
-    f[r].dadd = dadd;
-    f[r].xadd = x + r * nlm;
-    f[r].bsub = bsub ? bsub + r * nlm : nullptr;
-    f[r].out = y + r * nlm;
-  }
+  FinalizeArgs<double> f;
+  f.L = L;
+  f.dl_out = dl_out;
+  f.dadd = dadd;
+  f.xadd = x;
+  f.bsub = bsub;
+  f.out = y;
+  f.ld = nlm;
   TimerScope ts(P->timing, P->stream, "legendre_adjoint_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
   if (ds_use(a)) return launch_ds_adjoint(a, ph, nr, reinterpret_cast<double*>(part), f, P->stream);
-  int nb = 0;
-  rc = launch_leg_adjoint_mr(a, ph, ld_phase, nr, part, &nb, P->stream);
-  for (int r = 0; r < nr && !rc; ++r) {
-    f[r].partial = part + (int64_t)r * nb * nlm;
-    f[r].nblk = nb;
-    rc = launch_leg_finalize<double>(f[r], P->stream);
-  }
-  return rc;
+  if ((rc = launch_leg_adjoint_mr(a, ph, ld_phase, nr, part, &f.nblk, P->stream))) return rc;
+  f.partial = part;
+  f.nrhs = nr;
+  return launch_leg_finalize<double>(f, P->stream);
 }
 
 template int do_synth<double>(cr_plan*, const Grid&, int, const void*, void*, const double*);
@@ -1186,31 +1184,34 @@ int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t, b
                            P->d_tc_status, P->stream);
   }
   if (rc) return rc;
-  for (int r = 0; r < nr; ++r) {
-    FinalizeArgs<float> f;
-    f.partial = reinterpret_cast<const float2*>(P->tc_partial) + (int64_t)r * nblk * nlm;
-    f.nblk = nblk;
-    f.L = L;
-    f.dl_out = t.dl_out;
-    f.dadd = t.dadd;
-    f.xadd = t.xadd ? t.xadd + r * nlm : nullptr;
-    f.bsub = t.bsub ? t.bsub + r * nlm : nullptr;
-    f.accumulate = t.accumulate;
-    f.out = t.out + r * nlm;
-    TimerScope ts(P->timing, P->stream, "legendre_finalize_tc", (double)(nblk + 1) * nlm * sizeof(float2));
-    if ((rc = launch_leg_finalize<float>(f, P->stream))) return rc;
-  }
-  return CR_OK;
+  FinalizeArgs<float> f;
+  f.partial = reinterpret_cast<const float2*>(P->tc_partial);
+  f.nblk = nblk;
+  f.L = L;
+  f.dl_out = t.dl_out;
+  f.dadd = t.dadd;
+  f.xadd = t.xadd;
+  f.bsub = t.bsub;
+  f.accumulate = t.accumulate;
+  f.out = t.out;
+  f.nrhs = nr;
+  f.ld = nlm;
+  TimerScope ts(P->timing, P->stream, "legendre_finalize_tc", (double)nr * (nblk + 1) * nlm * sizeof(float2));
+  return launch_leg_finalize<float>(f, P->stream);
 }
 
-// ring FFT stage of phase slot r: mode 0 slot -> map_out, mode 1 map_in -> slot
-int tc_ring(cr_plan* P, const Grid& g, int L, int r, int mode, const float* map_in, float* map_out) {
+// ring FFT stage of phase slots r .. r + nr - 1 (maps follow on each other):
+// mode 0 slots -> map_out, mode 1 map_in -> slots
+int tc_ring(cr_plan* P, const Grid& g, int L, int r, int nr, int mode, const float* map_in, float* map_out) {
   RingArgs<float> ra = ring_args<float>(P, g, L);
   ra.phase = tc_slot(P, g, L, r);
   ra.map_in = map_in;
   ra.map_out = map_out;
+  ra.nrhs = nr;
+  ra.ld_phase = (int64_t)g.nring * (L + 1);
+  ra.ld_map = g.npix;
   TimerScope ts(P->timing, P->stream, mode == 0 ? "ring_fft_synth_f32" : "ring_fft_adjoint_f32",
-                fft_bytes<float>(g, L, 1));
+                nr * fft_bytes<float>(g, L, 1));
   return launch_ring_fft<float>(ra, mode, P->stream);
 }
 
@@ -1222,13 +1223,15 @@ int tc_sandwich(cr_plan* P, const Grid& g, int L, int nr, const float2* x, const
   const bool masked = masked_rings(P, g, pix);
   int rc = tc_synth_stage(P, g, L, x, nr, dl_in, masked);
   if (rc) return rc;
-  for (int r = 0; r < nr; ++r) {
+  {
     RingArgs<float> ra = ring_args<float>(P, g, L);
-    ra.phase = tc_slot(P, g, L, r);
+    ra.phase = tc_slot(P, g, L, 0);
     ra.pixdiag = pix;
+    ra.nrhs = nr;
+    ra.ld_phase = (int64_t)g.nring * (L + 1);
     if (masked) limit_rings(P, ra);
     TimerScope ts(P->timing, P->stream, "ring_fft_apply_f32",
-                  fft_bytes<float>(g, L, 1) + (double)g.nring * (L + 1) * sizeof(float2));
+                  nr * (fft_bytes<float>(g, L, 1) + (double)g.nring * (L + 1) * sizeof(float2)));
     if ((rc = launch_ring_fft<float>(ra, 2, P->stream))) return rc;
   }
   return tc_adjoint_tail(P, g, L, nr, t, masked);
@@ -1246,13 +1249,7 @@ static int tc_synth(cr_plan* P, const Grid& g, int L, const void* alm, void* map
     const int nr = std::min(16, nrhs - r0);
     if ((rc = tc_synth_stage(P, g, L, reinterpret_cast<const float2*>(alm) + (int64_t)r0 * nlm, nr, nullptr)))
       return rc;
-    for (int r = 0; r < nr; ++r) {
-      RingArgs<float> ra = ring_args<float>(P, g, L);
-      ra.phase = tc_slot(P, g, L, r);
-      ra.map_out = reinterpret_cast<float*>(map) + (int64_t)(r0 + r) * g.npix;
-      TimerScope ts(P->timing, P->stream, "ring_fft_synth_f32", fft_bytes<float>(g, L, 1));
-      if ((rc = launch_ring_fft<float>(ra, 0, P->stream))) return rc;
-    }
+    if ((rc = tc_ring(P, g, L, 0, nr, 0, nullptr, reinterpret_cast<float*>(map) + (int64_t)r0 * g.npix))) return rc;
   }
   return tc_end(P, "tensor-core synthesis: a completion wait gave up");
 }
@@ -1263,13 +1260,7 @@ static int tc_adjoint(cr_plan* P, const Grid& g, int L, const void* map, void* a
   const int64_t nlm = n_lm(L);
   for (int r0 = 0; r0 < nrhs; r0 += 16) {
     const int nr = std::min(16, nrhs - r0);
-    for (int r = 0; r < nr; ++r) {
-      RingArgs<float> ra = ring_args<float>(P, g, L);
-      ra.phase = tc_slot(P, g, L, r);
-      ra.map_in = reinterpret_cast<const float*>(map) + (int64_t)(r0 + r) * g.npix;
-      TimerScope ts(P->timing, P->stream, "ring_fft_adjoint_f32", fft_bytes<float>(g, L, 1));
-      if ((rc = launch_ring_fft<float>(ra, 1, P->stream))) return rc;
-    }
+    if ((rc = tc_ring(P, g, L, 0, nr, 1, reinterpret_cast<const float*>(map) + (int64_t)r0 * g.npix, nullptr))) return rc;
     TcTail t;
     t.out = reinterpret_cast<float2*>(alm) + r0 * nlm;
     if ((rc = tc_adjoint_tail(P, g, L, nr, t))) return rc;

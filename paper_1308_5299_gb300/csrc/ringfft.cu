@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
   const C* __restrict__ vh = a.vhat + f.vhat;
   const int n = f.n, nh = f.nh, M = f.M, lg = f.logM;
   const int twon = 2 * n;
-  C* row = a.phase + (int64_t)r * a.ldp;
+  C* row = a.phase + blockIdx.y * a.ld_phase + (int64_t)r * a.ldp;  // blockIdx.y: right-hand side
   const int L = a.L;
   const int tid = threadIdx.x;
   const int NT = blockDim.x;
@@ -300,13 +300,13 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
     // z_t = (map_{2t}, map_{2t+1}) = buf[t] (times the chirp for Bluestein rings)
     auto z_of = [&](int t) -> C { return f.bluestein ? cmul(buf[swz(t)], chirp(t)) : buf[swz(t)]; };
     if (MODE == 0) {
-      C* out = reinterpret_cast<C*>(a.map_out + f.off);
+      C* out = reinterpret_cast<C*>(a.map_out + blockIdx.y * a.ld_map + f.off);
       for (int t = tid; t < nh; t += NT) out[t] = z_of(t);
       return;
     }
     // MODE 2: multiply by the pixel diagonal and continue with the adjoint.
     const C* dg = reinterpret_cast<const C*>(a.pixdiag + f.off);
-    C* mo = a.map_out ? reinterpret_cast<C*>(a.map_out + f.off) : nullptr;
+    C* mo = a.map_out ? reinterpret_cast<C*>(a.map_out + blockIdx.y * a.ld_map + f.off) : nullptr;
     for (int t = tid; t < nh; t += NT) {
       C z = z_of(t);
       if (mo) mo[t] = z;
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
       for (int k = nh + tid; k < M; k += NT) buf[swz(k)] = mk((T)0, (T)0);
     __syncthreads();
   } else {
-    const C* in = reinterpret_cast<const C*>(a.map_in + f.off);
+    const C* in = reinterpret_cast<const C*>(a.map_in + blockIdx.y * a.ld_map + f.off);
     for (int t = tid; t < nh; t += NT) {
       const C z = in[t];
       buf[swz(t)] = f.bluestein ? cmul(cconj(z), chirp(t)) : z;
@@ -383,15 +383,15 @@ static int ring_fft_launch(const RingArgs<T>& b, int mode, int cnt, int nt, size
   switch (mode) {
     case 0:
       CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 0, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      { ring_fft_kernel<T, 0, BIG><<<cnt, nt, smem, st>>>(b); count_launch(); }
+      { ring_fft_kernel<T, 0, BIG><<<dim3(cnt, b.nrhs), nt, smem, st>>>(b); count_launch(); }
       break;
     case 1:
       CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 1, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      { ring_fft_kernel<T, 1, BIG><<<cnt, nt, smem, st>>>(b); count_launch(); }
+      { ring_fft_kernel<T, 1, BIG><<<dim3(cnt, b.nrhs), nt, smem, st>>>(b); count_launch(); }
       break;
     default:
       CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 2, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      { ring_fft_kernel<T, 2, BIG><<<cnt, nt, smem, st>>>(b); count_launch(); }
+      { ring_fft_kernel<T, 2, BIG><<<dim3(cnt, b.nrhs), nt, smem, st>>>(b); count_launch(); }
       break;
   }
   return CR_OK;

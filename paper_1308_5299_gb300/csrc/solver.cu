@@ -204,23 +204,23 @@ static int smooth_add_tc(cr_plan* P, int h, int nr, float2* X, const float2* R) 
   if (!rc && H.smoother_kind == 0 && nr > 1) {
     // every right-hand side's map, then the sweeps for all of them at once
     const int64_t np = g.npix;
-    for (int r = 0; r < nr && !rc; ++r) rc = tc_ring(P, g, L, r, 0, nullptr, H.d_mr_m1 + r * np);
+    rc = tc_ring(P, g, L, 0, nr, 0, nullptr, H.d_mr_m1);
     if (!rc) {
       const double bytes = 2.0 * lev.pat.nblocks * 64.0 * 64.0 * sizeof(float);
       TimerScope ts(P->timing, P->stream, "pixel_smoother", bytes);
       rc = apply_smoother_mr<float>(P, lev, nr, H.d_mr_m1, H.d_mr_m2, np);
     }
-    for (int r = 0; r < nr && !rc; ++r) rc = tc_ring(P, g, L, r, 1, H.d_mr_m2 + r * np, nullptr);
+    if (!rc) rc = tc_ring(P, g, L, 0, nr, 1, H.d_mr_m2, nullptr);
   }
   for (int r = 0; r < nr && !rc && !(H.smoother_kind == 0 && nr > 1); ++r) {
-    if ((rc = tc_ring(P, g, L, r, 0, nullptr, m1))) break;
+    if ((rc = tc_ring(P, g, L, r, 1, 0, nullptr, m1))) break;
     {
       const double bytes = H.smoother_kind == 1 ? lev.pat.ntile * 64.0 * 64.0 * sizeof(float)
                                                 : 2.0 * lev.pat.nblocks * 64.0 * 64.0 * sizeof(float);
       TimerScope ts(P->timing, P->stream, "pixel_smoother", bytes);
       if ((rc = apply_smoother<float>(P, lev, m1, m2))) break;
     }
-    rc = tc_ring(P, g, L, r, 1, m2, nullptr);
+    rc = tc_ring(P, g, L, r, 1, 1, m2, nullptr);
   }
   if (rc) return rc;
   TcTail t;
