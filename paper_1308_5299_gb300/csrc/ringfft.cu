@@ -163,9 +163,9 @@ __device__ __forceinline__ void fft_pass(C* buf, int M, int lg, const C* __restr
 }
 
 // BIG: up to 4 stages per pass (FP32 rings with M >= 4096: fewer barriers and
-// shared-memory round trips, at 75 registers); otherwise up to 3 (fewer
-// registers, so more CTAs per SM, which the small rings need).  Never more
-// stages than leave one group per thread.
+// shared-memory round trips); otherwise up to 3 (fewer registers, so more CTAs
+// per SM, which the small rings need).  Never more stages than leave one group
+// per thread.
 template <bool BIG>
 __device__ __forceinline__ int fft_pass_cap(int logM) {
   const int lt = 31 - __clz((int)blockDim.x);
@@ -201,8 +201,15 @@ __device__ void fft_run(C* buf, int M, int logM, const C* __restrict__ tw, int M
   if (logM == 0 && post) __syncthreads();
 }
 
+// CTAs per SM that the register allocation leaves room for: FP32 rings are bound
+// by the latency of their barriers and shared-memory round trips, so resident
+// CTAs count.  A (FP32, L = 2 Nside - 1; us at Nside 2048 / 1024 / 512) with
+// (BIG, other) CTAs unbounded: 1109 / 364 / 105; (3, -) 974 / 340 / 106;
+// (4, -) 932 / 315 / 106; (4, 5) 919 / 274 / 83; (4, 6) 920 / 271 / 85; (4, 8)
+// 934 / 282 / 97; three stages per pass in BIG instead of four: (4, -) 999.
+// FP64 rings are bound by the FP64 pipe and keep all registers they ask for.
 template <typename T, int MODE, bool BIG>
-__global__ void __launch_bounds__(RF_NT) ring_fft_kernel(RingArgs<T> a) {
+__global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 1 : BIG ? 4 : 5) ring_fft_kernel(RingArgs<T> a) {
   using C = typename Tr<T>::C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
