@@ -490,9 +490,11 @@ int64_t lf_partial_bytes(int npairs, int L) {
 }
 
 // ring pairs per thread where nothing was tuned: 4, or 2 where 4 would leave
-// fewer than 16 warps per SM
-static int lf_default_rp(const LegArgs<float>& a) {
-  return (int64_t)lf_nblocks(a, 4) * (a.L + 1) < 152 * 16 ? 2 : 4;
+// fewer than `least` warps per SM.  Measured (us, 2 against 4 pairs): synthesis
+// Nside 512 / 1023 81 : 94, Nside 1024 / 2047 504 : 497; adjoint Nside 128 / 384
+// 19 : 23, Nside 256 / 512 36 : 33.
+static int lf_default_rp(const LegArgs<float>& a, int least) {
+  return (int64_t)lf_nblocks(a, 4) * (a.L + 1) < 152 * (int64_t)least ? 2 : 4;
 }
 
 template <int RP>
@@ -504,7 +506,7 @@ static void lf_synth_launch(const LegArgs<float>& a, cudaStream_t st) {
 }
 
 int launch_lf_synth(const LegArgs<float>& a, cudaStream_t st) {
-  const int rp = a.rp_synth ? a.rp_synth : lf_default_rp(a);
+  const int rp = a.rp_synth ? a.rp_synth : lf_default_rp(a, 128);
   if (rp == 2) lf_synth_launch<2>(a, st);
   else if (rp == 8) lf_synth_launch<8>(a, st);
   else lf_synth_launch<4>(a, st);
@@ -538,7 +540,7 @@ static int lf_adjoint_launch(const LegArgs<float>& a, const FinalizeArgs<float>&
 }
 
 int launch_lf_adjoint(const LegArgs<float>& a, const FinalizeArgs<float>& f, cudaStream_t st) {
-  const int rp = a.rp_adj ? a.rp_adj : lf_default_rp(a);
+  const int rp = a.rp_adj ? a.rp_adj : lf_default_rp(a, 16);
   if (rp == 2) return lf_adjoint_launch<2>(a, f, st);
   if (rp == 8) return lf_adjoint_launch<8>(a, f, st);
   if (rp == 16) return lf_adjoint_launch<16>(a, f, st);
