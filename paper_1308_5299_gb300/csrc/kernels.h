@@ -109,6 +109,7 @@ struct RingArgs {
   int nring = 0;
   const int* rings = nullptr;  // ring indices ordered by FFT size (device)
   int rbase = 0;               // first entry of this launch's class
+  int stage = 0;               // where the row is kept in shared memory (elements; 0: nowhere)
   int nclass = 0;              // host: FFT-size classes
   const int* cls_M = nullptr;
   const int* cls_start = nullptr;

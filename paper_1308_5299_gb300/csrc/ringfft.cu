@@ -162,16 +162,14 @@ __device__ __forceinline__ void fft_pass(C* buf, int M, int lg, const C* __restr
   }
 }
 
-// BIG: up to 4 stages per pass (FP32 rings with M >= 4096: fewer barriers and
-// shared-memory round trips); otherwise up to 3 (fewer registers, so more CTAs
-// per SM, which the small rings need).  Never more stages than leave one group
-// per thread.
-template <bool BIG>
-__device__ __forceinline__ int fft_pass_cap(int logM) {
-  const int lt = 31 - __clz((int)blockDim.x);
-  return max(1, min(BIG ? 4 : 3, logM - lt));
-}
-
+// Stages per pass.  FP32: 4 in BIG (rings with M >= 4096: fewer barriers and
+// shared-memory round trips), 3 otherwise (fewer registers, so more CTAs per
+// SM), also where that leaves threads without a group: small rings wait for
+// barriers and round trips, not for arithmetic (A at Nside 64, lmax 383: 21.9 us
+// with one group per thread at least, 18.3 us so).  FP64 keeps a quarter of the
+// threads busy, as an SM's FP64 units are spread over its four schedulers
+// (Nside 32, lmax 95: 29.2 us with a group per thread, 27.4 us with a quarter,
+// 34.7 us without a limit).
 template <typename C, bool FWD, bool TRIV, bool BIG>
 __device__ __forceinline__ void fft_pass_ns(int ns, C* buf, int M, int lg, const C* __restrict__ tw, int Mmax,
                                             const C* __restrict__ post) {
@@ -187,7 +185,7 @@ __device__ __forceinline__ void fft_pass_ns(int ns, C* buf, int M, int lg, const
 template <bool FWD, bool BIG, typename C>
 __device__ void fft_run(C* buf, int M, int logM, const C* __restrict__ tw, int Mmax,
                         const C* __restrict__ post = nullptr) {
-  const int cap = fft_pass_cap<BIG>(logM);
+  const int cap = BIG ? 4 : sizeof(C) == 8 ? 3 : max(1, min(3, logM - 29 + __clz((int)blockDim.x)));
   int lg = 0;
   while (lg < logM) {
     const int ns = min(cap, logM - lg);
@@ -207,9 +205,13 @@ __device__ void fft_run(C* buf, int M, int logM, const C* __restrict__ tw, int M
 // (BIG, other) CTAs unbounded: 1109 / 364 / 105; (3, -) 974 / 340 / 106;
 // (4, -) 932 / 315 / 106; (4, 5) 919 / 274 / 83; (4, 6) 920 / 271 / 85; (4, 8)
 // 934 / 282 / 97; three stages per pass in BIG instead of four: (4, -) 999.
-// FP64 rings are bound by the FP64 pipe and keep all registers they ask for.
+// (With the folds four abreast these became 856 / 247 / 78.)
+// FP64 rings are bound by the FP64 pipe; 2 CTAs hold them to 128 registers
+// instead of 138 (A at Nside 1024, lmax 2047 2574 -> 2389 us, Nside 2048, lmax
+// 3000 10.45 -> 10.07 ms, eight right-hand sides at Nside 512 4.46 -> 4.20 ms;
+// Nside 128, lmax 383 57 -> 63 us; with 3 CTAs the same within 3 %).
 template <typename T, int MODE, bool BIG>
-__global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 1 : BIG ? 4 : 5) ring_fft_kernel(RingArgs<T> a) {
+__global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 2 : BIG ? 4 : 5) ring_fft_kernel(RingArgs<T> a) {
   using C = typename Tr<T>::C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
@@ -223,6 +225,10 @@ __global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 1 : BIG ? 4 : 5) ring_
   const int L = a.L;
   const int tid = threadIdx.x;
   const int NT = blockDim.x;
+  // rings with fewer bins than rows may keep the row in shared memory behind the
+  // FFT buffer
+  const bool staged = a.stage && n <= L;
+  C* srow = buf + a.stage;
   if (MODE == 2 && a.live && !a.live[r]) {
     if (min(r, a.nring - 1 - r) < a.np_live)
       for (int m = tid; m <= L; m += NT) row[m] = mk((T)0, (T)0);
@@ -232,68 +238,80 @@ __global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 1 : BIG ? 4 : 5) ring_
   auto chirp = [&](int k) -> C { return tab[(int)((2u * (unsigned)k * (unsigned)k) % (unsigned)twon)]; };
 
   if (MODE != 1) {
-    // sum over m = b + q n of F_m e^{i pi s m / n} (tab[s (b + (q mod 2) n)]);
-    // half of m = 0, which the two sums of bin 0 share
-    auto fold = [&](int b) -> C {
-      C h = mk((T)0, (T)0);
-      int u = f.shift ? b : 0;
-      const int du = f.shift ? n : 0;
-      for (int m = b; m <= L; m += n) {
-        C v = row[m];
-        if (f.shift) v = cmul(v, tab[u]);
-        if (m == 0) v = cscale(v, (T)0.5);
-        h = cadd(h, v);
-        u = (u + du < twon) ? u + du : u + du - twon;
+    // The folds of bins k and nh - k together: sums over m = b + q n, q = j mod g
+    // (b = k, n - k, nh - k, nh + k), four loads in flight a step; with
+    // e^{i pi s m / n} = e^{i pi s b / n} (-1)^{s q} the phase waits for the sum.
+    // A = H'_k and B = conj H'_{nh-k} (twice the Hermitian halves).
+    auto fold4 = [&](auto load, int k, int j, int g, C& A, C& B) {
+      const int b1 = k == 0 ? 0 : n - k, b2 = nh - k, b3 = nh + k;
+      C h0 = mk((T)0, (T)0), h1 = h0, h2 = h0, h3 = h0;
+      T sg = f.shift && (j & 1) ? (T)-1 : (T)1;
+      const T fl = f.shift && g == 1 ? (T)-1 : (T)1;
+      for (int q = j * n; q + k <= L; q += g * n) {
+        const C v0 = load(q + k);  // half of m = 0, which the two sums of bin 0 share
+        const C v1 = q + b1 <= L ? load(q + b1) : mk((T)0, (T)0);
+        const C v2 = q + b2 <= L ? load(q + b2) : mk((T)0, (T)0);
+        const C v3 = q + b3 <= L ? load(q + b3) : mk((T)0, (T)0);
+        const T s0 = q + k == 0 ? (T)0.5 * sg : sg;
+        h0 = mk(fma(s0, v0.x, h0.x), fma(s0, v0.y, h0.y));
+        const T s1 = q + b1 == 0 ? (T)0.5 * sg : sg;
+        h1 = mk(fma(s1, v1.x, h1.x), fma(s1, v1.y, h1.y));
+        h2 = mk(fma(sg, v2.x, h2.x), fma(sg, v2.y, h2.y));
+        h3 = mk(fma(sg, v3.x, h3.x), fma(sg, v3.y, h3.y));
+        sg *= fl;
       }
-      return h;
+      if (f.shift) {
+        h0 = cmul(h0, tab[k]);
+        h1 = cmul(h1, tab[b1]);
+        h2 = cmul(h2, tab[b2]);
+        h3 = cmul(h3, tab[b3]);
+      }
+      A = cadd(h0, cconj(h1));
+      B = cadd(cconj(h2), h3);
     };
-    auto Hp = [&](int b) -> C { return cadd(fold(b), cconj(fold(b == 0 ? 0 : n - b))); };
+    // with S = H'_k + conj H'_{nh-k} and T = i w^k (H'_k - conj H'_{nh-k}),
+    // Z_k = S + T and Z_{nh-k} = conj(S - T)
     auto put = [&](int k, C Z) {
       if (!f.bluestein) buf[swz(bitrev(k, lg))] = Z;
       else buf[swz(k)] = cmul(Z, chirp(k));
     };
-    // Rings with fewer bins than threads split each bin's fold over g lanes
-    // (a power of two <= 32; lane j of a group takes m = b + q n with
-    // q = j mod g, whose phase e^{i pi s m / n} is then constant) and sum the
-    // g partial Z in a fixed shuffle order: the long serial folds of the
-    // small polar rings become g short ones.
-    int g = 1;
-    while (g < 32 && nh * g * 2 <= NT) g <<= 1;
-    if (g == 1) {
-      // bins k and nh - k together: with S = H'_k + conj H'_{nh-k} and T = i w^k
-      // (H'_k - conj H'_{nh-k}), Z_k = S + T and Z_{nh-k} = conj(S - T)
-      for (int k = tid; 2 * k <= nh; k += NT) {
-        const C A = Hp(k);
-        const C B = cconj(Hp(nh - k));
-        const C S = cadd(A, B), D = cmuli(cmul(tab[2 * k], csub(A, B)));
-        put(k, cadd(S, D));
-        if (k > 0 && 2 * k < nh) put(nh - k, cconj(csub(S, D)));
-      }
-    } else {
-      const int k = tid / g, j = tid & (g - 1);
-      auto fold_part = [&](int b) -> C {
-        C h = mk((T)0, (T)0);
-#pragma unroll 4
-        for (int m = b + j * n; m <= L; m += g * n) {
-          const C F = row[m];
-          h = cadd(h, m == 0 ? cscale(F, (T)0.5) : F);
+    auto put2 = [&](int k, C A, C B) {
+      const C S = cadd(A, B), D = cmuli(cmul(tab[2 * k], csub(A, B)));
+      put(k, cadd(S, D));
+      if (k > 0 && 2 * k < nh) put(nh - k, cconj(csub(S, D)));
+    };
+    // rings with fewer bins than threads split each fold over g lanes (a power
+    // of two <= 32) and sum the parts in a fixed shuffle order
+    auto folds = [&](auto load) {
+      const int nk = nh / 2 + 1;
+      int g = 1;
+      while (g < 32 && nk * g * 2 <= NT) g <<= 1;
+      if (g == 1) {
+        for (int k = tid; k < nk; k += NT) {
+          C A, B;
+          fold4(load, k, 0, 1, A, B);
+          put2(k, A, B);
         }
-        return f.shift ? cmul(h, tab[b + ((j & 1) ? n : 0)]) : h;
-      };
-      auto Hpp = [&](int b) -> C {
-        return cadd(fold_part(b), cconj(fold_part(b == 0 ? 0 : n - b)));
-      };
-      C Z = mk((T)0, (T)0);
-      if (k < nh) {
-        const C A = Hpp(k);
-        const C B = cconj(Hpp(nh - k));
-        Z = cadd(cadd(A, B), cmuli(cmul(tab[2 * k], csub(A, B))));
+        return;
       }
+      const int k = tid / g, j = tid & (g - 1);
+      C A = mk((T)0, (T)0), B = A;
+      if (k < nk) fold4(load, k, j, g, A, B);
       for (int o = g >> 1; o > 0; o >>= 1) {
-        Z.x += __shfl_xor_sync(0xffffffffu, Z.x, o);
-        Z.y += __shfl_xor_sync(0xffffffffu, Z.y, o);
+        A.x += __shfl_xor_sync(0xffffffffu, A.x, o);
+        A.y += __shfl_xor_sync(0xffffffffu, A.y, o);
+        B.x += __shfl_xor_sync(0xffffffffu, B.x, o);
+        B.y += __shfl_xor_sync(0xffffffffu, B.y, o);
       }
-      if (k < nh && j == 0) put(k, Z);
+      if (k < nk && j == 0) put2(k, A, B);
+    };
+    if (!staged) {
+      folds([&](int m) -> C { return row[m]; });
+    } else {
+#pragma unroll 4
+      for (int m = tid; m <= L; m += NT) srow[swz(m)] = row[m];
+      __syncthreads();
+      folds([&](int m) -> C { return srow[swz(m)]; });
     }
     if (f.bluestein)
       for (int k = nh + tid; k < M; k += NT) buf[swz(k)] = mk((T)0, (T)0);
@@ -346,13 +364,11 @@ __global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 1 : BIG ? 4 : 5) ring_
   auto getZ = [&](int k) -> C {
     return f.bluestein ? cconj(cmul(buf[swz(k)], chirp(k))) : buf[swz(bitrev(k, lg))];
   };
-  if (n > L) {
-    // bins b and nh - b together: with E = (Z_b + conj Z_{nh-b}) / 2 and
-    // T = i w^-b (Z_b - conj Z_{nh-b}) / 2, Yhat_b = E - T and Yhat_{nh-b} =
-    // conj(E + T); row m is bin m, or the conjugate of bin n - m
-    auto out = [&](int m, C Y) {
-      if (m <= L) row[m] = f.shift ? cmul(Y, cconj(tab[m])) : Y;
-    };
+  // bins b and nh - b together: with E = (Z_b + conj Z_{nh-b}) / 2 and
+  // T = i w^-b (Z_b - conj Z_{nh-b}) / 2, Yhat_b = E - T and Yhat_{nh-b} =
+  // conj(E + T); row m is bin m mod n, or the conjugate of bin n - m mod n,
+  // times e^{-i pi s m / n}
+  auto bins = [&](auto out) {
     for (int b = tid; 2 * b <= nh; b += NT) {
       const C Zb = getZ(b);
       const C Zc = cconj(getZ(b == 0 ? 0 : nh - b));
@@ -366,22 +382,35 @@ __global__ void __launch_bounds__(RF_NT, sizeof(T) == 8 ? 1 : BIG ? 4 : 5) ring_
         if (b > 0) out(nh + b, cconj(Y1));
       }
     }
+  };
+  auto turn = [&](int m, C Y) -> C { return f.shift ? cmul(Y, cconj(tab[m])) : Y; };
+  if (!staged) {
+    // every row of a bin from its thread: e^{-i pi s m / n} turns by (-1)^s a period
+    bins([&](int b, C Y) {
+      if (b > L) return;
+      C v = turn(b, Y);
+      for (int m = b; m <= L; m += n) {
+        row[m] = v;
+        if (f.shift) v = mk(-v.x, -v.y);
+      }
+    });
     return;
   }
-  auto Yhat = [&](int b) -> C {  // b in [0, nh]
-    const C Zb = getZ(b == nh ? 0 : b);
-    const C Zc = cconj(getZ(b == 0 ? 0 : nh - b));
-    const C E = cscale(cadd(Zb, Zc), (T)0.5);
-    const C O = cscale(csub(Zb, Zc), (T)0.5);
-    const C wm = cconj(tab[2 * b]);  // e^{-2 pi i b / n}
-    // Yhat = E - i w^-b O
-    return csub(E, cmuli(cmul(wm, O)));
-  };
+  bins([&](int b, C Y) { srow[swz(b)] = turn(b, Y); });
+  __syncthreads();
+  int b = tid % n;
+  bool odd = f.shift && ((tid / n) & 1);
+  const int db = NT % n;
+  const bool dodd = f.shift && ((NT / n) & 1);
   for (int m = tid; m <= L; m += NT) {
-    const int b = m % n;
-    const C Y = (b <= nh) ? Yhat(b) : cconj(Yhat(n - b));
-    const C t = tab[f.shift ? m % twon : 0];
-    row[m] = cmul(Y, cconj(t));
+    const C v = srow[swz(b)];
+    row[m] = odd ? mk(-v.x, -v.y) : v;
+    b += db;
+    odd ^= dodd;
+    if (b >= n) {
+      b -= n;
+      odd ^= f.shift != 0;
+    }
   }
 }
 
@@ -413,11 +442,19 @@ int launch_ring_fft(const RingArgs<T>& a, int mode, cudaStream_t st) {
     const int M = a.cls_M[c];
     const int cnt = a.cls_start[c + 1] - a.cls_start[c];
     if (cnt <= 0) continue;
-    const size_t smem = (size_t)M * sizeof(C);
+    size_t smem = (size_t)M * sizeof(C);
     if (smem > 227 * 1024 || M > 65536) return fail(CR_EINVAL, "ring FFT buffer exceeds shared memory");
     // at least 128 threads: small rings split their folds over the idle lanes
     const int nt = std::max(128, std::min(RF_NT, M / 8));
     RingArgs<T> b = a;
+    // The smallest rings fold each row many times over: the row is staged where
+    // it is long.  A with | without staging: FP32 Nside 1024, lmax 2047 247 | 264
+    // us, Nside 2048, lmax 3000 856 | 891; FP64 10.44 | 10.59 ms; but FP32 Nside
+    // 512, lmax 1023 78.9 | 77.6 us, and staging the larger classes as well loses
+    // what the first gains (Nside 2048: 922 us; fewer CTAs per SM).
+    const size_t rows = ((size_t)a.L + 16) / 16 * 16 * sizeof(C);
+    b.stage = c == 0 && 2 * a.L > 3 * M && smem + rows <= 227 * 1024 ? M : 0;
+    if (b.stage) smem += rows;
     b.rbase = a.cls_start[c];
     // FP32 rings with M >= 4096: the 4-stage passes with computed twiddles
     int rc;
