@@ -1,0 +1,135 @@
+"""The kernels' dispatch at the edges of its rules, where a tile, a warp or a
+launch is nearly empty: digit-slice FP64 stages, two-step FP32 stages, ring
+FFTs of few bins, rings without weight, and explicit inverses of small levels.
+
+Tolerances: FP64 transforms of lmax <= 200 round at about lmax 2^-53 (2e-14)
+in the oracle's one-step recurrence, 1e-12 leaves a factor 50; FP32 stages
+have 1e-5 as elsewhere.  Two forms of the same FP32 level solve differ by
+rounding times the condition of a tile's factor, 2e-4 as for the sweeps
+against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import cuda_device, rel_l2
+from oracle import geometry, sht
+from paper_1308_5299_gb300 import binding, synthetic
+
+pytestmark = pytest.mark.gpu
+
+TOL = {torch.float64: 1e-12, torch.float32: 1e-5}
+
+
+@pytest.fixture(scope="module")
+def dev():
+    return cuda_device()
+
+
+def transforms(dev, grid, lmax, dtype):
+    """Relative errors of synthesis and adjoint against the oracle."""
+    kw = {"nside": grid} if isinstance(grid, int) else {"gl": grid}
+    g = geometry.healpix_grid(grid) if isinstance(grid, int) else geometry.gl_grid(*grid)
+    plan = binding.Plan(lmax, **kw)
+    a = synthetic.random_alm(lmax, seed=11)
+    y = synthetic.random_map(g["npix"], seed=12)
+    cdtype = torch.complex128 if dtype == torch.float64 else torch.complex64
+    m = torch.empty(g["npix"], dtype=dtype, device=dev)
+    plan.sht_synth(torch.from_numpy(a).to(cdtype).to(dev), m)
+    b = torch.empty(sht.n_lm(lmax), dtype=cdtype, device=dev)
+    plan.sht_adjoint(torch.from_numpy(y).to(dtype).to(dev), b)
+    return rel_l2(m.cpu().numpy(), sht.synth(a, lmax, g)), rel_l2(b.cpu().numpy(), sht.adjoint(y, lmax, g))
+
+
+# 64 pairs and lmax 64 are the smallest of the digit slices, 63 of either goes
+# the other way; 128 and 129 pairs fill a tile and begin the next; odd counts
+# have a ring on the equator; ring lengths of few bins fold rows many times,
+# with (2 lmax > 3 M) and without the row in shared memory
+@pytest.mark.parametrize("grid,lmax", [
+    (32, 63), (32, 64), (32, 191), ((125, 160), 70), ((127, 160), 64), ((128, 160), 65), ((255, 160), 79),
+    ((257, 160), 80), ((258, 162), 127), ((20, 4), 40), ((20, 6), 40), ((20, 34), 60), ((130, 10), 100),
+])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_transforms_at_the_edges(dev, grid, lmax, dtype):
+    for e in transforms(dev, grid, lmax, dtype):
+        assert e < TOL[dtype]
+
+
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 4, 5, 9])
+def test_digit_slices_of_several_right_hand_sides(dev, nrhs):
+    """Columns of one launch are independent: each equals its own call."""
+    lmax = 95
+    cl = 1.0 / np.arange(1.0, lmax + 2.0) ** 2
+    bl = np.exp(-0.5 * np.arange(lmax + 1) ** 2 * 1e-4)
+    ninv = np.abs(synthetic.random_map(12 * 32 * 32, seed=4)) + 0.1
+    plan = binding.Plan(lmax, nside=32, cl=cl, bl=bl, ninv=torch.from_numpy(ninv).to(dev))
+    x = torch.from_numpy(np.stack([synthetic.random_alm(lmax, seed=20 + j) * 10.0 ** (j - 4) for j in range(nrhs)])).to(dev)
+    y = torch.empty_like(x)
+    plan.apply_A(x, y)
+    for j in range(nrhs):
+        one = torch.empty_like(x[j])
+        plan.apply_A(x[j].contiguous(), one)
+        assert rel_l2(y[j].cpu().numpy(), one.cpu().numpy()) < 1e-13
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_digit_slices_pass_on_what_is_not_finite(dev, bad):
+    lmax, g = 95, geometry.healpix_grid(32)
+    plan = binding.Plan(lmax, nside=32)
+    a = torch.from_numpy(synthetic.random_alm(lmax, seed=1)).to(dev)
+    a[5] = bad  # m = 0
+    m = torch.empty(g["npix"], dtype=torch.float64, device=dev)
+    plan.sht_synth(a, m)
+    assert not torch.isfinite(m).any()
+    y = torch.from_numpy(synthetic.random_map(g["npix"], seed=2)).to(dev)
+    y[g["npix"] // 2] = bad
+    b = torch.empty(sht.n_lm(lmax), dtype=torch.complex128, device=dev)
+    plan.sht_adjoint(y, b)
+    assert not torch.isfinite(b.real).any()
+
+
+# rings without weight: none, one, both caps, all but one, all; every other
+# ring (pairs half masked); grids on either side of the digit slices
+@pytest.mark.parametrize("nside,lmax", [(8, 23), (32, 95), (64, 191)])
+@pytest.mark.parametrize("mask", ["none", "one", "caps", "north", "most", "all", "every other"])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_rings_without_weight_against_the_full_transforms(dev, nside, lmax, mask, dtype):
+    g = geometry.healpix_grid(nside)
+    nring = 4 * nside - 1
+    z = np.arange(nring)
+    off = {"none": z < 0, "one": z == nside, "caps": np.minimum(z, nring - 1 - z) < nside,
+           "north": z < nring // 2, "most": z != nring - 3, "all": z >= 0, "every other": z % 2 == 0}[mask]
+    n = np.where(np.minimum(z, nring - 1 - z) < nside, 4 * (np.minimum(z, nring - 1 - z) + 1), 4 * nside)
+    assert n.sum() == g["npix"]
+    ninv = np.abs(synthetic.random_map(g["npix"], seed=8)) + 0.1
+    ninv[np.repeat(off, n)] = 0.0
+    l = np.arange(lmax + 1)
+    cl, bl = 1.0 / (l + 1.0) ** 2, np.exp(-1e-4 * l * (l + 1.0))
+    plan = binding.Plan(lmax, nside=nside, cl=cl, bl=bl, ninv=torch.from_numpy(ninv).to(dev))
+    cdtype = torch.complex128 if dtype == torch.float64 else torch.complex64
+    x = torch.from_numpy(synthetic.random_alm(lmax, seed=9)).to(cdtype).to(dev)
+    y = torch.empty_like(x)
+    plan.apply_A(x, y)
+    ell = np.concatenate([np.arange(m, lmax + 1) for m in range(lmax + 1)])
+    b = torch.from_numpy(bl[ell]).to(dev)
+    p = torch.empty(g["npix"], dtype=torch.float64, device=dev)
+    plan.sht_synth(x.to(torch.complex128) * b, p)
+    t = torch.empty_like(x, dtype=torch.complex128)
+    plan.sht_adjoint(p * torch.from_numpy(ninv).to(dev), t)
+    full = x.to(torch.complex128) / torch.from_numpy(cl[ell]).to(dev) + b * t
+    assert rel_l2(y.cpu().numpy(), full.cpu().numpy()) < TOL[dtype]
+
+
+def test_explicit_inverse_of_small_levels_against_the_sweeps(dev):
+    """Levels up to 48 tiles multiply by the inverse of the sweeps' factor."""
+    cfg, cl, bl, ninv = synthetic.problem_inputs("nside32_lmax95")
+    kw = dict(nside=cfg["nside"], cl=cl, bl=bl, ninv=torch.from_numpy(ninv).to(dev), levels="default")
+    sweeps = binding.Plan(cfg["lmax"], smoother_sweep="per_colour", **kw)
+    ridges = [sweeps.level(h)["ridge"] for h in range(1, sweeps.nlevels() + 1)]
+    auto = binding.Plan(cfg["lmax"], ridge_alpha=ridges, **kw)
+    for h in range(1, sweeps.nlevels() + 1):
+        L = auto.level(h)["lmax_h"]
+        r = torch.from_numpy(synthetic.random_alm(L, seed=40 + h)).to(dev)
+        a, b = torch.empty_like(r), torch.empty_like(r)
+        auto.smooth(h, r, a)
+        sweeps.smooth(h, r, b)
+        assert rel_l2(a.cpu().numpy(), b.cpu().numpy()) < 2e-4, h
