@@ -1,5 +1,8 @@
 // Legendre stages of spherical-harmonic synthesis Y and adjoint synthesis Y^T
-// (Section 2.1, Eq. sh-synthesis; normalised P~_lm of Section 3.3).
+// (Section 2.1, Eq. sh-synthesis; normalised P~_lm of Section 3.3): the plan's
+// start tables, the dispatch, and the FP64 kernels of small grids and of the
+// smoother's diagonal.  FP32 stages are those of legendre_f32.cu, FP64 stages of
+// at least 64 ring pairs and lmax >= 64 those of legendre_ds.cu.
 //
 // For one m and one north/south ring pair (z, -z):
 //   synthesis  F_m(+-z) = sum_{l=m..L} a_lm P~_lm(+-z),

@@ -2,8 +2,9 @@
 //
 // On this GPU the FP64 pipe runs at 1/64 of the FP32 rate, so a Legendre
 // stage whose sums are FP64 fused multiply-adds is bound by that pipe.  Here
-// the FP64 pipe only advances the recurrence; the sums over l (synthesis) or
-// over ring pairs (adjoint) are exact integer products on the tensor cores.
+// the recurrence runs in 64-bit integers and the sums over l (synthesis) or
+// over ring pairs (adjoint) are exact integer products on the tensor cores; the
+// FP64 pipe only takes the first steps of a sequence and collects the sums.
 //
 // Digit slices.  Every operand is written as a fixed-point number of seven
 // signed base-256 digits (54 bits below a bound that holds for the whole row
@@ -28,20 +29,26 @@
 // and p_k obeys a three-term recurrence in z^2 (Ishioka, J. Meteor. Soc.
 // Japan 96, 2018).  Rescaled by sigma_k so that the last coefficient is one,
 //   q_{k+1} = (A_k z^2 + B_k) q_k - q_{k-1},
-// two FP64 operations per two l instead of four.  z^2 is rounded once for the
-// whole sequence, which would add up coherently; four copies of it that
-// differ in the last place and average to the exact square are used in turn,
-// and near the poles (z^2 > 1/2) the same is done with 1 - z^2 and
-// A_k + B_k.  Near the equator p_k grows like 1/z while P~ does not and the
-// even sums would cancel, so pairs with z <= DS_ZEQ run the one-step
-// recurrence of legendre.cu instead (every l its own column of the sums).
-// Against extended precision at Nside 2048 / lmax 3000 both forms are at or
-// below the error of the one-step form for z > 0.2 and far below it near the
-// poles (1e-12 instead of 3e-11 in the first rings).
+// one step for two l.  Once a pair's values have grown past the first steps
+// they are 64-bit fixed-point numbers, z^2 and the coefficients too (z^2 to
+// 2^-64, the factor A z^2 + B + 8 to 2^-60), so a step rounds at 2^-62 of the
+// bound of the functions and not at 2^-53 of the running value; the upper
+// bytes of the same integers are the digits of the products.  Near the poles
+// the first steps use 1 - z^2 and A_k + B_k.  Near the equator p_k grows like
+// 1/z while P~ does not and the even sums would cancel, so pairs with z <=
+// DS_ZEQ run the one-step recurrence of legendre.cu in the same integers (every
+// l its own column of the sums).  Against a double-double recurrence the whole
+// transforms are 2.5 to 4 times nearer than FP64 sums over an FP64 one-step
+// recurrence (Nside 1024, lmax 2047: synthesis 2.6e-15 instead of 7.0e-15,
+// adjoint 4.7e-15 instead of 1.8e-14).
 //
-// What bounds it: the FP64 pipe (2 instructions per two l and ring pair, 4
-// near the equator, plus 1/8 for collecting the accumulators), with about 45
-// integer and shared-memory instructions per two l hidden behind it.
+// What bounds it: instruction issue, at half of its rate (ncu at Nside 512 /
+// lmax 1023: 2.0 instructions a cycle, FP64 pipe 33 %, tensor pipe 16 %, 24 % of
+// the warp slots); the rest are waits for the coefficients, the block barrier
+// of a stage and the products.  About 42 instructions take a warp two l
+// further.  At Nside 2048 / lmax 3000 the synthesis stage went from 89.1 ms
+// (FP64 sums, one-step recurrence) to 17.4 ms and the adjoint from 99.9 to 21.7
+// ms; where rings carry no weight in A, to 13.0 and 16.1 ms.
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -1039,6 +1046,11 @@ int64_t ds_partial_bytes(int nis, int npairs, int L, int nr) {
   return (int64_t)nr * ds_tiles(nis, npairs) * ds_len(L) * 4 * (int64_t)sizeof(double);
 }
 
+// Below 64 ring pairs a CTA's 128 rows are more than half empty, and below 64
+// l a stage of 32 columns is mostly padding: the FP64 kernels of legendre.cu
+// run there, where a launch and one warp's chain of a few dozen steps take the
+// time.  Just above the line (Nside 32, lmax 95: 64 pairs) the synthesis stage is
+// 19 us here and 55 us there.
 bool ds_use(const LegArgs<double>& a) { return a.ds && !a.df && a.npairs >= 64 && a.L >= 64; }
 
 static DsArgs ds_args(const LegArgs<double>& la, int nr) {

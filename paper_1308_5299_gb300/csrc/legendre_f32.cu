@@ -24,7 +24,14 @@
 // stages the chunk's coefficients itself; a group of 8 k runs unchecked once
 // all of the warp's pairs have started (start tables, |P~| >= 2^-60).  Bound by
 // FP32 issue: 6.5 operations per pair and k beside two shared loads per k and
-// warp.
+// warp (ncu at Nside 1024 / lmax 2047: synthesis 2.9, adjoint 2.75 instructions a
+// cycle, the adjoint's transpose near the shared-memory rate as well).  At Nside
+// 2048 / lmax 3000 against the one-step kernels with two ring pairs packed into
+// an instruction and a launch each for polar and other pairs: synthesis 2.4 ->
+// 1.54 ms, adjoint 3.3 -> 2.05 ms; Nside 512 / lmax 1023 synthesis 130 -> 75 us,
+// adjoint 150 -> 103 us with its finalisation.
+#include <cmath>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -45,7 +52,7 @@ void lf_zones(const double* z, int npairs, int* n1, int* n2) {
 // arguments of a pair's steps: four copies of z^2 (middle), or 1 - z^2, or z^2
 void lf_args(const double* z, int npairs, int n1, int n2, float4* out) {
   for (int p = 0; p < npairs; ++p) {
-    const long double x = (long double)z[p] * z[p];
+    const double x = z[p] * z[p], xl = std::fma(z[p], z[p], -x);  // the exact square
     if (p < n1) {
       const double w = 1.0 - z[p];
       const float s = (float)(w * (2.0 - w));
@@ -56,7 +63,7 @@ void lf_args(const double* z, int npairs, int n1, int n2, float4* out) {
     } else {
       const float h = (float)x;
       const float up = nextafterf(h, 2.f) - h;
-      const int t = (int)lrint(4.0 * (double)(x - (long double)h) / up);
+      const int t = (int)lrint(4.0 * ((x - h) + xl) / up);
       float c[4];
       for (int j = 0; j < 4; ++j) c[j] = h + (j < abs(t) ? (t > 0 ? up : -up) : 0.f);
       out[p] = make_float4(c[0], c[1], c[2], c[3]);

@@ -1,6 +1,6 @@
 // FP64 Legendre stages of several right-hand sides at once (Section 2.1,
-// Eq. sh-synthesis and its transpose), for the batched solves' FP64 outer
-// residual r = b - A x of each right-hand side (iterative refinement).
+// Eq. sh-synthesis and its transpose), for grids below the digit slices'
+// sizes (legendre_ds.cu: fewer than 64 ring pairs, or lmax < 64).
 //
 // On this GPU the FP64 pipe runs at 1/64 of the FP32 rate, so these stages
 // are bound by FP64 fused multiply-adds and nothing else.  For one
