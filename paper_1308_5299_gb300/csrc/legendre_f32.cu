@@ -26,10 +26,9 @@
 // FP32 issue: 6.5 operations per pair and k beside two shared loads per k and
 // warp (ncu at Nside 1024 / lmax 2047: synthesis 2.9, adjoint 2.75 instructions a
 // cycle, the adjoint's transpose near the shared-memory rate as well).  At Nside
-// 2048 / lmax 3000 against the one-step kernels with two ring pairs packed into
-// an instruction and a launch each for polar and other pairs: synthesis 2.4 ->
-// 1.54 ms, adjoint 3.3 -> 2.05 ms; Nside 512 / lmax 1023 synthesis 130 -> 75 us,
-// adjoint 150 -> 103 us with its finalisation.
+// 2048 / lmax 3000, in A, against the one-step kernels with two ring pairs packed
+// into an instruction and a launch each for polar and other pairs: synthesis
+// 2.4 -> 1.54 ms, adjoint 3.3 -> 2.05 ms.
 #include <cmath>
 
 #include "common.cuh"

@@ -513,25 +513,27 @@ static double leg_work(const Grid& g, int L) { return 8.0 * g.npairs * (double)n
 // precisions use.  Counted once per (grid, band limit) from the table on the
 // host while timing is on (it synchronises, so not inside a graph capture,
 // where the dense count stands in).
-static double leg_work_exec(cr_plan* P, const Grid& gc, int L) {
+static double leg_work_exec(cr_plan* P, const Grid& gc, int L, bool masked = false) {
   if (!P->timing.enabled || L < 0) return 0.0;
   Grid& g = const_cast<Grid&>(gc);
-  auto it = g.exec_terms.find(L);
+  const int np = masked ? P->np_live : g.npairs;
+  const double dense = 8.0 * np * (double)n_lm(L);
+  auto it = g.exec_terms.find({L, np});
   if (it != g.exec_terms.end()) return 8.0 * it->second;
-  if (P->capturing || !g.d_ls32 || L > g.Lseed) return leg_work(g, L);
+  if (P->capturing || !g.d_ls32 || L > g.Lseed) return dense;
   std::vector<int> ls((size_t)(L + 1) * g.npairs);
   if (cudaStreamSynchronize(P->stream) != cudaSuccess ||
       cudaMemcpy(ls.data(), g.d_ls32, ls.size() * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return leg_work(g, L);
+    return dense;
   double n = 0.0;
   for (int m = 0; m <= L; ++m) {
     const int* row = ls.data() + (size_t)m * g.npairs;
     int64_t s = 0;
-    for (int p = 0; p < g.npairs; ++p)
+    for (int p = 0; p < np; ++p)
       if (row[p] <= L) s += L + 1 - row[p];
     n += (double)s;
   }
-  g.exec_terms[L] = n;
+  g.exec_terms[{L, np}] = n;
   return 8.0 * n;
 }
 // algorithmic HBM bytes of one ring-FFT stage: the phase array [nring][L+1]
@@ -595,7 +597,7 @@ int do_sandwich(cr_plan* P, const Grid& g, int L, const void* x, void* y, const 
   int rc;
   {
     TimerScope ts(P->timing, P->stream, std::string("legendre_synth") + ptag<T>(), leg_work(g, L),
-                  leg_work_exec(P, g, L));
+                  leg_work_exec(P, g, L, masked));
     rc = launch_leg_synth<T>(a, P->stream);
   }
   if (rc) return rc;
@@ -617,7 +619,7 @@ int do_sandwich(cr_plan* P, const Grid& g, int L, const void* x, void* y, const 
   f.bsub = reinterpret_cast<const typename Tr<T>::C*>(bsub);
   f.out = reinterpret_cast<typename Tr<T>::C*>(y);
   TimerScope ts(P->timing, P->stream, std::string("legendre_adjoint") + ptag<T>(), leg_work(g, L),
-                  leg_work_exec(P, g, L));
+                  leg_work_exec(P, g, L, masked));
   return launch_leg_adjoint<T>(a, f, P->stream);
 }
 
@@ -663,7 +665,7 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
   const bool masked = masked_rings(P, g, pix);
   if (masked) limit_pairs(P, a);
   {
-    TimerScope ts(P->timing, P->stream, "legendre_synth_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
+    TimerScope ts(P->timing, P->stream, "legendre_synth_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L, masked) * nr);
     rc = ds_use(a) ? launch_ds_synth(a, x, nlm, nr, ph, P->stream)
                    : launch_leg_synth_mr(a, x, nlm, nr, ph, ld_phase, P->stream);
   }
@@ -688,7 +690,7 @@ int do_sandwich_mr(cr_plan* P, const Grid& g, int L, int nr, const double2* x, d
   f.bsub = bsub;
   f.out = y;
   f.ld = nlm;
-  TimerScope ts(P->timing, P->stream, "legendre_adjoint_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
+  TimerScope ts(P->timing, P->stream, "legendre_adjoint_f64", leg_work(g, L) * nr, leg_work_exec(P, g, L, masked) * nr);
   if (ds_use(a)) return launch_ds_adjoint(a, ph, nr, reinterpret_cast<double*>(part), f, P->stream);
   if ((rc = launch_leg_adjoint_mr(a, ph, ld_phase, nr, part, &f.nblk, P->stream))) return rc;
   f.partial = part;
@@ -1165,7 +1167,7 @@ int tc_synth_stage(cr_plan* P, const Grid& g, int L, const float2* x, int nr, co
   LegArgs<float> la = leg_args<float>(P, g, L);
   la.dl = dl;
   if (masked) limit_pairs(P, la);
-  TimerScope ts(P->timing, P->stream, "legendre_synth_tc", leg_work(g, L) * nr, leg_work_exec(P, g, L) * nr);
+  TimerScope ts(P->timing, P->stream, "legendre_synth_tc", leg_work(g, L) * nr, leg_work_exec(P, g, L, masked) * nr);
   return launch_tc_synth(la, x, n_lm(L), nr, tc_slot(P, g, L, 0), P->d_tc_status, P->stream);
 }
 
@@ -1179,7 +1181,7 @@ int tc_adjoint_tail(cr_plan* P, const Grid& g, int L, int nr, const TcTail& t, b
   int nblk = 0, rc;
   {
     TimerScope ts(P->timing, P->stream, "legendre_adjoint_tc", leg_work(g, L) * nr,
-                  leg_work_exec(P, g, L) * nr);
+                  leg_work_exec(P, g, L, masked) * nr);
     rc = launch_tc_adjoint(la, tc_slot(P, g, L, 0), nr, reinterpret_cast<float2*>(P->tc_partial), &nblk,
                            P->d_tc_status, P->stream);
   }

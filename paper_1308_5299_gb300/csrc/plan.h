@@ -69,10 +69,10 @@ struct Grid {
   float2* d_sti = nullptr;     // state of the FP32 two-step sequence there (legendre_f32.cu)
   float4* d_zi = nullptr;      // [npairs] its arguments
   int n1 = 0, n2 = 0;          // its zones: pairs [0, n1) polar, [n2, npairs) equatorial
-  // number of (ring pair, l, m) terms the Legendre kernels evaluate at band
-  // limit L -- those at or past the 2^-60 start of each (m, pair) -- filled
+  // number of (ring pair, l, m) terms the Legendre kernels evaluate at (band
+  // limit, ring pairs taken part) -- those at or past the 2^-60 start of each (m, pair) -- filled
   // on demand from the start table (per-stage timing only)
-  std::map<int, double> exec_terms;
+  std::map<std::pair<int, int>, double> exec_terms;
 };
 
 // Scratch sizes for transforms at band limit L on a grid (ws_mr: the FP64
