@@ -1446,7 +1446,7 @@ __global__ void average_transpose_kernel(float* M, int n) {
   M[(int64_t)j * n + i] = a;
 }
 
-// out = M in, one warp per row; n a multiple of 128
+// out = M in, one warp per row; n a multiple of 64
 template <typename T>
 __global__ void __launch_bounds__(256) dense_apply_kernel(const float* __restrict__ M, const T* __restrict__ in, T* out,
                                                           int n) {
