@@ -153,9 +153,21 @@ __device__ __forceinline__ void fft_pass(C* buf, int M, int lg, const C* __restr
         }
       }
     }
+    // the last pass: h = 1, and a thread's R consecutive values in 16-byte loads (A
+    // in FP32, Nside 2048 / 1024 / 512: 857 / 247 / 78 -> 845 / 232 / 75 us; one
+    // value a load touched every line R times)
     if (post) {
+      if constexpr (sizeof(T) == 4) {
 #pragma unroll
-      for (int t = 0; t < R; ++t) e[t] = cmul(e[t], post[j0 + t * h]);
+        for (int t = 0; t < R; t += 2) {
+          const float4 v = *reinterpret_cast<const float4*>(post + j0 + t);
+          e[t] = cmul(e[t], mk(v.x, v.y));
+          e[t + 1] = cmul(e[t + 1], mk(v.z, v.w));
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < R; ++t) e[t] = cmul(e[t], post[j0 + t]);
+      }
     }
 #pragma unroll
     for (int t = 0; t < R; ++t) buf[swz(j0 + t * h)] = e[t];
@@ -205,7 +217,7 @@ __device__ void fft_run(C* buf, int M, int logM, const C* __restrict__ tw, int M
 // (BIG, other) CTAs unbounded: 1109 / 364 / 105; (3, -) 974 / 340 / 106;
 // (4, -) 932 / 315 / 106; (4, 5) 919 / 274 / 83; (4, 6) 920 / 271 / 85; (4, 8)
 // 934 / 282 / 97; three stages per pass in BIG instead of four: (4, -) 999.
-// (With the folds four abreast these became 856 / 247 / 78.)
+// (With later changes to the folds and the loads these became 845 / 232 / 75.)
 // FP64 rings are bound by the FP64 pipe; 2 CTAs hold them to 128 registers
 // instead of 138 (A at Nside 1024, lmax 2047 2574 -> 2389 us, Nside 2048, lmax
 // 3000 10.45 -> 10.07 ms, eight right-hand sides at Nside 512 4.46 -> 4.20 ms;
