@@ -20,14 +20,14 @@
 //
 // Length-nh DFTs: radix-2 in shared memory when nh is a power of two,
 // otherwise Bluestein's chirp-z with a power-of-two convolution of size
-// M >= 2 nh - 1 (decimation-in-frequency forward FFT, pointwise product with
-// the precomputed kernel spectrum stored in bit-reversed order,
-// decimation-in-time inverse FFT: no bit-reversal passes).  The chirp
+// M >= 2 nh - 1 (forward FFT from natural to bit-reversed order, pointwise
+// product with the precomputed kernel spectrum stored in bit-reversed order,
+// inverse FFT back to natural order: no bit-reversal passes).  The chirp
 // e^{i pi k^2 / nh} = e^{i pi (2 k^2 mod 2n) / n} comes from an exact integer
 // reduction into the ring length's table of e^{i pi u / n}, u < 2n.
 //
-// One CTA per ring; mode 2 keeps the ring's map in shared memory between the
-// synthesis and the adjoint (map * N^-1 never touches HBM).
+// One CTA per ring and right-hand side; mode 2 keeps the ring's map in shared
+// memory between the synthesis and the adjoint (map * N^-1 never touches HBM).
 #include <algorithm>
 #include <cstdio>
 #include <map>
