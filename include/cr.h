@@ -500,8 +500,8 @@ int cr_smooth(cr_plan* plan, int h, const void* r, void* c, int dtype);
  * block incomplete-Cholesky solve L^-T L^-1 in the tiles' elimination
  * order, or the additive Schwarz form).  map_in, map_out: DEVICE
  * [nrhs][12 nside_h^2], RING order of the level's grid, FP32 or FP64 (the
- * factor is FP32).  With several maps every factor block is read once for
- * all of them (the form the batched cycles use).  Errors: CR_EINVAL,
+ * factor is FP32).  map_out may be map_in.  With several maps every factor
+ * block is read once for all of them (the form the batched cycles use).  Errors: CR_EINVAL,
  * CR_ESTATE, CR_ECUDA. */
 int cr_pixel_smoother(cr_plan* plan, int h, const void* map_in, void* map_out, int nrhs, int dtype);
 /* x = A_bottom^-1 b on the bottom level (l <= lmax_dense), dense (FP64). */

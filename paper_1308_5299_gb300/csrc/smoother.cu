@@ -1446,9 +1446,10 @@ __global__ void average_transpose_kernel(float* M, int n) {
   M[(int64_t)j * n + i] = a;
 }
 
-// out = M in, one warp per row; n a multiple of 64
-template <typename T>
-__global__ void __launch_bounds__(256) dense_apply_kernel(const float* __restrict__ M, const T* __restrict__ in, T* out,
+// out = M in, one warp per row; n a multiple of 64.  Every warp reads all of
+// `in`, so `out` must not overlap it (apply_smoother).
+template <typename T, typename O>
+__global__ void __launch_bounds__(256) dense_apply_kernel(const float* __restrict__ M, const T* __restrict__ in, O* out,
                                                           int n) {
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const float4* m4 = reinterpret_cast<const float4*>(M + (int64_t)row * n);
@@ -1465,7 +1466,12 @@ __global__ void __launch_bounds__(256) dense_apply_kernel(const float* __restric
   float s = (acc.x + acc.y) + (acc.z + acc.w);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[row] = (T)s;
+  if (lane == 0) out[row] = (O)s;
+}
+
+template <typename T>
+__global__ void from_f32_kernel(const float* __restrict__ in, T* out, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = (T)in[i];
 }
 
 // the backward sweep's transposed copy of the factor, made on first use
@@ -1490,7 +1496,15 @@ int apply_smoother(cr_plan* P, PixLevel& lev, T* map_in, T* map_out) {
   }
   if (lev.inv_valid) {
     const int n = pat.ntile * TK;
-    { dense_apply_kernel<T><<<n / 8, 256, 0, P->stream>>>(lev.d_inv, map_in, map_out, n); count_launch(); }
+    const uintptr_t i0 = reinterpret_cast<uintptr_t>(map_in), o0 = reinterpret_cast<uintptr_t>(map_out);
+    if (i0 < o0 + n * sizeof(T) && o0 < i0 + n * sizeof(T)) {
+      // in place: the product goes through the tile work vector (the same numbers)
+      float* y = reinterpret_cast<float*>(P->hier_tile_work);
+      { dense_apply_kernel<T, float><<<n / 8, 256, 0, P->stream>>>(lev.d_inv, map_in, y, n); count_launch(); }
+      { from_f32_kernel<T><<<(n + 255) / 256, 256, 0, P->stream>>>(y, map_out, n); count_launch(); }
+    } else {
+      { dense_apply_kernel<T, T><<<n / 8, 256, 0, P->stream>>>(lev.d_inv, map_in, map_out, n); count_launch(); }
+    }
     CR_CHECK_LAUNCH("dense_apply_kernel");
     return CR_OK;
   }

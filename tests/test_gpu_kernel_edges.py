@@ -133,3 +133,27 @@ def test_explicit_inverse_of_small_levels_against_the_sweeps(dev):
         auto.smooth(h, r, a)
         sweeps.smooth(h, r, b)
         assert rel_l2(a.cpu().numpy(), b.cpu().numpy()) < 2e-4, h
+
+
+@pytest.fixture(scope="module")
+def levels256(dev):
+    cfg, cl, bl, ninv = synthetic.problem_inputs("nside256_lmax767")
+    return binding.Plan(cfg["lmax"], nside=cfg["nside"], cl=cl, bl=bl, ninv=torch.from_numpy(ninv).to(dev),
+                        levels="default")
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("nrhs", [1, 2, 16])
+def test_pixel_smoother_in_place(dev, levels256, nrhs, dtype):
+    """map_out may be map_in on every level, also where each output depends
+    on the whole input: the same numbers as with a buffer of its own."""
+    plan = levels256
+    for h in range(1, plan.nlevels() + 1):
+        npix = 12 * plan.level(h)["nside_h"] ** 2
+        m = torch.from_numpy(synthetic.random_map(nrhs * npix, seed=60 + h)).to(dtype).to(dev).reshape(nrhs, npix)
+        out = torch.empty_like(m)
+        plan.pixel_smoother(h, m, out)
+        for _ in range(5):
+            a = m.clone()
+            plan.pixel_smoother(h, a, a)
+            assert torch.equal(a, out), h
