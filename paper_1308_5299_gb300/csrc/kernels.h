@@ -13,7 +13,7 @@ struct DsTab {
   double *A = nullptr, *B = nullptr, *AB = nullptr;    // coefficients of the step that produces q_k
   double *sg = nullptr, *e0 = nullptr, *e1 = nullptr;  // sigma_k, and times e_o and e_{o+1}
   uint64_t *Ai = nullptr, *Bi = nullptr;               // A 2^57, (B + 8) 2^60: the integer steps' coefficients
-  float4 *rf = nullptr, *cf = nullptr;                 // FP32: (A, A + B - 2, B, B + 2); sigma_k times (1, e_o, e_{o+1})
+  float4 *rf = nullptr, *cf = nullptr;                 // FP32: (A, A + B - 2, B, 0); sigma_k times (1, e_o, e_{o+1})
   int Lc = -1;
 };
 

@@ -532,14 +532,15 @@ int launch_leg_diag(cr_plan* P, const double* ringval, double2* out) {
 }
 
 // The start state (value before k0, second value) of one pair of the FP32
-// two-step sequence (legendre_f32.cu), from the FP64
-// state (Q_{l-1}, Q_{l-2}) and Q_l at its start l: such that the zone's step
-// returns q_{k0}, k0 = (l - m) / 2.
-__device__ float2 lf_start(const DsTab& t, const double* s, int Lc, int m, int l, double z, int zone, double Q,
-                           double Q1, double Q2) {
+// sequences (legendre_f32.cu), from the FP64 state (Q_{l-1}, Q_{l-2}) and Q_l at
+// its start l: such that the zone's step returns q_{k0}, k0 = (l - m) / 2 (the
+// one-step zone: Q_{m + 2 k0}, one step back where l is the second of its two).
+__device__ float2 lf_start(const DsTab& t, const double* c, const double* s, int Lc, int m, int l, double z, int zone,
+                           double Q, double Q1, double Q2) {
   const int k0 = (l - m) >> 1;
   const int64_t oc = lm_off(Lc, m) + (l - m), ok = ((lm_off(t.Lc, m) >> 1) + m) + k0;
   const bool odd = (l - m) & 1;
+  if (zone == 2) return odd ? make_float2((float)Q2, (float)(c[oc - 1] * z * Q2 - Q1)) : make_float2((float)Q1, (float)Q2);
   const double P = s[oc] * Q;
   double q1 = 0.0;
   if (k0 > 0) q1 = (odd ? s[oc - 2] * Q2 : s[oc - 1] * Q1) / (z * t.sg[ok - 1]);
@@ -550,9 +551,7 @@ __device__ float2 lf_start(const DsTab& t, const double* s, int Lc, int m, int l
     return make_float2((float)q1, (float)(qk - q1 - e * q1));
   }
   const double e = k0 > 0 ? fma(t.A[ok], z * z, t.B[ok]) : 0.0;
-  if (zone == 1) return make_float2((float)q1, (float)(e * q1 - qk));
-  const double sg = (k0 & 1) ? -1.0 : 1.0;
-  return make_float2((float)(-sg * q1), (float)(sg * (qk + q1 - (k0 > 0 ? (e + 2.0) * q1 : 0.0))));
+  return make_float2((float)q1, (float)(e * q1 - qk));
 }
 
 // Start tables (see Grid): for each m <= Lseed and ring pair, the scaled FP64
@@ -587,7 +586,7 @@ __global__ void start_kernel(const double* z, const double* seed, const int* lev
         f32 = l;
         s32 = (p < npolar32) ? make_float2((float)q1, (float)(q1 - q2)) : make_float2((float)q1, (float)q2);
         s64b = make_double2(q1, q2);
-        si = lf_start(t, s, Lc, m, l, zz, p < n1 ? 0 : p < n2 ? 1 : 2, q, q1, q2);
+        si = lf_start(t, c, s, Lc, m, l, zz, p < n1 ? 0 : p < n2 ? 1 : 2, q, q1, q2);
         break;
       }
     }

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(DST_NT) ds_tab_kernel(DsTab t) {
       t.B[off + k + 1] = B.h;
       const dd2 AB = dd_mul(A, S1);
       t.AB[off + k + 1] = AB.h;
-      t.rf[off + k + 1] = make_float4((float)A.h, (float)((AB.h - 2.0) + AB.l), (float)B.h, (float)((B.h + 2.0) + B.l));
+      t.rf[off + k + 1] = make_float4((float)A.h, (float)((AB.h - 2.0) + AB.l), (float)B.h, 0.f);
       // fixed point: A 2^57 and (B + 8) 2^60 (modulo 2^64); the integer steps
       // start where A < 100
       const double n = rint(B.h);

@@ -5,19 +5,26 @@
 //   c_k = e_o a_{o-1} + e_{o+1} a_{o+1},  d_k = a_o,
 // and q_k = p_k / sigma_k obeys q_{k+1} = e_k q_k - q_{k-1}, e_k = A_k z^2 + B_k.
 // Per two l and ring pair that is 2 (or 3) operations of recurrence and 4 of
-// sums, where the one-step recurrence took 4 (or 6) and 4.  Three forms of the
+// sums, where the one-step recurrence takes 4 (or 6) and 4.  Three forms of the
 // step keep FP32's rounding down, each on a range of pairs (a warp has one):
 //  - polar, z > LF_ZPOLAR: the difference form on s = 1 - z^2,
 //      d = ((A + B - 2) - A s) q + d, q = q + d
 //    (q varies slowly in k there; e - 2 is carried at full relative precision);
-//  - middle: q_{k+1} = (A z^2 + B) q_k - q_{k-1} with four copies of z^2 that
-//    differ in the last place and average to the exact square, used in turn
-//    (one rounded square would act the same way at every k);
-//  - equatorial, z < LF_ZEQ: q alternates in sign; v_k = (-1)^k q_k takes the
-//    difference form with -(B + 2) - A z^2, and the sign goes to the
-//    coefficients (synthesis) or the sums (adjoint).
-// In FP32 emulated against extended precision (white spectrum, Nside 2048 /
-// lmax 3000) the error is 5e-6 where the one-step form's was 1.5e-5.
+//  - middle: q_{k+1} = (A z^2 + B) q_k - q_{k-1};
+//  - equatorial, z < LF_ZEQ: the one-step recurrence, P~_l = s_l q_l, q_l = c_l z
+//    q_{l-1} - q_{l-2}.  p_k grows like min(L, 1 / z) there while P~ does not, so
+//    that the two-step form's even sums cancel by that factor (the ring on the
+//    equator would be off by 5e-6, 1.4e-5, 4e-5 at lmax 384, 1023, 3000).
+// The argument of each has four copies that differ in the last place and
+// average to the exact value, used in turn: a single rounded one would act the
+// same way at every step.  The lines lie where the forms on either side are
+// about equally near or the cheaper one is.
+// Ring by ring against FP64 (white spectrum, Nside 64 / lmax 384, 512 / 1023, 2048 /
+// 3000): 3e-7, 5e-7, 8e-7 for z < 0.015, at most 5e-7, 1e-6, 2.5e-6 for z < LF_ZEQ,
+// 2e-6, 4.7e-6, 1.3e-5 just below LF_ZPOLAR, 1.2e-6, 2.8e-6, 7e-6 above it; over the
+// map 7.5e-7, 1.6e-6, 4.9e-6.  One-step kernels with rounded arguments throughout:
+// 3e-7, 5e-7, 9e-7 for z < 0.015, 3.8e-6, 9e-6, 2.5e-5 at z = 0.7, 1.8e-6, 4.4e-6,
+// 1.2e-5 over the map.  No ring is further off than theirs.
 //
 // One warp per block of 32 RP pairs of one m (RP per thread), without block
 // barriers; m in blockIdx.y, so the longest warps start first.  Each warp
@@ -48,33 +55,35 @@ void lf_zones(const double* z, int npairs, int* n1, int* n2) {
   *n2 = i;
 }
 
-// arguments of a pair's steps: four copies of z^2 (middle), or 1 - z^2, or z^2
+// arguments of a pair's steps: four copies of 1 - z^2 (polar), z^2 (middle) or z
 void lf_args(const double* z, int npairs, int n1, int n2, float4* out) {
   for (int p = 0; p < npairs; ++p) {
-    const double x = z[p] * z[p], xl = std::fma(z[p], z[p], -x);  // the exact square
+    // the exact value as x + xl
+    double x = z[p], xl = 0.0;
     if (p < n1) {
-      const double w = 1.0 - z[p];
-      const float s = (float)(w * (2.0 - w));
-      out[p] = make_float4(s, s, s, s);
-    } else if (p >= n2) {
-      const float s = (float)x;
-      out[p] = make_float4(s, s, s, s);
-    } else {
-      const float h = (float)x;
+      const double w = 1.0 - z[p], u = 2.0 * w;  // exact
+      x = std::fma(-w, w, u);
+      xl = std::fma(-w, w, u - x);
+    } else if (p < n2) {
+      x = z[p] * z[p];
+      xl = std::fma(z[p], z[p], -x);
+    }
+    const float h = (float)x;
+    float c[4] = {h, h, h, h};
+    if (h > 0.f) {
       const float up = nextafterf(h, 2.f) - h;
       const int t = (int)lrint(4.0 * ((x - h) + xl) / up);
-      float c[4];
       for (int j = 0; j < 4; ++j) c[j] = h + (j < abs(t) ? (t > 0 ? up : -up) : 0.f);
-      out[p] = make_float4(c[0], c[1], c[2], c[3]);
     }
+    out[p] = make_float4(c[0], c[1], c[2], c[3]);
   }
 }
 
-// One warp's pairs: arguments, states, start indices.
+// One warp's pairs: arguments, states, start indices.  ZONE 0 polar, 1 middle,
+// 2 equatorial (one-step: two l, of either parity of l - m, per k).
 template <int ZONE, int RP>
 struct LfPairs {
-  static constexpr int NZ = ZONE == 1 ? 4 : 1;
-  float q1[RP], q2[RP], Z[RP][NZ];
+  float q1[RP], q2[RP], Z[RP][4];
   int k0[RP], p[RP];
   int kmin, kmax;  // first and last start of the warp's live pairs
 
@@ -102,34 +111,47 @@ struct LfPairs {
         }
       }
       Z[j][0] = z.x;
-      if (NZ == 4) {
-        Z[j][NZ > 1 ? 1 : 0] = z.y;
-        Z[j][NZ > 2 ? 2 : 0] = z.z;
-        Z[j][NZ > 3 ? 3 : 0] = z.w;
-      }
+      Z[j][1] = z.y;
+      Z[j][2] = z.z;
+      Z[j][3] = z.w;
     }
     kmin = __reduce_min_sync(0xffffffffu, lo);
     kmax = __reduce_max_sync(0xffffffffu, hi);
   }
-  // the next value of pair j; u: its k modulo 4
-  __device__ __forceinline__ float next(float2 r, int j, int u, float& second) const {
-    const float e = fmaf(r.x, Z[j][NZ == 4 ? u & 3 : 0], r.y);
-    if (ZONE == 1) {
+  // the next value of pair j, for the even and the odd sums (ZONE 2: the next
+  // two), and the state behind it if `on`; u: its k modulo 4
+  __device__ __forceinline__ float2 next(float2 r, int j, int u, bool on) {
+    const float z = Z[j][u & 3];
+    float qe, qo, second;
+    if (ZONE == 2) {
+      qe = fmaf(r.x * z, q1[j], -q2[j]);
+      qo = fmaf(r.y * z, qe, -q1[j]);
+      second = qe;
+    } else if (ZONE == 1) {
+      qe = qo = fmaf(fmaf(r.x, z, r.y), q1[j], -q2[j]);
       second = q1[j];
-      return fmaf(e, q1[j], -q2[j]);
+    } else {
+      second = fmaf(fmaf(r.x, z, r.y), q1[j], q2[j]);
+      qe = qo = q1[j] + second;
     }
-    const float d = fmaf(e, q1[j], q2[j]);
-    second = d;
-    return q1[j] + d;
+    if (on) {
+      q2[j] = second;
+      q1[j] = qo;
+    }
+    return make_float2(qe, qo);
   }
 };
 
-// (factor of the argument, constant) of a zone's step, from (A, A + B - 2, B, B + 2)
+// coefficients of step k: (factor of the argument, constant) from (A, A + B - 2,
+// B), or those of l = m + 2k and l + 1 (ZONE 2)
 template <int ZONE>
-__device__ __forceinline__ float2 lf_coef(float4 t) {
-  if (ZONE == 0) return make_float2(-t.x, t.y);
-  if (ZONE == 1) return make_float2(t.x, t.z);
-  return make_float2(-t.x, -t.w);
+__device__ __forceinline__ float2 lf_step(const LegArgs<float>& a, int m, int k) {
+  if (ZONE == 2) {
+    const float* c = a.c + lm_off(a.Lc, m) + 2 * k;
+    return make_float2(c[0], m + 2 * k + 1 <= a.L ? c[1] : 0.f);
+  }
+  const float4 t = a.rf[(lm_off(a.Lc, m) >> 1) + m + k];
+  return ZONE == 0 ? make_float2(-t.x, t.y) : make_float2(t.x, t.z);
 }
 
 struct LfStage {
@@ -158,12 +180,21 @@ __device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, i
       const int k = kc + i;
       if (i < n) {
         const int l = m + 2 * k;
-        const float4 t = a.rf[offk + k], g = a.cf[offk + k];
         const float2* x = a.alm + offa + 2 * k;
         const float2 x0 = x[0];
         const float2 x1 = l + 1 <= L ? x[1] : make_float2(0.f, 0.f);
-        const float2 x2 = l + 2 <= L ? x[2] : make_float2(0.f, 0.f);
-        float f0 = g.y, f1 = g.x, f2 = g.z;
+        const float2 x2 = ZONE < 2 && l + 2 <= L ? x[2] : make_float2(0.f, 0.f);
+        float f0, f1, f2 = 0.f;
+        if (ZONE == 2) {
+          const float* s1 = a.s + lm_off(a.Lc, m) + 2 * k;
+          f0 = s1[0];
+          f1 = l + 1 <= L ? s1[1] : 0.f;
+        } else {
+          const float4 g = a.cf[offk + k];
+          f0 = g.y;
+          f1 = g.x;
+          f2 = g.z;
+        }
         if (a.dl) {
           f0 *= a.dl[l];
           f1 *= l + 1 <= L ? a.dl[l + 1] : 0.f;
@@ -171,9 +202,8 @@ __device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, i
         }
         float4 c = make_float4(fmaf(f0, x0.x, f2 * x2.x), fmaf(f0, x0.y, f2 * x2.y), f1 * x1.x, f1 * x1.y);
         if (m == 0) c.y = c.w = 0.f;
-        if (ZONE == 2 && (k & 1)) c = make_float4(-c.x, -c.y, -c.z, -c.w);
         sh.c[i] = c;
-        sh.r[i] = lf_coef<ZONE>(t);
+        sh.r[i] = lf_step<ZONE>(a, m, k);
       }
     }
     __syncwarp();
@@ -187,14 +217,11 @@ __device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, i
           const float4 c = sh.c[i8 + u];
 #pragma unroll
           for (int j = 0; j < RP; ++j) {
-            float d;
-            const float q = s.next(r, j, u, d);
-            s.q2[j] = d;
-            s.q1[j] = q;
-            cx[j] = fmaf(q, c.x, cx[j]);
-            cy[j] = fmaf(q, c.y, cy[j]);
-            dx[j] = fmaf(q, c.z, dx[j]);
-            dy[j] = fmaf(q, c.w, dy[j]);
+            const float2 q = s.next(r, j, u, true);
+            cx[j] = fmaf(q.x, c.x, cx[j]);
+            cy[j] = fmaf(q.x, c.y, cy[j]);
+            dx[j] = fmaf(q.y, c.z, dx[j]);
+            dy[j] = fmaf(q.y, c.w, dy[j]);
           }
         }
       } else {
@@ -205,15 +232,13 @@ __device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, i
           const float4 c = sh.c[i8 + u];
 #pragma unroll
           for (int j = 0; j < RP; ++j) {
-            float d;
-            const float q = s.next(r, j, u, d);
-            if (k + u >= s.k0[j]) {
-              s.q2[j] = d;
-              s.q1[j] = q;
-              cx[j] = fmaf(q, c.x, cx[j]);
-              cy[j] = fmaf(q, c.y, cy[j]);
-              dx[j] = fmaf(q, c.z, dx[j]);
-              dy[j] = fmaf(q, c.w, dy[j]);
+            const bool on = k + u >= s.k0[j];
+            const float2 q = s.next(r, j, u, on);
+            if (on) {
+              cx[j] = fmaf(q.x, c.x, cx[j]);
+              cy[j] = fmaf(q.x, c.y, cy[j]);
+              dx[j] = fmaf(q.y, c.z, dx[j]);
+              dy[j] = fmaf(q.y, c.w, dy[j]);
             }
           }
         }
@@ -224,15 +249,23 @@ __device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, i
   for (int j = 0; j < RP; ++j)
     if (s.p[j] < pend) {
       const int rn = s.p[j], rs = a.nring - 1 - rn;
-      const float z = a.z[rn];
+      const float z = ZONE == 2 ? 1.f : a.z[rn];
       a.phase[(int64_t)rn * a.ldp + m] = make_float2(fmaf(z, dx[j], cx[j]), fmaf(z, dy[j], cy[j]));
       if (rs != rn) a.phase[(int64_t)rs * a.ldp + m] = make_float2(fmaf(-z, dx[j], cx[j]), fmaf(-z, dy[j], cy[j]));
     }
 }
 
-// warp blocks of the three zones
+// warp blocks of a zone of n pairs
 template <int RP>
 __host__ __device__ inline int lf_blocks(int n) { return (n + 32 * RP - 1) / (32 * RP); }
+
+// The equatorial zone, whose steps are the longest and whose pairs often fill
+// less than half of a warp's: half as many per thread then.
+template <int RP>
+__device__ __forceinline__ void lf_synth_eq(const LegArgs<float>& a, LfStage& sh, int m, int base) {
+  if (a.npairs - base <= 16 * RP) lf_synth<2, RP / 2>(a, sh, m, base, a.npairs);
+  else lf_synth<2, RP>(a, sh, m, base, a.npairs);
+}
 
 template <int RP, int MT>
 __global__ void __launch_bounds__(32) lf_synth_kernel(LegArgs<float> a) {
@@ -245,7 +278,7 @@ __global__ void __launch_bounds__(32) lf_synth_kernel(LegArgs<float> a) {
     if (mi > 0 && m <= (int)blockIdx.y) break;
     if (b < b0) lf_synth<0, RP>(a, sh, m, b * 32 * RP, a.n1);
     else if (b < b0 + b1) lf_synth<1, RP>(a, sh, m, a.n1 + (b - b0) * 32 * RP, a.n2);
-    else lf_synth<2, RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, a.npairs);
+    else lf_synth_eq<RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP);
     __syncwarp();
   }
 }
@@ -253,6 +286,7 @@ __global__ void __launch_bounds__(32) lf_synth_kernel(LegArgs<float> a) {
 // ---- adjoint -----------------------------------------------------------------
 // u_k = sum_pairs q_k (G_m(z) + G_m(-z)), v_k = sum_pairs q_k z (G_m(z) - G_m(-z));
 // a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k, a_{o+1} += sigma_k e_{o+1} u_k.
+// ZONE 2: the sums of q_l themselves, l = m + 2k and m + 2k + 1; a_l = s_l times it.
 // The four real sums of a k over a thread's RP pairs go to a shared-memory
 // row; per 8 k, lane (k, part) adds every fourth lane's entry and two exchange
 // steps leave one of the four sums per lane, 128 contiguous bytes of the
@@ -285,14 +319,13 @@ __device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& 
     ge[j] = go[j] = make_float2(0.f, 0.f);
     if (s.k0[j] < nk) {
       const int rn = s.p[j], rs = a.nring - 1 - rn;
-      const float z = a.z[rn];
+      const float z = ZONE == 2 ? 1.f : a.z[rn];
       const float2 gn = a.phase[(int64_t)rn * a.ldp + m];
       const float2 gs = rs != rn ? a.phase[(int64_t)rs * a.ldp + m] : make_float2(0.f, 0.f);
       ge[j] = cadd(gn, gs);
       go[j] = make_float2(z * (gn.x - gs.x), z * (gn.y - gs.y));
     }
   }
-  const int64_t offk = (lm_off(a.Lc, m) >> 1) + m;
   const int kbeg = min(s.kmin, nk) & ~7;
   for (int i = lane; i < 4 * kbeg; i += 32) row[i] = 0.f;  // before the first start
   if (s.kmin >= nk) {
@@ -304,7 +337,7 @@ __device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& 
     __syncwarp();
 #pragma unroll
     for (int i = lane; i < LF_CH; i += 32)
-      if (i < n) sh.r[i] = lf_coef<ZONE>(a.rf[offk + kc + i]);
+      if (i < n) sh.r[i] = lf_step<ZONE>(a, m, kc + i);
     __syncwarp();
     for (int i8 = 0; i8 < n; i8 += 8) {
       const int k = kc + i8;
@@ -316,14 +349,11 @@ __device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& 
           float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int j = 0; j < RP; ++j) {
-            float d;
-            const float q = s.next(r, j, u, d);
-            s.q2[j] = d;
-            s.q1[j] = q;
-            t.x = fmaf(q, ge[j].x, t.x);
-            t.y = fmaf(q, ge[j].y, t.y);
-            t.z = fmaf(q, go[j].x, t.z);
-            t.w = fmaf(q, go[j].y, t.w);
+            const float2 q = s.next(r, j, u, true);
+            t.x = fmaf(q.x, ge[j].x, t.x);
+            t.y = fmaf(q.x, ge[j].y, t.y);
+            t.z = fmaf(q.y, go[j].x, t.z);
+            t.w = fmaf(q.y, go[j].y, t.w);
           }
           sh.b[u][lane] = t;
         }
@@ -335,15 +365,13 @@ __device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& 
             const float2 r = sh.r[i8 + u];
 #pragma unroll
             for (int j = 0; j < RP; ++j) {
-              float d;
-              const float q = s.next(r, j, u, d);
-              if (k + u >= s.k0[j]) {
-                s.q2[j] = d;
-                s.q1[j] = q;
-                t.x = fmaf(q, ge[j].x, t.x);
-                t.y = fmaf(q, ge[j].y, t.y);
-                t.z = fmaf(q, go[j].x, t.z);
-                t.w = fmaf(q, go[j].y, t.w);
+              const bool on = k + u >= s.k0[j];
+              const float2 q = s.next(r, j, u, on);
+              if (on) {
+                t.x = fmaf(q.x, ge[j].x, t.x);
+                t.y = fmaf(q.x, ge[j].y, t.y);
+                t.z = fmaf(q.y, go[j].x, t.z);
+                t.w = fmaf(q.y, go[j].y, t.w);
               }
             }
           }
@@ -368,10 +396,15 @@ __device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& 
       const float s1 = __shfl_xor_sync(0xffffffffu, hi ? tu.y : tv.y, 2);
       const float w0 = (hi ? tv.x : tu.x) + s0, w1 = (hi ? tv.y : tu.y) + s1;
       float w = (im ? w1 : w0) + __shfl_xor_sync(0xffffffffu, im ? w0 : w1, 1);
-      if (ZONE == 2 && (u & 1)) w = -w;  // k is a multiple of 8
       if (i8 + u < n) row[4 * (k + u) + part] = w;
     }
   }
+}
+
+template <int RP>
+__device__ __forceinline__ void lf_adjoint_eq(const LegArgs<float>& a, LfAdjStage& sh, int m, int base, float* row) {
+  if (a.npairs - base <= 16 * RP) lf_adjoint<2, RP / 2>(a, sh, m, base, a.npairs, row);
+  else lf_adjoint<2, RP>(a, sh, m, base, a.npairs, row);
 }
 
 template <int RP, int MT>
@@ -386,16 +419,17 @@ __global__ void __launch_bounds__(32) lf_adjoint_kernel(LegArgs<float> a, float*
     float* row = partial + ((int64_t)b * nkk + ((lm_off(a.L, m) >> 1) + m)) * 4;
     if (b < b0) lf_adjoint<0, RP>(a, sh, m, b * 32 * RP, a.n1, row);
     else if (b < b0 + b1) lf_adjoint<1, RP>(a, sh, m, a.n1 + (b - b0) * 32 * RP, a.n2, row);
-    else lf_adjoint<2, RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, a.npairs, row);
+    else lf_adjoint_eq<RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, row);
     __syncwarp();
   }
 }
 
-// a_l (l = m + 2k + w) from the summed (u_k, v_k), u_{k-1}, and the epilogue of
-// leg_finalize_kernel
+// a_l (l = m + 2k + w) from the summed (u_k, v_k), u_{k-1} and the one-step
+// zone's sums q, and the epilogue of leg_finalize_kernel
 __device__ __forceinline__ void lf_emit(const LegArgs<float>& a, const FinalizeArgs<float>& f, int m, int k, float4 t,
-                                        float2 um) {
+                                        float2 um, float4 q) {
   const int L = a.L;
+  const float* sl = a.s + lm_off(a.Lc, m) + 2 * k;
   const int64_t ok = (lm_off(a.Lc, m) >> 1) + m + k;
   const float4 g = a.cf[ok];
   const float g1 = k > 0 ? a.cf[ok - 1].z : 0.f;
@@ -405,6 +439,8 @@ __device__ __forceinline__ void lf_emit(const LegArgs<float>& a, const FinalizeA
     if (l > L) break;
     float2 y = w == 0 ? make_float2(fmaf(g.y, t.x, g1 * um.x), fmaf(g.y, t.y, g1 * um.y))
                       : make_float2(g.x * t.z, g.x * t.w);
+    y.x = fmaf(sl[w], w == 0 ? q.x : q.z, y.x);
+    y.y = fmaf(sl[w], w == 0 ? q.y : q.w, y.y);
     const int64_t i = lm_off(L, m) + (l - m);
     if (f.dl_out) y = cscale(y, f.dl_out[l]);
     if (f.dadd) {
@@ -422,35 +458,36 @@ __device__ __forceinline__ void lf_emit(const LegArgs<float>& a, const FinalizeA
   }
 }
 
-// The warps' rows in a fixed order; thread = one k.
+// The warps' rows in a fixed order (n2s of the two-step zones, then the one-step
+// zone's); thread = one k.
 __global__ void __launch_bounds__(128) lf_finalize_kernel(LegArgs<float> a, FinalizeArgs<float> f, const float4* partial,
-                                                          int64_t nkk, int nblk) {
+                                                          int64_t nkk, int n2s, int nblk) {
   const int m = blockIdx.y;
   const int nk = (a.L - m) / 2 + 1;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if ((int)(blockIdx.x * blockDim.x) >= nk) return;  // whole CTA
   const float4* row = partial + ((lm_off(a.L, m) >> 1) + m);
-  auto sum = [&](int kk) {
+  auto sum = [&](int kk, int b0, int b1) {
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-    for (int b = 0; b < nblk; ++b) {
+    for (int b = b0; b < b1; ++b) {
       const float4 w = row[b * nkk + kk];
       t = make_float4(t.x + w.x, t.y + w.y, t.z + w.z, t.w + w.w);
     }
     return t;
   };
   float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (k < nk) t = sum(k);
+  if (k < nk) t = sum(k, 0, n2s);
   float2 um = make_float2(__shfl_up_sync(0xffffffffu, t.x, 1), __shfl_up_sync(0xffffffffu, t.y, 1));
   if (k >= nk) return;
   if ((threadIdx.x & 31) == 0) {
     um = make_float2(0.f, 0.f);
     if (k > 0) {
-      const float4 w = sum(k - 1);
+      const float4 w = sum(k - 1, 0, n2s);
       um = make_float2(w.x, w.y);
     }
   }
-  lf_emit(a, f, m, k, t, um);
+  lf_emit(a, f, m, k, t, um, sum(k, n2s, nblk));
 }
 
 // All warps of one m in one CTA (grids of few pairs): the rows stay in shared
@@ -468,12 +505,13 @@ __global__ void __launch_bounds__(32 * LF_FUSED) lf_adjoint_fused_kernel(LegArgs
   float* row = reinterpret_cast<float*>(rows + b * ld);
   if (b < b0) lf_adjoint<0, RP>(a, sh, m, b * 32 * RP, a.n1, row);
   else if (b < b0 + b1) lf_adjoint<1, RP>(a, sh, m, a.n1 + (b - b0) * 32 * RP, a.n2, row);
-  else lf_adjoint<2, RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, a.npairs, row);
+  else lf_adjoint_eq<RP>(a, sh, m, a.n2 + (b - b0 - b1) * 32 * RP, row);
   __syncthreads();
   for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f), q = t;
     float2 um = make_float2(0.f, 0.f);
-    for (int w = 0; w < nw; ++w) {
+    const int n2s = b0 + b1;
+    for (int w = 0; w < n2s; ++w) {
       const float4 x = rows[w * ld + k];
       t = make_float4(t.x + x.x, t.y + x.y, t.z + x.z, t.w + x.w);
       if (k > 0) {
@@ -481,15 +519,23 @@ __global__ void __launch_bounds__(32 * LF_FUSED) lf_adjoint_fused_kernel(LegArgs
         um = make_float2(um.x + y.x, um.y + y.y);
       }
     }
-    lf_emit(a, f, m, k, t, um);
+    for (int w = n2s; w < nw; ++w) {
+      const float4 x = rows[w * ld + k];
+      q = make_float4(q.x + x.x, q.y + x.y, q.z + x.z, q.w + x.w);
+    }
+    lf_emit(a, f, m, k, t, um, q);
   }
 }
 
 // ---- launchers ---------------------------------------------------------------
 
-static int lf_nblocks(const LegArgs<float>& a, int rp) {
+// warps of one m: those of the two-step zones, and of all zones
+static int lf_blocks2(const LegArgs<float>& a, int rp) {
   auto nb = [&](int n) { return (n + 32 * rp - 1) / (32 * rp); };
-  return nb(a.n1) + nb(a.n2 - a.n1) + nb(a.npairs - a.n2);
+  return nb(a.n1) + nb(a.n2 - a.n1);
+}
+static int lf_nblocks(const LegArgs<float>& a, int rp) {
+  return lf_blocks2(a, rp) + (a.npairs - a.n2 + 32 * rp - 1) / (32 * rp);
 }
 int64_t lf_partial_bytes(int npairs, int L) {
   return (int64_t)((npairs + 63) / 64 + 3) * ds_len(L) * (int64_t)sizeof(float4);
@@ -540,7 +586,8 @@ static int lf_adjoint_launch(const LegArgs<float>& a, const FinalizeArgs<float>&
   count_launch();
   CR_CHECK_LAUNCH("lf_adjoint_kernel");
   const dim3 grid((a.L / 2 + 1 + 127) / 128, a.L + 1);
-  { lf_finalize_kernel<<<grid, 128, 0, st>>>(a, f, reinterpret_cast<const float4*>(part), nkk, nb); count_launch(); }
+  { lf_finalize_kernel<<<grid, 128, 0, st>>>(a, f, reinterpret_cast<const float4*>(part), nkk,
+                                           lf_blocks2(a, RP), nb); count_launch(); }
   CR_CHECK_LAUNCH("lf_finalize_kernel");
   return CR_OK;
 }

@@ -66,9 +66,9 @@ struct Grid {
   int* d_ls32 = nullptr;
   float2* d_st32 = nullptr;
   double2* d_st64b = nullptr;  // FP64 state at the FP32 start (double-float kernels)
-  float2* d_sti = nullptr;     // state of the FP32 two-step sequence there (legendre_f32.cu)
-  float4* d_zi = nullptr;      // [npairs] its arguments
-  int n1 = 0, n2 = 0;          // its zones: pairs [0, n1) polar, [n2, npairs) equatorial
+  float2* d_sti = nullptr;     // state of the FP32 sequences there (legendre_f32.cu)
+  float4* d_zi = nullptr;      // [npairs] their arguments
+  int n1 = 0, n2 = 0;          // their zones: pairs [0, n1) polar, [n2, npairs) equatorial
   // number of (ring pair, l, m) terms the Legendre kernels evaluate at (band
   // limit, ring pairs taken part) -- those at or past the 2^-60 start of each (m, pair) -- filled
   // on demand from the start table (per-stage timing only)

@@ -157,3 +157,37 @@ def test_pixel_smoother_in_place(dev, levels256, nrhs, dtype):
             a = m.clone()
             plan.pixel_smoother(h, a, a)
             assert torch.equal(a, out), h
+
+
+@pytest.mark.parametrize("grid,lmax", [(64, 384), (512, 1023), ((901, 1802), 900), ((258, 520), 257)])
+def test_fp32_ring_by_ring(dev, grid, lmax):
+    """Every ring of an FP32 synthesis, and the FP32 adjoint of single rings
+    next to the equator, against FP64: the sums of about lmax / 2 terms round
+    as a random walk, sqrt(lmax) 2^-24, and a rounding of the argument shifts
+    the phase of P~_l by l z 2^-24; twice their sum is allowed."""
+    if isinstance(grid, int):
+        z, n = (np.asarray(v) for v in synthetic.healpix_ring_table(grid)[:2])
+        plan = binding.Plan(lmax, nside=grid)
+    else:
+        z, n = np.polynomial.legendre.leggauss(grid[0])[0], np.full(grid[0], grid[1])
+        plan = binding.Plan(lmax, gl=grid)
+    tol = 2.0**-23 * (np.sqrt(lmax) + 2.0 * lmax * np.abs(z))
+    ring = np.repeat(np.arange(len(n)), n)
+    a = torch.from_numpy(synthetic.random_alm(lmax, seed=13)).to(dev).to(torch.complex64)
+    m32 = torch.empty(len(ring), dtype=torch.float32, device=dev)
+    m64 = torch.empty(len(ring), dtype=torch.float64, device=dev)
+    plan.sht_synth(a, m32)
+    plan.sht_synth(a.to(torch.complex128), m64)
+    ref = m64.cpu().numpy()
+    err = np.sqrt(np.bincount(ring, (m32.cpu().numpy() - ref) ** 2) / np.bincount(ring, ref**2))
+    assert (err < tol).all(), (err / tol).max()
+    near = np.argsort(np.abs(z), kind="stable")
+    for k in (0, 1, 3, 7, 15, 31):
+        i = near[k]
+        y = torch.zeros(len(ring), dtype=torch.float32, device=dev)
+        y[torch.from_numpy(ring == i).to(dev)] = torch.from_numpy(synthetic.random_map(n[i], seed=80 + k)).to(dev).float()
+        b32 = torch.empty(sht.n_lm(lmax), dtype=torch.complex64, device=dev)
+        b64 = torch.empty(sht.n_lm(lmax), dtype=torch.complex128, device=dev)
+        plan.sht_adjoint(y, b32)
+        plan.sht_adjoint(y.double(), b64)
+        assert rel_l2(b32.cpu().numpy().astype(np.complex128), b64.cpu().numpy()) < tol[i], k
