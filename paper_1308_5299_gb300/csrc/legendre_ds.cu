@@ -7,14 +7,21 @@
 // FP64 pipe only takes the first steps of a sequence and collects the sums.
 //
 // Digit slices.  Every operand is written as a fixed-point number of seven
-// signed base-256 digits (54 bits below a bound that holds for the whole row
-// or block).  Digits are small integers, exact in FP16; products of two
-// digits summed over at most 128 terms and at most seven digit pairs of the
-// same weight stay below 2^24, so the FP32 accumulators of the tensor cores
-// are exact, and the sums of equal weight (order s = i + j of the digits'
-// positions) can share one accumulator.  Orders 0..7 are kept: the dropped
-// ones are below the last digit of either operand.  Per term the error is
-// thus an absolute 2^-54 of the operands' bounds, where a chain of FP64
+// base-256 digits (54 bits below a bound that holds for the whole row or
+// block): the sequence's 0..255 below a signed leading one, the other
+// operand's -128..127; leading ones are within 64.  Digits are small integers,
+// exact in FP16, their products exact integers, and the sums of products of
+// equal weight (order s = i + j of the digits' positions) share one FP32
+// accumulator.  Below 2^24 an accumulator is exact: always in the orders that
+// count (the assertions at DSS_KB and DSA_CB); in the last two (three in the
+// adjoint, when four accumulators are added up) the largest possible sums, all
+// digits extreme and of one sign, reach 1.2 (1.5) times 2^24 and may lose units
+// there.  A unit of order s is 2^(-8 s - 12) of the operands' bounds, and one or
+// two are lost in an addition: at most 2^-53 a block of the synthesis (42
+// products into an order) and 2^-51 of the adjoint, under 3 and 7 % of the 96
+// and 128 2^-54 that the digits not kept amount to.  Orders 0..7 are kept: the
+// dropped ones are below the last digit of either operand.  Per term the error
+// is thus an absolute 2^-54 of the operands' bounds, where a chain of FP64
 // multiply-adds rounds to 2^-53 of the running sum at each step.  (The
 // splitting of an accurate product into exact low-precision products is the
 // scheme of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012.)
@@ -31,7 +38,7 @@
 //   q_{k+1} = (A_k z^2 + B_k) q_k - q_{k-1},
 // one step for two l.  Once a pair's values have grown past the first steps
 // they are 64-bit fixed-point numbers, z^2 and the coefficients too (z^2 to
-// 2^-64, the factor A z^2 + B + 8 to 2^-60), so a step rounds at 2^-62 of the
+// 2^-64, the factor A z^2 + B + 8 to 2^-57), so a step rounds at 2^-58 of the
 // bound of the functions and not at 2^-53 of the running value; the upper
 // bytes of the same integers are the digits of the products.  Near the poles
 // the first steps use 1 - z^2 and A_k + B_k.  Near the equator p_k grows like
@@ -71,6 +78,14 @@ constexpr uint64_t DS_BIAS = 0x8000000000000080ull;  // zero (sign bit flipped) 
 // (L - m) / 2 + 1 entries each
 __host__ __device__ inline int64_t ds_off(int L, int m) { return (lm_off(L, m) >> 1) + m; }
 int64_t ds_len(int L) { return (ds_off(L, L + 1) + 3) & ~(int64_t)1; }  // even: 16-byte alignment of what follows
+
+// largest |sum| of order s over `terms` products of the two operands' digits
+constexpr int64_t ds_order_sum(int s, int terms) {
+  int64_t n = 0;
+  for (int i = 0; i < DS_DIG; ++i)
+    if (s - i >= 0 && s - i < DS_DIG) n += (i == 0 ? 64 : 255) * (s - i == 0 ? 64 : 128);
+  return n * terms;
+}
 
 // ---- plan tables -------------------------------------------------------------
 // Double-double helpers (Knuth's TwoSum, Dekker's product by FMA).
@@ -578,6 +593,7 @@ __device__ __forceinline__ void ds_wait(DsShared& sh, int n, bool& ok) {
 constexpr int DSS_STAGE = DS_DIG * DS_PAIRS * 16 * 2;     // 28 KB
 constexpr int DSS_BSTEP = 16 * DS_ORD * 16 * 2;           // 16 columns x 8 digits (the last zero) x K 16
 constexpr int DSS_KB = 96;                                // k per block
+static_assert(ds_order_sum(5, DSS_KB) < (1 << 24) && ds_order_sum(7, DSS_KB) < (5 << 22), "see the bounds above");
 constexpr int DSS_SMEM = DSS_STAGE + (DSS_KB / 16) * DSS_BSTEP;
 constexpr int DSS_TMEM = 128;
 
@@ -775,11 +791,11 @@ __global__ void __launch_bounds__(DS_PAIRS, NR == 1 ? 4 : 3) ds_synth_kernel(DsA
 // pairs' phases G = (even combination, z times the odd one) x (Re, Im) of up
 // to NR right-hand sides are split into digits once: row (digit, column) of a
 // K-major operand, 8 columns per digit (64 rows), with zero rows around.  The
-// other operand holds 32 sequence values of the 128 pairs per stage, MN-major,
+// other operand holds 16 sequence values of the 128 pairs per stage, MN-major,
 // so a thread writes 8 consecutive values of its own pair.  A tensor-core
 // instruction takes at least 48 cycles here up to N = 64 and N / 2 beyond,
-// whatever M, so four digits of the sequence share one instruction (N = 128,
-// then 96 for the other three, read against G's digits shifted down by four):
+// whatever M, so four digits of the sequence share one instruction (N = 64,
+// then 48 for the other three, read against G's digits shifted down by four):
 // 16 per stage instead of 56, which the instruction rate would bind (30 ms
 // against 18 at Nside 2048 / lmax 3000).  Row s of the accumulator of digits
 // d and d + 4 is order s + d.  One partial row per (tile, right-hand side):
@@ -788,6 +804,9 @@ __global__ void __launch_bounds__(DS_PAIRS, NR == 1 ? 4 : 3) ds_synth_kernel(DsA
 // the equator.
 constexpr int DSA_N = 16;                                  // sequence values per stage
 constexpr int DSA_CB = 8;                                  // columns per digit of G
+// an accumulator takes digits d and d + 4 of the sequence against one digit each
+static_assert(2 * 255 * 128 * DS_PAIRS < (1 << 24) && ds_order_sum(4, DS_PAIRS) < (1 << 24) &&
+                  ds_order_sum(7, DS_PAIRS) < (3 << 23), "see the bounds above");
 constexpr int DSA_A = 12 * DSA_CB * DS_PAIRS * 2;          // G: 4 CB zero rows, the digits, CB zero rows
 constexpr int DSA_B = DS_DIG * DSA_N * DS_PAIRS * 2;       // a stage: digits 0..3, digits 4..6
 constexpr int DSA_FS = 24;                                 // row stride of the collected accumulators
@@ -1047,7 +1066,7 @@ int64_t ds_partial_bytes(int nis, int npairs, int L, int nr) {
 }
 
 // Below 64 ring pairs a CTA's 128 rows are more than half empty, and below 64
-// l a stage of 32 columns is mostly padding: the FP64 kernels of legendre.cu
+// l a stage of 16 columns is mostly padding: the FP64 kernels of legendre.cu
 // run there, where a launch and one warp's chain of a few dozen steps take the
 // time.  Just above the line (Nside 32, lmax 95: 64 pairs) the synthesis stage is
 // 19 us here and 55 us there.
