@@ -56,6 +56,18 @@ extern "C" {
 #define CR_EIO (-9)        /* checkpoint file could not be read or written */
 
 /* arithmetic of a call */
+/* FP64.  From 64 ring pairs and lmax 64 on, the sums over l (synthesis) and
+ * over rings (adjoint) are integer sums of fixed-point numbers with 54 bits
+ * below a bound: of P~_lm at a ring, its largest value over l; of the
+ * coefficients, the largest of 192 neighbouring l of one m; of the rings'
+ * F_m, the largest of F_m P~ among 128 ring pairs.  Whole transforms are
+ * nearer than with FP64 multiply-adds; but a part that is small beside the
+ * others under one bound (a coefficient 1e-8 of what a ring 1e10 times
+ * brighter than its neighbours gives the same m, a ring's F_m from a_lm that
+ * fall by orders within 192 l) keeps about 2^-54 of the large ones, not of
+ * itself.  Terms with |P~_lm| < 2^-60 before its first larger value are left
+ * out everywhere.  Values below 2^-987 count as zero, F_m above 2^1009 may
+ * overflow to NaN. */
 #define CR_F64 0
 #define CR_F32 1
 /* dtype of cr_sht_synth, cr_sht_adjoint and cr_apply_A (level 0): FP32 data

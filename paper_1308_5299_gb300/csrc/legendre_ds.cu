@@ -352,6 +352,26 @@ __device__ __forceinline__ void ds_ld16(uint32_t taddr, float f[16]) {
                : "memory");
 }
 
+// log2 of how far all |P~_lm(z)|, l <= L + 1, stay below their bound at the
+// turning point of l = L + 1, for rings nearer to the pole than it (else 0).
+// y = P~ sqrt(sin) obeys y'' = Q y, Q = (m^2 - 1/4) / sin^2 - (l + 1/2)^2, in theta,
+// and g = y' / y stays above sqrt(Q) from the pole to the turning point (g' = Q -
+// g^2 is 0 where they meet, and sqrt(Q) falls), so y is at most its value there
+// times exp of minus the integral of sqrt(Q): m log((m z + u) / (sin D)) - nu
+// log((nu z + u) / D) with u^2 = m^2 - nu^2 sin^2, D^2 = nu^2 - m^2, nu = l + 1/2.  Without it such a ring's digits
+// would end 2^-54 below a bound far above its values: those 1e-6 (1e-9) of the
+// largest ring's lost 5e-9 (1e-5) of themselves to it.  (Against the recurrence at
+// lmax 64 to 8000 the bound is 0.2 to 5 bits above the largest value; the margins
+// are FP32's rounding.)
+__device__ __forceinline__ float ds_decay(int L, int m, float z, float s2) {
+  const float nu = (float)L + 1.5f, mm = (float)m * (float)m - 0.25f;
+  const float u2 = mm - nu * nu * s2;
+  if (m == 0 || u2 <= 0.f) return 0.f;
+  const float mf = sqrtf(mm), u = sqrtf(u2), D = rsqrtf((nu - mf) * (nu + mf));
+  const float S = mf * log2f((mf * z + u) * D * rsqrtf(s2)) - nu * log2f((nu * z + u) * D);
+  return fminf(80.f, fmaxf(0.f, 0.999f * S - 0.07f - 3e-5f * nu));
+}
+
 // One ring pair's sequence.  The first few steps, where the functions can grow
 // by large factors, run in FP64 (mode 0); then in integers with an exponent
 // per pair (mode 1: (Q - 2^63) 2^-62 2^(eb - 1023 - x), x falling to zero as
@@ -380,15 +400,15 @@ struct DsPair {
     // bounds |P~_lm| <= sqrt((2 l + 1) / 4 pi) and 0.3 (l + 1)^(1/4) / sqrt(sin)
     // (the supremum over l, m and z is 0.29965 at every l tried to 3000),
     // over the rescaling at its smallest
-    const float fl = (float)(L + 1);
-    float b = fminf(0.2821f * sqrtf(2.f * fl), 0.305f * sqrtf(sqrtf(fl)) * rsqrtf(sqrtf(fmaxf((float)(1.0 - zz), 1e-20f))));
+    const float fl = (float)(L + 1), s2 = fmaxf((float)(1.0 - zz), 1e-20f);
+    float b = fminf(0.2821f * sqrtf(2.f * fl), 0.305f * sqrtf(sqrtf(fl)) * rsqrtf(sqrtf(s2)));
     if (EQ) {
       const int64_t c = lm_off(a.Lc, m) + (L - m);
       b /= fminf((float)fmin(a.s[c], L > m ? a.s[c - 1] : 1.0), 1.f);
     } else {
       b /= (float)z;
     }
-    eb = 1023 + (int)ceilf(log2f(b) + 0.1f);
+    eb = 1023 + (int)ceilf(log2f(b) + 0.1f - ds_decay(L, m, (float)z, s2));
     if (ls > L) return;
     const int64_t oc = lm_off(a.Lc, m) + (ls - m);
     const double c = ls > m ? a.c[oc] : 0.0;
