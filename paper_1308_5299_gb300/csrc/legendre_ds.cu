@@ -1085,12 +1085,13 @@ int64_t ds_partial_bytes(int nis, int npairs, int L, int nr) {
   return (int64_t)nr * ds_tiles(nis, npairs) * ds_len(L) * 4 * (int64_t)sizeof(double);
 }
 
-// Below 64 ring pairs a CTA's 128 rows are more than half empty, and below 64
-// l a stage of 16 columns is mostly padding: the FP64 kernels of legendre.cu
-// run there, where a launch and one warp's chain of a few dozen steps take the
-// time.  Just above the line (Nside 32, lmax 95: 64 pairs) the synthesis stage is
-// 19 us here and 55 us there.
-bool ds_use(const LegArgs<double>& a) { return a.ds && !a.df && a.npairs >= 64 && a.L >= 64; }
+// By the grid, not by the pairs that a mask leaves: A at Nside 32 / lmax 95 with
+// 55 of 64 pairs takes 64 us here and 147 us with the FP64 sums of legendre.cu, at
+// Nside 2048 / lmax 3000 with 1 and 63 pairs 624 and 690 us against 3.7 and 4.0 ms:
+// one warp's chain of FP64 steps, however few the pairs.  The smallest grids and
+// band limits stay with the plain FP64 sums (60 pairs, lmax 64: synthesis 33 us here,
+// 57 us there; 8 pairs: 33 and 56 us).
+bool ds_use(const LegArgs<double>& a) { return a.ds && !a.df && (a.nring + 1) / 2 >= 64 && a.L >= 64; }
 
 static DsArgs ds_args(const LegArgs<double>& la, int nr) {
   DsArgs a;
