@@ -893,10 +893,16 @@ def main():
     # Legendre autotuner: ring-block choice per grid, band limit, precision
     t3 = time.perf_counter()
     table = plan.autotune()
+
+    def choice(t):
+        if "pairs_per_thread" not in t:
+            return {"variant": t["variant"]}
+        if len(set(t["ms"].values()) | set(t["ms_m_tile2"].values())) == 1:
+            return {"form": "digit slices"}  # one form, no shapes
+        return {"pairs_per_thread": t["pairs_per_thread"], "m_tile": t["m_tile"]}
+
     autotune = {"s": time.perf_counter() - t3,
-                "observation_grid": {"%s_%s" % (t["precision"], t["stage"]):
-                                     ({"pairs_per_thread": t["pairs_per_thread"], "m_tile": t["m_tile"]}
-                                      if "pairs_per_thread" in t else {"variant": t["variant"]})
+                "observation_grid": {"%s_%s" % (t["precision"], t["stage"]): choice(t)
                                      for t in table if t["nring"] == 4 * nside - 1 and t["lmax"] == lmax},
                 "m_tile_2_chosen": sum(1 for t in table if t.get("m_tile") == 2),
                 "entries": len(table)}

@@ -249,7 +249,10 @@ int cr_plan_create(cr_plan** out, const cr_params* p);
  * every grid and band limit the plan transforms on, and keeps the fastest
  * shape.  Choices are cached for the process per (grid shape, band limit,
  * precision, stage) and used by every plan with those shapes; shapes already
- * in the cache are not re-timed.  Untuned shapes use 4 and 1.  *nentries (may be
+ * in the cache are not re-timed.  The FP64 stages from 64 ring pairs and lmax
+ * 64 on have one form: it is timed once, and its time stands under every
+ * choice.  Untuned FP64 shapes use 4 and 1, untuned FP32 ones 1 and the pairs
+ * per thread (2 or 4) that leave the GPU enough warps.  *nentries (may be
  * NULL) receives the size of the cache.  Synchronous; a few seconds at
  * Nside 2048.  The batched tensor-core synthesis (16 right-hand sides) is
  * tuned too: its stage shape (variant 0: K 32 per parity, 2 pipeline

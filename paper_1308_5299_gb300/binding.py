@@ -225,7 +225,8 @@ def tune_table():
     "synthesis"/"adjoint"): the chosen pairs per thread and m tile (1: one m
     per CTA, 2: m and L - m per CTA) and the measured ms of 2, 4, 8 (and,
     for the FP32 adjoint, 16) pairs per thread with m tile 1 (``ms``) and 2
-    (``ms_m_tile2``).  The batched tensor-core synthesis (precision "bf16",
+    (``ms_m_tile2``); an FP64 stage of one form has its time under every
+    choice.  The batched tensor-core synthesis (precision "bf16",
     stage "tc_synthesis"): the chosen stage-shape variant (0: K 32 per
     parity, 2 stages; 1: K 32, 3 stages; 2: K 16, 3 stages) and the measured
     ms of each."""

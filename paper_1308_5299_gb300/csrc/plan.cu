@@ -726,7 +726,10 @@ static const Grid* grid_of(cr_plan* P, int grid, int* L) {
 // pairs per thread (16 for the FP32 adjoint), each with one m per CTA and
 // with m paired with L - m (one untimed launch, then `reps` timed with CUDA
 // events on the plan's stream; native kernels, zero coefficients -- the work
-// does not depend on the data) and record the fastest shape.
+// does not depend on the data) and record the fastest shape.  The digit-slice
+// FP64 stages have no shapes: timed once, the time stands for every shape and
+// the first one is recorded (timing six shapes that nothing runs on took 4.5 s
+// of the 10.7 s of a plan at Nside 2048).
 template <typename T>
 static int tune_stage(cr_plan* P, const Grid& g, int L, int stage, int reps) {
   using C = typename Tr<T>::C;
@@ -742,13 +745,18 @@ static int tune_stage(cr_plan* P, const Grid& g, int L, int stage, int reps) {
   TuneVal v{4, 1, {-1.0, -1.0, -1.0, -1.0, -1.0, -1.0, -1.0, -1.0}};
   const int rps[4] = {2, 4, 8, 16};
   const int nchoice = rp_allowed(16, (int)sizeof(T), stage) ? 4 : 3;
+  LegArgs<T> a = leg_args<T>(P, g, L);
+  a.df = 0;
+  a.alm = alm;
+  bool one_form = false;
+  if constexpr (sizeof(T) == 8) one_form = ds_use(a);
   for (int ci = 0; ci < 8 && !rc; ++ci) {
     const int i = ci & 3, mt = 1 + (ci >> 2);
     if (i >= nchoice) continue;
-    LegArgs<T> a = leg_args<T>(P, g, L);
-    a.df = 0;
-    a.ds = nullptr;  // the shapes are those of the CUDA-core kernels
-    a.alm = alm;
+    if (one_form && ci > 0) {
+      v.ms[ci] = v.ms[0];
+      continue;
+    }
     a.rp_synth = a.rp_adj = rps[i];
     a.mt_synth = a.mt_adj = mt;
     FinalizeArgs<T> f;
@@ -764,7 +772,7 @@ static int tune_stage(cr_plan* P, const Grid& g, int L, int stage, int reps) {
     v.ms[ci] = ms / reps;
   }
   if (!rc) {
-    int best = 1;
+    int best = one_form ? 0 : 1;
     for (int ci = 0; ci < 8; ++ci)
       if (v.ms[ci] >= 0.0 && v.ms[ci] < v.ms[best]) best = ci;
     v.rp = rps[best & 3];

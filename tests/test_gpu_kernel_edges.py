@@ -224,3 +224,32 @@ def test_fp64_small_parts_beside_large_ones(dev, nside, lmax):
         plan.sht_adjoint(torch.from_numpy(y).to(dev), b)
         ref = sht.adjoint(y, lmax, g)
         check(b.cpu().numpy() - ref, ref, ms, 3e-10)
+
+
+@pytest.mark.parametrize("mt", [1, 2])
+@pytest.mark.parametrize("rp", [2, 4, 8])
+@pytest.mark.parametrize("grid,lmax", [(8, 23), (16, 47), (16, 64), ((125, 130), 63), ((300, 130), 48)])
+def test_fp64_shapes_below_the_digit_slices(dev, grid, lmax, rp, mt):
+    """Every ring-block shape of the plain FP64 kernels on the grids that run
+    on them: fewer than 64 ring pairs, or lmax below 64."""
+    g = geometry.healpix_grid(grid) if isinstance(grid, int) else geometry.gl_grid(*grid)
+    for stage in ("synthesis", "adjoint"):
+        binding.tune_set(g["nring"], g["npix"], lmax, "f64", stage, rp, m_tile=mt)
+    for e in transforms(dev, grid, lmax, torch.float64):
+        assert e < TOL[torch.float64]
+
+
+def test_autotuner_times_what_runs(dev):
+    """FP64 stages on digit slices have one form: one time under every choice;
+    smaller grids time every choice."""
+    for nside, lmax, forms in ((32, 70, 1), (16, 50, 6)):
+        plan = binding.Plan(lmax, nside=nside)
+        rows = [t for t in plan.autotune() if (t["nring"], t["lmax"], t["precision"]) == (4 * nside - 1, lmax, "f64")]
+        assert len(rows) == 2
+        for t in rows:
+            ms = list(t["ms"].values()) + list(t["ms_m_tile2"].values())
+            assert len(ms) == 6 and all(v > 0 for v in ms)
+            if forms == 1:
+                assert len(set(ms)) == 1
+            else:
+                assert len(set(ms)) > 1
