@@ -46,6 +46,7 @@ namespace cr {
 constexpr double LF_ZPOLAR = 0.8, LF_ZEQ = 0.15;
 constexpr int LF_CH = 128;       // k per staged chunk
 constexpr int LF_FUSED = 8;      // most warps of one m whose sums one CTA collects
+constexpr int LF_FUSED_SMEM = 64 * 1024;  // and its shared memory: three CTAs per SM
 
 void lf_zones(const double* z, int npairs, int* n1, int* n2) {
   int i = 0;
@@ -571,9 +572,10 @@ static int lf_adjoint_launch(const LegArgs<float>& a, const FinalizeArgs<float>&
   const int nb = lf_nblocks(a, RP);
   const size_t smem = nb * (sizeof(LfAdjStage) + (size_t)(a.L / 2 + 1) * sizeof(float4));
   if constexpr (RP <= 4) {
-    // few pairs: one CTA per m (up to LF_FUSED warps, 64 KB: three CTAs per SM)
-    if (a.mt_adj == 1 && nb <= LF_FUSED && smem <= 64 * 1024) {
-      CR_CUDA(cudaFuncSetAttribute(lf_adjoint_fused_kernel<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // few pairs: one CTA per m.  The kernel's limit is the most it may take, not
+    // this launch's size, which another thread's launch could exceed.
+    if (a.mt_adj == 1 && nb <= LF_FUSED && smem <= LF_FUSED_SMEM) {
+      CR_CUDA(cudaFuncSetAttribute(lf_adjoint_fused_kernel<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, LF_FUSED_SMEM));
       { lf_adjoint_fused_kernel<RP><<<a.L + 1, 32 * nb, smem, st>>>(a, f); count_launch(); }
       CR_CHECK_LAUNCH("lf_adjoint_fused_kernel");
       return CR_OK;

@@ -39,6 +39,10 @@
 namespace cr {
 
 constexpr int RF_NT = 256;
+// The most shared memory of a CTA.  The kernels' limit is set to it whatever a
+// launch takes: it is one per kernel and process, so a limit of a launch's own
+// size could fall below that of another thread's launch.
+constexpr int RF_SMEM = 227 * 1024;
 
 // Shared-memory position of FFT buffer element i: bits 4..15 XOR-folded into
 // bits 0..3 (a bijection on [0, 2^16)).  With 8-byte elements a bank pair
@@ -430,15 +434,15 @@ template <typename T, bool BIG>
 static int ring_fft_launch(const RingArgs<T>& b, int mode, int cnt, int nt, size_t smem, cudaStream_t st) {
   switch (mode) {
     case 0:
-      CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 0, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 0, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
       { ring_fft_kernel<T, 0, BIG><<<dim3(cnt, b.nrhs), nt, smem, st>>>(b); count_launch(); }
       break;
     case 1:
-      CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 1, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 1, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
       { ring_fft_kernel<T, 1, BIG><<<dim3(cnt, b.nrhs), nt, smem, st>>>(b); count_launch(); }
       break;
     default:
-      CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 2, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      CR_CUDA(cudaFuncSetAttribute(ring_fft_kernel<T, 2, BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
       { ring_fft_kernel<T, 2, BIG><<<dim3(cnt, b.nrhs), nt, smem, st>>>(b); count_launch(); }
       break;
   }
@@ -455,7 +459,7 @@ int launch_ring_fft(const RingArgs<T>& a, int mode, cudaStream_t st) {
     const int cnt = a.cls_start[c + 1] - a.cls_start[c];
     if (cnt <= 0) continue;
     size_t smem = (size_t)M * sizeof(C);
-    if (smem > 227 * 1024 || M > 65536) return fail(CR_EINVAL, "ring FFT buffer exceeds shared memory");
+    if (smem > RF_SMEM || M > 65536) return fail(CR_EINVAL, "ring FFT buffer exceeds shared memory");
     // at least 128 threads: small rings split their folds over the idle lanes
     const int nt = std::max(128, std::min(RF_NT, M / 8));
     RingArgs<T> b = a;
@@ -465,7 +469,7 @@ int launch_ring_fft(const RingArgs<T>& a, int mode, cudaStream_t st) {
     // 512, lmax 1023 78.9 | 77.6 us, and staging the larger classes as well loses
     // what the first gains (Nside 2048: 922 us; fewer CTAs per SM).
     const size_t rows = ((size_t)a.L + 16) / 16 * 16 * sizeof(C);
-    b.stage = c == 0 && 2 * a.L > 3 * M && smem + rows <= 227 * 1024 ? M : 0;
+    b.stage = c == 0 && 2 * a.L > 3 * M && smem + rows <= RF_SMEM ? M : 0;
     if (b.stage) smem += rows;
     b.rbase = a.cls_start[c];
     // FP32 rings with M >= 4096: the 4-stage passes with computed twiddles
@@ -576,7 +580,7 @@ int build_fft_tables(Grid& g, cudaStream_t st) {
     f.tab = d.tab;
     f.vhat = d.vhat;
   }
-  if ((size_t)Mmax * sizeof(double2) > 227 * 1024) return fail(CR_EINVAL, "ring too long for the shared-memory FFT");
+  if ((size_t)Mmax * sizeof(double2) > RF_SMEM) return fail(CR_EINVAL, "ring too long for the shared-memory FFT");
   g.Mmax = Mmax;
   g.tab_len = tab_len;
   g.vhat_len = vhat_len;
@@ -595,7 +599,7 @@ int build_fft_tables(Grid& g, cudaStream_t st) {
   CR_CHECK_LAUNCH("tw_kernel");
   if (vhat_len > 0) {
     const size_t smem = (size_t)Mmax * sizeof(double2);
-    CR_CUDA(cudaFuncSetAttribute(vhat_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CR_CUDA(cudaFuncSetAttribute(vhat_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_SMEM));
     vhat_kernel<<<(int)lens.size(), 256, smem, st>>>(d_lens, g.d_tab, g.d_tw, Mmax, g.d_vhat);
     CR_CHECK_LAUNCH("vhat_kernel");
   }

@@ -253,3 +253,36 @@ def test_autotuner_times_what_runs(dev):
                 assert len(set(ms)) == 1
             else:
                 assert len(set(ms)) > 1
+
+
+def test_two_threads_with_plans_of_different_sizes(dev):
+    """Two host threads, a plan and a stream each: launches that take much and
+    little shared memory of the same kernels at the same time."""
+    import threading
+
+    def work(gl, lmax, dtype, errors):
+        try:
+            s = torch.cuda.Stream()
+            plan = binding.Plan(lmax, gl=gl, stream=s)
+            cdtype = torch.complex128 if dtype == torch.float64 else torch.complex64
+            a = torch.from_numpy(synthetic.random_alm(lmax, seed=3)).to(dev).to(cdtype)
+            m = torch.from_numpy(synthetic.random_map(gl[0] * gl[1], seed=4)).to(dev).to(dtype)
+            b, o = torch.empty_like(a), torch.empty_like(m)
+            torch.cuda.synchronize()
+            for _ in range(2000):
+                plan.sht_synth(a, o)
+                plan.sht_adjoint(m, b)
+            s.synchronize()
+        except Exception as e:
+            errors.append(e)
+
+    # ring FFTs of 64 and 16 KB in FP64; fused adjoints of 51 and 20 KB in FP32
+    for dtype, big, small in ((torch.float64, ((33, 3000), 40), ((33, 82), 40)),
+                              (torch.float32, ((255, 1802), 900), ((33, 82), 40))):
+        errors = []
+        t = [threading.Thread(target=work, args=(gl, lmax, dtype, errors)) for gl, lmax in (big, small)]
+        for x in t:
+            x.start()
+        for x in t:
+            x.join()
+        assert not errors, errors
