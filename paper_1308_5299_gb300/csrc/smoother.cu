@@ -1632,15 +1632,25 @@ static int sweep_mr(cr_plan* P, PixLevel& lev, int nr, const T* map_in, T* map_o
 }
 // The explicit inverse of a level with few tiles from its present factor
 // (once per factor, at the end of the precompute); only where the form of the
-// sweeps was left to the library.
+// sweeps was left to the library.  Where the memory for a first inverse cannot
+// be had the level keeps the sweeps; an inverse that exists, which a captured
+// graph may apply, is rebuilt or the call fails.
 int build_dense_inverse(cr_plan* P, PixLevel& lev) {
   const Hierarchy& H = *P->hier;
   lev.inv_valid = false;
   if (H.smoother_kind != 0 || H.sweep_mode != 0 || lev.pat.ntile > DI_TILES) return CR_OK;
   const int n = lev.pat.ntile * TK;
-  if (!lev.d_inv) CR_CUDA(cudaMalloc(&lev.d_inv, (size_t)n * n * sizeof(float)));
   float* tmp = nullptr;
-  CR_CUDA(cudaMalloc(&tmp, (size_t)2 * SM_NR * n * sizeof(float)));
+  const bool first = !lev.d_inv;
+  cudaError_t e = first ? cudaMalloc(&lev.d_inv, (size_t)n * n * sizeof(float)) : cudaSuccess;
+  if (e == cudaSuccess) e = cudaMalloc(&tmp, (size_t)2 * SM_NR * n * sizeof(float));
+  if (first && e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();  // handled
+    if (lev.d_inv) cudaFree(lev.d_inv);
+    lev.d_inv = nullptr;
+    return CR_OK;
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "dense inverse");
   int rc = CR_OK;
   for (int j0 = 0; j0 < n && !rc; j0 += SM_NR) {
     unit_panel_kernel<<<152, 256, 0, P->stream>>>(tmp, n, j0);
@@ -1650,7 +1660,7 @@ int build_dense_inverse(cr_plan* P, PixLevel& lev) {
   if (!rc) {
     average_transpose_kernel<<<dim3((n + 31) / 32, (n + 7) / 8), dim3(32, 8), 0, P->stream>>>(lev.d_inv, n);
     count_launch();
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "dense inverse");
   }
