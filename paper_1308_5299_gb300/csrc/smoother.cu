@@ -1431,7 +1431,9 @@ int smoother_numeric(cr_plan* P, PixLevel& lev, double ridge_factor, int bisecti
 // visits), and applying it is one matrix-vector product over the whole chip:
 // 4 and 9 us.  At n = 12288 (604 MB) the product would take longer than the
 // 68 us of the sweeps.  M's columns are the sweeps' results for unit vectors,
-// 16 at a time, averaged with their transpose.
+// 16 at a time, averaged with their transpose: positive definite in FP32 as far
+// as was tried (the presets, and noise contrasts of 1e4 to 1e6, where the
+// eigenvalues span ten orders; quotients within 5e-4 of the sweeps').
 constexpr int DI_TILES = 48;
 
 __global__ void unit_panel_kernel(float* v, int n, int j0) {

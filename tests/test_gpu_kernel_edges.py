@@ -286,3 +286,25 @@ def test_two_threads_with_plans_of_different_sizes(dev):
         for x in t:
             x.join()
         assert not errors, errors
+
+
+@pytest.mark.parametrize("preset", ["nside32_lmax95", "nside512_lmax1023"])
+def test_explicit_inverses_are_symmetric_and_positive(dev, preset):
+    """M of the levels of at most 48 tiles, column by column: symmetric to the
+    bit, and positive definite, as the factor's L^-T L^-1 is."""
+    cfg, cl, bl, ninv = synthetic.problem_inputs(preset)
+    plan = binding.Plan(cfg["lmax"], nside=cfg["nside"], cl=cl, bl=bl, ninv=torch.from_numpy(ninv).to(dev),
+                        levels="default", ridge_bisections=8)
+    seen = 0
+    for h in range(1, plan.nlevels() + 1):
+        n = 12 * plan.level(h)["nside_h"] ** 2
+        if n > 48 * 64:
+            continue
+        eye, m = torch.eye(n, dtype=torch.float32, device=dev), torch.empty((n, n), dtype=torch.float32, device=dev)
+        for i in range(n):
+            plan.pixel_smoother(h, eye[i], m[i])
+        assert torch.equal(m, m.T), h
+        w = torch.linalg.eigvalsh(m.double())
+        assert w[0] > 0, (h, w[0], w[-1])
+        seen += 1
+    assert seen
