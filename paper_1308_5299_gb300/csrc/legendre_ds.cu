@@ -925,7 +925,8 @@ __device__ __forceinline__ void ds_adjoint_body(const DsArgs& a, DsShared& sh, u
           }
         }
         tc::fence_before_sync();
-        __syncthreads();
+        // the sums below are of all warps' loads: one wait that gave up marks them all
+        ok = __syncthreads_and(ok ? 1 : 0) != 0;
         const int w = tid & 3, kk = tid >> 2, k = kbeg + it * DSA_N + kk;
         if (kk >= DSA_N) continue;
         float c[DS_ORD];
