@@ -170,7 +170,7 @@ int launch_ds_adjoint(const LegArgs<double>& la, const double2* phase, int nr, d
 // FP32 stages (legendre_f32.cu)
 int64_t ds_len(int L);
 void lf_zones(const double* z, int npairs, int* n1, int* n2);
-void lf_args(const double* z, int npairs, int n1, int n2, float4* out);
+void lf_args(const double* z, int npairs, int n1, float4* out);
 int64_t lf_partial_bytes(int npairs, int L);
 int launch_lf_synth(const LegArgs<float>& a, cudaStream_t st);
 int launch_lf_adjoint(const LegArgs<float>& a, const FinalizeArgs<float>& f, cudaStream_t st);

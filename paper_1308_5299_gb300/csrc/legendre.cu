@@ -534,13 +534,15 @@ int launch_leg_diag(cr_plan* P, const double* ringval, double2* out) {
 // The start state (value before k0, second value) of one pair of the FP32
 // sequences (legendre_f32.cu), from the FP64 state (Q_{l-1}, Q_{l-2}) and Q_l at
 // its start l: such that the zone's step returns q_{k0}, k0 = (l - m) / 2 (the
-// one-step zone: Q_{m + 2 k0}, one step back where l is the second of its two).
+// one-step zone: (z Q, Q) before Q_{m + 2 k0}, one step back where l is the second
+// of its two).
 __device__ float2 lf_start(const DsTab& t, const double* c, const double* s, int Lc, int m, int l, double z, int zone,
                            double Q, double Q1, double Q2) {
   const int k0 = (l - m) >> 1;
   const int64_t oc = lm_off(Lc, m) + (l - m), ok = ((lm_off(t.Lc, m) >> 1) + m) + k0;
   const bool odd = (l - m) & 1;
-  if (zone == 2) return odd ? make_float2((float)Q2, (float)(c[oc - 1] * z * Q2 - Q1)) : make_float2((float)Q1, (float)Q2);
+  if (zone == 2)
+    return odd ? make_float2((float)(z * Q2), (float)(c[oc - 1] * z * Q2 - Q1)) : make_float2((float)(z * Q1), (float)Q2);
   const double P = s[oc] * Q;
   double q1 = 0.0;
   if (k0 > 0) q1 = (odd ? s[oc - 2] * Q2 : s[oc - 1] * Q1) / (z * t.sg[ok - 1]);

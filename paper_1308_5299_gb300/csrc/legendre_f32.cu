@@ -12,7 +12,9 @@
 //    (q varies slowly in k there; e - 2 is carried at full relative precision);
 //  - middle: q_{k+1} = (A z^2 + B) q_k - q_{k-1};
 //  - equatorial, z < LF_ZEQ: the one-step recurrence, P~_l = s_l q_l, q_l = c_l z
-//    q_{l-1} - q_{l-2}.  p_k grows like min(L, 1 / z) there while P~ does not, so
+//    q_{l-1} - q_{l-2}, with w = z q at odd l - m (q_l = c_l w_{l-1} - q_{l-2}, w_l =
+//    c_l z^2 q_{l-1} - w_{l-2}: one product less; the odd sums are divided by z).
+//    p_k grows like min(L, 1 / z) there while P~ does not, so
 //    that the two-step form's even sums cancel by that factor (the ring on the
 //    equator would be off by 5e-6, 1.4e-5, 4e-5 at lmax 384, 1023, 3000).
 // The argument of each has four copies that differ in the last place and
@@ -56,16 +58,16 @@ void lf_zones(const double* z, int npairs, int* n1, int* n2) {
   *n2 = i;
 }
 
-// arguments of a pair's steps: four copies of 1 - z^2 (polar), z^2 (middle) or z
-void lf_args(const double* z, int npairs, int n1, int n2, float4* out) {
+// arguments of a pair's steps: four copies of 1 - z^2 (polar) or z^2
+void lf_args(const double* z, int npairs, int n1, float4* out) {
   for (int p = 0; p < npairs; ++p) {
     // the exact value as x + xl
-    double x = z[p], xl = 0.0;
+    double x, xl;
     if (p < n1) {
       const double w = 1.0 - z[p], u = 2.0 * w;  // exact
       x = std::fma(-w, w, u);
       xl = std::fma(-w, w, u - x);
-    } else if (p < n2) {
+    } else {
       x = z[p] * z[p];
       xl = std::fma(z[p], z[p], -x);
     }
@@ -120,12 +122,12 @@ struct LfPairs {
     kmax = __reduce_max_sync(0xffffffffu, hi);
   }
   // the next value of pair j, for the even and the odd sums (ZONE 2: the next
-  // two), and the state behind it if `on`; u: its k modulo 4
+  // q and w), and the state behind it if `on`; u: its k modulo 4
   __device__ __forceinline__ float2 next(float2 r, int j, int u, bool on) {
     const float z = Z[j][u & 3];
     float qe, qo, second;
     if (ZONE == 2) {
-      qe = fmaf(r.x * z, q1[j], -q2[j]);
+      qe = fmaf(r.x, q1[j], -q2[j]);
       qo = fmaf(r.y * z, qe, -q1[j]);
       second = qe;
     } else if (ZONE == 1) {
@@ -154,6 +156,10 @@ __device__ __forceinline__ float2 lf_step(const LegArgs<float>& a, int m, int k)
   const float4 t = a.rf[(lm_off(a.Lc, m) >> 1) + m + k];
   return ZONE == 0 ? make_float2(-t.x, t.y) : make_float2(t.x, t.z);
 }
+
+// factor of the odd sums (on the equator they are zero)
+template <int ZONE>
+__device__ __forceinline__ float lf_odd(float z) { return ZONE < 2 ? z : z > 0.f ? 1.f / z : 0.f; }
 
 struct LfStage {
   float2 r[LF_CH];
@@ -250,7 +256,7 @@ __device__ __forceinline__ void lf_synth(const LegArgs<float>& a, LfStage& sh, i
   for (int j = 0; j < RP; ++j)
     if (s.p[j] < pend) {
       const int rn = s.p[j], rs = a.nring - 1 - rn;
-      const float z = ZONE == 2 ? 1.f : a.z[rn];
+      const float z = lf_odd<ZONE>(a.z[rn]);
       a.phase[(int64_t)rn * a.ldp + m] = make_float2(fmaf(z, dx[j], cx[j]), fmaf(z, dy[j], cy[j]));
       if (rs != rn) a.phase[(int64_t)rs * a.ldp + m] = make_float2(fmaf(-z, dx[j], cx[j]), fmaf(-z, dy[j], cy[j]));
     }
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(32) lf_synth_kernel(LegArgs<float> a) {
 // ---- adjoint -----------------------------------------------------------------
 // u_k = sum_pairs q_k (G_m(z) + G_m(-z)), v_k = sum_pairs q_k z (G_m(z) - G_m(-z));
 // a_o = sigma_k v_k, a_{o-1} += sigma_k e_o u_k, a_{o+1} += sigma_k e_{o+1} u_k.
-// ZONE 2: the sums of q_l themselves, l = m + 2k and m + 2k + 1; a_l = s_l times it.
+// ZONE 2: the sums of q_l (w_l / z) themselves, l = m + 2k and m + 2k + 1; a_l = s_l times it.
 // The four real sums of a k over a thread's RP pairs go to a shared-memory
 // row; per 8 k, lane (k, part) adds every fourth lane's entry and two exchange
 // steps leave one of the four sums per lane, 128 contiguous bytes of the
@@ -320,7 +326,7 @@ __device__ __forceinline__ void lf_adjoint(const LegArgs<float>& a, LfAdjStage& 
     ge[j] = go[j] = make_float2(0.f, 0.f);
     if (s.k0[j] < nk) {
       const int rn = s.p[j], rs = a.nring - 1 - rn;
-      const float z = ZONE == 2 ? 1.f : a.z[rn];
+      const float z = lf_odd<ZONE>(a.z[rn]);
       const float2 gn = a.phase[(int64_t)rn * a.ldp + m];
       const float2 gs = rs != rn ? a.phase[(int64_t)rs * a.ldp + m] : make_float2(0.f, 0.f);
       ge[j] = cadd(gn, gs);

@@ -215,7 +215,7 @@ int grid_upload(Grid& g, int Lseed, cudaStream_t st) {
   g.nis = ds_first_equatorial(g.z.data(), g.npairs);
   lf_zones(g.z.data(), g.npairs, &g.n1, &g.n2);
   std::vector<float4> zi(g.npairs);
-  lf_args(g.z.data(), g.npairs, g.n1, g.n2, zi.data());
+  lf_args(g.z.data(), g.npairs, g.n1, zi.data());
   CR_CUDA(cudaMalloc(&g.d_zi, g.npairs * sizeof(float4)));
   CR_CUDA(cudaMemcpyAsync(g.d_zi, zi.data(), g.npairs * sizeof(float4), cudaMemcpyHostToDevice, st));
   int rc = build_fft_tables(g, st);
