@@ -195,8 +195,10 @@ typedef struct cr_params {
   /* fp64_df: 1 = evaluate the FP64 Legendre stages (FP64 transforms, FP64
    * A, the outer residual of CR_MIXED) in double-float arithmetic on the
    * FP32 pipes -- pairs of floats with error-free sums and products, about
-   * 2^-44 relative per operation -- which GB300 runs several times faster
-   * than native FP64; 0 = native FP64. */
+   * 2^-44 relative per operation; 0 = the FP64 stages described at CR_F64,
+   * which are both faster (FP64 A at Nside 2048, lmax 3000: 39 ms against
+   * 69 ms with the option) and nearer.  The option has its own use where
+   * every part has to keep a relative precision of its own. */
   int fp64_df;
   /* defer_precompute: 1 = build the level structure (grids, tile patterns,
    * the observation-dependent inverse-noise terms) but not the
@@ -216,11 +218,14 @@ typedef struct cr_params {
    * ridge_factor) and raised under ridge_lambda_target. */
   int smoother;
   /* triangular sweeps of the ICC(0) smoother: 0 = automatic (levels of at
-   * most 1024 tiles, Nside_h <= 64, run both sweeps of one application in
-   * one cooperative persistent launch, larger levels one launch per
-   * colour); 1 = one launch
-   * per colour on every level; 2 = the cooperative launch wherever the
-   * device supports it.  The same operator either way. */
+   * most 48 tiles, Nside_h <= 16, multiply a map by the explicit inverse,
+   * formed with the factor where its memory -- 38 MB at 48 tiles -- is to be
+   * had; other levels of at most 1024 tiles, Nside_h <= 64, run both sweeps
+   * of one application in one cooperative persistent launch; larger levels
+   * one launch per colour); 1 = one launch per colour on every level; 2 =
+   * the cooperative launch wherever the device supports it.  Batches of maps
+   * take the sweeps in every mode.  The two forms of the sweeps give the
+   * same numbers; the inverse is the same operator up to FP32 rounding. */
   int smoother_sweep;
   /* tensor-core contractions of batched right-hand sides (CR_TC, and the
    * cycles of CR_TC_CYCLES): 0 = BF16 operands (about 2^-9 relative per

@@ -1,8 +1,10 @@
 // FP64 Legendre stages evaluated in double-float arithmetic on the FP32 pipes.
 //
 // GB300 executes FP64 FMAs at 1/64 of the FP32 rate, so the FP64 synthesis
-// and adjoint (used by the outer residual of the mixed-precision solve) can
-// instead carry every value as an unevaluated sum hi + lo of two floats.
+// and adjoint can instead carry every value as an unevaluated sum hi + lo of
+// two floats (a plan option: against FP64 sums it is 2.4 times faster, against
+// the digit slices of legendre_ds.cu, the default, 1.8 times slower: A at Nside
+// 2048 / lmax 3000 69 and 39 ms).
 // Sums use Knuth's error-free TwoSum, products Dekker's exact product through
 // a fused multiply-add, so each operation is accurate to about 2^-44 relative
 // (Dekker 1971; Knuth, TAOCP vol. 2, 4.2.2).  Inputs and outputs stay FP64
