@@ -33,11 +33,11 @@
 // stages the chunk's coefficients itself; a group of 8 k runs unchecked once
 // all of the warp's pairs have started (start tables, |P~| >= 2^-60).  Bound by
 // FP32 issue: 6.5 operations per pair and k beside two shared loads per k and
-// warp (ncu at Nside 1024 / lmax 2047: synthesis 2.9, adjoint 2.75 instructions a
+// warp (ncu at Nside 1024 / lmax 2047: synthesis 2.8, adjoint 2.65 instructions a
 // cycle, the adjoint's transpose near the shared-memory rate as well).  At Nside
 // 2048 / lmax 3000, in A, against the one-step kernels with two ring pairs packed
 // into an instruction and a launch each for polar and other pairs: synthesis
-// 2.4 -> 1.54 ms, adjoint 3.3 -> 2.05 ms.
+// 2.4 -> 1.52 ms, adjoint 3.3 -> 2.06 ms; alone, with every ring, 1.92 and 2.58 ms.
 #include <cmath>
 
 #include "common.cuh"
@@ -414,8 +414,12 @@ __device__ __forceinline__ void lf_adjoint_eq(const LegArgs<float>& a, LfAdjStag
   else lf_adjoint<2, RP>(a, sh, m, base, a.npairs, row);
 }
 
+// Warps per SM that the registers leave room for.  32, all that an SM takes of
+// CTAs this small, cost 8 registers at RP = 4 (72 without the bound): adjoint at
+// Nside 2048 / lmax 3000 2610 -> 2577 us, 1024 / 2047 677 -> 661, 512 / 1023 134 -> 132
+// (in A there, with a mask, 108 -> 111).
 template <int RP, int MT>
-__global__ void __launch_bounds__(32) lf_adjoint_kernel(LegArgs<float> a, float* partial, int64_t nkk) {
+__global__ void __launch_bounds__(32, RP <= 2 ? 32 : RP == 4 ? (MT == 1 ? 32 : 24) : RP == 8 ? 16 : 8) lf_adjoint_kernel(LegArgs<float> a, float* partial, int64_t nkk) {
   __shared__ LfAdjStage sh;
   const int b0 = lf_blocks<RP>(a.n1), b1 = lf_blocks<RP>(a.n2 - a.n1);
   const int b = blockIdx.x;
@@ -474,27 +478,30 @@ __global__ void __launch_bounds__(128) lf_finalize_kernel(LegArgs<float> a, Fina
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if ((int)(blockIdx.x * blockDim.x) >= nk) return;  // whole CTA
   const float4* row = partial + ((lm_off(a.L, m) >> 1) + m);
-  auto sum = [&](int kk, int b0, int b1) {
-    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+  // two-step rows to t, one-step rows to q, all loads in one loop
+  auto sum = [&](int kk, float4& t, float4& q) {
+    t = q = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-    for (int b = b0; b < b1; ++b) {
+    for (int b = 0; b < nblk; ++b) {
       const float4 w = row[b * nkk + kk];
-      t = make_float4(t.x + w.x, t.y + w.y, t.z + w.z, t.w + w.w);
+      const bool two = b < n2s;
+      t = make_float4(t.x + (two ? w.x : 0.f), t.y + (two ? w.y : 0.f), t.z + (two ? w.z : 0.f), t.w + (two ? w.w : 0.f));
+      q = make_float4(q.x + (two ? 0.f : w.x), q.y + (two ? 0.f : w.y), q.z + (two ? 0.f : w.z), q.w + (two ? 0.f : w.w));
     }
-    return t;
   };
-  float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (k < nk) t = sum(k, 0, n2s);
+  float4 t = make_float4(0.f, 0.f, 0.f, 0.f), q = t;
+  if (k < nk) sum(k, t, q);
   float2 um = make_float2(__shfl_up_sync(0xffffffffu, t.x, 1), __shfl_up_sync(0xffffffffu, t.y, 1));
   if (k >= nk) return;
   if ((threadIdx.x & 31) == 0) {
     um = make_float2(0.f, 0.f);
     if (k > 0) {
-      const float4 w = sum(k - 1, 0, n2s);
+      float4 w, wq;
+      sum(k - 1, w, wq);
       um = make_float2(w.x, w.y);
     }
   }
-  lf_emit(a, f, m, k, t, um, sum(k, n2s, nblk));
+  lf_emit(a, f, m, k, t, um, q);
 }
 
 // All warps of one m in one CTA (grids of few pairs): the rows stay in shared
