@@ -258,7 +258,7 @@ int cr_plan_create(cr_plan** out, const cr_params* p);
  * 64 on have one form: it is timed once, and its time stands under every
  * choice.  Untuned FP64 shapes use 4 and 1, untuned FP32 ones 1 and the pairs
  * per thread (2 or 4) that leave the GPU enough warps.  *nentries (may be
- * NULL) receives the size of the cache.  Synchronous; a few seconds at
+ * NULL) receives the size of the cache.  Synchronous; about a second at
  * Nside 2048.  The batched tensor-core synthesis (16 right-hand sides) is
  * tuned too: its stage shape (variant 0: K 32 per parity, 2 pipeline
  * stages; 1: K 32, 3 stages; 2: K 16, 3 stages), cached with precision 2

@@ -50,12 +50,12 @@
 // adjoint 4.7e-15 instead of 1.8e-14).
 //
 // What bounds it: instruction issue, at half of its rate (ncu at Nside 512 /
-// lmax 1023: 2.0 instructions a cycle, FP64 pipe 33 %, tensor pipe 16 %, 24 % of
+// lmax 1023: 1.8 instructions a cycle, FP64 pipe 31 %, tensor pipe 17 %, 24 % of
 // the warp slots); the rest are waits for the coefficients, the block barrier
 // of a stage and the products.  About 42 instructions take a warp two l
 // further.  At Nside 2048 / lmax 3000 the synthesis stage went from 89.1 ms
-// (FP64 sums, one-step recurrence) to 17.4 ms and the adjoint from 99.9 to 21.7
-// ms; where rings carry no weight in A, to 13.0 and 16.1 ms.
+// (FP64 sums, one-step recurrence) to 17.5 ms and the adjoint from 99.9 to 21.7
+// ms; where rings carry no weight in A, to 13.0 and 16.2 ms.
 #include <cuda_fp16.h>
 
 #include <cmath>
